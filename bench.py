@@ -4,7 +4,7 @@
 Workload (default): the Taylor-Green vortex (Re 1600, Mach 0.1, Pr 0.71) on
 32^3 elements at P = 3, 16^3 at P = 6 and 16^3 at P = 8, FP32 operator with FP64
 state and FP64 RK3 accumulation.  One step = one RK3 time step (three stages, each a
-BR1-gradient launch and a flux/lift/RK-update launch) on each of the three meshes.
+gradient-and-volume launch and an interface/RK-update launch) on each of the three meshes.
 A DOF is a node carrying five variables (dof = N_el (P+1)^3); one DOF-stage update is
 one node advanced through one RK stage.
 
@@ -608,11 +608,11 @@ def run_ours(args, rank, ws):
     kernels = []
     for p in prof:
         for kind in ("flux", "gradient"):
-            kernels.append({"kernel": "k_flux" if kind == "flux" else "k_gradient", "workload": p["workload"],
+            kernels.append({"kernel": "k_surface" if kind == "flux" else "k_volume", "workload": p["workload"],
                             "ms": p[f"ms_{kind}"], "launches": p[f"launches_{kind}"],
                             "bytes_per_launch": p[f"{kind}_bytes_per_launch"],
                             "share": p[f"ms_{kind}"] / total_ms,
-                            "traffic_per_launch": measured_traffic("k_flux" if kind == "flux" else "k_gradient",
+                            "traffic_per_launch": measured_traffic("k_surface" if kind == "flux" else "k_volume",
                                                                    p["workload"])})
     dom = max(kernels, key=lambda k: k["ms"])
     dom_achieved = dom["bytes_per_launch"] / (dom["ms"] / dom["launches"] / 1e3) / 1e9
@@ -624,14 +624,14 @@ def run_ours(args, rank, ws):
     traffics = [k["traffic_per_launch"] for k in kernels]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": peak_kind, "bytes_per_dof_stage": FLOOR_BYTES,
-                "kernel": "one RK stage of the three meshes (k_gradient + k_flux per mesh)",
+                "kernel": "one RK stage of the three meshes (k_volume + k_surface per mesh)",
                 "bytes_per_launch": unit_bytes,
                 "traffic": sum(traffics) if all(t is not None for t in traffics) else None,
                 "per_mesh": {m: round(v["frac"], 4) for m, v in per_mesh.items()},
                 "note": "algorithmic floor 160 B per DOF-stage (q read, RK register read + write, q write, "
                         "FP64); traffic = ncu DRAM bytes of the six launches of one stage, null unless taken "
                         "on the current kernel sources"}
-    # the implementation's own bytes (stage state, stored stresses, FP32 increments: each
+    # the implementation's own bytes (stage states, volume terms, face fluxes, FP32 increments: each
     # value read or written once) over the whole timed step and for the dominant kernel
     step_bytes = sum(3 * (p["flux_bytes_per_launch"] + p["gradient_bytes_per_launch"]) for p in prof)
     step_gbs = step_bytes / (ms / args.steps / 1e3) / 1e9
@@ -741,8 +741,12 @@ def run_ours(args, rank, ws):
 
 # ----------------------------------------------------------------------------- batched instances
 
-# FP32-operator algorithmic bytes per node of one RK3 step (both launches of all stages)
-STEP_BYTES_PER_NODE = 676.0
+def step_bytes_per_node(P):
+    """FP32-operator algorithmic bytes per node of one RK3 step (both launches of all
+    stages): 500 of node values and 96 / (P + 1) of face fluxes six times."""
+    return 500.0 + 576.0 / (P + 1)
+
+
 BATCH_NAME = ("12 independent TGV instances, (K, P, Re) drawn with seed 12 from {8,12,16} x {3,6} x "
               "{30,200,1600}, Mach 0.1, one batch, graph replay")
 
@@ -831,7 +835,8 @@ def batched_measure(args, rank, ws, steps, with_clocks=False):
            "call": "dg_batch_rk3_step (pinned host states copied in and out every step)"}
     peak, peak_kind = peaks()
     floor = FLOOR_BYTES * value / ws / 1e9
-    impl = STEP_BYTES_PER_NODE * sum(nodes) * steps / (ms / 1e3) / 1e9
+    step_bytes = sum(step_bytes_per_node(P) * n for (_, P, _), n in zip(members, nodes))
+    impl = step_bytes * steps / (ms / 1e3) / 1e9
     groups = len({P for _, P, _ in members})
     dg.dg_batch_destroy(b)
     return {"value": value, "unit": UNIT, "ms_per_step": ms / steps, "steps": steps, "clocks": clk,
@@ -841,7 +846,7 @@ def batched_measure(args, rank, ws, steps, with_clocks=False):
             "roofline": {"bound": "hbm", "achieved": floor, "peak": peak, "unit": "GB/s", "frac": floor / peak,
                          "peak_source": peak_kind, "bytes_per_dof_stage": FLOOR_BYTES,
                          "kernel": "whole batched step (all launches)", "traffic": None,
-                         "implementation": {"bytes_per_dof_stage": STEP_BYTES_PER_NODE / 3, "achieved": impl,
+                         "implementation": {"bytes_per_dof_stage": step_bytes / (3 * sum(nodes)), "achieved": impl,
                                             "frac": impl / peak}},
             "e2e": e2e, "gpu_launches": 6 * groups * steps}
 

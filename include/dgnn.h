@@ -66,10 +66,11 @@ typedef struct {
   double Prt;         /* turbulent Prandtl number, default 0.9 */
   double les_delta;   /* LES filter width; <= 0 selects h/(P+1) (default) */
   int elems_per_block;/* elements per CUDA block; <= 0 selects the tuned default for P */
-  int block_shape;    /* 0: blocks of elems_per_block consecutive elements (default);
-                         1: 2 x 2 x 2 cubes of elements (P <= 3 and even K only, else
-                         DG_ERR_INVALID_ARG): a cube's twelve internal faces need no halo
-                         and their interface fluxes are formed once for both sides */
+  int block_shape;    /* blocks of the gradient and volume phase: 0: elems_per_block
+                         consecutive elements (default); 1: 2 x 2 x 2 cubes of elements
+                         (P <= 3 and even K only, else DG_ERR_INVALID_ARG), whose twelve
+                         internal faces need no halo.  The interface phase picks its own
+                         blocks */
   int volume_flux;    /* 0: standard strong-form volume term (default, the paper's);
                          1: kinetic-energy-preserving split form, 2 sum_m D_im F#(q_i, q_m)
                          with Pirozzoli's two-point flux for the Euler part (a robustness
@@ -131,8 +132,8 @@ int dg_rhs(dg_ctx* ctx, const double* q, double* dqdt, const nn_model* forcing, 
  * synchronise the device, as cudaMalloc and cudaFree may).  The mesh and flow are given
  * as in dg_create (default dg_opts apart from precision, no forcing).  q, dqdt: DEVICE,
  * 5 N doubles, N = K^3 (P+1)^3.
- * The two intermediate fields of the operator live in one scratch array inside the
- * library's device image (3.7 MB, kept by every GPU that loads the library until exit):
+ * The intermediate fields of the operator live in one scratch array inside the
+ * library's device image (5.8 MB, kept by every GPU that loads the library until exit):
  * N may be at most 32768 nodes, larger meshes return DG_ERR_INVALID_ARG.  The first call
  * on a device (with that device current) does the set-up: it looks up the array's device
  * address and uploads the FP32 kernels' constant tables (synchronous copies, whatever the

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "dg_aux.h"
+#include "dg_bulk.cuh"
 #include "dg_kernels.cuh"
 #include "nn_bridge.h"
 #include "tc_common.cuh"
@@ -22,9 +23,13 @@ thread_local std::string g_last_error;
 constexpr double kRkA[3] = {0.0, -5.0 / 9.0, -153.0 / 128.0};
 constexpr double kRkB[3] = {1.0 / 3.0, 15.0 / 16.0, 8.0 / 15.0};
 
-int default_elems_per_block(int P) {
-  static const int E[9] = {0, 32, 16, 4, 2, 2, 1, 1, 1};
-  return E[P];
+// Phase-A elements per block.  FP32 RK3 steps on GB300 at these against the neighbouring
+// choices: P1 32^3 70 us (E = 32: 73), P2 32^3 206 (E = 8: 211), P3 8^3 29.4 (E = 8: 30.6) and
+// 32^3 328 (E = 1: 427, half a warp), P4 15^3 91.5 (E = 2: 95.8), P5 15^3 133 (E = 2: 149);
+// FP64: P2 12^3 221 (E = 4: 256), P3 8^3 164 (E = 2: 190).
+int default_elems_per_block(int P, bool f32) {
+  static const int E32[9] = {0, 8, 4, 2, 1, 1, 1, 1, 1}, E64[9] = {0, 8, 8, 4, 1, 1, 1, 1, 1};
+  return f32 ? E32[P] : E64[P];
 }
 
 int max_elems_per_block(int P) {
@@ -44,28 +49,18 @@ int cuda_fail(cudaError_t err, const char* what) {
   return fail(DG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
 }
 
-cudaError_t launch_gradient(const dg_ctx* c, const double* q, int src, cudaStream_t st) {
+RkStage rk_stage(int k) { return RkStage{kRkA[k], kRkB[k], 1.0 / kRkB[0], kRkB[2] * kRkA[2]}; }
+
+cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_t st) {
   const bool f32 = c->opts.precision == DG_PREC_FP32;
-  if (c->part) return f32 ? gradient_f32_slab(c, q, src, st) : gradient_f64_slab(c, q, src, st);
-  return f32 ? gradient_f32(c, q, src, st) : gradient_f64(c, q, src, st);
+  if (c->geom.split) return f32 ? volume_split_f32(c, q, src, st) : volume_split_f64(c, q, src, st);
+  return f32 ? volume_f32(c, q, src, st) : volume_f64(c, q, src, st);
 }
 
-cudaError_t launch_flux(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                        double dt, cudaStream_t st) {
-  const double invB1 = 1.0 / kRkB[0];
-  if (c->part) {
-    const bool f32 = c->opts.precision == DG_PREC_FP32;
-    if (c->geom.split)
-      return f32 ? flux_split_f32_slab(c, q, dqdt, f, mode, A, B, dt, invB1, st)
-                 : flux_split_f64_slab(c, q, dqdt, f, mode, A, B, dt, invB1, st);
-    return f32 ? flux_f32_slab(c, q, dqdt, f, mode, A, B, dt, invB1, st)
-               : flux_f64_slab(c, q, dqdt, f, mode, A, B, dt, invB1, st);
-  }
-  if (c->geom.split)
-    return c->opts.precision == DG_PREC_FP32 ? flux_split_f32(c, q, dqdt, f, mode, A, B, dt, invB1, st)
-                                             : flux_split_f64(c, q, dqdt, f, mode, A, B, dt, invB1, st);
-  return c->opts.precision == DG_PREC_FP32 ? flux_f32(c, q, dqdt, f, mode, A, B, dt, invB1, st)
-                                           : flux_f64(c, q, dqdt, f, mode, A, B, dt, invB1, st);
+cudaError_t launch_surface(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,
+                           double dt, cudaStream_t st) {
+  return c->opts.precision == DG_PREC_FP32 ? surface_f32(c, q, dqdt, f, mode, rk, dt, st)
+                                           : surface_f64(c, q, dqdt, f, mode, rk, dt, st);
 }
 
 // Launch plan of RK stage k (0, 1, 2): source of the phase-A stage state and phase-B mode.
@@ -82,15 +77,12 @@ static void stage_plan(const dg_ctx* c, int k, int* src, int* mode) {
 // Algorithmic bytes per node of the phase-A and phase-B launches of stage k: every value
 // the kernel must read or write once (neighbour interface reads are L2 hits, not counted).
 static void stage_bytes(const dg_ctx* c, int k, double* grad, double* flux) {
-  if (c->opts.precision == DG_PREC_FP32) {
-    const double A[3] = {40 + 20 + 20 + 36, 20 + 20 + 20 + 36, 20 + 20 + 20 + 36};
-    const double B[3] = {20 + 36 + 20, 20 + 36 + 20 + 20 + 20, 20 + 36 + 20 + 20 + 40 + 40};
-    *grad = A[k];
-    *flux = B[k];
-  } else {
-    *grad = 40 + 40 + 72;
-    *flux = 40 + 72 + (k ? 40 : 0) + 40 + 40 + 40;
-  }
+  const bool f32 = c->opts.precision == DG_PREC_FP32;
+  const double T = f32 ? 4 : 8, face = 24.0 * T / c->n;   // four viscous values on six faces
+  *grad = (f32 && k > 0 ? 5 * T : 40 + 5 * T) + 5 * T + face;
+  *flux = 10 * T + face;
+  if (!f32) *flux += 40 + (k ? 40 : 0) + 80;
+  else *flux += k == 0 ? 10 * T : k == 1 ? 20 * T : 5 * T + 80;
 }
 
 // Evaluates the network forcing on the current state q (all elements) into c->s_buf;
@@ -146,7 +138,8 @@ static int rhs_into_n(dg_ctx* const* cs, int n, double* const* qs, double* const
   if (rc) return rc;
   const bool feats = n == 1 && net && nn_phase_a_features(net, cs[0], &cs[0]->feat_out);
   for (int i = 0; i < n; ++i) {
-    const cudaError_t e = launch_gradient(cs[i], qs[i], 0, st);
+    cs[i]->cur = cs[i]->qf;
+    const cudaError_t e = launch_volume(cs[i], qs[i], 0, st);
     cs[i]->feat_out = FeatureOut{};
     DG_CUDA(e);
   }
@@ -157,7 +150,7 @@ static int rhs_into_n(dg_ctx* const* cs, int n, double* const* qs, double* const
   }
   rc = exchange_traces(cs, n, qs, kWhatPhaseB, st);
   if (rc) return rc;
-  for (int i = 0; i < n; ++i) DG_CUDA(launch_flux(cs[i], qs[i], outs[i], f, 0, 0.0, 0.0, 0.0, st));
+  for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], outs[i], f, 0, RkStage{}, 0.0, st));
   return DG_OK;
 }
 
@@ -180,13 +173,14 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
     for (int k = 0; k < 3; ++k) {
       int src, mode;
       stage_plan(c, k, &src, &mode);
+      for (int i = 0; i < n; ++i) cs[i]->cur = stage_buffer(cs[i], k);
       int rc = exchange ? exchange_traces(cs, n, qs, phase_a_what(c, src), st) : DG_OK;
       if (rc) return rc;
       // the forcing's input features come out of the phase-A launch when the network allows
       const bool want = net && (!post || k == 0);
       const bool feats = want && n == 1 && nn_phase_a_features(net, c, &c->feat_out);
       for (int i = 0; i < n; ++i) {
-        const cudaError_t e = launch_gradient(cs[i], qs[i], src, st);
+        const cudaError_t e = launch_volume(cs[i], qs[i], src, st);
         cs[i]->feat_out = FeatureOut{};
         DG_CUDA(e);
       }
@@ -201,7 +195,7 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
       }
       rc = exchange ? exchange_traces(cs, n, qs, kWhatPhaseB, st) : DG_OK;
       if (rc) return rc;
-      for (int i = 0; i < n; ++i) DG_CUDA(launch_flux(cs[i], qs[i], nullptr, f, mode, kRkA[k], kRkB[k], dt, st));
+      for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], nullptr, f, mode, rk_stage(k), dt, st));
     }
     if (post) DG_CUDA(launch_add_forcing(c, qs[0], fpost, dt, st));
   }
@@ -295,7 +289,7 @@ int setup_ctx(dg_ctx* c, int K, int P, double Re, double Mach, double Pr, int cl
   c->geom.K = K;
   c->geom.nel = c->nel;
   c->geom.N = c->N;
-  c->geom.E = o.elems_per_block > 0 ? o.elems_per_block : default_elems_per_block(P);
+  c->geom.E = o.elems_per_block > 0 ? o.elems_per_block : default_elems_per_block(P, o.precision == DG_PREC_FP32);
   c->geom.cube = o.block_shape;
   if (c->geom.cube) c->geom.E = kCubeElems;
   c->geom.split = o.volume_flux;
@@ -380,13 +374,6 @@ int dg_create_part(int K, int P, double Re, double Mach, double Pr, int closure,
   dg_ctx* c = nullptr;
   int rc = dg_create_local(K, P, Re, Mach, Pr, closure, &o, z_count + 2, &c);
   if (rc) return rc;
-  if (o.precision == DG_PREC_FP32) {
-    const cudaError_t ec = prepare_f32_slab_constants();
-    if (ec != cudaSuccess) {
-      dg_destroy(c);
-      return cuda_fail(ec, "dg_create_part: constant tables");
-    }
-  }
   c->part = 1;
   c->z_begin = z_begin;
   c->z_count = z_count;
@@ -397,8 +384,6 @@ int dg_create_part(int K, int P, double Re, double Mach, double Pr, int closure,
   c->trace_bytes = tb;
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaMalloc(&c->trace[i], tb);
-  // the ghost layers' FP32 increment stays zero: their stage state arrives whole in qn32
-  if (e == cudaSuccess && c->dlt) e = cudaMemset(c->dlt, 0, 5 * c->N * sizeof(float));
   if (e != cudaSuccess) {
     dg_destroy(c);
     return cuda_fail(e, "dg_create_part: trace buffers");
@@ -554,7 +539,9 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
   const bool f32 = o.precision == DG_PREC_FP32;
   if (f32) {
     cudaError_t ec = prepare_f32_constants();
+    if (ec == cudaSuccess) ec = prepare_split_constants();
     if (ec == cudaSuccess) ec = prepare_batch_f32_constants();
+    if (ec == cudaSuccess) ec = prepare_batch_persist_constants();
     if (ec != cudaSuccess) {
       delete c;
       return cuda_fail(ec, "dg_create: constant tables");
@@ -563,11 +550,14 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
   const size_t tsz = f32 ? sizeof(float) : sizeof(double);
   c->red_blocks = kDiagBlocks;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaMalloc(&c->qf, 5 * c->N * tsz);
-  if (e == cudaSuccess) e = cudaMalloc(&c->vis, 9 * c->N * tsz);
-  if (e == cudaSuccess) e = cudaMalloc(&c->g, 5 * c->N * tsz);
-  if (f32 && e == cudaSuccess) e = cudaMalloc(&c->qn32, 5 * c->N * sizeof(float));
-  if (f32 && e == cudaSuccess) e = cudaMalloc(&c->dlt, 5 * c->N * sizeof(float));
+  const size_t rec = (size_t)c->nel * state_record(c->n), frec = (size_t)c->nel * face_record(c->n);
+  if (e == cudaSuccess) e = cudaMalloc(&c->qf, rec * tsz);
+  if (e == cudaSuccess) e = cudaMalloc(&c->rv, rec * tsz);
+  if (e == cudaSuccess) e = cudaMalloc(&c->vt, frec * tsz);
+  if (!f32 && e == cudaSuccess) e = cudaMalloc(&c->g, rec * tsz);
+  if (f32 && e == cudaSuccess) e = cudaMalloc(&c->qy, rec * tsz);
+  if (f32 && e == cudaSuccess) e = cudaMalloc(&c->dlt, rec * tsz);
+  c->cur = c->qf;
   if (e == cudaSuccess) e = cudaMalloc(&c->rhs_tmp, 5 * c->N * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->red, (size_t)(c->red_blocks + 1) * kDiagLen * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost(&c->red_host, (kDiagLen + 1) * sizeof(double));
@@ -589,9 +579,10 @@ int dg_destroy(dg_ctx* c) {
   if (!c) return fail(DG_ERR_INVALID_ARG, "dg_destroy: NULL");
   if (c->borrowed) return fail(DG_ERR_INVALID_ARG, "dg_destroy: the context belongs to a batch (dg_batch_destroy)");
   cudaFree(c->qf);
-  cudaFree(c->vis);
+  cudaFree(c->qy);
+  cudaFree(c->rv);
+  cudaFree(c->vt);
   cudaFree(c->g);
-  cudaFree(c->qn32);
   cudaFree(c->dlt);
   cudaFree(c->rhs_tmp);
   cudaFree(c->red);
@@ -798,11 +789,12 @@ int dg_profile_rk3(dg_ctx* c, double* q, double dt, int nsteps, double* ms_gradi
         stage_bytes(c, k, &gb, &fb);
         bg += gb;
         bf += fb;
+        c->cur = stage_buffer(c, k);
         cudaEventRecord(ev[i], st);
-        e = launch_gradient(c, q, src, st);
+        e = launch_volume(c, q, src, st);
         cudaEventRecord(ev[i + 1], st);
         cudaEventRecord(ev[i + 2], st);
-        if (e == cudaSuccess) e = launch_flux(c, q, nullptr, Forcing{}, mode, kRkA[k], kRkB[k], dt, st);
+        if (e == cudaSuccess) e = launch_surface(c, q, nullptr, Forcing{}, mode, rk_stage(k), dt, st);
         cudaEventRecord(ev[i + 3], st);
       }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -897,7 +889,7 @@ extern "C" int dg_set_forcing_mode(dg_ctx* c, int mode) {
 
 namespace dgnn {
 // Two bounded waits on mbarriers that never complete (no arrivals): out[0] from the
-// operator's bulk-copy wait, out[1] from the tensor-core wait; 1 = reported completion.
+// bulk-copy wait, out[1] from the tensor-core wait; 1 = reported completion.
 __global__ void k_wait_selfcheck(int* out) {
   __shared__ unsigned long long bars[2];
   if (threadIdx.x == 0) {

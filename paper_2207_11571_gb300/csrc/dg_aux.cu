@@ -259,26 +259,23 @@ size_t trace_bytes_for(const dg_ctx* c, int what) {
   return (size_t)comps * esize * c->K * c->K * c->n * c->n;
 }
 
-// Source (component v) of a trace value: pointer to node 0 of component v's array.
-template <typename T>
-__device__ __forceinline__ const T* trace_src(int what, int v, const double* q, const float* qn32, const T* qf,
-                                              const T* vis, long long N) {
-  if (what == 0) return reinterpret_cast<const T*>(q + v * N);
-  if (what == 1) return reinterpret_cast<const T*>(qn32 + v * N);
-  // stage state, then tau_xz, tau_yz, tau_zz, k theta_z (indices 4, 5, 2, 8 of the 9-vector:
-  // symmetric tensor (xx, yy, zz, xy, xz, yz), then the heat flux)
-  if (v < 5) return qf + v * N;
-  const int vi[4] = {4, 5, 2, 8};
-  return vis + vi[v - 5] * N;
-}
-
 // One thread per (component, element of the layer, face node); side 0 = lo, 1 = hi.
 template <typename T>
-__global__ void k_trace_pack(const double* __restrict__ q, const float* __restrict__ qn32,
-                             const float* __restrict__ dlt, const T* __restrict__ qf, const T* __restrict__ vis,
-                             int what, int comps, int K, int n, int z_lo, int z_hi, long long N, T* __restrict__ lo,
-                             T* __restrict__ hi) {
-  const int n2 = n * n, K2 = K * K, np = n2 * n;
+__device__ __forceinline__ T* trace_value(double* q, T* s, T* vt, int what, int v, int n, long long e, int ab, int upper,
+                                          long long N) {
+  const int n2 = n * n;
+  const int node = ab + (upper ? n2 * (n - 1) : 0);   // upper face k = P, lower face k = 0
+  if (what == 0) return reinterpret_cast<T*>(q + v * N + e * (n2 * n) + node);
+  if (v < 5) return s + e * state_record(n) + v * node_stride(n) + node;
+  return vt + e * face_record(n) + (4 + upper) * (kFaceVis * n2) + (v - 5) * n2 + ab;
+}
+
+// PACK: lo takes the lower faces of layer z_lo, hi the upper faces of layer z_hi; else the
+// upper faces of (ghost) layer z_lo come from lo, the lower faces of layer z_hi from hi.
+template <typename T, bool PACK>
+__global__ void k_trace(double* __restrict__ q, T* __restrict__ s, T* __restrict__ vt, int what, int comps, int K, int n,
+                        int z_lo, int z_hi, long long N, T* __restrict__ lo, T* __restrict__ hi) {
+  const int n2 = n * n, K2 = K * K;
   const long long per_side = (long long)comps * K2 * n2;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= 2 * per_side) return;
@@ -287,82 +284,36 @@ __global__ void k_trace_pack(const double* __restrict__ q, const float* __restri
   const int v = (int)(u / ((long long)K2 * n2));
   const int r = (int)(u - (long long)v * K2 * n2);
   const int el = r / n2, ab = r - el * n2;
-  const long long e = (long long)(side ? z_hi : z_lo) * K2 + el;
-  const long long node = e * np + ab + (side ? n2 * (n - 1) : 0);   // upper face k = P, lower face k = 0
-  T val;
-  if (what == 1) {
-    val = T(qn32[v * N + node] + dlt[v * N + node]);     // the stage state the neighbour's phase A forms
-  } else {
-    val = trace_src<T>(what, v, q, qn32, qf, vis, N)[node];
-  }
-  (side ? hi : lo)[u] = val;
+  T* value = trace_value<T>(q, s, vt, what, v, n, (long long)(side ? z_hi : z_lo) * K2 + el, ab, PACK ? side : !side, N);
+  T* buf = (side ? hi : lo) + u;
+  if (PACK) *buf = *value;
+  else *value = *buf;
 }
 
-template <typename T>
-__global__ void k_trace_unpack(double* __restrict__ q, float* __restrict__ qn32, float* __restrict__ dlt,
-                               T* __restrict__ qf, T* __restrict__ vis, int what, int comps, int K, int n,
-                               int z_glo, int z_ghi, long long N, const T* __restrict__ lo,
-                               const T* __restrict__ hi) {
-  const int n2 = n * n, K2 = K * K, np = n2 * n;
-  const long long per_side = (long long)comps * K2 * n2;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= 2 * per_side) return;
-  const int side = t >= per_side;
-  const long long u = t - side * per_side;
-  const int v = (int)(u / ((long long)K2 * n2));
-  const int r = (int)(u - (long long)v * K2 * n2);
-  const int el = r / n2, ab = r - el * n2;
-  // lower ghost layer: its upper face (k = P) faces the first owned layer; upper ghost
-  // layer: its lower face (k = 0)
-  const long long e = (long long)(side ? z_ghi : z_glo) * K2 + el;
-  const long long node = e * np + ab + (side ? 0 : n2 * (n - 1));
-  const T val = (side ? hi : lo)[u];
-  T* dst;
-  if (what == 0) dst = reinterpret_cast<T*>(q + v * N);
-  else if (what == 1) dst = reinterpret_cast<T*>(qn32 + v * N);
-  else if (v < 5) dst = qf + v * N;
-  else {
-    const int vi[4] = {4, 5, 2, 8};
-    dst = vis + vi[v - 5] * N;
-  }
-  dst[node] = val;
-}
-
-template <typename T>
-static cudaError_t trace_pack_t(const dg_ctx* c, const double* q, int what, void* lo, void* hi, cudaStream_t st) {
+template <typename T, bool PACK>
+static cudaError_t trace_t(const dg_ctx* c, double* q, int what, void* lo, void* hi, cudaStream_t st) {
   int comps, esize;
   trace_shape(c, what, &comps, &esize);
   const long long total = 2LL * comps * c->K * c->K * c->n * c->n;
-  k_trace_pack<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
-      q, c->qn32, c->dlt, static_cast<const T*>(c->qf), static_cast<const T*>(c->vis), what, comps, c->K, c->n, 1,
-      c->z_count, c->N, static_cast<T*>(lo), static_cast<T*>(hi));
-  return cudaGetLastError();
-}
-
-template <typename T>
-static cudaError_t trace_unpack_t(const dg_ctx* c, double* q, int what, const void* lo, const void* hi,
-                                  cudaStream_t st) {
-  int comps, esize;
-  trace_shape(c, what, &comps, &esize);
-  const long long total = 2LL * comps * c->K * c->K * c->n * c->n;
-  k_trace_unpack<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
-      q, c->qn32, c->dlt, static_cast<T*>(c->qf), static_cast<T*>(c->vis), what, comps, c->K, c->n, 0,
-      c->z_count + 1, c->N, static_cast<const T*>(lo), static_cast<const T*>(hi));
+  k_trace<T, PACK><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+      q, static_cast<T*>(c->cur), static_cast<T*>(c->vt), what, comps, c->K, c->n, PACK ? 1 : 0,
+      PACK ? c->z_count : c->z_count + 1, c->N, static_cast<T*>(lo), static_cast<T*>(hi));
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace_pack(const dg_ctx* c, const double* q, int what, void* lo, void* hi, cudaStream_t st) {
   int comps, esize;
   trace_shape(c, what, &comps, &esize);
-  return esize == 8 ? trace_pack_t<double>(c, q, what, lo, hi, st) : trace_pack_t<float>(c, q, what, lo, hi, st);
+  double* qq = const_cast<double*>(q);   // read only
+  return esize == 8 ? trace_t<double, true>(c, qq, what, lo, hi, st) : trace_t<float, true>(c, qq, what, lo, hi, st);
 }
 
 cudaError_t launch_trace_unpack(const dg_ctx* c, double* q, int what, const void* lo, const void* hi,
                                 cudaStream_t st) {
   int comps, esize;
   trace_shape(c, what, &comps, &esize);
-  return esize == 8 ? trace_unpack_t<double>(c, q, what, lo, hi, st)
-                    : trace_unpack_t<float>(c, q, what, lo, hi, st);
+  void *l = const_cast<void*>(lo), *h = const_cast<void*>(hi);   // read only
+  return esize == 8 ? trace_t<double, false>(c, q, what, l, h, st) : trace_t<float, false>(c, q, what, l, h, st);
 }
 
 // ---------------------------------------------------------------- Algorithm 1 pairs

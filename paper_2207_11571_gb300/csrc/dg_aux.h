@@ -61,10 +61,10 @@ cudaError_t launch_make_pairs(const dg_ctx* lo, const double* qb_n, const double
 // upper faces, recv_hi into the upper ghost layer's lower faces.  Buffer layout
 // [component][element of the layer][face node].
 //   what 0: the FP64 state q (5 doubles per face node);
-//   what 1: the FP32 stage state qn32 + dlt (5 floats; unpacked into qn32, the ghost dlt
-//           stays zero);
-//   what 2: the operator-precision stage state qf and the z-normal viscous quantities
-//           (tau_xz, tau_yz, tau_zz, k theta_z): 9 values.
+//   what 1: the FP32 stage state (5 floats);
+//   what 2: the operator-precision stage state and the viscous fluxes normal to the face
+//           (4 values, as phase A stored them): 9 values.
+// The stage state is the context's current one (c->cur).
 cudaError_t launch_trace_pack(const dg_ctx* c, const double* q, int what, void* send_lo, void* send_hi,
                               cudaStream_t st);
 cudaError_t launch_trace_unpack(const dg_ctx* c, double* q, int what, const void* recv_lo, const void* recv_hi,
@@ -75,46 +75,34 @@ size_t trace_bytes_for(const dg_ctx* c, int what);
 // q += dt s on the forced variables (Algorithm 1's correction after the step).
 cudaError_t launch_add_forcing(const dg_ctx* c, double* q, const Forcing& f, double dt, cudaStream_t st);
 
-// Operator kernels per precision (dg_kernels_f32.cu / dg_kernels_f64.cu).
-cudaError_t gradient_f32(const dg_ctx* c, const double* q, int src, cudaStream_t st);
-cudaError_t gradient_f64(const dg_ctx* c, const double* q, int src, cudaStream_t st);
-cudaError_t flux_f32(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                     double dt, double invB1, cudaStream_t st);
-cudaError_t flux_split_f32(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                           double dt, double invB1, cudaStream_t st);
-cudaError_t flux_split_f64(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                           double dt, double invB1, cudaStream_t st);
-cudaError_t flux_f64(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                     double dt, double invB1, cudaStream_t st);
+// Operator kernels per precision (dg_kernels_*.cu, dg_split.cu, dg_surface_*.cu); src and
+// mode as launch_volume and launch_surface.
+cudaError_t volume_f32(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+cudaError_t volume_f64(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+cudaError_t volume_split_f32(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+cudaError_t volume_split_f64(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+cudaError_t surface_f32(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,
+                        double dt, cudaStream_t st);
+cudaError_t surface_f64(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,
+                        double dt, cudaStream_t st);
 
-// The same for slab contexts (dg_kernels_f32_slab.cu, dg_kernels_f64_slab.cu).
-cudaError_t gradient_f32_slab(const dg_ctx* c, const double* q, int src, cudaStream_t st);
-cudaError_t gradient_f64_slab(const dg_ctx* c, const double* q, int src, cudaStream_t st);
-cudaError_t flux_f32_slab(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                          double dt, double invB1, cudaStream_t st);
-cudaError_t flux_f64_slab(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A, double B,
-                          double dt, double invB1, cudaStream_t st);
-cudaError_t flux_split_f32_slab(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A,
-                                double B, double dt, double invB1, cudaStream_t st);
-cudaError_t flux_split_f64_slab(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, double A,
-                                double B, double dt, double invB1, cudaStream_t st);
-cudaError_t prepare_f32_slab_constants();
-
-// Derivative matrices in the constant memory of the FP32 kernels (dg_kernels_f32.cu,
-// dg_batch_f32.cu); once per device, before the first FP32 launch.
+// Derivative matrices in the constant memory of the FP32 kernels of each translation unit
+// that holds some; once per device, before the first FP32 launch.
 cudaError_t prepare_f32_constants();
+cudaError_t prepare_split_constants();
 cudaError_t prepare_batch_f32_constants();
+cudaError_t prepare_batch_persist_constants();
 
 // Batched RK stage k for n instances of order P sharing precision and elements per block
 // (dg_batch_f32.cu / dg_batch_f64.cu): q[i] is instance i's FP64 state, dt[i] its step.
-cudaError_t batch_stage_f32(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k, double A,
-                            double B, double invB1, cudaStream_t st);
+cudaError_t batch_stage_f32(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
+                            const RkStage& rk, cudaStream_t st);
 // Sets the kernels' shared-memory attributes for order P at E elements per block; call
 // before batch_stage_* (never inside a stream capture).
 cudaError_t batch_prepare_f32(int P, int E);
 cudaError_t batch_prepare_f64(int P, int E);
-cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k, double A,
-                            double B, double invB1, cudaStream_t st);
+cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
+                            const RkStage& rk, cudaStream_t st);
 
 // Persistent batched RK stage (dg_batch_persist.cu, FP32 operator, orders 1..6): one
 // cooperative launch per stage for every member; bar: the grid barrier's two counters
@@ -122,7 +110,7 @@ cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const d
 // attribute for the orders present and returns the shared memory and co-resident grid.
 bool batch_persistent_ok(int P);
 cudaError_t batch_persistent_prepare(const int* orders, int n, size_t* smem, int* grid);
-cudaError_t batch_persistent_stage(dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k, double A,
-                                   double B, double invB1, unsigned* bar, size_t smem, int grid, cudaStream_t st);
+cudaError_t batch_persistent_stage(dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
+                                   const RkStage& rk, unsigned* bar, size_t smem, int grid, cudaStream_t st);
 
 }  // namespace dgnn

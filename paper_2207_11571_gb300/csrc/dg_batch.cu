@@ -2,8 +2,8 @@
 //
 // Each member is an ordinary context (its own mesh, flow, closure and workspace).  A
 // batched RK3 step groups the members by order P: every group runs one phase-A and one
-// phase-B launch per stage covering all of its members' element blocks (k_gradient_batch,
-// k_flux_batch), so twelve small meshes cost six launches per step per order instead of
+// phase-B launch per stage covering all of its members' element blocks (k_volume_batch,
+// k_surface_batch), so twelve small meshes cost six launches per step per order instead of
 // six per mesh.  Groups of different orders do not depend on each other and run as
 // parallel branches.  The whole step is recorded once into a CUDA graph on private
 // streams and replayed on the caller's stream; it is recorded again when the member
@@ -16,10 +16,6 @@
 
 namespace dgnn {
 namespace {
-
-// Williamson 2N RK3 (the same coefficients as the single-mesh path).
-constexpr double kA[3] = {0.0, -5.0 / 9.0, -153.0 / 128.0};
-constexpr double kB[3] = {1.0 / 3.0, 15.0 / 16.0, 8.0 / 15.0};
 
 struct Group {
   int P = 0;
@@ -65,9 +61,8 @@ cudaError_t stage_group(const dg_batch* b, const Group& g, double* const* q, con
     qs[j] = q[g.members[j]];
     dts[j] = dt[g.members[j]];
   }
-  const double invB1 = 1.0 / kB[0];
-  return b->precision == DG_PREC_FP32 ? batch_stage_f32(g.P, ctx, qs, dts, n, k, kA[k], kB[k], invB1, st)
-                                      : batch_stage_f64(g.P, ctx, qs, dts, n, k, kA[k], kB[k], invB1, st);
+  return b->precision == DG_PREC_FP32 ? batch_stage_f32(g.P, ctx, qs, dts, n, k, rk_stage(k), st)
+                                      : batch_stage_f64(g.P, ctx, qs, dts, n, k, rk_stage(k), st);
 }
 
 cudaError_t prepare_groups(const dg_batch* b) {
@@ -97,9 +92,8 @@ cudaError_t step_persistent(const dg_batch* b, double* const* q, const double* d
                             cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), st);
   const int n = (int)b->inst.size();
-  const double invB1 = 1.0 / kB[0];
   for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-    e = batch_persistent_stage(b->inst.data(), q, dt, n, k, kA[k], kB[k], invB1, b->bar, smem, grid, st);
+    e = batch_persistent_stage(b->inst.data(), q, dt, n, k, rk_stage(k), b->bar, smem, grid, st);
   return e;
 }
 

@@ -1,12 +1,12 @@
-// FP64 instantiation of the batched RK-stage kernels (several meshes of one
+// F64 instantiation of the batched RK-stage kernels (several meshes of one
 // order per launch).
 #include "dg_aux.h"
 #include "dg_launch.cuh"
 
 namespace dgnn {
-cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k, double A,
-                            double B, double invB1, cudaStream_t st) {
-  return batch_stage_t<double>(P, ctx, q, dt, n, k, A, B, invB1, st);
+cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
+                           const RkStage& rk, cudaStream_t st) {
+  return batch_stage_t<double>(P, ctx, q, dt, n, k, rk, st);
 }
 cudaError_t batch_prepare_f64(int P, int E) { return batch_prepare_t<double>(P, E); }
 }  // namespace dgnn

@@ -4,8 +4,8 @@
 // Each block of kPersistThreads threads walks the phase-A work items of all members
 // (blocks of E_P consecutive elements of a member, E_P = the elements of order P that
 // fill the block), meets every other block at a grid barrier, then walks the phase-B items
-// of all members.  The per-item arithmetic is the single-mesh kernels' (gradient_block,
-// flux_block), so a member computes what it computes alone; only the blocking differs.
+// of all members.  The per-item arithmetic is the single-mesh kernels' (volume_block,
+// surface_block), so a member computes what it computes alone; only the blocking differs.
 // The grid holds as many blocks as are resident at once (a cooperative launch), and the
 // barrier's wait is bounded (about a second): on expiry the block sets the batch's error
 // flag and returns.  The launches of a step form one CUDA graph, after a reset of the
@@ -16,7 +16,9 @@
 namespace dgnn {
 
 constexpr int kPersistThreads = 384;
-__host__ __device__ constexpr int persist_elems(int P) { return kPersistThreads / ((P + 1) * (P + 1) * (P + 1)); }
+__host__ __device__ constexpr int persist_elems(int P) {
+  return kPersistThreads / (use_rows4(P, sizeof(float), false) ? 16 : (P + 1) * (P + 1) * (P + 1));
+}
 
 struct PersistTable {
   BatchTable<float> tb;   // block_start: first work item of each member (the same items in both phases)
@@ -60,11 +62,10 @@ __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const _
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int i = batch_instance(tb.block_start, tb.n, item);
     const int blk = item - tb.block_start[i];
-    float* qn32_out = SRC == 0 ? tb.qn32[i] : nullptr;
     switch (pt.P[i]) {
-#define DG_PA(PP)                                                                                                  \
-  case PP:                                                                                                         \
-    gradient_block<PP, float, SRC>(blk, tb.q[i], tb.qn32[i], tb.dlt[i], tb.qf[i], qn32_out, tb.vis[i], tb.C[i]); \
+#define DG_PA(PP)                                                                                   \
+  case PP:                                                                                          \
+    volume_phase<PP, float, SRC>(blk, tb.a[i].q, tb.qs[i], tb.rv[i], tb.vt[i], tb.C[i]);            \
     break;
       DG_PA(1) DG_PA(2) DG_PA(3) DG_PA(4) DG_PA(5) DG_PA(6)
 #undef DG_PA
@@ -79,10 +80,10 @@ __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const _
     const int i = batch_instance(tb.block_start, tb.n, item);
     const int blk = item - tb.block_start[i];
     switch (pt.P[i]) {
-#define DG_PB(PP)                                                                                                 \
-  case PP:                                                                                                        \
-    flux_block<PP, float, MODE>(blk, tb.q[i], tb.qf[i], tb.vis[i], nullptr, tb.g[i], tb.dlt[i], Forcing{}, tb.C[i], \
-                                tb.rk[i]);                                                                        \
+#define DG_PB(PP)                                                                                   \
+  case PP:                                                                                          \
+    surface_prologue<PP, float, false>(blk, persist_elems(PP), tb.C[i]);                            \
+    surface_block<PP, float, MODE>(blk, persist_elems(PP), tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);  \
     break;
       DG_PB(1) DG_PB(2) DG_PB(3) DG_PB(4) DG_PB(5) DG_PB(6)
 #undef DG_PB
@@ -96,8 +97,10 @@ namespace {
 // Shared memory of one work item of order P in the persistent kernel (the larger phase).
 size_t persist_smem_p(int P) {
   switch (P) {
-#define DG_SM(PP) \
-  case PP: return std::max(gradient_smem<PP, float>(persist_elems(PP)), flux_smem<PP, float>(persist_elems(PP)));
+#define DG_SM(PP)                                                                                                     \
+  case PP:                                                                                                            \
+    return std::max(volume_smem<PP, float, false>(persist_elems(PP), false),                                          \
+                    surface_smem_bytes<PP, float>(persist_elems(PP)));
     DG_SM(1) DG_SM(2) DG_SM(3) DG_SM(4) DG_SM(5) DG_SM(6)
 #undef DG_SM
   }
@@ -111,6 +114,9 @@ PersistKernel persist_kernel(int k) {
 }
 
 }  // namespace
+
+// Constant-memory tables of this unit's kernels (see upload_const_D).
+cudaError_t prepare_batch_persist_constants() { return upload_const_D(); }
 
 bool batch_persistent_ok(int P) { return P >= 1 && P <= 6; }
 
@@ -137,11 +143,11 @@ cudaError_t batch_persistent_prepare(const int* orders, int n, size_t* smem_out,
   return cudaSuccess;
 }
 
-cudaError_t batch_persistent_stage(dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k, double A,
-                                   double B, double invB1, unsigned* bar, size_t smem, int grid, cudaStream_t st) {
+cudaError_t batch_persistent_stage(dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
+                                   const RkStage& rk, unsigned* bar, size_t smem, int grid, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
   PersistTable pt;
-  fill_batch<float>(&pt.tb, ctx, q, dt, n, A, B, invB1);
+  fill_batch<float>(&pt.tb, ctx, q, dt, n, k, rk);
   // work items of E_P elements per member, whatever blocking the member uses alone
   int items = 0;
   for (int i = 0; i < n; ++i) {

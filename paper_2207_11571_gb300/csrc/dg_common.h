@@ -13,6 +13,13 @@ namespace dgnn {
 constexpr int kMaxP = 8;
 constexpr int kMaxN1 = kMaxP + 1;
 
+// Element-major workspace records (dg_kernels.cuh), n = P + 1: node stride of a component,
+// and sizes of the state and face records in values.
+__host__ __device__ constexpr int node_stride(int n) { return (n * n * n + 3) & ~3; }
+__host__ __device__ constexpr int state_record(int n) { return 5 * node_stride(n); }
+constexpr int kFaceVis = 4;   // viscous values of a face node
+__host__ __device__ constexpr int face_record(int n) { return 6 * kFaceVis * n * n; }
+
 // Thread-local error message; returns the status for convenient `return fail(...)`.
 int fail(int status, const std::string& msg);
 int cuda_fail(cudaError_t err, const char* what);
@@ -118,11 +125,14 @@ struct dg_ctx {
   dg_exchange_fn xfn = nullptr;  // exchange of a slab's traces with its neighbours (dg_part_set_exchange)
   void* xuser = nullptr;
   // workspace (device)
-  void* qf = nullptr;     // operator-precision stage state (reference-shifted), [5][N]
-  float* qn32 = nullptr;  // FP32 operator: reference-shifted FP32 image of q at the step start, [5][N]
-  float* dlt = nullptr;   // FP32 operator: RK increment accumulated within the step, [5][N]
-  void* vis = nullptr;    // viscous stresses and heat flux, [9][N] operator precision
-  void* g = nullptr;      // RK register [5][N] (double or float)
+  // element-major records (dg_kernels.cuh), operator precision unless said otherwise
+  void* qf = nullptr;     // stage state: [elem][5][node] (FP32: stages 1 and 3, reference-shifted)
+  void* qy = nullptr;     // FP32 operator: stage state of stage 2, [elem][5][node]
+  void* cur = nullptr;    // the stage state of the stage being evaluated (qf or qy)
+  void* rv = nullptr;     // volume term, [elem][5][node]
+  void* vt = nullptr;     // face-normal viscous fluxes, [elem][6][4][face node]
+  void* g = nullptr;      // FP64 operator: RK register, [elem][5][node]
+  float* dlt = nullptr;   // FP32 operator: RK increment, [elem][5][node]
   double* rhs_tmp = nullptr;  // [5][N] FP64 operator value for diagnostics
   double* red = nullptr;  // reduction partials
   int red_blocks = 0;
@@ -148,15 +158,26 @@ struct dg_ctx {
 
 namespace dgnn {
 
-// Launchers of the operator kernels.  All return cudaError_t.
-// Phase A.  src 0: stage state from q (FP64); src 1: from qn32 + dlt (FP32 operator,
-// RK stages 2 and 3).
-cudaError_t launch_gradient(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+// One stage of the 2N-storage RK3 scheme: its coefficients, 1 / B of stage 1 and B A of
+// stage 3 (the FP32 increment scheme, see dg_kernels.cuh).
+struct RkStage {
+  double A, B, invB1, wc;
+};
+RkStage rk_stage(int k);
+// Stage state buffer of RK stage k (0, 1, 2).
+inline void* stage_buffer(const dg_ctx* c, int k) {
+  return (c->opts.precision == DG_PREC_FP32 && k == 1) ? c->qy : c->qf;
+}
+
+// Launchers of the operator kernels on the stage state c->cur.  All return cudaError_t.
+// Phase A.  src 0: the stage state is formed from q (FP64) in c->qf; src 1 (FP32 operator,
+// RK stages 2 and 3): it is in c->cur.
+cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_t st);
 // Phase B.  mode 0: dqdt = R (+ s).  mode 1: FP64 RK stage, g = A g + dt R, q += B g.
 // modes 2, 3, 4: FP32 operator RK stages 1, 2, 3 on the FP32 increment; stage 3 adds
 // the increment to the FP64 state.
-cudaError_t launch_flux(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode,
-                        double rkA, double rkB, double dt, cudaStream_t st);
+cudaError_t launch_surface(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,
+                           double dt, cudaStream_t st);
 
 // Fills the sizes, basis, geometry and physics constants of a context from validated
 // arguments (host only; no device memory is touched).  Shared by dg_create and the

@@ -1,33 +1,40 @@
 // The two phases of one evaluation of the DGSEM operator p(q) (Sec. 2, Eq. 3):
 //
-//  phase A (k_gradient): BR1 lifted gradient of (v1, v2, v3, theta)
+//  phase A (k_volume): BR1 lifted gradient of (v1, v2, v3, theta)
 //     G_d = (2/h) [ D_d U + (U^ - U)|right / w_P - (U^ - U)|left / w_0 ],  U^ central,
-//     then the viscous stresses and heat flux of Appendix A (Eq. A.3), optionally with
-//     the Smagorinsky viscosity.  Writes them (9 values per node) and the stage state s
-//     (reference-shifted, operator precision) that phase B and the neighbours read.
-//  phase B (k_flux): volume term -(2/h) sum_d D_d (f^a_d - f^nu_d), Roe + central-BR1
-//     interface fluxes and their lifting (strong form), optional forcing s (Eq. 4), then
-//     writes dq/dt or applies one stage of the low-storage RK3.
+//     the viscous stresses and heat flux of Appendix A (Eq. A.3), optionally with the
+//     Smagorinsky viscosity, and from them the whole volume term of the element,
+//     -(2/h) sum_d D_d (f^a_d - f^nu_d).  Writes the volume term (5 values per node), the
+//     viscous flux normal to each face (4 values per face node) and, from an FP64 state,
+//     the stage state in operator precision.
+//  phase B (k_surface): Roe + central-BR1 interface fluxes and their lifting (strong
+//     form), optional forcing s (Eq. 4), then dq/dt or one stage of the low-storage RK3.
+//
+// A node's viscous quantities enter the operator twice: in its own element's volume term
+// and, on a face, in the interface flux.  Forming the volume term where the stresses are
+// formed therefore leaves only the face values to hand over: 20 + 96/n bytes per node
+// and way in FP32 instead of the 36 of all nine viscous quantities, and the state's
+// primitives and fluxes are formed once.
 //
 // RK3 in the FP32 operator: the state q stays FP64 and is read and written once per
-// step.  Within a step the stage state is qn32 + dlt (FP32 image of q at the step start
-// plus the FP32 increment accumulated by the stages); stage 3 adds the increment to q
-// in FP64.  The Williamson register of stage 1 is recovered as g1 = dlt1 / B1, so only
-// stage 2 stores it.  In the FP64 operator every stage updates q in FP64 (the plain
-// 2N scheme).
+// step.  The stages work on FP32 stage states in two alternating buffers: phase A of
+// stage 1 forms s1 = q - reference in qf, phase B of stage 1 writes s2 = s1 + d1 to qy and
+// the increment d1 to dlt, phase B of stage 2 writes s3 = s1 + d2 over s1 in qf (phase B
+// reads neighbours from qy only) and folds what stage 3 needs, d2 + B3 A3 g2, into dlt;
+// stage 3 adds dlt + B3 dt R to q in FP64.  In the FP64 operator every stage updates q in
+// FP64 (the plain 2N scheme) and qf holds the stage's copy of q.
 //
-// Each CUDA block owns E consecutive elements (or, at P <= 3 on even K, a 2 x 2 x 2 cube
-// of elements whose twelve internal faces need no halo and whose internal interface
-// fluxes are computed once for both sides), one thread per node for the nodal work.
-// At kernel start the block issues all its global loads: its own nodes into registers
-// and a halo (the neighbours' face nodes of all six faces of its elements) into shared
-// memory.  Interface fluxes are dense work items, one per (element, face, face node),
-// so that every lane does useful Roe work; items are ordered (face node, side,
-// direction, element) so that a warp shares one face direction and every index divisor
-// is a compile-time constant.  Node threads add the lifted results in a fixed order.
-// The 1D derivative contractions read element tiles in shared memory.  All constants
-// arrive in the operator precision (OpConst): no FP64 arithmetic or conversion runs per
-// node except where the FP64 state is read or written.
+// Workspace layout: element-major records [elem][component][node] (node stride padded to a
+// multiple of 4 values), face values [elem][face][component][face node], face = 2 d + side.
+// Every component of a node or face node is then at a compile-time offset from one address.
+//
+// Phase A: a block owns E consecutive elements (or, at P <= 3 on even K, a 2 x 2 x 2 cube
+// of elements whose twelve internal faces need no halo), one thread per node.  Phase B: a
+// block owns surf_elems(P) elements; its interface terms are dense work items, one per
+// (element, face, face node), so that every lane does useful Roe work, and its nodes add
+// the lifted results in a fixed order.  All constants arrive in the operator precision
+// (OpConst): no FP64 arithmetic or conversion runs per node except where the FP64 state
+// is read or written.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -46,7 +53,7 @@ namespace dgnn {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Maximum threads per block for order P (one node per thread, E elements per block).
+// Maximum threads per phase-A block for order P (one node per thread, E elements per block).
 __host__ __device__ constexpr int max_threads_for(int P) {
   return P == 1 ? 256 : P <= 4 ? 512 : P == 5 ? 448 : P == 6 ? 352 : P == 7 ? 512 : 736;
 }
@@ -91,23 +98,6 @@ __device__ __forceinline__ int wrap_step(int x, int shift, int K) {
   return x < 0 ? x + K : (x >= K ? x - K : x);
 }
 
-// Element index of block element hl shifted by +/-1 along d (periodic; Kz layers along z),
-// without division.
-__device__ __forceinline__ int neighbour_of(const BlockCoords& b, int hl, int K, int Kz, int d, int shift) {
-  int x = b.x + hl, y = b.y, z = b.z;
-  while (x >= K) {
-    x -= K;
-    if (++y >= K) {
-      y = 0;
-      ++z;
-    }
-  }
-  if (d == 0) x = wrap_step(x, shift, K);
-  else if (d == 1) y = wrap_step(y, shift, K);
-  else z = wrap_step(z, shift, Kz);
-  return x + K * (y + K * z);
-}
-
 
 // 2 x 2 x 2 element blocks ("cubes", even K): block b covers the elements 2 c + l,
 // l in {0, 1}^3, of the (K/2)^3 grid of cubes; local element hl = lx + 2 ly + 4 lz.
@@ -130,13 +120,21 @@ __device__ __forceinline__ int cube_element(const BlockCoords& c, int hl, int K)
   return (c.x + (hl & 1)) + K * ((c.y + ((hl >> 1) & 1)) + K * (c.z + (hl >> 2)));
 }
 
-// Element index of local element hl shifted by +/-1 along d (periodic).
-__device__ __forceinline__ int cube_neighbour(const BlockCoords& c, int hl, int K, int d, int shift) {
-  int x = c.x + (hl & 1), y = c.y + ((hl >> 1) & 1), z = c.z + (hl >> 2);
-  if (d == 0) x = wrap_step(x, shift, K);
-  else if (d == 1) y = wrap_step(y, shift, K);
-  else z = wrap_step(z, shift, K);
-  return x + K * (y + K * z);
+
+// Element across face 2 d + side of element e (periodic; Kz layers along z).
+__device__ __forceinline__ int element_across(int e, int face, int K, int Kz) {
+  BlockCoords c = block_coords(e, K);
+  const int step = (face & 1) ? 1 : -1, d = face >> 1;
+  if (d == 0) c.x = wrap_step(c.x, step, K);
+  else if (d == 1) c.y = wrap_step(c.y, step, K);
+  else c.z = wrap_step(c.z, step, Kz);
+  return c.x + K * (c.y + K * c.z);
+}
+
+// Internal faces of a cube, u <-> (ab, p, d): face p (0..3) normal to d joins the local
+// elements hlL (bit d clear) and hlL | 1 << d.
+__device__ __forceinline__ int cube_left_of_pair(int p, int d) {
+  return ((p >> d) << (d + 1)) | (p & ((1 << d) - 1));
 }
 
 // Node of the face normal to d at normal index m with tangential index ab.
@@ -154,51 +152,11 @@ __device__ __forceinline__ int face_ab(int d, const int idx[3]) {
   return d == 0 ? idx[1] + n * idx[2] : d == 1 ? idx[0] + n * idx[2] : idx[0] + n * idx[1];
 }
 
-// Derivative matrices of every order in FP32, in constant memory (one copy per
-// translation unit, filled by upload_const_D on the host before the first streamed
-// launch).  Read with compile-time indices, so each entry is an FFMA operand straight
-// from the constant bank.
-__constant__ float c_D32[kMaxP + 1][kMaxN1 * kMaxN1];
 
-// Derivative of component f along direction D for one line of nodes (tangential index
-// ab): out[node(i)] = sum_m D[i][m] f[node(m)], i = 0..P.  Each operand is read from
-// shared memory once for the whole line (instead of once per output node).
-template <int P, int D>
-__device__ __forceinline__ void line_derivative(const float* __restrict__ f, float* __restrict__ out, int ab) {
-  constexpr int n = P + 1;
-  float v[n];
-#pragma unroll
-  for (int m = 0; m < n; ++m) v[m] = f[face_node<P>(D, m, ab)];
-#pragma unroll
-  for (int i = 0; i < n; ++i) {
-    float acc = 0.f;
-#pragma unroll
-    for (int m = 0; m < n; ++m) acc += c_D32[P][i * n + m] * v[m];
-    out[face_node<P>(D, i, ab)] = acc;
-  }
-}
-
-// line_derivative in place: the line's values are all read before any is written, and
-// no other task touches the line, so the derivative may overwrite its operand.
-template <int P, int D>
-__device__ __forceinline__ void line_derivative_inplace(float* f, int ab) {
-  constexpr int n = P + 1;
-  float v[n];
-#pragma unroll
-  for (int m = 0; m < n; ++m) v[m] = f[face_node<P>(D, m, ab)];
-#pragma unroll
-  for (int i = 0; i < n; ++i) {
-    float acc = 0.f;
-#pragma unroll
-    for (int m = 0; m < n; ++m) acc += c_D32[P][i * n + m] * v[m];
-    f[face_node<P>(D, i, ab)] = acc;
-  }
-}
-
-// Halo / interface item t <-> (ab, side, d, hl), ab fastest, element slowest.
+// Face item t <-> (ab, face, hl), ab fastest, element slowest; face = 2 d + side.
 template <int P>
 struct Item {
-  int ab, side, d, hl;
+  int ab, face, hl;
 };
 
 template <int P>
@@ -206,18 +164,16 @@ __device__ __forceinline__ Item<P> item_of(int t) {
   constexpr int n2 = (P + 1) * (P + 1);
   Item<P> it;
   it.ab = t % n2;
-  int r = t / n2;
-  it.side = r & 1;
-  r >>= 1;
-  it.d = r % 3;
-  it.hl = r / 3;
+  const int r = t / n2;
+  it.face = r % 6;
+  it.hl = r / 6;
   return it;
 }
 
 template <int P>
-__device__ __forceinline__ int item_index(int ab, int side, int d, int hl) {
+__device__ __forceinline__ int item_index(int ab, int face, int hl) {
   constexpr int n2 = (P + 1) * (P + 1);
-  return ab + n2 * (side + 2 * (d + 3 * hl));
+  return ab + n2 * (face + 6 * hl);
 }
 
 // External face items of a cube, t <-> (ab, hl, d), ab fastest, direction slowest (a warp
@@ -229,8 +185,8 @@ __device__ __forceinline__ Item<P> cube_item_of(int t) {
   it.ab = t % n2;
   const int r = t / n2;
   it.hl = r % kCubeElems;
-  it.d = r / kCubeElems;
-  it.side = (it.hl >> it.d) & 1;
+  const int d = r / kCubeElems;
+  it.face = 2 * d + ((it.hl >> d) & 1);
   return it;
 }
 
@@ -240,10 +196,194 @@ __device__ __forceinline__ int cube_item_index(int ab, int d, int hl) {
   return ab + n2 * (hl + kCubeElems * d);
 }
 
-// Internal faces of a cube, u <-> (ab, p, d): face p (0..3) normal to d joins the local
-// elements hlL (bit d clear) and hlL | 1 << d.
-__device__ __forceinline__ int cube_left_of_pair(int p, int d) {
-  return ((p >> d) << (d + 1)) | (p & ((1 << d) - 1));
+// Multiply, add and fused multiply-add with no contraction left to the compiler.
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// ---------------------------------------------------------------- shared-memory tiles
+
+// Four values of a node in shared memory, read and written as vectors: FP32 one plane of
+// 16-byte quads, FP64 two planes of 16-byte pairs (cnt entries each).
+__device__ __forceinline__ void quad_store(float* base, int, int i, const float v[4]) {
+  reinterpret_cast<float4*>(base)[i] = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void quad_store(double* base, int cnt, int i, const double v[4]) {
+  double2* p = reinterpret_cast<double2*>(base);
+  p[i] = make_double2(v[0], v[1]);
+  p[cnt + i] = make_double2(v[2], v[3]);
+}
+__device__ __forceinline__ void quad_load(const float* base, int, int i, float v[4]) {
+  const float4 a = reinterpret_cast<const float4*>(base)[i];
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = a.z;
+  v[3] = a.w;
+}
+__device__ __forceinline__ void quad_load(const double* base, int cnt, int i, double v[4]) {
+  const double2* p = reinterpret_cast<const double2*>(base);
+  const double2 a = p[i], b = p[cnt + i];
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
+}
+
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf).  The FP32 rate is the
+// same as fmaf's (measured 37.4 against 35.6 T multiply-adds/s), the issue slots are half.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 p, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+
+// An entry of the derivative matrix as the contractions use it: FP32 a duplicated pair.
+template <typename T>
+struct DEntry {
+  using type = T;
+  __device__ static __forceinline__ T make(T x) { return x; }
+};
+template <>
+struct DEntry<float> {
+  using type = f32x2;
+  __device__ static __forceinline__ f32x2 make(float x) { return pack2(x, x); }
+};
+
+// Running sum over a line of D entry x quad.
+template <typename T>
+struct QuadSum {
+  T a[4] = {T(0), T(0), T(0), T(0)};
+  __device__ __forceinline__ void add(T d, const T* base, int cnt, int i) {
+    T v[4];
+    quad_load(base, cnt, i, v);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] += d * v[k];
+  }
+  __device__ __forceinline__ void get(T out[4]) const {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = a[k];
+  }
+};
+template <>
+struct QuadSum<float> {
+  f32x2 a[2] = {0ull, 0ull};
+  __device__ __forceinline__ void add(f32x2 d, const float* base, int, int i) {
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(base)[i];
+    fma2(a[0], d, v.x);
+    fma2(a[1], d, v.y);
+  }
+  __device__ __forceinline__ void get(float out[4]) const {
+    unpack2(a[0], out[0], out[1]);
+    unpack2(a[1], out[2], out[3]);
+  }
+};
+__device__ __forceinline__ double d_scalar(double d) { return d; }
+__device__ __forceinline__ float d_scalar(f32x2 d) {
+  float a, b;
+  unpack2(d, a, b);
+  return a;
+}
+
+// ---------------------------------------------------------------- line contractions
+
+// FP32 at P >= 5: the contractions run line by line, one task per (direction, pair of
+// components, line) computing the derivative at every node of the line, so that each
+// operand is read from shared memory once per line instead of once per output node.
+template <typename T>
+__host__ __device__ constexpr bool use_lines(int P) {
+  return std::is_same<T, float>::value && P >= 5;
+}
+// Shared-memory index of a node: rows of odd length, so that the lanes of a warp reading
+// consecutive x-lines fall on different banks.
+__host__ __device__ constexpr int line_row(int n) { return n | 1; }
+__host__ __device__ constexpr int line_nodes(int n) { return line_row(n) * n * n; }
+
+// The derivative matrix changes sign when rows and columns are reversed, D[P-i][P-m] =
+// -D[i][m], so a line's derivative splits into the sums and differences of its mirrored
+// values: with e_m = f_m + f_{P-m}, o_m = f_m - f_{P-m},
+//   E_i = sum_m (D[i][m] + D[i][P-m])/2 e_m (+ D[i][c] f_c),  O_i = sum_m (D[i][m] - D[i][P-m])/2 o_m,
+//   out_i = O_i + E_i,  out_{P-i} = O_i - E_i,  m < n/2, c the middle node of an odd n.
+// That is about half the multiply-adds and half the matrix entries.  The energy flux has a
+// large common part at low Mach numbers, whose rounding the sums e_m would double; D
+// annihilates constants, so its lines (REF) are taken relative to a node r of the line,
+// e_m = (f_m - f_r) + (f_{P-m} - f_r), with r = c for an odd n and n/2 - 1 for an even one
+// (16^3/P8 RK3 step against 64 bits: 4.6e-10 as a plain sum, 5.7e-10 without r, 4.3e-10 with).
+// c_D32 holds the entries of every order as duplicated FP32 pairs, in constant memory (one
+// copy per translation unit, filled by upload_const_D on the host before the first launch):
+// row i (i <= n/2): the E entries (n+1)/2, then the O entries n/2.  Read with compile-time
+// indices.
+__constant__ float2 c_D32[kMaxP + 1][kMaxN1 * kMaxN1];
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 line_add(f32x2 a, f32x2 b) { return add2(a, b); }
+__device__ __forceinline__ f32x2 line_sub(f32x2 a, f32x2 b) {   // a - b in one instruction: -1 x b + a
+  fma2(a, 0xBF800000BF800000ull, b);
+  return a;
+}
+__device__ __forceinline__ float line_add(float a, float b) { return a + b; }
+__device__ __forceinline__ float line_sub(float a, float b) { return a - b; }
+__device__ __forceinline__ void line_fma(f32x2& acc, float2 d, f32x2 v) { fma2(acc, pack2(d.x, d.y), v); }
+__device__ __forceinline__ void line_fma(float& acc, float2 d, float v) { acc = fmaf(d.x, v, acc); }
+
+// out[node(i)] = sum_m D[i][m] f[node(m)], i = 0..P, for the line of nodes along direction
+// D with tangential index ab; f and out may be the same array (the line's values are all
+// read before any is written, and no other task touches the line).
+template <int P, int D, bool REF, typename V>
+__device__ __forceinline__ void line_derivative(const V* f, V* out, int ab) {
+  constexpr int n = P + 1, rs = line_row(n), h = n / 2, he = (n + 1) / 2;
+  constexpr int ne = REF ? h : he;   // the reference is the middle node of an odd n: its entry drops out
+  const int a = ab % n, b = ab / n;
+  const int base = D == 0 ? rs * (a + n * b) : D == 1 ? a + rs * n * b : a + rs * b;
+  constexpr int st = D == 0 ? 1 : D == 1 ? rs : rs * n;
+  V e[ne], o[h];
+  V r = V(0);
+  if (REF) r = f[base + (n & 1 ? h : h - 1) * st];
+#pragma unroll
+  for (int m = 0; m < h; ++m) {
+    const V x = f[base + m * st], y = f[base + (P - m) * st];
+    if (!REF) e[m] = line_add(x, y);
+    else if (!(n & 1) && m == h - 1) e[m] = line_sub(y, r);   // f_m is the reference itself
+    else e[m] = line_add(line_sub(x, r), line_sub(y, r));
+    o[m] = line_sub(x, y);
+  }
+  if (!REF && (n & 1)) e[ne - 1] = f[base + h * st];
+#pragma unroll
+  for (int i = 0; i < h; ++i) {
+    V E = V(0), O = V(0);
+#pragma unroll
+    for (int m = 0; m < ne; ++m) line_fma(E, c_D32[P][i * n + m], e[m]);
+#pragma unroll
+    for (int m = 0; m < h; ++m) line_fma(O, c_D32[P][i * n + he + m], o[m]);
+    out[base + i * st] = line_add(O, E);
+    out[base + (P - i) * st] = line_sub(O, E);
+  }
+  if (n & 1) {   // the middle row: D[c][P-m] = -D[c][m]
+    V O = V(0);
+#pragma unroll
+    for (int m = 0; m < h; ++m) line_fma(O, c_D32[P][h * n + he + m], o[m]);
+    out[base + h * st] = O;
+  }
+}
+
+template <int P, bool REF, typename V>
+__device__ __forceinline__ void line_derivative_dir(int d, const V* f, V* out, int ab) {
+  if (d == 0) line_derivative<P, 0, REF>(f, out, ab);
+  else if (d == 1) line_derivative<P, 1, REF>(f, out, ab);
+  else line_derivative<P, 2, REF>(f, out, ab);
 }
 
 template <typename T>
@@ -251,24 +391,17 @@ __device__ __forceinline__ Prim<T> prim_c(const T s[5], const OpConst<T>& C) {
   return primitives(s, C.rho_ref, C.gm1);
 }
 
-// Stage state of node gi.  SRC 0: from the FP64 state q; SRC 1: qn32 + dlt (FP32).
-template <typename T, int SRC>
-__device__ __forceinline__ void stage_state(const double* __restrict__ q, const float* __restrict__ qn32,
-                                            const float* __restrict__ dlt, long long N, long long gi,
-                                            const OpConst<T>& C, T s[5]) {
-  if (SRC == 0) {
-    double qd[5];
+// Stage state of an element's node from the FP64 state q ([var][node], gi = elem n^3 + node).
+template <typename T>
+__device__ __forceinline__ void state_from_q(const double* __restrict__ q, long long gi, const OpConst<T>& C, T s[5]) {
+  double qd[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) qd[v] = q[v * N + gi];
-    s[0] = from_double<T>(qd[0] - C.drho_ref);
-    s[1] = from_double<T>(qd[1]);
-    s[2] = from_double<T>(qd[2]);
-    s[3] = from_double<T>(qd[3]);
-    s[4] = from_double<T>(qd[4] - C.dE_ref);
-  } else {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) s[v] = T(qn32[v * N + gi] + dlt[v * N + gi]);
-  }
+  for (int v = 0; v < 5; ++v) qd[v] = q[v * C.N + gi];
+  s[0] = from_double<T>(qd[0] - C.drho_ref);
+  s[1] = from_double<T>(qd[1]);
+  s[2] = from_double<T>(qd[2]);
+  s[3] = from_double<T>(qd[3]);
+  s[4] = from_double<T>(qd[4] - C.dE_ref);
 }
 
 // Effective viscosity and heat coefficient (Smagorinsky when les != 0).
@@ -290,315 +423,6 @@ __device__ __forceinline__ void transport_c(const OpConst<T>& C, T rho, const T 
   }
   *mu = m;
   *lam = l;
-}
-
-// Phase A of block `blk` of one mesh (the body of k_gradient and k_gradient_batch).
-// CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the external
-// faces, internal faces take the neighbour's values from the own tile.  SLAB: a slab of
-// element layers (owned range from C.e_begin, C.Kz local layers); a whole mesh compiles
-// without it.  FEAT: also write the forcing network's input features (C.feat).
-template <int P, typename T, int SRC, bool CUBE = false, bool SLAB = false, bool FEAT = false>
-__device__ __forceinline__ void gradient_block(int blk, const double* __restrict__ q,
-                                               const float* __restrict__ qn32_in, const float* __restrict__ dlt,
-                                               T* __restrict__ qf, float* __restrict__ qn32_out,
-                                               T* __restrict__ vis, const OpConst<T>& C) {
-  constexpr int n = P + 1, n2 = n * n, np = n2 * n;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int E = CUBE ? kCubeElems : C.E;
-  const int tileN = E * np;
-  const int haloN = CUBE ? 3 * kCubeElems * n2 : E * 6 * n2;
-  T* sD = reinterpret_cast<T*>(smem_raw);
-  T* sU = sD + n2;            // [4][E np]
-  T* sH = sU + 4 * tileN;     // [4][haloN]: neighbours' gradient variables on the (external) faces
-  const int e0 = (SLAB ? C.e_begin : 0) + blk * E;
-  const BlockCoords bc = CUBE ? cube_coords(blk, C.K) : block_coords(e0, C.K);
-  for (int t = threadIdx.x; t < n2; t += blockDim.x) sD[t] = C.D[t];
-
-  const int le = threadIdx.x / np;
-  const int node = threadIdx.x - le * np;
-  const int e = CUBE ? cube_element(bc, le, C.K) : e0 + le;
-  const bool active = CUBE ? (le < kCubeElems) : (le < E) && (e < C.nel);
-  const long long N = C.N;
-  const long long gi = (long long)e * np + node;
-
-  T s[5], U[4];
-  Prim<T> w;
-  if (active) {
-    stage_state<T, SRC>(q, qn32_in, dlt, N, gi, C, s);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) qf[v * N + gi] = s[v];
-    if (SRC == 0 && qn32_out != nullptr) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) qn32_out[v * N + gi] = float(s[v]);
-    }
-    if (FEAT) {
-      // the forcing network's input features of this node, from the stage state just
-      // formed: the same arithmetic as the separate feature kernels of the network
-      __nv_bfloat16* fo = static_cast<__nv_bfloat16*>(C.feat.out) + (long long)e * C.feat.ld + node;
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const int slot = v - C.feat.first_var;
-        if (slot < 0 || slot >= C.feat.n_vars) continue;
-        const int f = slot * np + node;
-        float x;
-        if constexpr (sizeof(T) == 4) x = (float(s[v]) - C.feat.shift32[f]) / C.feat.sd[f];
-        else x = d2f_rn(double(s[v]) - C.feat.mean64[f]) / C.feat.sd[f];
-        fo[slot * np] = __float2bfloat16_rn(x);
-      }
-    }
-    w = prim_c(s, C);
-    gradient_vars(s, w, C.theta_ref, U);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) sU[a * tileN + le * np + node] = U[a];
-  }
-  // halo: gradient variables of the neighbours' face nodes
-  for (int t = threadIdx.x; t < haloN; t += blockDim.x) {
-    const Item<P> it = CUBE ? cube_item_of<P>(t) : item_of<P>(t);
-    if (!CUBE && e0 + it.hl >= C.nel) continue;
-    const int enb = CUBE ? cube_neighbour(bc, it.hl, C.K, it.d, it.side ? 1 : -1)
-                         : neighbour_of(bc, it.hl, C.K, SLAB ? C.Kz : C.K, it.d, it.side ? 1 : -1);
-    const long long gnb = (long long)enb * np + face_node<P>(it.d, it.side ? 0 : P, it.ab);
-    T sn[5], Un[4];
-    stage_state<T, SRC>(q, qn32_in, dlt, N, gnb, C, sn);
-    const Prim<T> wn = prim_c(sn, C);
-    gradient_vars(sn, wn, C.theta_ref, Un);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) sH[a * haloN + t] = Un[a];
-  }
-  __syncthreads();
-  // FP32 at P >= 7 (one element per block): line-wise contraction, one task per
-  // (direction, variable, line) computing the derivative at every node of the line into
-  // sG [3][4][np]; each operand is read from shared memory once per line (measured: -5 %
-  // at P = 8, +5 % at P = 6, where the extra barrier and buffer cost more than they save)
-  constexpr bool kLines = std::is_same<T, float>::value && P >= 7;
-  T* sG = sH + 4 * haloN;
-  if constexpr (kLines) {
-    if (E == 1) {
-      for (int task = threadIdx.x; task < 12 * n2; task += blockDim.x) {
-        const int da = task / n2, ab = task - da * n2;
-        const float* f = reinterpret_cast<const float*>(sU) + (da % 4) * np;
-        float* o = reinterpret_cast<float*>(sG) + da * np;
-        if (da < 4) line_derivative<P, 0>(f, o, ab);
-        else if (da < 8) line_derivative<P, 1>(f, o, ab);
-        else line_derivative<P, 2>(f, o, ab);
-      }
-      __syncthreads();
-    }
-  }
-  if (!active) return;
-
-  const int idx[3] = {node % n, (node / n) % n, node / n2};
-  const int stride[3] = {1, n, n2};
-  const T lift = C.s2h * C.winv * T(0.5);
-  T G[3][4];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const T* Drow = sD + idx[d] * n;
-    const int base = le * np + node - idx[d] * stride[d];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      T acc = T(0);
-      if (kLines && E == 1) {
-        acc = sG[(4 * d + a) * np + node];
-      } else if (P == 3 && !CUBE && std::is_same<T, float>::value && d < 2) {
-        // P3 rows: an element's 64 nodes are two whole warps (node i + 4 j + 16 k), so its
-        // x- and y-lines lie within one warp: the line's values come by warp shuffles of
-        // the threads' own U (same products, same order: the same bits as from shared
-        // memory; measured -1 % per 32^3 RK3 step); z-lines span the two warps
-        const int l0 = (threadIdx.x & 31) - idx[d] * stride[d];
-#pragma unroll
-        for (int m = 0; m < n; ++m) acc += Drow[m] * __shfl_sync(0xffffffffu, U[a], l0 + m * stride[d]);
-      } else {
-#pragma unroll
-        for (int m = 0; m < n; ++m) acc += Drow[m] * sU[a * tileN + base + m * stride[d]];
-      }
-      G[d][a] = C.s2h * acc;
-    }
-    // interface lifting with the central U^ = (U + U_nb) / 2
-    const bool right = (idx[d] == P), left = (idx[d] == 0);
-    if (right || left) {
-      const int ab = face_ab<P>(d, idx);
-      const T sgn = right ? lift : -lift;
-      const T* nb;  // the neighbour's four values, stride st
-      int st;
-      if (CUBE && (right ? 1 : 0) != ((le >> d) & 1)) {
-        nb = sU + (le ^ (1 << d)) * np + face_node<P>(d, right ? 0 : P, ab);   // internal face
-        st = tileN;
-      } else {
-        nb = sH + (CUBE ? cube_item_index<P>(ab, d, le) : item_index<P>(ab, right ? 1 : 0, d, le));
-        st = haloN;
-      }
-#pragma unroll
-      for (int a = 0; a < 4; ++a) G[d][a] += sgn * (nb[a * st] - U[a]);
-    }
-  }
-
-  T mu, lam;
-  transport_c(C, w.rho, G, &mu, &lam);
-  const T div = G[0][0] + G[1][1] + G[2][2];
-  const T t23 = T(2.0 / 3.0) * mu * div;
-  // G[d][a] = d u_a / d x_d, tau_ab = mu (du_a/dx_b + du_b/dx_a) - 2/3 mu div delta_ab
-  T out[9];
-  out[0] = T(2) * mu * G[0][0] - t23;
-  out[1] = T(2) * mu * G[1][1] - t23;
-  out[2] = T(2) * mu * G[2][2] - t23;
-  out[3] = mu * (G[1][0] + G[0][1]);
-  out[4] = mu * (G[2][0] + G[0][2]);
-  out[5] = mu * (G[2][1] + G[1][2]);
-  out[6] = lam * G[0][3];
-  out[7] = lam * G[1][3];
-  out[8] = lam * G[2][3];
-#pragma unroll
-  for (int c = 0; c < 9; ++c) vis[c * N + gi] = out[c];
-}
-
-template <int P, typename T, int SRC, bool CUBE = false, bool SLAB = false, bool FEAT = false>
-__global__ void __launch_bounds__(max_threads_for(P))
-k_gradient(const double* __restrict__ q, const float* __restrict__ qn32_in, const float* __restrict__ dlt,
-           T* __restrict__ qf, float* __restrict__ qn32_out, T* __restrict__ vis, const OpConst<T> C) {
-  pdl_wait();
-  pdl_release();
-  gradient_block<P, T, SRC, CUBE, SLAB, FEAT>(blockIdx.x, q, qn32_in, dlt, qf, qn32_out, vis, C);
-}
-
-// Per-launch RK data of phase B in the arithmetic of the update.
-template <typename R>
-struct RkArgs {
-  R A, B, dt;   // Williamson coefficients of the stage and the step size
-  R invB1;      // 1 / B of stage 1 (the FP32 increment scheme recovers g1 = dlt1 / B1)
-};
-
-// Halo and own-node components of an interface item: stage state (5) and the viscous
-// quantities entering the flux normal to the face (tau_0d, tau_1d, tau_2d, k theta_d).
-constexpr int kFaceComponents = 9;
-// Components of the own-element tile: stage state (5) and all viscous quantities (9);
-// the tile is reused for the three directions' volume fluxes (15).
-constexpr int kTileComponents = 15;
-
-// Column D of the viscous flux from the face-normal viscous quantities t4 = (tau_0D,
-// tau_1D, tau_2D, k theta_D): (0, tau_0D, tau_1D, tau_2D, v . tau_D + k theta_D).
-template <typename T>
-__device__ __forceinline__ void viscous_flux4(const T t4[4], const T v[3], T f[5]) {
-  f[0] = T(0);
-  f[1] = t4[0];
-  f[2] = t4[1];
-  f[3] = t4[2];
-  f[4] = v[0] * t4[0] + v[1] * t4[1] + v[2] * t4[2] + t4[3];
-}
-
-// One interface work item normal to D (compile-time, so flux arrays stay in registers):
-//   F* - F = (f_nb - f_own - diss)/2 + (f^nu_own - f^nu_nb)/2, lifted with -/+ (2/h)/w on
-// the right / left face; diss = |A~|(q_R - q_L) in the face's left/right order.
-template <int D, typename T>
-__device__ __forceinline__ void interface_item(const T so[5], const T to[4], const T sn[5], const T tn[4], T* out,
-                                               int ostride, int side, const OpConst<T>& C) {
-  const Prim<T> wo = primitives(so, C.rho_ref, C.gm1), wn = primitives(sn, C.rho_ref, C.gm1);
-  T fo[5], fnb[5], fvo[5], fvn[5], diss[5];
-  euler_flux(so, wo, C.Hc, D, fo);
-  euler_flux(sn, wn, C.Hc, D, fnb);
-  {
-    // the face's left and right states by selection, not by branching: the two sides of
-    // a face sit in one warp, and a branch would run the Roe solver twice
-    T sL[5], sR[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      sL[v] = side ? so[v] : sn[v];
-      sR[v] = side ? sn[v] : so[v];
-    }
-    Prim<T> wL, wR;
-    wL.rho = side ? wo.rho : wn.rho;
-    wR.rho = side ? wn.rho : wo.rho;
-    wL.ir = side ? wo.ir : wn.ir;
-    wR.ir = side ? wn.ir : wo.ir;
-    wL.pp = side ? wo.pp : wn.pp;
-    wR.pp = side ? wn.pp : wo.pp;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      wL.v[i] = side ? wo.v[i] : wn.v[i];
-      wR.v[i] = side ? wn.v[i] : wo.v[i];
-    }
-    roe_dissipation(sL, wL, sR, wR, D, C.gm1, C.Hc, diss);
-  }
-  viscous_flux4(to, wo.v, fvo);
-  viscous_flux4(tn, wn.v, fvn);
-  const T lift = C.s2h * C.winv;
-  const T sgn = side ? -lift : lift;
-  if (sizeof(T) == 8) {
-    // FP64 parity path: the plain form, F* assembled first and F subtracted after
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const T fstar = T(0.5) * (fo[c] + fnb[c] - diss[c]) - T(0.5) * (fvo[c] + fvn[c]);
-      out[c * ostride] = sgn * (fstar - (fo[c] - fvo[c]));
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 5; ++c)
-      out[c * ostride] = sgn * (T(0.5) * (fnb[c] - fo[c] - diss[c]) + T(0.5) * (fvo[c] - fvn[c]));
-  }
-}
-
-// Both sides of an internal face of a cube at once: the Roe dissipation, fluxes and
-// primitives are formed once; each side's lifted term is the expression interface_item
-// evaluates for it (own = left element on its side 1, own = right element on its side 0).
-template <int D, typename T>
-__device__ __forceinline__ void interface_pair(const T sl[5], const T tl[4], const T sr[5], const T tr[4], T* outL,
-                                               T* outR, int ostride, const OpConst<T>& C) {
-  const Prim<T> wl = primitives(sl, C.rho_ref, C.gm1), wr = primitives(sr, C.rho_ref, C.gm1);
-  T fl[5], fr[5], fvl[5], fvr[5], diss[5];
-  euler_flux(sl, wl, C.Hc, D, fl);
-  euler_flux(sr, wr, C.Hc, D, fr);
-  roe_dissipation(sl, wl, sr, wr, D, C.gm1, C.Hc, diss);
-  viscous_flux4(tl, wl.v, fvl);
-  viscous_flux4(tr, wr.v, fvr);
-  const T lift = C.s2h * C.winv;
-  if (sizeof(T) == 8) {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const T fstar = T(0.5) * (fl[c] + fr[c] - diss[c]) - T(0.5) * (fvl[c] + fvr[c]);
-      outL[c * ostride] = -lift * (fstar - (fl[c] - fvl[c]));
-      outR[c * ostride] = lift * (fstar - (fr[c] - fvr[c]));
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      outL[c * ostride] = -lift * (T(0.5) * (fr[c] - fl[c] - diss[c]) + T(0.5) * (fvl[c] - fvr[c]));
-      outR[c * ostride] = lift * (T(0.5) * (fl[c] - fr[c] - diss[c]) + T(0.5) * (fvr[c] - fvl[c]));
-    }
-  }
-}
-
-// Index of viscous component i of the face-normal set of direction d in the 9-vector.
-__device__ __forceinline__ int face_vis_index(int d, int i) { return i < 3 ? sym_index(i, d) : 6 + d; }
-
-// Halo entry t of a phase-B block: the neighbour's stage state (5) and its viscous
-// quantities normal to the face (4), for a face normal to D (compile-time, so the
-// component offsets are constants).
-template <int D, typename T>
-__device__ __forceinline__ void load_face_data(const T* __restrict__ qf, const T* __restrict__ vis, long long N,
-                                               long long g, T* dst, int stride) {
-  const T* s = qf + g;
-  const T* w = vis + g;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) dst[v * stride] = s[v * N];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) dst[(5 + i) * stride] = w[face_vis_index(D, i) * N];
-}
-
-// Nodes per thread of the flux kernel.  At P >= 6 one element has 343 to 729 nodes; two
-// nodes per thread halve the block so that more blocks fit an SM's registers and one
-// block's barriers overlap the others' work.
-__host__ __device__ constexpr int flux_npt(int P) { return P >= 6 ? 2 : 1; }
-
-// Maximum threads per flux block.
-__host__ __device__ constexpr int flux_max_threads(int P) {
-  return flux_npt(P) == 1 ? max_threads_for(P) : ((max_threads_for(P) / 2 + 31) / 32) * 32;
-}
-
-// Blocks per SM the flux kernel is compiled for (register budget, about 80 registers per
-// thread in FP32): several, so that one block's barriers overlap another's work; one in
-// FP64 (the parity path), whose doubled register footprint would otherwise spill.
-__host__ __device__ constexpr int min_blocks_for(int P, int tsize) {
-  return tsize == 8 ? 1 : P == 6 ? 4 : P == 7 ? 3 : 2;
 }
 
 // Split form: a node's primitives for the two-point flux, (rho, v1, v2, v3, p', H) with
@@ -627,365 +451,1127 @@ __device__ __forceinline__ void kep_flux_prims(const T a[6], const T b[6], int d
   F[4] = m * (T(0.5) * (a[5] + b[5]));
 }
 
-// Phase B forms the volume fluxes before the interface phase, in a tile of their own
-// (FP32 at P = 4, 5, one node per thread): one barrier less for a larger shared
-// footprint.  Measured per RK3 step, 24^3/P4 408 vs 415 us, 20^3/P5 431 vs 439 us, but
-// 32^3/P3 465 vs 458 us, so P <= 3 and FP64 keep the smaller footprint.
-__host__ __device__ constexpr bool flux_early(int P, int tsize) { return tsize == 4 && (P == 4 || P == 5); }
 
-// MODE 0: dqdt = R.  MODE 1: FP64 RK stage (g = A g + dt R; q += B g).
-// MODES 2, 3, 4: FP32 increment scheme, stages 1, 2, 3.
-// Phase B of block `blk` of one mesh (the body of k_flux and k_flux_batch).
-//
-// Thread j-th node: tile index tix = threadIdx.x + j blockDim.x, j < NPT.  With one node
-// per thread the own state and viscous values stay in registers across the interface
-// phase and the RK operands are loaded first; with two, they are read back from the
-// tile and the RK operands are loaded after the interface phase (register budget).
-// CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the external
-// faces, and each internal face is one work item that writes both sides' lifted terms.
-// SPLIT: the Euler part of the volume term in the kinetic-energy-preserving split form,
-// 2 sum_m D_im F#(q_i, q_m) along each line with Pirozzoli's two-point flux F# (mass flux
-// {rho}{v_d}; momentum m {v_j} + {p'} delta_jd; energy m {H}), from a tile of primitives;
-// the viscous part and the surface terms keep the standard form.
-template <int P, typename T, int MODE, bool CUBE = false, bool SPLIT = false, bool SLAB = false>
-__device__ __forceinline__ void flux_block(int blk, double* __restrict__ q, const T* __restrict__ qf,
-                                           const T* __restrict__ vis, double* __restrict__ dqdt,
-                                           T* __restrict__ greg, float* __restrict__ dlt, const Forcing& fc,
-                                           const OpConst<T>& C, const RkArgs<T>& rk) {
-  constexpr int n = P + 1, n2 = n * n, np = n2 * n;
-  constexpr int FC = kFaceComponents;
-  constexpr int NPT = flux_npt(P);
-  constexpr bool kHold = (NPT == 1);
+// Shared memory of a phase-A block (values of T unless said otherwise), in this order:
+// neighbour elements [6 E] (int), D entries [n^2] (direct contraction), then
+//   direct: U quads [4][E np], halo quads [4][faces], flux quads [3][4][E np] and energy
+//           fluxes [3][E np] (quads need 16-byte alignment), split form: primitives [6][E np];
+//   lines:  U pairs [2][E ln], halo pairs [2][faces], derivatives and then fluxes pairs
+//           [6][E ln], energy fluxes [3][E ln], split form: primitives [6][E np].
+template <int P, typename T>
+__host__ __device__ constexpr size_t volume_smem_bytes(int E, int faces, bool split) {
+  constexpr int n = P + 1, n2 = n * n, np = n2 * n, ln = line_nodes(n);
+  const size_t head = ((6 * E + 3) & ~3) * sizeof(int);
+  const size_t prims = split ? (size_t)6 * E * np : 0;
+  if (use_lines<T>(P)) return head + sizeof(float) * ((size_t)E * ln * (4 + 12 + 3) + 4 * (size_t)faces + prims);
+  return head + sizeof(typename DEntry<T>::type) * ((n2 + 1) & ~1) + sizeof(T) * ((size_t)E * np * (4 + 15) + 4 * (size_t)faces + prims);
+}
+
+// Phase A of block `blk` of one mesh (the body of k_volume and k_volume_batch).
+// SRC 0: the stage state is formed from the FP64 state q and written to qf; SRC 1: it is
+// read from qf.  CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the
+// external faces, internal faces take the neighbour's values from the own tile.  FEAT:
+// also write the forcing network's input features (C.feat).  SPLIT: the Euler part of the
+// volume term in the kinetic-energy-preserving split form, 2 sum_m D_im F#(q_i, q_m) along
+// each line with Pirozzoli's two-point flux F# (mass flux {rho}{v_d}; momentum m {v_j} +
+// {p'} delta_jd; energy m {H}), from a tile of primitives; the viscous part keeps the
+// standard form.
+template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
+__device__ __forceinline__ void volume_block(int blk, const double* __restrict__ q, T* __restrict__ qf,
+                                             T* __restrict__ rv, T* __restrict__ vt, const OpConst<T>& C) {
+  constexpr int n = P + 1, n2 = n * n, np = n2 * n, ns = node_stride(n);
+  constexpr bool kLines = use_lines<T>(P);
+  constexpr int tn = kLines ? line_nodes(n) : np;   // tile entries per element
+  using DT = typename DEntry<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int E = CUBE ? kCubeElems : C.E;
-  const int tileN = E * np;
-  const int faceN = E * 6 * n2;                          // lifted terms: every face of every element
-  const int haloN = CUBE ? 3 * kCubeElems * n2 : faceN;  // neighbours' face data: external faces
-  // flux_early: the volume fluxes are formed right after the own loads, into their own
-  // tile, so that the interface phase and the contraction need one barrier less.
-  // Otherwise they overwrite the own tile after the interface phase (register and
-  // shared-memory budget).
-  constexpr bool kEarlyF = flux_early(P, sizeof(T));
-  T* sD = reinterpret_cast<T*>(smem_raw);
-  T* sX = sD + n2;                        // own data [14][E np] (late fluxes: [15], then the fluxes)
-  T* sF = kEarlyF ? sX + 14 * tileN : sX; // [15][E np]: volume fluxes
-  T* sH = kEarlyF ? sF + kTileComponents * tileN : sX + kTileComponents * tileN;  // [9][E 6 n2]
-  T* sS = sH + FC * haloN;                // [5][E 6 n2]: lifted interface terms
-  T* sW = sS + 5 * faceN;                 // SPLIT: primitives [6][E np] (rho, v, p', H)
-  const int e0 = (SLAB ? C.e_begin : 0) + blk * E;
-  const BlockCoords bc = CUBE ? cube_coords(blk, C.K) : block_coords(e0, C.K);
-  for (int t = threadIdx.x; t < n2; t += blockDim.x) sD[t] = C.D[t];
-  const long long N = C.N;
+  const int tileN = E * tn;
+  const int haloN = CUBE ? 3 * kCubeElems * n2 : E * 6 * n2;
+  int* sNb = reinterpret_cast<int*>(smem_raw);                      // element across each face
+  DT* sD = reinterpret_cast<DT*>(sNb + ((6 * E + 3) & ~3));         // direct contraction only
+  T* sU = kLines ? reinterpret_cast<T*>(sD) : reinterpret_cast<T*>(sD + ((n2 + 1) & ~1));
+  T* sH = sU + 4 * tileN;                                           // neighbours' gradient variables
+  T* sF = sH + 4 * haloN;
+  const int e0 = C.e_begin + blk * E;
+  const BlockCoords bc = CUBE ? cube_coords(blk, C.K) : BlockCoords{0, 0, 0};
 
-  int le[NPT], node[NPT], tix[NPT];
-  long long gi[NPT];
-  bool active[NPT];
+  const int le = threadIdx.x / np;
+  const int node = threadIdx.x - le * np;
+  const int e = CUBE ? cube_element(bc, le, C.K) : e0 + le;
+  const bool active = CUBE ? (le < kCubeElems) : (le < E) && (e < C.nel);
+  T* qe = qf + (size_t)e * state_record(n) + node;
+
+  T s[5];
+  if (active) {
+    if (SRC == 0) {
+      state_from_q(q, (long long)e * np + node, C, s);
 #pragma unroll
-  for (int j = 0; j < NPT; ++j) {
-    tix[j] = threadIdx.x + j * blockDim.x;
-    le[j] = tix[j] / np;
-    node[j] = tix[j] - le[j] * np;
-    active[j] = CUBE ? (le[j] < kCubeElems) : (le[j] < E) && (e0 + le[j] < C.nel);
-    gi[j] = (long long)(CUBE ? cube_element(bc, le[j], C.K) : e0 + le[j]) * np + node[j];
+      for (int v = 0; v < 5; ++v) qe[v * ns] = s[v];
+    } else {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) s[v] = qe[v * ns];
+    }
+  }
+  // set-up that the own loads' latency covers
+  for (int t = threadIdx.x; t < 6 * E; t += blockDim.x) {
+    const int hl = t / 6, eh = CUBE ? cube_element(bc, hl, C.K) : e0 + hl;
+    sNb[t] = element_across(eh, t - 6 * hl, C.K, C.Kz);
+  }
+  if (!kLines)
+    for (int t = threadIdx.x; t < n2; t += blockDim.x) sD[t] = DEntry<T>::make(C.D[t]);
+  __syncthreads();
+
+  // halo: gradient variables of the neighbours' face nodes
+  for (int t = threadIdx.x; t < haloN; t += blockDim.x) {
+    const Item<P> it = CUBE ? cube_item_of<P>(t) : item_of<P>(t);
+    if (!CUBE && e0 + it.hl >= C.nel) continue;
+    const int enb = sNb[6 * it.hl + it.face];
+    const int fn = face_node<P>(it.face >> 1, (it.face & 1) ? 0 : P, it.ab);
+    T sn[5], Un[4];
+    if (SRC == 0) {
+      state_from_q(q, (long long)enb * np + fn, C, sn);
+    } else {
+      const T* qn = qf + (size_t)enb * state_record(n) + fn;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sn[v] = qn[v * ns];
+    }
+    const Prim<T> wn = prim_c(sn, C);
+    gradient_vars(sn, wn, C.theta_ref, Un);
+    if constexpr (kLines) {
+      f32x2* h = reinterpret_cast<f32x2*>(sH);
+      h[t] = pack2(Un[0], Un[1]);
+      h[haloN + t] = pack2(Un[2], Un[3]);
+    } else {
+      quad_store(sH, haloN, t, Un);
+    }
   }
 
-  // RK operands of the update (loaded first with one node per thread, late with two)
-  T gold[NPT][5], dold[NPT][5];
-  // P3 rows in FP32: the x- and y-direction volume fluxes stay in registers and the
-  // contraction takes a line's values by warp shuffles (an element is two whole warps, its
-  // x- and y-lines lie within one); the z-fluxes go through shared memory
-  constexpr bool kShfl = (P == 3) && !CUBE && !SPLIT && std::is_same<T, float>::value && !flux_early(P, sizeof(T));
-  T Fr[NPT][2][5];
-  auto load_rk = [&](int j) {
-    if (MODE == 3 || MODE == 4) {
+  const int idx[3] = {node % n, (node / n) % n, node / n2};
+  const int ti = kLines ? le * tn + node + (node / n) * (line_row(n) - n) : le * np + node;  // own tile entry
+  T U[4];
+  Prim<T> w;
+  if (active) {
+    if (FEAT) {
+      // the forcing network's input features of this node, from the stage state: the same
+      // arithmetic as the separate feature kernels of the network
+      __nv_bfloat16* fo = static_cast<__nv_bfloat16*>(C.feat.out) + (long long)e * C.feat.ld + node;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) dold[j][v] = T(dlt[v * N + gi[j]]);
-    }
-    if (MODE == 4 || MODE == 1) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) gold[j][v] = (MODE == 1 && rk.A == T(0)) ? T(0) : greg[v * N + gi[j]];
-      // the FP64 state is read only by the final update: start its lines towards L1 now, so
-      // that read does not wait on DRAM at the end of the block (no registers held)
-#pragma unroll
-      for (int v = 0; v < 5; ++v) asm volatile("prefetch.global.L1 [%0];" ::"l"(q + v * N + gi[j]));
-    }
-    if (fc.s != nullptr) {   // likewise the forcing, added to R at the end
-      const float* fs = fc.s + (gi[j] / np) * fc.stride + node[j];
-      for (int slot = 0; slot < fc.n_vars; ++slot) asm volatile("prefetch.global.L1 [%0];" ::"l"(fs + slot * np));
-    }
-  };
-
-  // own loads first (all independent)
-  T s[NPT][5], vs[NPT][9];
-  auto own_loads = [&](int j) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) s[j][v] = qf[v * N + gi[j]];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) vs[j][c] = vis[c * N + gi[j]];
-    if (kHold) load_rk(j);
-  };
-  auto own_stores = [&](int j) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) sX[v * tileN + tix[j]] = s[j][v];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) sX[(5 + c) * tileN + tix[j]] = vs[j][c];
-    if (kEarlyF) {
-      const Prim<T> w = prim_c(s[j], C);
-      if (SPLIT) store_split_prims(s[j], w, C, sW + tix[j], tileN);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        T F[5], fv[5];
-        euler_flux(s[j], w, C.Hc, d, F);
-        viscous_flux(vs[j], w.v, d, fv);
-#pragma unroll
-        for (int c = 0; c < 5; ++c) sF[(5 * d + c) * tileN + tix[j]] = SPLIT ? -fv[c] : F[c] - fv[c];
+      for (int v = 0; v < 5; ++v) {
+        const int slot = v - C.feat.first_var;
+        if (slot < 0 || slot >= C.feat.n_vars) continue;
+        const int f = slot * np + node;
+        float x;
+        if constexpr (sizeof(T) == 4) x = (float(s[v]) - C.feat.shift32[f]) / C.feat.sd[f];
+        else x = d2f_rn(double(s[v]) - C.feat.mean64[f]) / C.feat.sd[f];
+        fo[slot * np] = __float2bfloat16_rn(x);
       }
     }
-  };
-  // halo: neighbours' stage state and face-normal viscous quantities on every face
-  auto halo_gather = [&]() {
-    for (int t = threadIdx.x; t < haloN; t += blockDim.x) {
-      const Item<P> it = CUBE ? cube_item_of<P>(t) : item_of<P>(t);
-      if (!CUBE && e0 + it.hl >= C.nel) continue;
-      const int enb = CUBE ? cube_neighbour(bc, it.hl, C.K, it.d, it.side ? 1 : -1)
-                           : neighbour_of(bc, it.hl, C.K, SLAB ? C.Kz : C.K, it.d, it.side ? 1 : -1);
-      const long long gnb = (long long)enb * np + face_node<P>(it.d, it.side ? 0 : P, it.ab);
-      switch (it.d) {
-        case 0: load_face_data<0>(qf, vis, N, gnb, sH + t, haloN); break;
-        case 1: load_face_data<1>(qf, vis, N, gnb, sH + t, haloN); break;
-        default: load_face_data<2>(qf, vis, N, gnb, sH + t, haloN);
-      }
+    w = prim_c(s, C);
+    gradient_vars(s, w, C.theta_ref, U);
+    if constexpr (kLines) {
+      f32x2* u2 = reinterpret_cast<f32x2*>(sU);
+      u2[ti] = pack2(U[0], U[1]);
+      u2[tileN + ti] = pack2(U[2], U[3]);
+    } else {
+      quad_store(sU, tileN, ti, U);
     }
-  };
-  if (kHold) {
-    // one node per thread: the own values stay in registers anyway, so their tile stores
-    // wait until the halo gathers are issued and the two latencies overlap
-#pragma unroll
-    for (int j = 0; j < NPT; ++j)
-      if (active[j]) own_loads(j);
-    halo_gather();
-#pragma unroll
-    for (int j = 0; j < NPT; ++j)
-      if (active[j]) own_stores(j);
-  } else {
-#pragma unroll
-    for (int j = 0; j < NPT; ++j)
-      if (active[j]) {
-        own_loads(j);
-        own_stores(j);
-      }
-    halo_gather();
   }
   __syncthreads();
 
-  // interface terms, one work item per (element, face, face node); in a cube, the
-  // external faces first, then one item per internal face node for both sides
-  const int nItems = CUBE ? haloN + 12 * n2 : haloN;
-  for (int t = threadIdx.x; t < nItems; t += blockDim.x) {
-    if (!CUBE || t < haloN) {
-      const Item<P> it = CUBE ? cube_item_of<P>(t) : item_of<P>(t);
-      if (!CUBE && e0 + it.hl >= C.nel) continue;
-      const int o = it.hl * np + face_node<P>(it.d, it.side ? P : 0, it.ab);
-      T* out = sS + (CUBE ? item_index<P>(it.ab, it.side, it.d, it.hl) : t);
-      T so[5], to[4], sn[5], tn[4];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) so[v] = sX[v * tileN + o];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) sn[v] = sH[v * haloN + t];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) tn[i] = sH[(5 + i) * haloN + t];
-      switch (it.d) {
-        case 0:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(0, i)) * tileN + o];
-          interface_item<0>(so, to, sn, tn, out, faceN, it.side, C);
-          break;
-        case 1:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(1, i)) * tileN + o];
-          interface_item<1>(so, to, sn, tn, out, faceN, it.side, C);
-          break;
-        default:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(2, i)) * tileN + o];
-          interface_item<2>(so, to, sn, tn, out, faceN, it.side, C);
-      }
-    } else {
-      const int u = t - haloN;
-      const int ab = u % n2, r = u / n2, d = r >> 2;
-      const int hlL = cube_left_of_pair(r & 3, d), hlR = hlL | (1 << d);
-      const int oL = hlL * np + face_node<P>(d, P, ab), oR = hlR * np + face_node<P>(d, 0, ab);
-      T* outL = sS + item_index<P>(ab, 1, d, hlL);
-      T* outR = sS + item_index<P>(ab, 0, d, hlR);
-      T sl[5], tl[4], sr[5], tr[4];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) sl[v] = sX[v * tileN + oL];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) sr[v] = sX[v * tileN + oR];
-      switch (d) {
-        case 0:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tl[i] = sX[(5 + face_vis_index(0, i)) * tileN + oL];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tr[i] = sX[(5 + face_vis_index(0, i)) * tileN + oR];
-          interface_pair<0>(sl, tl, sr, tr, outL, outR, faceN, C);
-          break;
-        case 1:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tl[i] = sX[(5 + face_vis_index(1, i)) * tileN + oL];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tr[i] = sX[(5 + face_vis_index(1, i)) * tileN + oR];
-          interface_pair<1>(sl, tl, sr, tr, outL, outR, faceN, C);
-          break;
-        default:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tl[i] = sX[(5 + face_vis_index(2, i)) * tileN + oL];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) tr[i] = sX[(5 + face_vis_index(2, i)) * tileN + oR];
-          interface_pair<2>(sl, tl, sr, tr, outL, outR, faceN, C);
-      }
+  T G[3][4];
+  DT Dr[3][kLines ? 1 : n];
+  constexpr int stride[3] = {1, n, n2};
+  if constexpr (kLines) {
+    f32x2* u2 = reinterpret_cast<f32x2*>(sU);
+    f32x2* g2 = reinterpret_cast<f32x2*>(sF);
+    for (int task = threadIdx.x; task < E * 6 * n2; task += blockDim.x) {
+      const int r = task / n2, ab = task - r * n2, hl = r / 6, dp = r - 6 * hl;   // dp = 2 d + pair
+      line_derivative_dir<P, false>(dp >> 1, u2 + (dp & 1) * tileN + hl * tn, g2 + dp * tileN + hl * tn, ab);
     }
-  }
-  __syncthreads();  // own-data tile no longer needed: (late fluxes) it now takes the volume fluxes
-
-#pragma unroll
-  for (int j = 0; j < NPT; ++j) {
-    if (kEarlyF || !active[j]) continue;
-    if (!kHold) {
-      load_rk(j);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) s[j][v] = sX[v * tileN + tix[j]];
-#pragma unroll
-      for (int c = 0; c < 9; ++c) vs[j][c] = sX[(5 + c) * tileN + tix[j]];
-    }
-    const Prim<T> w = prim_c(s[j], C);
-    if (SPLIT) store_split_prims(s[j], w, C, sW + tix[j], tileN);
+    __syncthreads();
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      T F[5], fv[5];
-      euler_flux(s[j], w, C.Hc, d, F);
-      viscous_flux(vs[j], w.v, d, fv);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const T fd = SPLIT ? -fv[c] : F[c] - fv[c];
-        if (kShfl && d < 2) Fr[j][d][c] = fd;
-        else sX[(5 * d + c) * tileN + tix[j]] = fd;
-      }
+      if (!active) continue;
+      unpack2(g2[(2 * d) * tileN + ti], G[d][0], G[d][1]);
+      unpack2(g2[(2 * d + 1) * tileN + ti], G[d][2], G[d][3]);
     }
-  }
-  if (!kEarlyF) __syncthreads();
-
-#pragma unroll
-  for (int j = 0; j < NPT; ++j) {
-    if (!active[j]) continue;
-    const int nd = node[j], lj = le[j];
-    const long long g = gi[j];
-    // volume term -(2/h) sum_d D_d F_d, then the lifted interface terms (fixed order x, y, z)
-    const int idx[3] = {nd % n, (nd / n) % n, nd / n2};
-    const int stride[3] = {1, n, n2};
-    T R[5] = {T(0), T(0), T(0), T(0), T(0)};
+  } else if (active) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const T* Drow = sD + idx[d] * n;
-      const int base = lj * np + nd - idx[d] * stride[d];
+      const DT* Drow = sD + idx[d] * n;
+      const int base = ti - idx[d] * stride[d];
+      QuadSum<T> sum;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        T acc = T(0);
-        if (kShfl && d < 2) {
-          const int l0 = (threadIdx.x & 31) - idx[d] * stride[d];
+      for (int m = 0; m < n; ++m) {
+        Dr[d][m] = Drow[m];
+        sum.add(Dr[d][m], sU, tileN, base + m * stride[d]);
+      }
+      sum.get(G[d]);
+    }
+  }
+
+  T vis[9];
+  if (active) {
+    const T lift = C.s2h * C.winv * T(0.5);
 #pragma unroll
-          for (int m = 0; m < n; ++m) acc += Drow[m] * __shfl_sync(0xffffffffu, Fr[j][d][c], l0 + m * stride[d]);
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a) G[d][a] *= C.s2h;
+      // interface lifting with the central U^ = (U + U_nb) / 2
+      const bool right = (idx[d] == P), left = (idx[d] == 0);
+      if (right || left) {
+        const int ab = face_ab<P>(d, idx);
+        const T sgn = right ? lift : -lift;
+        T Un[4];
+        if (CUBE && (right ? 1 : 0) != ((le >> d) & 1)) {   // internal face: the neighbour's tile entry
+          const int o = (le ^ (1 << d)) * np + face_node<P>(d, right ? 0 : P, ab);
+          quad_load(sU, tileN, o, Un);
         } else {
-#pragma unroll
-          for (int m = 0; m < n; ++m) acc += Drow[m] * sF[(5 * d + c) * tileN + base + m * stride[d]];
-        }
-        R[c] -= C.s2h * acc;
-      }
-    }
-    if (SPLIT) {
-      const int ti = tix[j];
-      T wi[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) wi[k] = sW[k * tileN + ti];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const T* Drow = sD + idx[d] * n;
-        const int base = lj * np + nd - idx[d] * stride[d];
-        T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-        for (int m = 0; m < n; ++m) {
-          const int o = base + m * stride[d];
-          T wm[6];
-#pragma unroll
-          for (int k = 0; k < 6; ++k) wm[k] = sW[k * tileN + o];
-          T F[5];
-          kep_flux_prims(wi, wm, d, F);
-#pragma unroll
-          for (int c = 0; c < 5; ++c) acc[c] += Drow[m] * F[c];
+          const int o = CUBE ? cube_item_index<P>(ab, d, le) : item_index<P>(ab, 2 * d + (right ? 1 : 0), le);
+          if constexpr (kLines) {
+            const f32x2* h = reinterpret_cast<const f32x2*>(sH);
+            unpack2(h[o], Un[0], Un[1]);
+            unpack2(h[haloN + o], Un[2], Un[3]);
+          } else {
+            quad_load(sH, haloN, o, Un);
+          }
         }
 #pragma unroll
-        for (int c = 0; c < 5; ++c) R[c] -= C.s2h * (T(2) * acc[c]);
+        for (int a = 0; a < 4; ++a) G[d][a] += sgn * (Un[a] - U[a]);
       }
     }
+    T mu, lam;
+    transport_c(C, w.rho, G, &mu, &lam);
+    const T div = G[0][0] + G[1][1] + G[2][2];
+    const T t23 = T(2.0 / 3.0) * mu * div;
+    // G[d][a] = d u_a / d x_d, tau_ab = mu (du_a/dx_b + du_b/dx_a) - 2/3 mu div delta_ab
+    vis[0] = T(2) * mu * G[0][0] - t23;
+    vis[1] = T(2) * mu * G[1][1] - t23;
+    vis[2] = T(2) * mu * G[2][2] - t23;
+    vis[3] = mu * (G[1][0] + G[0][1]);
+    vis[4] = mu * (G[2][0] + G[0][2]);
+    vis[5] = mu * (G[2][1] + G[1][2]);
+    vis[6] = lam * G[0][3];
+    vis[7] = lam * G[1][3];
+    vis[8] = lam * G[2][3];
+    // viscous flux normal to each face the node lies on, in the face's frame (see face_terms):
+    // (tau_nn, s tau_nt1, s tau_nt2, s k theta_n) with s = +1 on the right, -1 on the left
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const bool right = (idx[d] == P), left = (idx[d] == 0);
       if (!(right || left)) continue;
-      const int h = item_index<P>(face_ab<P>(d, idx), right ? 1 : 0, d, lj);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) R[c] += sS[c * faceN + h];
+      const T sg = right ? T(1) : T(-1);
+      T* o = vt + (size_t)e * face_record(n) + (2 * d + (right ? 1 : 0)) * (kFaceVis * n2) + face_ab<P>(d, idx);
+      const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+      o[0] = vis[d];
+      o[n2] = sg * vis[sym_index(t1, d)];
+      o[2 * n2] = sg * vis[sym_index(t2, d)];
+      o[3 * n2] = sg * vis[6 + d];
     }
-
-    if (fc.s != nullptr) {
-      const long long base = (g / np) * fc.stride + nd;
+    // volume fluxes of the three directions
+    T* sW = sF + 15 * tileN;
+    if (SPLIT) store_split_prims(s, w, C, sW + le * np + node, E * np);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const int slot = c - fc.first_var;
-        if (slot >= 0 && slot < fc.n_vars) R[c] += T(fc.s[base + (long long)slot * np]);
+    for (int d = 0; d < 3; ++d) {
+      T F[5], fv[5];
+      viscous_flux(vis, w.v, d, fv);
+      if (SPLIT) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) F[c] = -fv[c];
+      } else {
+        euler_flux(s, w, C.Hc, d, F);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) F[c] -= fv[c];
+      }
+      if constexpr (kLines) {
+        // over this node's own derivative entries, already read
+        f32x2* f2 = reinterpret_cast<f32x2*>(sF);
+        f2[(2 * d) * tileN + ti] = pack2(F[0], F[1]);
+        f2[(2 * d + 1) * tileN + ti] = pack2(F[2], F[3]);
+        sF[(12 + d) * tileN + ti] = F[4];
+      } else {
+        quad_store(sF + 4 * d * tileN, tileN, ti, F);
+        sF[(12 + d) * tileN + ti] = F[4];
       }
     }
+  }
+  __syncthreads();
 
-    if (MODE == 0) {
+  T R[5] = {T(0), T(0), T(0), T(0), T(0)};
+  if constexpr (kLines) {
+    f32x2* f2 = reinterpret_cast<f32x2*>(sF);
+    T* f1 = sF + 12 * tileN;
+    for (int task = threadIdx.x; task < E * 9 * n2; task += blockDim.x) {
+      const int r = task / n2, ab = task - r * n2, hl = r / 9, k = r - 9 * hl;
+      if (k < 6) line_derivative_dir<P, false>(k >> 1, f2 + k * tileN + hl * tn, f2 + k * tileN + hl * tn, ab);
+      else line_derivative_dir<P, true>(k - 6, f1 + (k - 6) * tileN + hl * tn, f1 + (k - 6) * tileN + hl * tn, ab);
+    }
+    __syncthreads();
+    if (!active) return;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) dqdt[c * N + g] = double(R[c]);
-    } else if (MODE == 1) {
-      // FP64 operator: plain 2N update of the FP64 state
+    for (int d = 0; d < 3; ++d) {
+      T a[5];
+      unpack2(f2[(2 * d) * tileN + ti], a[0], a[1]);
+      unpack2(f2[(2 * d + 1) * tileN + ti], a[2], a[3]);
+      a[4] = f1[d * tileN + ti];
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const long long o = c * N + g;
-        T gnew = rk.dt * R[c];
-        if (rk.A != T(0)) gnew = rk.A * gold[j][c] + gnew;
-        greg[o] = gnew;
-        q[o] = double(rk.B) * double(gnew) + q[o];
+      for (int c = 0; c < 5; ++c) R[c] -= C.s2h * a[c];
+    }
+  } else {
+    if (!active) return;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int base = ti - idx[d] * stride[d];
+      QuadSum<T> sum;
+      T a[5];
+      a[4] = T(0);
+#pragma unroll
+      for (int m = 0; m < n; ++m) {
+        sum.add(Dr[d][m], sF + 4 * d * tileN, tileN, base + m * stride[d]);
+        a[4] += d_scalar(Dr[d][m]) * sF[(12 + d) * tileN + base + m * stride[d]];
       }
+      sum.get(a);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) R[c] -= C.s2h * a[c];
+    }
+  }
+  if (SPLIT) {
+    const T* sW = sF + 15 * tileN;
+    const int wN = E * np, wi0 = le * np + node;
+    T wi[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) wi[k] = sW[k * wN + wi0];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int base = wi0 - idx[d] * stride[d];
+      T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
+      for (int m = 0; m < n; ++m) {
+        const int o = base + m * stride[d];
+        T wm[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) wm[k] = sW[k * wN + o];
+        T F[5];
+        kep_flux_prims(wi, wm, d, F);
+        const T dm = kLines ? C.D[idx[d] * n + m] : d_scalar(Dr[d][kLines ? 0 : m]);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[c] += dm * F[c];
+      }
+#pragma unroll
+      for (int c = 0; c < 5; ++c) R[c] -= C.s2h * (T(2) * acc[c]);
+    }
+  }
+  T* re = rv + (size_t)e * state_record(n) + node;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) re[v * ns] = R[v];
+}
+
+// ---------------------------------------------------------------- phase A at P = 3, FP32
+//
+// n = 4 makes a row of nodes along x one 16-byte vector, so a thread owns a row: its
+// x-derivatives stay in registers, its y- and z-derivatives read whole rows, and every
+// global and shared access moves four nodes.  An element is 16 threads of one warp, and
+// its 16 halo rows along y and z (4 faces of 4 rows) are one per thread, so the kernel needs
+// warp-level synchronisation only.  Against one node per thread (k_volume at P = 3 as the
+// other orders have it) shared-memory traffic, which bounded that, falls from 133 to 80
+// floats per node and warp instructions to less than half.
+__host__ __device__ constexpr bool use_rows4(int P, int tsize, bool split) { return P == 3 && tsize == 4 && !split; }
+
+// Four consecutive values as two pairs.
+struct Row {
+  f32x2 lo, hi;
+};
+__device__ __forceinline__ Row row_load(const float* p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  return Row{v.x, v.y};
+}
+__device__ __forceinline__ void row_unpack(const Row& r, float v[4]) {
+  unpack2(r.lo, v[0], v[1]);
+  unpack2(r.hi, v[2], v[3]);
+}
+__device__ __forceinline__ void row_store(float* p, const float v[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void row_read(const float* p, float v[4]) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = a.z;
+  v[3] = a.w;
+}
+// sum_m d[m] row(m) of the rows base, base + step, ...
+__device__ __forceinline__ void rows_contract(const float* base, int step, const f32x2 d[4], float out[4]) {
+  Row acc{0ull, 0ull};
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const Row r = row_load(base + m * step);
+    fma2(acc.lo, d[m], r.lo);
+    fma2(acc.hi, d[m], r.hi);
+  }
+  row_unpack(acc, out);
+}
+
+// Four consecutive FP64 values (two 16-byte loads where the address allows).
+__device__ __forceinline__ void row_read64(const double* p, bool wide, double v[4]) {
+  if (wide) {
+    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = b.x;
+    v[3] = b.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = p[i];
+  }
+}
+
+// Stage state of the row of four nodes at node index `node` of element e.
+template <int SRC>
+__device__ __forceinline__ void state_row(const double* __restrict__ q, const float* qf, int e, int node, bool wide,
+                                          const OpConst<float>& C, float s[5][4]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    if (SRC == 0) {
+      double d[4];
+      row_read64(q + v * C.N + (long long)e * 64 + node, wide, d);
+      const double ref = v == 0 ? C.drho_ref : v == 4 ? C.dE_ref : 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[v][i] = d2f_rn(v == 0 || v == 4 ? d[i] - ref : d[i]);
     } else {
-      // FP32 increment scheme
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const long long o = c * N + g;
-        if (MODE == 2) {
-          dlt[o] = float(rk.B * (rk.dt * R[c]));                 // g1 = dt R1; dlt1 = B1 g1
-        } else if (MODE == 3) {
-          const T g2 = rk.A * (dold[j][c] * rk.invB1) + rk.dt * R[c];
-          greg[o] = g2;
-          dlt[o] = float(dold[j][c] + rk.B * g2);
-        } else {
-          const T g3 = rk.A * gold[j][c] + rk.dt * R[c];
-          const float d3 = float(dold[j][c] + rk.B * g3);
-          q[o] = q[o] + f2d(d3);                                 // once per step, in FP64
-        }
-      }
+      row_read(qf + (size_t)e * state_record(4) + v * 64 + node, s[v]);
     }
   }
 }
 
-template <int P, typename T, int MODE, bool CUBE = false, bool SPLIT = false, bool SLAB = false>
-__global__ void __launch_bounds__(flux_max_threads(P), min_blocks_for(P, sizeof(T)))
-k_flux(double* __restrict__ q, const T* __restrict__ qf, const T* __restrict__ vis, double* __restrict__ dqdt,
-       T* __restrict__ greg, float* __restrict__ dlt, Forcing fc, const OpConst<T> C, RkArgs<T> rk) {
+constexpr int kRows4Floats = 18 * 64;   // shared floats per element: U, halo rows (4 + 4), y- and z-fluxes (10)
+
+template <int SRC, bool CUBE, bool FEAT>
+__device__ __forceinline__ void volume4_block(int blk, const double* __restrict__ q, float* qf, float* __restrict__ rv,
+                                              float* __restrict__ vt, const OpConst<float>& C) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int E = CUBE ? kCubeElems : C.E;
+  const int le = threadIdx.x >> 4, r = threadIdx.x & 15, j = r & 3, k = r >> 2;
+  const int e = CUBE ? cube_element(cube_coords(blk, C.K), le, C.K) : C.e_begin + blk * E + le;
+  // an element's 16 threads are half a warp: with an odd number of elements the other half idles
+  const bool active = le < E && e < C.nel;
+  const unsigned half = 0xffffu << (threadIdx.x & 16);
+  if (!active) return;
+  float* sU = reinterpret_cast<float*>(smem_raw) + le * kRows4Floats;   // [4][16 rows][4]
+  float* sH = sU + 4 * 64;                                              // [4][16 halo rows][4]
+  float* sF = sU + 8 * 64;                                              // [2][5][16 rows][4]
+  const bool wide = (reinterpret_cast<size_t>(q) & 15) == 0;
+
+  // own row; halo row r: faces y-, y+ (r / 4 = 0, 1; row k = r % 4), then z-, z+ (row j = r % 4);
+  // the x faces' one node on each side
+  const int hside = (r >> 2) & 1, hz = r >> 3;
+  const int hrow = hz ? (r & 3) + (hside ? 0 : 12) : (hside ? 0 : 3) + 4 * (r & 3);
+  const BlockCoords bc = block_coords(e, C.K);
+  const int base_y = C.K * (bc.y + C.K * bc.z);
+  const int exl = wrap_step(bc.x, -1, C.K) + base_y, exr = wrap_step(bc.x, 1, C.K) + base_y;
+  const int hstep = hside ? 1 : -1;
+  const int eh = hz ? bc.x + C.K * (bc.y + C.K * wrap_step(bc.z, hstep, C.Kz))
+                    : bc.x + C.K * (wrap_step(bc.y, hstep, C.K) + C.K * bc.z);
+
+  float s[5][4];
+  state_row<SRC>(q, qf, e, 4 * r, wide, C, s);
+  float UL[4], UR[4];
+  {
+    float hs[5][4], xl[5], xr[5];
+    state_row<SRC>(q, qf, eh, 4 * hrow, wide, C, hs);
+    if (SRC == 0) {
+      state_from_q(q, (long long)exl * 64 + 4 * r + 3, C, xl);
+      state_from_q(q, (long long)exr * 64 + 4 * r, C, xr);
+    } else {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) xl[v] = qf[(size_t)exl * state_record(4) + v * 64 + 4 * r + 3];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) xr[v] = qf[(size_t)exr * state_record(4) + v * 64 + 4 * r];
+    }
+    float hU[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float t[5] = {hs[0][i], hs[1][i], hs[2][i], hs[3][i], hs[4][i]};
+      float u[4];
+      gradient_vars(t, prim_c(t, C), C.theta_ref, u);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) hU[a][i] = u[a];
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) row_store(sH + a * 64 + 4 * r, hU[a]);
+    gradient_vars(xl, prim_c(xl, C), C.theta_ref, UL);
+    gradient_vars(xr, prim_c(xr, C), C.theta_ref, UR);
+  }
+  float U[4][4], pp[4], rho[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float t[5] = {s[0][i], s[1][i], s[2][i], s[3][i], s[4][i]};
+    const Prim<float> w = prim_c(t, C);
+    float u[4];
+    gradient_vars(t, w, C.theta_ref, u);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) U[a][i] = u[a];
+    pp[i] = w.pp;
+    rho[i] = w.rho;
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) row_store(sU + a * 64 + 4 * r, U[a]);
+  if (SRC == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) row_store(qf + (size_t)e * state_record(4) + v * 64 + 4 * r, s[v]);
+  }
+  if (FEAT) {
+    // the forcing network's input features, from the stage state: the same arithmetic as the
+    // separate feature kernels of the network
+    __nv_bfloat16* fo = static_cast<__nv_bfloat16*>(C.feat.out) + (long long)e * C.feat.ld + 4 * r;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const int slot = v - C.feat.first_var;
+      if (slot < 0 || slot >= C.feat.n_vars) continue;
+      const int f = slot * 64 + 4 * r;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        fo[slot * 64 + i] = __float2bfloat16_rn((s[v][i] - C.feat.shift32[f + i]) / C.feat.sd[f + i]);
+    }
+  }
+  f32x2 Dy[4], Dz[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const float dy = C.D[4 * j + m], dz = C.D[4 * k + m];
+    Dy[m] = pack2(dy, dy);
+    Dz[m] = pack2(dz, dz);
+  }
+  __syncwarp(half);
+
+  // BR1 gradient G[d][a][node], lifted with the central U^ = (U + U_nb) / 2
+  float G[3][4][4];
+  const float lift = C.s2h * C.winv * 0.5f;
+  const int ky = 4 * k, jz = 4 * j;   // first float of the y-line's and z-line's rows: 4 (0 + 4 k), 4 (j + 0)
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float g = 0.f;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) g += C.D[4 * i + m] * U[a][m];
+      G[0][a][i] = mul_(C.s2h, g);
+    }
+    G[0][a][0] = fma_(-lift, UL[a] - U[a][0], G[0][a][0]);
+    G[0][a][3] = fma_(lift, UR[a] - U[a][3], G[0][a][3]);
+    rows_contract(sU + a * 64 + 4 * ky, 4, Dy, G[1][a]);
+    rows_contract(sU + a * 64 + jz, 16, Dz, G[2][a]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      G[1][a][i] = mul_(C.s2h, G[1][a][i]);
+      G[2][a][i] = mul_(C.s2h, G[2][a][i]);
+    }
+  }
+  if (j == 0 || j == 3) {
+    const float sg = j ? lift : -lift;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      float nb[4];
+      row_read(sH + a * 64 + 4 * ((j ? 4 : 0) + k), nb);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) G[1][a][i] = fma_(sg, nb[i] - U[a][i], G[1][a][i]);
+    }
+  }
+  if (k == 0 || k == 3) {
+    const float sg = k ? lift : -lift;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      float nb[4];
+      row_read(sH + a * 64 + 4 * (8 + (k ? 4 : 0) + j), nb);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) G[2][a][i] = fma_(sg, nb[i] - U[a][i], G[2][a][i]);
+    }
+  }
+
+  // viscous quantities (xx, yy, zz, xy, xz, yz, k th_x, k th_y, k th_z)
+  float vis[9][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float g[3][4];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) g[d][a] = G[d][a][i];
+    float mu, lam;
+    transport_c(C, rho[i], g, &mu, &lam);
+    const float t23 = float(2.0 / 3.0) * mu * (g[0][0] + g[1][1] + g[2][2]);
+    vis[0][i] = 2.f * mu * g[0][0] - t23;
+    vis[1][i] = 2.f * mu * g[1][1] - t23;
+    vis[2][i] = 2.f * mu * g[2][2] - t23;
+    vis[3][i] = mu * (g[1][0] + g[0][1]);
+    vis[4][i] = mu * (g[2][0] + g[0][2]);
+    vis[5][i] = mu * (g[2][1] + g[1][2]);
+    vis[6][i] = lam * g[0][3];
+    vis[7][i] = lam * g[1][3];
+    vis[8][i] = lam * g[2][3];
+  }
+  // face-normal viscous fluxes in the faces' frames (see volume_block)
+  float* ve = vt + (size_t)e * face_record(4);
+  ve[r] = vis[0][0];                        // x-: tau_xx, -tau_xy, -tau_xz, -k th_x
+  ve[16 + r] = -vis[3][0];
+  ve[32 + r] = -vis[4][0];
+  ve[48 + r] = -vis[6][0];
+  ve[64 + r] = vis[0][3];                   // x+
+  ve[80 + r] = vis[3][3];
+  ve[96 + r] = vis[4][3];
+  ve[112 + r] = vis[6][3];
+  if (j == 0 || j == 3) {                   // y: tau_yy, tau_yz, tau_yx, k th_y
+    const float sg = j ? 1.f : -1.f;
+    float* o = ve + (j ? 192 : 128) + ky;
+    float t[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      t[0][i] = sg * vis[5][i];
+      t[1][i] = sg * vis[3][i];
+      t[2][i] = sg * vis[7][i];
+    }
+    row_store(o, vis[1]);
+    row_store(o + 16, t[0]);
+    row_store(o + 32, t[1]);
+    row_store(o + 48, t[2]);
+  }
+  if (k == 0 || k == 3) {                   // z: tau_zz, tau_zx, tau_zy, k th_z
+    const float sg = k ? 1.f : -1.f;
+    float* o = ve + (k ? 320 : 256) + jz;
+    float t[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      t[0][i] = sg * vis[4][i];
+      t[1][i] = sg * vis[5][i];
+      t[2][i] = sg * vis[8][i];
+    }
+    row_store(o, vis[2]);
+    row_store(o + 16, t[0]);
+    row_store(o + 32, t[1]);
+    row_store(o + 48, t[2]);
+  }
+
+  // volume fluxes: x contracted in registers, y and z through shared memory
+  float R[5][4];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    float F[5][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float t[5] = {s[0][i], s[1][i], s[2][i], s[3][i], s[4][i]};
+      Prim<float> w;
+      w.v[0] = U[0][i];
+      w.v[1] = U[1][i];
+      w.v[2] = U[2][i];
+      w.pp = pp[i];
+      float f[5], fv[5], vi[9];
+#pragma unroll
+      for (int c = 0; c < 9; ++c) vi[c] = vis[c][i];
+      euler_flux(t, w, C.Hc, d, f);
+      viscous_flux(vi, w.v, d, fv);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) F[c][i] = f[c] - fv[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      if (d == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float g = 0.f;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) g += C.D[4 * i + m] * F[c][m];
+          R[c][i] = mul_(-C.s2h, g);
+        }
+      } else {
+        row_store(sF + (5 * (d - 1) + c) * 64 + 4 * r, F[c]);
+      }
+    }
+  }
+  __syncwarp(half);
+  float* re = rv + (size_t)e * state_record(4) + 4 * r;
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    float y[4], z[4];
+    rows_contract(sF + c * 64 + 4 * ky, 4, Dy, y);
+    rows_contract(sF + (5 + c) * 64 + jz, 16, Dz, z);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      R[c][i] = fma_(-C.s2h, z[i], fma_(-C.s2h, y[i], R[c][i]));
+    }
+    row_store(re + c * 64, R[c]);
+  }
+}
+
+// Threads, shared memory and register budget of a phase-A block of E elements.
+template <int P, typename T, bool SPLIT>
+__host__ __device__ constexpr int volume_threads(int E) {
+  const int t = use_rows4(P, sizeof(T), SPLIT) ? 16 * E : E * (P + 1) * (P + 1) * (P + 1);
+  return (t + 31) / 32 * 32;
+}
+template <int P, typename T, bool SPLIT>
+__host__ __device__ constexpr size_t volume_smem(int E, bool cube) {
+  return use_rows4(P, sizeof(T), SPLIT)
+             ? sizeof(float) * (size_t)kRows4Floats * E
+             : volume_smem_bytes<P, T>(E, (cube ? 3 : 6) * E * (P + 1) * (P + 1), SPLIT);
+}
+template <int P, typename T, bool SPLIT>
+__host__ __device__ constexpr int volume_max_threads() {
+  return use_rows4(P, sizeof(T), SPLIT) ? 128 : max_threads_for(P);
+}
+template <int P, typename T, bool SPLIT>
+__host__ __device__ constexpr int volume_min_blocks() {
+  return use_rows4(P, sizeof(T), SPLIT) ? 4 : sizeof(T) == 8 ? 1 : P == 1 ? 4 : P == 6 ? 3 : 2;
+}
+
+template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
+__device__ __forceinline__ void volume_phase(int blk, const double* __restrict__ q, T* qf, T* __restrict__ rv,
+                                             T* __restrict__ vt, const OpConst<T>& C) {
+  if constexpr (use_rows4(P, sizeof(T), SPLIT)) volume4_block<SRC, CUBE, FEAT>(blk, q, qf, rv, vt, C);
+  else volume_block<P, T, SRC, CUBE, FEAT, SPLIT>(blk, q, qf, rv, vt, C);
+}
+
+template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
+__global__ void __launch_bounds__(volume_max_threads<P, T, SPLIT>(), volume_min_blocks<P, T, SPLIT>())
+k_volume(const double* __restrict__ q, T* __restrict__ qf, T* __restrict__ rv, T* __restrict__ vt,
+         const OpConst<T> C) {
   pdl_wait();
   pdl_release();
-  flux_block<P, T, MODE, CUBE, SPLIT, SLAB>(blockIdx.x, q, qf, vis, dqdt, greg, dlt, fc, C, rk);
+  volume_phase<P, T, SRC, CUBE, FEAT, SPLIT>(blockIdx.x, q, qf, rv, vt, C);
+}
+
+// ---------------------------------------------------------------- phase B
+
+// Per-launch RK data of phase B in the arithmetic of the update.
+template <typename R>
+struct RkArgs {
+  R A, B, dt;   // Williamson coefficients of the stage and the step size
+  R invB1;      // 1 / B of stage 1 (the FP32 increment scheme recovers g1 = dlt1 / B1)
+  R wc;         // B A of stage 3: the share of g2 in the final increment
+};
+
+// Operands of phase B on one mesh.
+template <typename T>
+struct SurfArgs {
+  double* q;          // FP64 state
+  const T* s;         // stage state of this stage
+  const T* rv;        // volume term
+  const T* vt;        // face-normal viscous fluxes
+  double* dqdt;       // MODE 0
+  T* g;               // MODE 1: RK register
+  T* x;               // MODE 2: s1 (read); MODE 3: s1, replaced by s3
+  T* y;               // MODE 2: s2 (written)
+  float* dlt;         // MODES 2, 3, 4: increment (see the head of this file)
+};
+
+// The FP32 increment scheme, one value.  Stage 1: g1 = dt R, d1 = B1 g1, s2 = s1 + d1.
+// Stage 2: g2 = A2 g1 + dt R with g1 = d1 / B1, d2 = d1 + B2 g2, s3 = s1 + d2, and
+// w = d2 + B3 A3 g2, all that stage 3 needs of them.  Stage 3: d3 = d2 + B3 (A3 g2 + dt R).
+template <typename T>
+__device__ __forceinline__ void rk_stage1(const RkArgs<T>& rk, T R, T s1, T& d1, T& s2) {
+  d1 = mul_(rk.B, mul_(rk.dt, R));
+  s2 = add_(s1, d1);
+}
+template <typename T>
+__device__ __forceinline__ void rk_stage2(const RkArgs<T>& rk, T R, T s1, T d1, T& w, T& s3) {
+  const T g2 = fma_(rk.A, mul_(d1, rk.invB1), mul_(rk.dt, R));
+  const T d2 = fma_(rk.B, g2, d1);
+  s3 = add_(s1, d2);
+  w = fma_(rk.wc, g2, d2);
+}
+template <typename T>
+__device__ __forceinline__ T rk_stage3(const RkArgs<T>& rk, T R, T w) {
+  return fma_(rk.B, mul_(rk.dt, R), w);
+}
+
+// Square root and its square's inverse of c2 = c^2, from one reciprocal square root (FP32:
+// the approximate instruction).
+__device__ __forceinline__ void sound(float c2, float* c, float* inv_c2) {
+  const float r = rsqrtf(c2);
+  *c = c2 * r;
+  *inv_c2 = r * r;
+}
+__device__ __forceinline__ void sound(double c2, double* c, double* inv_c2) {
+  const double r = rsqrt(c2);
+  *c = mul_(c2, r);
+  *inv_c2 = mul_(r, r);
+}
+
+// One side of an interface in the face's frame: normal component first, pointing out of
+// the element the frame belongs to.
+template <typename T>
+struct FaceState {
+  T s[5];     // rho', m_n, m_t1, m_t2, e (reference-shifted)
+  T rho, ir, vn, v1, v2, pp, h;   // h = rho e + p
+};
+
+template <typename T>
+__device__ __forceinline__ void face_state(FaceState<T>& f, const OpConst<T>& C) {
+  f.vn = mul_(f.s[1], f.ir);
+  f.v1 = mul_(f.s[2], f.ir);
+  f.v2 = mul_(f.s[3], f.ir);
+  const T mv = fma_(f.s[1], f.vn, fma_(f.s[2], f.v1, mul_(f.s[3], f.v2)));
+  f.pp = mul_(C.gm1, fma_(T(-0.5), mv, f.s[4]));
+  f.h = add_(add_(f.s[4], f.pp), C.Hc);
+}
+
+// Densities of both sides of a face, their reciprocals, rt = sqrt(rho_o rho_b) and
+// wd = 1 / (sqrt rho_o + sqrt rho_b)^2 = 1 / (rho_o + rho_b + 2 rt).  FP64: one division
+// serves all three reciprocals (the FP64 pipe bounds that operator).
+__device__ __forceinline__ void face_densities(FaceState<float>& o, FaceState<float>& b, float rho_ref, float& rt,
+                                               float& wd) {
+  o.rho = add_(o.s[0], rho_ref);
+  b.rho = add_(b.s[0], rho_ref);
+  o.ir = drcp(o.rho);
+  b.ir = drcp(b.rho);
+  rt = dsqrt(mul_(o.rho, b.rho));
+  wd = drcp(fma_(2.f, rt, add_(o.rho, b.rho)));
+}
+__device__ __forceinline__ void face_densities(FaceState<double>& o, FaceState<double>& b, double rho_ref, double& rt,
+                                               double& wd) {
+  o.rho = add_(o.s[0], rho_ref);
+  b.rho = add_(b.s[0], rho_ref);
+  const double pr = mul_(o.rho, b.rho);
+  rt = sqrt(pr);
+  const double den = fma_(2.0, rt, add_(o.rho, b.rho));
+  const double inv = 1.0 / mul_(pr, den), ipr = mul_(inv, den);
+  wd = mul_(inv, pr);
+  o.ir = mul_(b.rho, ipr);
+  b.ir = mul_(o.rho, ipr);
+}
+
+// Interface terms of one face node in the frame of the own element (o) looking at its
+// neighbour (b): with the outward fluxes f and f^nu, A = (f_b - f_o)/2 + (f^nu_o - f^nu_b)/2
+// and B = |A~|(q_b - q_o)/2, so that f* - f = A - B on the own side.  to, tb: the viscous
+// values each element stored for its side (volume_block), each in its own frame.
+//
+// The right and left element of a face evaluate the same expressions in mirrored frames
+// (normal components change sign, own and neighbour exchange roles), and every expression
+// here is exactly even or odd under that exchange: sums over the two sides are formed
+// without contraction, the acoustic strengths enter as a1 + a5 and a5 - a1.  Both
+// sides of a face therefore get the same flux to the last bit, without selecting left
+// and right states.
+//
+// The Roe averages (sqrt rho_o u_o + sqrt rho_b u_b) / (sqrt rho_o + sqrt rho_b) are taken
+// with numerator and denominator multiplied by the latter: (m_o + m_b + rt (u_o + u_b)) wd,
+// which needs one square root instead of two.
+template <typename T>
+__device__ __forceinline__ void face_terms(FaceState<T>& o, FaceState<T>& b, const T to[4], const T tb[4],
+                                           const OpConst<T>& C, T A[5], T B[5]) {
+  const T half = T(0.5);
+  T rt, wd;
+  face_densities(o, b, C.rho_ref, rt, wd);
+  face_state(o, C);
+  face_state(b, C);
+  const T un = mul_(fma_(rt, add_(o.vn, b.vn), add_(o.s[1], b.s[1])), wd);
+  const T u1 = mul_(fma_(rt, add_(o.v1, b.v1), add_(o.s[2], b.s[2])), wd);
+  const T u2 = mul_(fma_(rt, add_(o.v2, b.v2), add_(o.s[3], b.s[3])), wd);
+  const T H = mul_(fma_(rt, add_(mul_(o.h, o.ir), mul_(b.h, b.ir)), add_(o.h, b.h)), wd);
+  const T ke = mul_(half, fma_(un, un, fma_(u1, u1, mul_(u2, u2))));
+  T c, ic2;
+  sound(mul_(C.gm1, add_(H, -ke)), &c, &ic2);
+  const T dr = add_(b.s[0], -o.s[0]), dp = add_(b.pp, -o.pp), dn = add_(b.vn, -o.vn);
+  const T hc = mul_(half, ic2), x = mul_(rt, c);
+  const T l1 = mul_(fabs(add_(un, -c)), mul_(fma_(-x, dn, dp), hc));
+  const T l5 = mul_(fabs(add_(un, c)), mul_(fma_(x, dn, dp), hc));
+  const T l2 = fabs(un), a2 = fma_(-dp, ic2, dr);
+  const T ls = add_(l1, l5), ld = mul_(add_(l5, -l1), c);
+  const T h1 = mul_(rt, add_(b.v1, -o.v1)), h2 = mul_(rt, add_(b.v2, -o.v2));   // shear waves
+  B[0] = mul_(half, fma_(l2, a2, ls));
+  B[1] = mul_(half, fma_(ls, un, fma_(l2, mul_(a2, un), ld)));
+  B[2] = mul_(half, fma_(ls, u1, mul_(l2, fma_(a2, u1, h1))));
+  B[3] = mul_(half, fma_(ls, u2, mul_(l2, fma_(a2, u2, h2))));
+  B[4] = mul_(half, fma_(ls, H, fma_(ld, un, mul_(l2, fma_(a2, ke, fma_(u1, h1, mul_(u2, h2)))))));
+  // outward fluxes; the neighbour stored its viscous values in its own frame
+  const T eo = fma_(o.vn, to[0], fma_(o.v1, to[1], fma_(o.v2, to[2], to[3])));
+  const T eb = fma_(b.vn, tb[0], -fma_(b.v1, tb[1], fma_(b.v2, tb[2], tb[3])));
+  A[0] = mul_(half, add_(b.s[1], -o.s[1]));
+  A[1] = mul_(half, add_(add_(fma_(b.s[1], b.vn, b.pp), -fma_(o.s[1], o.vn, o.pp)), add_(to[0], -tb[0])));
+  A[2] = mul_(half, add_(add_(mul_(b.s[2], b.vn), -mul_(o.s[2], o.vn)), add_(to[1], tb[1])));
+  A[3] = mul_(half, add_(add_(mul_(b.s[3], b.vn), -mul_(o.s[3], o.vn)), add_(to[2], tb[2])));
+  A[4] = mul_(half, add_(add_(mul_(b.vn, b.h), -mul_(o.vn, o.h)), add_(eo, -eb)));
+}
+
+// Loads one side of a face item: the stage state at node fn of element record se and the
+// viscous values at ve, in the frame with outward sign sg (the state's normal momentum).
+template <int P, typename T>
+__device__ __forceinline__ void load_side(const T* __restrict__ se, int fn, int d, T sg, T s[5]) {
+  constexpr int ns = node_stride(P + 1);
+  const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+  const T* p = se + fn;
+  s[0] = p[0];
+  s[1] = sg * p[(1 + d) * ns];
+  s[2] = p[(1 + d1) * ns];
+  s[3] = p[(1 + d2) * ns];
+  s[4] = p[4 * ns];
+}
+
+// Elements and threads of a phase-B block (rows of elements).
+__host__ __device__ constexpr int surf_elems(int P) {
+  return P == 1 ? 16 : P == 2 ? 8 : P == 3 ? 8 : P == 4 ? 2 : 1;
+}
+__host__ __device__ constexpr int surf_threads(int P) {
+  return P == 1 ? 128 : P == 2 ? 224 : P == 3 ? 128 : P == 4 ? 160 : P == 5 ? 224 : P == 6 ? 192 : P == 7 ? 128 : 256;
+}
+__host__ __device__ constexpr int surf_threads_cube(int P) { return P == 1 ? 96 : 192; }
+// Orders whose phase-B blocks are cubes on a whole mesh of even K.  The cube's 36 face
+// evaluations instead of 48 pay where those bound the launch: FP64 (the FP64 pipe; 16^3/P3
+// 910 -> 844, 12^3/P2 248 -> 221 us per RK3 step) and FP32 at P = 3 (8^3 32.8 -> 29.5, 16^3
+// 72.0 -> 57.7, 32^3 327 -> 330 us); in FP32 at P = 2 (16^3 38.2 -> 43.1 us) and P = 1 rows win.
+__host__ __device__ constexpr bool surf_cube(int P, int tsize) { return tsize == 8 ? P <= 3 : P == 3; }
+// Blocks per SM the phase-B kernel is compiled for: 64 registers per thread in FP32, 128 in FP64.
+__host__ __device__ constexpr int surf_min_blocks(int threads, int tsize) {
+  return tsize == 8 ? 512 / threads : 1024 / threads;
+}
+
+// Shared memory of a phase-B block: neighbour elements [6 E] (int), lifted interface terms
+// [5][E 6 n^2].
+template <int P, typename T>
+__host__ __device__ constexpr size_t surface_smem_bytes(int E) {
+  return ((6 * E + 3) & ~3) * sizeof(int) + sizeof(T) * 5 * E * 6 * (P + 1) * (P + 1);
+}
+
+// MODE 0: dqdt = R.  MODE 1: FP64 RK stage (g = A g + dt R; q += B g).
+// MODES 2, 3, 4: FP32 increment scheme, stages 1, 2, 3.
+// Phase B of block `blk` of one mesh, E elements (the body of k_surface and k_surface_batch).
+// prologue: work that may run before the previous launch has completed.
+template <int P, typename T, bool CUBE>
+__device__ __forceinline__ void surface_prologue(int blk, int E, const OpConst<T>& C) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* sNb = reinterpret_cast<int*>(smem_raw);
+  const int e0 = C.e_begin + blk * E;
+  const BlockCoords bc = CUBE ? cube_coords(blk, C.K) : BlockCoords{0, 0, 0};
+  for (int t = threadIdx.x; t < 6 * E; t += blockDim.x) {
+    const int hl = t / 6, eh = CUBE ? cube_element(bc, hl, C.K) : e0 + hl;
+    sNb[t] = element_across(eh, t - 6 * hl, C.K, C.Kz);
+  }
+  __syncthreads();
+}
+
+template <int P, typename T, int MODE, bool CUBE = false>
+__device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>& a, const Forcing& fc,
+                                              const OpConst<T>& C, const RkArgs<T>& rk) {
+  constexpr int n = P + 1, n2 = n * n, np = n2 * n, ns = node_stride(n);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int* sNb = reinterpret_cast<const int*>(smem_raw);
+  T* sS = reinterpret_cast<T*>(smem_raw + ((6 * E + 3) & ~3) * sizeof(int));   // [5][E 6 n2]
+  const int faceN = E * 6 * n2;
+  const int e0 = C.e_begin + blk * E;
+  const BlockCoords bc = CUBE ? cube_coords(blk, C.K) : BlockCoords{0, 0, 0};
+  const T lift = C.s2h * C.winv;
+
+  // interface terms; in a cube the external faces first, then one item per internal face
+  // node for both sides
+  const int extN = CUBE ? 3 * kCubeElems * n2 : faceN;
+  const int nItems = CUBE ? extN + 12 * n2 : faceN;
+  for (int t = threadIdx.x; t < nItems; t += blockDim.x) {
+    Item<P> it;
+    if (!CUBE) {
+      it = item_of<P>(t);
+      if (e0 + it.hl >= C.nel) continue;
+    } else if (t < extN) {
+      it = cube_item_of<P>(t);
+    } else {   // internal face node: the left element's right side
+      const int u = t - extN, r = u / n2, d = r >> 2;
+      it.ab = u - r * n2;
+      it.hl = cube_left_of_pair(r & 3, d);
+      it.face = 2 * d + 1;
+    }
+    const int d = it.face >> 1;
+    const bool right = it.face & 1;
+    const T sg = right ? T(1) : T(-1);
+    const int e = CUBE ? cube_element(bc, it.hl, C.K) : e0 + it.hl;
+    const int enb = sNb[6 * it.hl + it.face];
+    const int st = d == 0 ? 1 : d == 1 ? n : n2;
+    const int f0 = face_node<P>(d, 0, it.ab);
+    FaceState<T> o, b;
+    T to[4], tb[4];
+    load_side<P>(a.s + (size_t)e * state_record(n), right ? f0 + P * st : f0, d, sg, o.s);
+    load_side<P>(a.s + (size_t)enb * state_record(n), right ? f0 : f0 + P * st, d, sg, b.s);
+    const T* vo = a.vt + (size_t)e * face_record(n) + it.face * (kFaceVis * n2) + it.ab;
+    const T* vb = a.vt + (size_t)enb * face_record(n) + (it.face ^ 1) * (kFaceVis * n2) + it.ab;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) to[i] = vo[i * n2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tb[i] = vb[i * n2];
+    T A[5], B[5];
+    face_terms(o, b, to, tb, C, A, B);
+    // lifted terms -(2/h)/w (f* - f) back in mesh components
+    const int cn = (1 + d) * faceN, c1 = (1 + (d == 2 ? 0 : d + 1)) * faceN, c2 = (1 + (d == 0 ? 2 : d - 1)) * faceN;
+    T* out = sS + item_index<P>(it.ab, it.face, it.hl);
+    out[0] = mul_(-lift, add_(A[0], -B[0]));
+    out[cn] = mul_(-lift * sg, add_(A[1], -B[1]));
+    out[c1] = mul_(-lift, add_(A[2], -B[2]));
+    out[c2] = mul_(-lift, add_(A[3], -B[3]));
+    out[4 * faceN] = mul_(-lift, add_(A[4], -B[4]));
+    if (CUBE && t >= extN) {
+      // the right element's left side: A and B of the mirrored frame
+      T* ob = sS + item_index<P>(it.ab, it.face ^ 1, it.hl | (1 << d));
+      ob[0] = mul_(-lift, add_(A[0], B[0]));
+      ob[cn] = mul_(lift, add_(-A[1], -B[1]));
+      ob[c1] = mul_(-lift, add_(A[2], B[2]));
+      ob[c2] = mul_(-lift, add_(A[3], B[3]));
+      ob[4 * faceN] = mul_(-lift, add_(A[4], B[4]));
+    }
+  }
+  __syncthreads();
+
+  if constexpr (P == 3 && sizeof(T) == 4) {
+    // a thread owns a row of four nodes along x: every access is a 16-byte vector
+    const bool wide = (reinterpret_cast<size_t>(MODE == 0 ? a.dqdt : a.q) & 15) == 0;
+    for (int t = threadIdx.x; t < E * 16; t += blockDim.x) {
+      const int le = t >> 4, r = t & 15, j = r & 3, k = r >> 2;
+      const int e = CUBE ? cube_element(bc, le, C.K) : e0 + le;
+      if (!CUBE && e >= C.nel) break;
+      const size_t o = (size_t)e * state_record(n) + 4 * r;
+      const long long g = (long long)e * 64 + 4 * r;
+      float R[5][4];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) row_read(a.rv + o + c * 64, R[c]);
+      // the lifted interface terms in a fixed order (x, y, z)
+      const float* ss = sS + le * 96;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        R[c][0] += ss[c * faceN + r];
+        R[c][3] += ss[c * faceN + 16 + r];
+      }
+      if (j == 0 || j == 3) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          float l[4];
+          row_read(ss + c * faceN + (j ? 48 : 32) + 4 * k, l);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) R[c][i] += l[i];
+        }
+      }
+      if (k == 0 || k == 3) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          float l[4];
+          row_read(ss + c * faceN + (k ? 80 : 64) + 4 * j, l);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) R[c][i] += l[i];
+        }
+      }
+      if (fc.s != nullptr) {
+        const float* fs = fc.s + (long long)e * fc.stride + 4 * r;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          const int slot = c - fc.first_var;
+          if (slot < 0 || slot >= fc.n_vars) continue;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) R[c][i] += fs[slot * 64 + i];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        double q1[4];
+        float u[4], v[4], x1[4], g1[4];
+        if (MODE == 2 || MODE == 3) row_read(a.x + o + c * 64, x1);
+        if (MODE == 3 || MODE == 4) row_read(a.dlt + o + c * 64, g1);
+        if (MODE == 4) row_read64(a.q + c * C.N + g, wide, q1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (MODE == 0) q1[i] = double(R[c][i]);
+          else if (MODE == 2) rk_stage1(rk, R[c][i], x1[i], u[i], v[i]);
+          else if (MODE == 3) rk_stage2(rk, R[c][i], x1[i], g1[i], u[i], v[i]);
+          else q1[i] += f2d(rk_stage3(rk, R[c][i], g1[i]));
+        }
+        if (MODE == 2 || MODE == 3) {
+          row_store(a.dlt + o + c * 64, u);
+          row_store((MODE == 2 ? a.y : a.x) + o + c * 64, v);
+        } else {
+          double* out = (MODE == 0 ? a.dqdt : a.q) + c * C.N + g;
+          if (wide) {
+            reinterpret_cast<double2*>(out)[0] = make_double2(q1[0], q1[1]);
+            reinterpret_cast<double2*>(out)[1] = make_double2(q1[2], q1[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) out[i] = q1[i];
+          }
+        }
+      }
+    }
+  } else {
+  for (int t = threadIdx.x; t < E * np; t += blockDim.x) {
+    const int le = t / np, node = t - le * np;
+    const int e = CUBE ? cube_element(bc, le, C.K) : e0 + le;
+    if (!CUBE && e >= C.nel) break;
+    const size_t o = (size_t)e * state_record(n) + node;
+    const long long g = (long long)e * np + node;
+    T R[5], g1[5], x1[5];
+    double q1[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) R[c] = a.rv[o + c * ns];
+    if (MODE == 2 || MODE == 3) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) x1[c] = a.x[o + c * ns];
+    }
+    if (MODE == 3 || MODE == 4) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) g1[c] = T(a.dlt[o + c * ns]);
+    }
+    if (MODE == 1) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) g1[c] = rk.A == T(0) ? T(0) : a.g[o + c * ns];
+    }
+    if (MODE == 1 || MODE == 4) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) q1[c] = a.q[c * C.N + g];
+    }
+    const int idx[3] = {node % n, (node / n) % n, node / n2};
+    // the lifted interface terms in a fixed order (x, y, z)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const bool right = (idx[d] == P), left = (idx[d] == 0);
+      if (!(right || left)) continue;
+      const int h = item_index<P>(face_ab<P>(d, idx), 2 * d + (right ? 1 : 0), le);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) R[c] += sS[c * faceN + h];
+    }
+    if (fc.s != nullptr) {
+      const float* fs = fc.s + (long long)e * fc.stride + node;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        const int slot = c - fc.first_var;
+        if (slot >= 0 && slot < fc.n_vars) R[c] += T(fs[slot * np]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      if (MODE == 0) {
+        a.dqdt[c * C.N + g] = double(R[c]);
+      } else if (MODE == 1) {   // FP64 operator: plain 2N update of the FP64 state
+        T gnew = mul_(rk.dt, R[c]);
+        if (rk.A != T(0)) gnew = fma_(rk.A, g1[c], gnew);
+        a.g[o + c * ns] = gnew;
+        a.q[c * C.N + g] = fma_(double(rk.B), double(gnew), q1[c]);
+      } else if (MODE == 2) {
+        T d1, s2;
+        rk_stage1(rk, R[c], x1[c], d1, s2);
+        a.dlt[o + c * ns] = float(d1);
+        a.y[o + c * ns] = s2;
+      } else if (MODE == 3) {
+        T w, s3;
+        rk_stage2(rk, R[c], x1[c], g1[c], w, s3);
+        a.x[o + c * ns] = s3;
+        a.dlt[o + c * ns] = float(w);
+      } else {
+        a.q[c * C.N + g] = q1[c] + f2d(float(rk_stage3(rk, R[c], g1[c])));
+      }
+    }
+  }
+  }
+}
+
+template <int P, typename T, int MODE, bool CUBE = false>
+__global__ void __launch_bounds__(CUBE ? surf_threads_cube(P) : surf_threads(P),
+                                  surf_min_blocks(CUBE ? surf_threads_cube(P) : surf_threads(P), sizeof(T)))
+k_surface(SurfArgs<T> a, Forcing fc, const OpConst<T> C, RkArgs<T> rk) {
+  constexpr int E = CUBE ? kCubeElems : surf_elems(P);
+  // last block first: phase A has just written the end of the mesh, which is still in L2
+  const int blk = gridDim.x - 1 - blockIdx.x;
+  surface_prologue<P, T, CUBE>(blk, E, C);
+  pdl_wait();
+  pdl_release();
+  surface_block<P, T, MODE, CUBE>(blk, E, a, fc, C, rk);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -998,16 +1584,14 @@ constexpr int kMaxBatch = 16;
 template <typename T>
 struct BatchTable {
   int n;                             // instances in this launch
-  int block_start[kMaxBatch + 1];    // first block of each instance; block_start[n] = grid
-  double* q[kMaxBatch];              // FP64 states
-  float* qn32[kMaxBatch];            // FP32 operator: step-start image (NULL in FP64)
-  float* dlt[kMaxBatch];             // FP32 operator: stage increment (NULL in FP64)
-  T* qf[kMaxBatch];                  // stage state
-  T* vis[kMaxBatch];                 // viscous quantities
-  T* g[kMaxBatch];                   // RK register
+  int block_start[kMaxBatch + 1];    // first phase-A block of each instance; block_start[n] = grid
+  int surf_start[kMaxBatch + 1];     // the same for phase B
+  T* qs[kMaxBatch];                  // stage state of this stage
+  T* rv[kMaxBatch];                  // volume term
+  T* vt[kMaxBatch];                  // face-normal viscous fluxes
+  SurfArgs<T> a[kMaxBatch];
   RkArgs<T> rk[kMaxBatch];
   OpConst<T> C[kMaxBatch];
-  int bulk[kMaxBatch];               // streamed phase B: own tiles by TMA bulk copies (see StreamMesh)
   int* err[kMaxBatch];               // device error flag of the instance (may be NULL)
 };
 
@@ -1018,411 +1602,24 @@ __device__ __forceinline__ int batch_instance(const int* start, int n, int b) {
 }
 
 template <int P, typename T, int SRC>
-__global__ void __launch_bounds__(max_threads_for(P))
-k_gradient_batch(const __grid_constant__ BatchTable<T> tb) {
+__global__ void __launch_bounds__(volume_max_threads<P, T, false>(), volume_min_blocks<P, T, false>())
+k_volume_batch(const __grid_constant__ BatchTable<T> tb) {
   pdl_wait();
   pdl_release();
   const int i = batch_instance(tb.block_start, tb.n, blockIdx.x);
-  gradient_block<P, T, SRC>(blockIdx.x - tb.block_start[i], tb.q[i], tb.qn32[i], tb.dlt[i], tb.qf[i],
-                            SRC == 0 ? tb.qn32[i] : nullptr, tb.vis[i], tb.C[i]);
+  volume_phase<P, T, SRC>(blockIdx.x - tb.block_start[i], tb.a[i].q, tb.qs[i], tb.rv[i], tb.vt[i], tb.C[i]);
 }
 
 template <int P, typename T, int MODE>
-__global__ void __launch_bounds__(flux_max_threads(P), min_blocks_for(P, sizeof(T)))
-k_flux_batch(const __grid_constant__ BatchTable<T> tb) {
+__global__ void __launch_bounds__(surf_threads(P), surf_min_blocks(surf_threads(P), sizeof(T)))
+k_surface_batch(const __grid_constant__ BatchTable<T> tb) {
+  const int b = gridDim.x - 1 - blockIdx.x;
+  const int i = batch_instance(tb.surf_start, tb.n, b);
+  const int blk = b - tb.surf_start[i];
+  surface_prologue<P, T, false>(blk, surf_elems(P), tb.C[i]);
   pdl_wait();
   pdl_release();
-  const int i = batch_instance(tb.block_start, tb.n, blockIdx.x);
-  flux_block<P, T, MODE>(blockIdx.x - tb.block_start[i], tb.q[i], tb.qf[i], tb.vis[i], nullptr, tb.g[i],
-                         tb.dlt[i], Forcing{}, tb.C[i], tb.rk[i]);
-}
-
-// ---------------------------------------------------------------------------------------
-// Streamed phase B for high orders (FP32 operator, P >= 6, one element per work item).
-//
-// At P >= 6 an element's phase B is latency-bound when its loads and its arithmetic
-// alternate: the block waits for the own tile and the face halo, then computes with no
-// memory traffic in flight.  The streamed kernel is persistent: each block walks the
-// elements blockIdx.x, blockIdx.x + gridDim.x, ... and, while it computes element k,
-// copies element k + 1's tile (TMA bulk copies, one per component row) and face halo
-// (4-byte cp.async) into the other half of a double buffer, straight to shared memory
-// with no registers held.  The per-node and per-item arithmetic is flux_block's.
-
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// TMA bulk copies (cp.async.bulk, global -> shared, completion counted in bytes on an
-// mbarrier).  Addresses 16-byte aligned, size a multiple of 16 bytes.
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bulk_bar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_bar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void bulk_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
-// Bounded wait for the phase with the given parity (about a second); false on expiry.
-__device__ __forceinline__ bool bulk_wait(unsigned long long* bar, unsigned parity) {
-  const long long t0 = clock64();
-  for (;;) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > 2000000000LL) return false;
-  }
-}
-
-// load_face_data with cp.async (no registers held while the copies fly).
-template <int D>
-__device__ __forceinline__ void copy_face_data(const float* qf, const float* vis, long long N, long long g,
-                                               float* dst, int stride) {
-  const float* s = qf + g;
-  const float* w = vis + g;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) cp_async4(dst + v * stride, s + v * N);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) cp_async4(dst + (5 + i) * stride, w + face_vis_index(D, i) * N);
-}
-
-// Threads of a streamed block: one per node.
-// One warp more where that saves a round of the 15 (P+1)^2 line-derivative tasks (P = 6:
-// 735 tasks take two rounds of 384 threads instead of three of 352).
-__host__ __device__ constexpr int stream_threads(int P) {
-  return ((15 * (P + 1) * (P + 1) + ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32) - 1) /
-              ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32) >
-          (15 * (P + 1) * (P + 1) + ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32 + 32) - 1) /
-              ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32 + 32))
-             ? ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32 + 32)
-             : ((((P + 1) * (P + 1) * (P + 1) + 31) / 32) * 32);
-}
-static_assert(stream_threads(6) == 384 && stream_threads(7) == 512 && stream_threads(8) == 736, "stream block sizes");
-// Blocks per SM the streamed kernel is compiled for (shared memory allows two at P <= 7).
-__host__ __device__ constexpr int stream_min_blocks(int P) { return P <= 7 ? 2 : 1; }
-
-// One mesh's operands as seen by a streamed work item.
-struct StreamItem {
-  double* q;
-  const float* qf;
-  const float* vis;
-  double* dqdt;
-  float* greg;
-  float* dlt;
-  const OpConst<float>* C;
-  const RkArgs<float>* rk;
-  Forcing fc;
-  int e;     // element
-  int bulk;  // own tile by TMA bulk copies (every component row 16-byte aligned modulo the element shift)
-  int* err;  // device error flag (may be NULL)
-};
-
-// Shared memory of the streamed kernel, in floats: two mbarriers (4 floats), the
-// per-direction volume fluxes and then their derivatives [3][5][np], and two 16-byte
-// aligned buffers of (own tile [14][kTS], halo [9][6 n2]); the interface items write
-// their lifted terms over the halo slots they read (components 0-4), so that the
-// footprint leaves room for the L1 cache that the halo gathers and RK loads go through.  An own-tile row has
-// room for the element's 0-3 float misalignment (node nd of component c at c kTS + sh + nd,
-// sh = (e np) mod 4), so that the bulk copies land on 16-byte boundaries.
-template <int P>
-__host__ __device__ constexpr int stream_tile_stride() { return ((P + 1) * (P + 1) * (P + 1) + 3 + 3) & ~3; }
-template <int P>
-__host__ __device__ constexpr int stream_buf_floats() {
-  return (14 * stream_tile_stride<P>() + kFaceComponents * 6 * (P + 1) * (P + 1) + 3) & ~3;
-}
-template <int P>
-__host__ __device__ constexpr int stream_buf_offset() {
-  return (4 + 15 * (P + 1) * (P + 1) * (P + 1) + 3) & ~3;
-}
-template <int P>
-__host__ __device__ constexpr int stream_smem_floats() {
-  return stream_buf_offset<P>() + 2 * stream_buf_floats<P>();
-}
-
-
-
-template <int P, int MODE, class Src>
-__device__ __forceinline__ void flux_stream(const Src& src, int n_items) {
-  using T = float;
-  constexpr int n = P + 1, n2 = n * n, np = n2 * n, haloN = 6 * n2;
-  constexpr int FC = kFaceComponents;
-  constexpr int kTS = stream_tile_stride<P>();
-  constexpr int kBuf = stream_buf_floats<P>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw);  // one per buffer
-  T* sV = reinterpret_cast<T*>(smem_raw) + 4;  // [3][5][np]: volume fluxes, then their derivatives
-  T* buf0 = reinterpret_cast<T*>(smem_raw) + stream_buf_offset<P>();  // two buffers: own tile, halo
-
-  // element k + 1's own tile and halo into buffer bi; the own tile's rows by one bulk
-  // copy each (16-byte aligned interior, issued by thread 0, counted on bar[bi]) and their
-  // 0-3 float ragged ends by 4-byte cp.async, or (unaligned layouts) all by cp.async
-  auto prefetch = [&](int item, int bi) {
-    const StreamItem m = src.at(item);
-    T* b = buf0 + bi * kBuf;
-    const long long N = m.C->N;
-    const long long e0 = (long long)m.e * np;
-    const int sh = (int)(e0 & 3);
-    if (m.bulk) {
-      const int hd = (4 - sh) & 3, tl = (sh + np) & 3, L = np - hd - tl;
-      if (threadIdx.x == 0) {
-        bulk_expect_tx(&bar[bi], 14u * 4u * (unsigned)L);
-        for (int c = 0; c < 14; ++c) {
-          const float* g = (c < 5 ? m.qf + c * N : m.vis + (c - 5) * N) + e0;
-          bulk_copy(b + c * kTS + sh + hd, g + hd, 4u * (unsigned)L, &bar[bi]);
-        }
-      }
-      for (int i = threadIdx.x; i < 14 * 8; i += blockDim.x) {
-        const int c = i >> 3, j = i & 7;
-        if (j < 4 ? j >= hd : j - 4 >= tl) continue;
-        const int nd = j < 4 ? j : np - tl + (j - 4);
-        const float* g = (c < 5 ? m.qf + c * N : m.vis + (c - 5) * N) + e0;
-        cp_async4(b + c * kTS + sh + nd, g + nd);
-      }
-    } else {
-      for (int nd = threadIdx.x; nd < np; nd += blockDim.x) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async4(b + v * kTS + sh + nd, m.qf + v * N + e0 + nd);
-#pragma unroll
-        for (int c = 0; c < 9; ++c) cp_async4(b + (5 + c) * kTS + sh + nd, m.vis + c * N + e0 + nd);
-      }
-    }
-    const BlockCoords bc = block_coords(m.e, m.C->K);
-    T* h = b + 14 * kTS;
-    for (int t = threadIdx.x; t < haloN; t += blockDim.x) {
-      const Item<P> it = item_of<P>(t);
-      const int enb = neighbour_of(bc, 0, m.C->K, Src::kSlab ? m.C->Kz : m.C->K, it.d, it.side ? 1 : -1);
-      const long long gnb = (long long)enb * np + face_node<P>(it.d, it.side ? 0 : P, it.ab);
-      switch (it.d) {
-        case 0: copy_face_data<0>(m.qf, m.vis, N, gnb, h + t, haloN); break;
-        case 1: copy_face_data<1>(m.qf, m.vis, N, gnb, h + t, haloN); break;
-        default: copy_face_data<2>(m.qf, m.vis, N, gnb, h + t, haloN);
-      }
-    }
-    cp_async_commit();
-  };
-
-  pdl_wait();
-  int item = blockIdx.x;
-  if (item >= n_items) return;
-  if (threadIdx.x == 0) {
-    bulk_bar_init(&bar[0]);
-    bulk_bar_init(&bar[1]);
-    bulk_bar_fence_init();
-  }
-  __syncthreads();
-  prefetch(item, 0);
-  const int node = threadIdx.x;
-  const bool active = node < np;
-  const int idx[3] = {node % n, (node / n) % n, node / n2};
-
-  unsigned phases = 0u;   // bit i: parity of buffer i's next bulk phase (members may mix modes)
-  for (int k = 0; item < n_items; item += gridDim.x, ++k) {
-    const StreamItem m = src.at(item);
-    T* b = buf0 + (k & 1) * kBuf;
-    cp_async_wait_all();
-    bool landed = true;
-    if (m.bulk) {
-      landed = bulk_wait(&bar[k & 1], (phases >> (k & 1)) & 1u);
-      phases ^= 1u << (k & 1);
-    }
-    if (__syncthreads_or(!landed)) {       // this item's data landed; the other buffer is free
-      if (threadIdx.x == 0 && m.err) atomicExch(m.err, 1);
-      break;                               // a bounded wait expired: give up (host reports it)
-    }
-    const int next = item + gridDim.x;
-    if (next < n_items) prefetch(next, (k + 1) & 1);
-    else pdl_release();   // this block's last element: the successor may launch
-
-    const OpConst<T>& C = *m.C;
-    const RkArgs<T>& rk = *m.rk;
-    const long long N = C.N;
-    const long long gi = (long long)m.e * np + node;
-    T* sX = b + (int)(((long long)m.e * np) & 3);   // own tile: component c of node nd at sX[c kTS + nd]
-    T* sH = b + 14 * kTS;
-
-    // RK operands of this thread's node, loaded now and used at the end
-    T gold[5], dold[5];
-    double qold[5];
-    if (active) {
-      if (MODE == 3 || MODE == 4) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) dold[v] = m.dlt[v * N + gi];
-      }
-      if (MODE == 4) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) gold[v] = m.greg[v * N + gi];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) qold[v] = m.q[v * N + gi];
-      }
-    }
-
-    // volume fluxes of this thread's node into sV (the own tile stays intact for the
-    // interface items, so no barrier separates the two)
-    if (active) {
-      T s[5], vs[9];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) s[v] = sX[v * kTS + node];
-#pragma unroll
-      for (int c = 0; c < 9; ++c) vs[c] = sX[(5 + c) * kTS + node];
-      const Prim<T> w = prim_c(s, C);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        T F[5], fv[5];
-        euler_flux(s, w, C.Hc, d, F);
-        viscous_flux(vs, w.v, d, fv);
-#pragma unroll
-        for (int c = 0; c < 5; ++c) sV[(5 * d + c) * np + node] = F[c] - fv[c];
-      }
-    }
-
-    // interface terms, one work item per (face, face node); each item reads its halo slot
-    // and then writes its lifted terms over components 0-4 of that slot
-    for (int t = threadIdx.x; t < haloN; t += blockDim.x) {
-      const Item<P> it = item_of<P>(t);
-      const int o = face_node<P>(it.d, it.side ? P : 0, it.ab);
-      T so[5], to[4], sn[5], tn[4];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) so[v] = sX[v * kTS + o];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) sn[v] = sH[v * haloN + t];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) tn[i] = sH[(5 + i) * haloN + t];
-      switch (it.d) {
-        case 0:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(0, i)) * kTS + o];
-          interface_item<0>(so, to, sn, tn, sH + t, haloN, it.side, C);
-          break;
-        case 1:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(1, i)) * kTS + o];
-          interface_item<1>(so, to, sn, tn, sH + t, haloN, it.side, C);
-          break;
-        default:
-#pragma unroll
-          for (int i = 0; i < 4; ++i) to[i] = sX[(5 + face_vis_index(2, i)) * kTS + o];
-          interface_item<2>(so, to, sn, tn, sH + t, haloN, it.side, C);
-      }
-    }
-    __syncthreads();
-
-    // volume term: one task per (direction, component, line) replaces the line's fluxes
-    // by their derivative; tasks are direction-major so that a warp shares d
-    for (int task = threadIdx.x; task < 15 * n2; task += blockDim.x) {
-      const int dc = task / n2, ab = task - dc * n2;
-      float* f = sV + dc * np;
-      if (dc < 5) line_derivative_inplace<P, 0>(f, ab);
-      else if (dc < 10) line_derivative_inplace<P, 1>(f, ab);
-      else line_derivative_inplace<P, 2>(f, ab);
-    }
-    __syncthreads();
-    if (!active) continue;
-
-    T R[5] = {T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-#pragma unroll
-      for (int c = 0; c < 5; ++c) R[c] -= C.s2h * sV[(5 * d + c) * np + node];
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const bool right = (idx[d] == P), left = (idx[d] == 0);
-      if (!(right || left)) continue;
-      const int h = item_index<P>(face_ab<P>(d, idx), right ? 1 : 0, d, 0);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) R[c] += sH[c * haloN + h];   // lifted terms over the halo slots
-    }
-    if (m.fc.s != nullptr) {
-      const long long fb = (long long)m.e * m.fc.stride + node;
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const int slot = c - m.fc.first_var;
-        if (slot >= 0 && slot < m.fc.n_vars) R[c] += T(m.fc.s[fb + (long long)slot * np]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const long long o = c * N + gi;
-      if (MODE == 0) {
-        m.dqdt[o] = double(R[c]);
-      } else if (MODE == 2) {
-        m.dlt[o] = float(rk.B * (rk.dt * R[c]));
-      } else if (MODE == 3) {
-        const T g2 = rk.A * (dold[c] * rk.invB1) + rk.dt * R[c];
-        m.greg[o] = g2;
-        m.dlt[o] = float(dold[c] + rk.B * g2);
-      } else if (MODE == 4) {
-        const T g3 = rk.A * gold[c] + rk.dt * R[c];
-        const float d3 = float(dold[c] + rk.B * g3);
-        m.q[o] = qold[c] + f2d(d3);
-      }
-    }
-  }
-  cp_async_wait_all();
-}
-
-// Operands of one mesh for the streamed kernel (kernel parameter).
-struct StreamMesh {
-  double* q;
-  const float* qf;
-  const float* vis;
-  double* dqdt;
-  float* greg;
-  float* dlt;
-  Forcing fc;
-  OpConst<float> C;
-  RkArgs<float> rk;
-  int bulk;  // qf and vis 16-byte aligned and N a multiple of 4: own tiles by TMA bulk copies
-  int* err;  // device error flag (may be NULL)
-};
-
-template <bool SLAB>
-struct SingleSource {
-  static constexpr bool kSlab = SLAB;
-  const StreamMesh& m;
-  __device__ __forceinline__ StreamItem at(int item) const {
-    return StreamItem{m.q, m.qf, m.vis, m.dqdt, m.greg, m.dlt, &m.C, &m.rk, m.fc, (SLAB ? m.C.e_begin : 0) + item,
-                      m.bulk, m.err};
-  }
-};
-
-struct BatchSource {
-  static constexpr bool kSlab = false;
-  const BatchTable<float>& tb;
-  __device__ __forceinline__ StreamItem at(int item) const {
-    const int i = batch_instance(tb.block_start, tb.n, item);
-    return StreamItem{tb.q[i], tb.qf[i], tb.vis[i], nullptr, tb.g[i], tb.dlt[i], &tb.C[i], &tb.rk[i], Forcing{},
-                      item - tb.block_start[i], tb.bulk[i], tb.err[i]};
-  }
-};
-
-template <int P, int MODE, bool SLAB = false>
-__global__ void __launch_bounds__(stream_threads(P), stream_min_blocks(P))
-k_flux_stream(const __grid_constant__ StreamMesh mesh) {
-  flux_stream<P, MODE>(SingleSource<SLAB>{mesh}, mesh.C.nel - (SLAB ? mesh.C.e_begin : 0));
-}
-
-// Batched streamed phase B: members of order P, one element per work item
-// (block_start counts elements).
-template <int P, int MODE>
-__global__ void __launch_bounds__(stream_threads(P), stream_min_blocks(P))
-k_flux_stream_batch(const __grid_constant__ BatchTable<float> tb) {
-  flux_stream<P, MODE>(BatchSource{tb}, tb.block_start[tb.n]);
+  surface_block<P, T, MODE>(blk, surf_elems(P), tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);
 }
 
 }  // namespace dgnn

@@ -4,14 +4,13 @@
 // allowed or not wanted -- an in-situ analysis hook inside another solver's time loop
 // whose device memory was budgeted and locked at start-up, or a host thread that must
 // not take the allocator's locks or synchronise the device (cudaMalloc and cudaFree may
-// do both).  dg_create allocates its workspace (stage state and viscous stresses, ~112
-// bytes per node in FP64); this entry point instead uses one fixed scratch array that
+// do both).  dg_create allocates its workspace (stage state, volume term and face fluxes); this entry point instead uses one fixed scratch array that
 // lives in the library's own device image.
 //
-// The scratch array holds the two intermediate fields of one operator evaluation: the
-// stage state (5 values per node) and the viscous stresses and heat flux (9 values per
-// node), at most kNoallocMaxNodes nodes.  Every GPU that loads the library keeps it
-// (3.7 MB) until the process exits.  All calls on a device share it and it keeps the
+// The scratch array holds the three intermediate fields of one operator evaluation: the
+// stage state and the volume term (5 values per node each) and the viscous fluxes normal to
+// the faces (4 values per face node), at most kNoallocMaxNodes nodes.  Every GPU that loads the library keeps it
+// (5.8 MB) until the process exits.  All calls on a device share it and it keeps the
 // last call's contents; nothing in it needs to start at zero, because the first kernel
 // of every call writes every entry it later reads.  Calls whose work overlaps on the GPU
 // (different streams, or different host threads) race on the array: serialise them.
@@ -32,7 +31,9 @@ namespace dgnn {
 namespace {
 
 constexpr long long kNoallocMaxNodes = 32768;  // e.g. 8^3 elements at P = 3, 4^3 at P = 7
-constexpr long long kNoallocDoubles = 14 * kNoallocMaxNodes;
+// values per node of the three fields, at most (P = 1): 2 x 5 node values and 24 per face
+// node over the (P + 1) nodes behind it
+constexpr long long kNoallocDoubles = 22 * kNoallocMaxNodes;
 constexpr int kNoallocMaxDevices = 64;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocDoubles];
@@ -93,19 +94,18 @@ extern "C" int dg_rhs_noalloc(int K, int P, double Re, double Mach, double Pr, i
   dg_ctx c;
   rc = setup_ctx(&c, K, P, Re, Mach, Pr, closure, o);
   if (rc) return rc;
-  // stage state then viscous quantities, in the operator precision
-  if (precision == DG_PREC_FP32) {
-    float* s = reinterpret_cast<float*>(scratch);
-    c.qf = s;
-    c.vis = s + 5 * nodes;
-  } else {
-    c.qf = scratch;
-    c.vis = scratch + 5 * nodes;
-  }
+  // stage state, volume term and face-normal viscous fluxes, in the operator precision
+  const size_t rec = (size_t)c.nel * state_record(c.n), tsz = precision == DG_PREC_FP32 ? 4 : 8;
+  static_assert(2 * state_record(2) + face_record(2) <= 22 * 8 && 2 * state_record(3) + face_record(3) <= 22 * 27,
+                "scratch values per node (the padding and faces weigh most at low order)");
+  unsigned char* s = reinterpret_cast<unsigned char*>(scratch);
+  c.qf = c.cur = s;
+  c.rv = s + rec * tsz;
+  c.vt = s + 2 * rec * tsz;
   cudaStream_t st = (cudaStream_t)stream;
-  DG_CUDA(launch_gradient(&c, q, 0, st));
-  DG_CUDA(launch_flux(&c, const_cast<double*>(q), dqdt, Forcing{}, 0, 0.0, 0.0, 0.0, st));
+  DG_CUDA(launch_volume(&c, q, 0, st));
+  DG_CUDA(launch_surface(&c, const_cast<double*>(q), dqdt, Forcing{}, 0, RkStage{}, 0.0, st));
   // the context lives on the stack and owns nothing: keep its destructor-free fields empty
-  c.qf = c.vis = nullptr;
+  c.qf = c.cur = c.rv = c.vt = nullptr;
   return DG_OK;
 }

@@ -109,9 +109,9 @@ __global__ void k_prep_state(const double* __restrict__ q, long long N, int np, 
   out[t] = __float2bfloat16_rn(v);
 }
 
-// Same from the FP32 reference-shifted stage state qf[var][elem][node] of an FP32 context;
-// mshift = mean - reference, formed on the host in FP64.
-__global__ void k_prep_state_f32(const float* __restrict__ qf, long long N, int np, int first_var, int n_vars, int e0,
+// Same from the FP32 reference-shifted stage state of an FP32 context, element-major
+// records s[elem][var][node] of rec values with node stride ns; mshift = mean - reference, formed on the host in FP64.
+__global__ void k_prep_state_f32(const float* __restrict__ s, int rec, int ns, int np, int first_var, int n_vars, int e0,
                                  int rows, int ld, const float* __restrict__ mshift, const float* __restrict__ sd,
                                  bf16* __restrict__ out) {
   pdl_enter();
@@ -121,7 +121,7 @@ __global__ void k_prep_state_f32(const float* __restrict__ qf, long long N, int 
   float v = 0.f;
   if (f < n_vars * np) {
     const int slot = f / np, node = f - slot * np;
-    const float x = qf[(long long)(first_var + slot) * N + (long long)(e0 + r) * np + node];
+    const float x = s[(long long)(e0 + r) * rec + (first_var + slot) * ns + node];
     v = (x - mshift[f]) / sd[f];
   }
   out[t] = __float2bfloat16_rn(v);
@@ -561,7 +561,8 @@ int nn_forcing_on_state(const nn_model* m, const dg_ctx* c, const double* q, flo
     if (features_ready && rows == c->nel) {
       // the phase-A launch before this call wrote the features (nn_phase_a_features)
     } else if (f32) {
-      DG_CUDA(pdl_launch(k_prep_state_f32, dim3(blocks_for(tot, 256)), dim3(256), st, static_cast<const float*>(c->qf), c->N, c->np,
+      DG_CUDA(pdl_launch(k_prep_state_f32, dim3(blocks_for(tot, 256)), dim3(256), st, static_cast<const float*>(c->cur), state_record(c->n),
+                                                             node_stride(c->n), c->np,
                                                              m->d.first_var, m->d.n_vars, e0, rows, m->pad[0],
                                                              m->mean_shift, m->std_in, m->act[0]));
     } else {
@@ -854,7 +855,10 @@ int nn_forcing_infer(const nn_model* m, const dg_ctx* c, const double* q, float*
   if (!m || !c || !q || !s) return fail(DG_ERR_INVALID_ARG, "nn_forcing_infer: NULL argument");
   cudaStream_t st = (cudaStream_t)stream;
   // the FP32 operator feeds the network its stage state: build it from q (phase A)
-  if (c->opts.precision == DG_PREC_FP32) DG_CUDA(launch_gradient(c, q, 0, st));
+  if (c->opts.precision == DG_PREC_FP32) {
+    const_cast<dg_ctx*>(c)->cur = c->qf;
+    DG_CUDA(launch_volume(c, q, 0, st));
+  }
   return nn_forcing_on_state(m, c, q, s, nullptr, nullptr, st);
 }
 
