@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "dg_aux.h"
@@ -63,15 +64,11 @@ cudaError_t launch_surface(const dg_ctx* c, double* q, double* dqdt, const Forci
                                            : surface_f64(c, q, dqdt, f, mode, rk, dt, st);
 }
 
-// Launch plan of RK stage k (0, 1, 2): source of the phase-A stage state and phase-B mode.
-static void stage_plan(const dg_ctx* c, int k, int* src, int* mode) {
-  if (c->opts.precision == DG_PREC_FP32) {
-    *src = (k == 0) ? 0 : 1;
-    *mode = 2 + k;
-  } else {
-    *src = 0;
-    *mode = 1;
-  }
+// Mode of phase B in RK stage k; more: another step follows in the same call, on the state
+// this one leaves (FP32: stage 3 then also forms its stage state).
+static int stage_mode(const dg_ctx* c, int k, bool more) {
+  if (c->opts.precision != DG_PREC_FP32) return 1;
+  return k == 2 && more ? 5 : 2 + k;
 }
 
 // Algorithmic bytes per node of the phase-A and phase-B launches of stage k: every value
@@ -127,8 +124,8 @@ static int exchange_traces(dg_ctx* const* cs, int n, double* const* qs, int what
   return DG_OK;
 }
 
-// Phase-A trace of stage state source src (0: the FP64 state; 1: the FP32 increment scheme).
-static int phase_a_what(const dg_ctx* c, int src) { return (c->opts.precision == DG_PREC_FP32 && src == 1) ? 1 : 0; }
+// Trace before phase A of stage k (0: the FP64 state; 1: the FP32 stage state).
+static int phase_a_what(const dg_ctx* c, int k) { return (c->opts.precision == DG_PREC_FP32 && k > 0) ? 1 : 0; }
 constexpr int kWhatPhaseB = 2;
 
 // dq/dt of n contexts: one whole mesh, or the slabs of one mesh exchanging traces.
@@ -168,19 +165,21 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
                        cudaStream_t st, bool exchange = true) {
   dg_ctx* c = cs[0];
   const bool post = net && c->forcing_mode == DG_FORCING_POST;
+  const bool f32 = c->opts.precision == DG_PREC_FP32;
+  bool ready = false;   // the step's first stage state is in qf
   for (int s = 0; s < nsteps; ++s) {
+    // slabs rebuild it from the exchanged FP64 state, the post form changes q after the step
+    const bool more = s + 1 < nsteps && !c->part && !post;
     Forcing fpost;
     for (int k = 0; k < 3; ++k) {
-      int src, mode;
-      stage_plan(c, k, &src, &mode);
       for (int i = 0; i < n; ++i) cs[i]->cur = stage_buffer(cs[i], k);
-      int rc = exchange ? exchange_traces(cs, n, qs, phase_a_what(c, src), st) : DG_OK;
+      int rc = exchange ? exchange_traces(cs, n, qs, phase_a_what(c, k), st) : DG_OK;
       if (rc) return rc;
       // the forcing's input features come out of the phase-A launch when the network allows
       const bool want = net && (!post || k == 0);
       const bool feats = want && n == 1 && nn_phase_a_features(net, c, &c->feat_out);
       for (int i = 0; i < n; ++i) {
-        const cudaError_t e = launch_volume(cs[i], qs[i], src, st);
+        const cudaError_t e = launch_volume(cs[i], qs[i], f32 && (k > 0 || ready), st);
         cs[i]->feat_out = FeatureOut{};
         DG_CUDA(e);
       }
@@ -195,8 +194,10 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
       }
       rc = exchange ? exchange_traces(cs, n, qs, kWhatPhaseB, st) : DG_OK;
       if (rc) return rc;
-      for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], nullptr, f, mode, rk_stage(k), dt, st));
+      for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], nullptr, f, stage_mode(c, k, more), rk_stage(k), dt, st));
     }
+    ready = f32 && more;
+    if (ready) std::swap(c->qf, c->qy);   // the next step's s1 is in qy
     if (post) DG_CUDA(launch_add_forcing(c, qs[0], fpost, dt, st));
   }
   return DG_OK;
@@ -783,18 +784,16 @@ int dg_profile_rk3(dg_ctx* c, double* q, double dt, int nsteps, double* ms_gradi
     for (int s = 0; s < nsteps && e == cudaSuccess; ++s)
       for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
         const int i = 4 * (3 * s + k);
-        int src, mode;
-        stage_plan(c, k, &src, &mode);
         double gb, fb;
         stage_bytes(c, k, &gb, &fb);
         bg += gb;
         bf += fb;
         c->cur = stage_buffer(c, k);
         cudaEventRecord(ev[i], st);
-        e = launch_volume(c, q, src, st);
+        e = launch_volume(c, q, k > 0 && c->opts.precision == DG_PREC_FP32, st);
         cudaEventRecord(ev[i + 1], st);
         cudaEventRecord(ev[i + 2], st);
-        if (e == cudaSuccess) e = launch_surface(c, q, nullptr, Forcing{}, mode, rk_stage(k), dt, st);
+        if (e == cudaSuccess) e = launch_surface(c, q, nullptr, Forcing{}, stage_mode(c, k, false), rk_stage(k), dt, st);
         cudaEventRecord(ev[i + 3], st);
       }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -391,6 +391,15 @@ __device__ __forceinline__ Prim<T> prim_c(const T s[5], const OpConst<T>& C) {
   return primitives(s, C.rho_ref, C.gm1);
 }
 
+// Variable v of the stage state: the FP64 value relative to the reference, rounded once.
+// The difference is volatile so that the compiler does not form it, on the slow FP64 pipe,
+// for the variables without a reference too.
+template <typename T>
+__device__ __forceinline__ T shifted(double x, int v, const OpConst<T>& C) {
+  if (v == 0 || v == 4) asm volatile("sub.rn.f64 %0, %0, %1;" : "+d"(x) : "d"(v == 0 ? C.drho_ref : C.dE_ref));
+  return from_double<T>(x);
+}
+
 // Stage state of an element's node from the FP64 state q ([var][node], gi = elem n^3 + node).
 template <typename T>
 __device__ __forceinline__ void state_from_q(const double* __restrict__ q, long long gi, const OpConst<T>& C, T s[5]) {
@@ -799,12 +808,16 @@ __device__ __forceinline__ void row_read(const float* p, float v[4]) {
   v[2] = a.z;
   v[3] = a.w;
 }
-// sum_m d[m] row(m) of the rows base, base + step, ...
-__device__ __forceinline__ void rows_contract(const float* base, int step, const f32x2 d[4], float out[4]) {
+// d[0] own + sum_{m = 1..3} d[m] row(at[m - 1]) of the rows at base + at[...]: the thread's own
+// row of a line and the three others.
+__device__ __forceinline__ void rows_contract(const float own[4], const float* base, const int at[3],
+                                              const f32x2 d[4], float out[4]) {
   Row acc{0ull, 0ull};
+  fma2(acc.lo, d[0], pack2(own[0], own[1]));
+  fma2(acc.hi, d[0], pack2(own[2], own[3]));
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const Row r = row_load(base + m * step);
+  for (int m = 1; m < 4; ++m) {
+    const Row r = row_load(base + at[m - 1]);
     fma2(acc.lo, d[m], r.lo);
     fma2(acc.hi, d[m], r.hi);
   }
@@ -834,13 +847,37 @@ __device__ __forceinline__ void state_row(const double* __restrict__ q, const fl
     if (SRC == 0) {
       double d[4];
       row_read64(q + v * C.N + (long long)e * 64 + node, wide, d);
-      const double ref = v == 0 ? C.drho_ref : v == 4 ? C.dE_ref : 0.0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) s[v][i] = d2f_rn(v == 0 || v == 4 ? d[i] - ref : d[i]);
+      for (int i = 0; i < 4; ++i) s[v][i] = shifted(d[i], v, C);
     } else {
       row_read(qf + (size_t)e * state_record(4) + v * 64 + node, s[v]);
     }
   }
+}
+
+// The stage state s1 from the FP64 state, one thread per node, in a pass of its own ahead of a
+// volume4_block<1> launch.  Formed in that launch, a state is converted 2.5 times (own row
+// and neighbours' faces) with the FP64 pipe 63 % busy; one pass moves 60 bytes per node and
+// converts once (32^3 RK3 step 331 -> 306 us, 16^3 58.2 -> 54.1, 8^3 29.7 -> 27.1; a thread per
+// row of four nodes here: 16^3 58.6).  At the other orders, whose kernels hide the
+// conversions, it does not pay (16^3/P8 516 -> 521 us).
+constexpr int kStateElems = 4;   // per block of 256 threads
+__device__ __forceinline__ void state4_block(int blk, const double* __restrict__ q, float* __restrict__ qf, int nel,
+                                             const OpConst<float>& C) {
+  const int e = blk * kStateElems + (threadIdx.x >> 6), node = threadIdx.x & 63;
+  if (e >= nel) return;
+  float s[5];
+  state_from_q(q, (long long)e * 64 + node, C, s);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) qf[(size_t)e * state_record(4) + v * 64 + node] = s[v];
+}
+
+template <typename T>   // float only
+__global__ void __launch_bounds__(256) k_state4(const double* __restrict__ q, T* __restrict__ qf, int nel,
+                                                const OpConst<T> C) {
+  pdl_wait();
+  pdl_release();
+  state4_block(blockIdx.x, q, qf, nel, C);
 }
 
 constexpr int kRows4Floats = 18 * 64;   // shared floats per element: U, halo rows (4 + 4), y- and z-fluxes (10)
@@ -933,19 +970,24 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
         fo[slot * 64 + i] = __float2bfloat16_rn((s[v][i] - C.feat.shift32[f + i]) / C.feat.sd[f + i]);
     }
   }
+  // the other rows of this row's y- and z-line (j ^ m, k ^ m) and their matrix entries
   f32x2 Dy[4], Dz[4];
+  int yat[3], zat[3];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    const float dy = C.D[4 * j + m], dz = C.D[4 * k + m];
+    const float dy = C.D[4 * j + (j ^ m)], dz = C.D[4 * k + (k ^ m)];
     Dy[m] = pack2(dy, dy);
     Dz[m] = pack2(dz, dz);
+    if (m) {
+      yat[m - 1] = 4 * ((j ^ m) + 4 * k);
+      zat[m - 1] = 4 * (j + 4 * (k ^ m));
+    }
   }
   __syncwarp(half);
 
   // BR1 gradient G[d][a][node], lifted with the central U^ = (U + U_nb) / 2
   float G[3][4][4];
   const float lift = C.s2h * C.winv * 0.5f;
-  const int ky = 4 * k, jz = 4 * j;   // first float of the y-line's and z-line's rows: 4 (0 + 4 k), 4 (j + 0)
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
 #pragma unroll
@@ -957,8 +999,8 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
     }
     G[0][a][0] = fma_(-lift, UL[a] - U[a][0], G[0][a][0]);
     G[0][a][3] = fma_(lift, UR[a] - U[a][3], G[0][a][3]);
-    rows_contract(sU + a * 64 + 4 * ky, 4, Dy, G[1][a]);
-    rows_contract(sU + a * 64 + jz, 16, Dz, G[2][a]);
+    rows_contract(U[a], sU + a * 64, yat, Dy, G[1][a]);
+    rows_contract(U[a], sU + a * 64, zat, Dz, G[2][a]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       G[1][a][i] = mul_(C.s2h, G[1][a][i]);
@@ -1020,7 +1062,7 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   ve[112 + r] = vis[6][3];
   if (j == 0 || j == 3) {                   // y: tau_yy, tau_yz, tau_yx, k th_y
     const float sg = j ? 1.f : -1.f;
-    float* o = ve + (j ? 192 : 128) + ky;
+    float* o = ve + (j ? 192 : 128) + 4 * k;
     float t[3][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1035,7 +1077,7 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   }
   if (k == 0 || k == 3) {                   // z: tau_zz, tau_zx, tau_zy, k th_z
     const float sg = k ? 1.f : -1.f;
-    float* o = ve + (k ? 320 : 256) + jz;
+    float* o = ve + (k ? 320 : 256) + 4 * j;
     float t[3][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1073,15 +1115,24 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       if (d == 0) {
+        // the energy flux relative to the row's first node: D annihilates constants, and the
+        // large common part at low Mach numbers stays out of the rounding
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float g = 0.f;
 #pragma unroll
-          for (int m = 0; m < 4; ++m) g += C.D[4 * i + m] * F[c][m];
+          for (int m = c == 4 ? 1 : 0; m < 4; ++m)
+            g = fma_(C.D[4 * i + m], c == 4 ? add_(F[4][m], -F[4][0]) : F[c][m], g);
           R[c][i] = mul_(-C.s2h, g);
         }
       } else {
         row_store(sF + (5 * (d - 1) + c) * 64 + 4 * r, F[c]);
+        if (c < 4) {   // the own row's share now, the others' after the exchange
+          float own, other;
+          unpack2(d == 1 ? Dy[0] : Dz[0], own, other);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h * own, F[c][i], R[c][i]);
+        }
       }
     }
   }
@@ -1089,13 +1140,27 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   float* re = rv + (size_t)e * state_record(4) + 4 * r;
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    float y[4], z[4];
-    rows_contract(sF + c * 64 + 4 * ky, 4, Dy, y);
-    rows_contract(sF + (5 + c) * 64 + jz, 16, Dz, z);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      R[c][i] = fma_(-C.s2h, z[i], fma_(-C.s2h, y[i], R[c][i]));
+    Row acc{0ull, 0ull}, y0, z0;
+    if (c == 4) {   // the energy flux relative to the own row, as above
+      y0 = row_load(sF + c * 64 + 4 * r);
+      z0 = row_load(sF + (5 + c) * 64 + 4 * r);
     }
+#pragma unroll
+    for (int m = 1; m < 4; ++m) {
+      Row y = row_load(sF + c * 64 + yat[m - 1]), z = row_load(sF + (5 + c) * 64 + zat[m - 1]);
+      if (c == 4) {
+        y = Row{line_sub(y.lo, y0.lo), line_sub(y.hi, y0.hi)};
+        z = Row{line_sub(z.lo, z0.lo), line_sub(z.hi, z0.hi)};
+      }
+      fma2(acc.lo, Dy[m], y.lo);
+      fma2(acc.hi, Dy[m], y.hi);
+      fma2(acc.lo, Dz[m], z.lo);
+      fma2(acc.hi, Dz[m], z.hi);
+    }
+    float g[4];
+    row_unpack(acc, g);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
     row_store(re + c * 64, R[c]);
   }
 }
@@ -1157,8 +1222,8 @@ struct SurfArgs {
   double* dqdt;       // MODE 0
   T* g;               // MODE 1: RK register
   T* x;               // MODE 2: s1 (read); MODE 3: s1, replaced by s3
-  T* y;               // MODE 2: s2 (written)
-  float* dlt;         // MODES 2, 3, 4: increment (see the head of this file)
+  T* y;               // MODE 2: s2, MODE 5: the next step's s1 (written)
+  float* dlt;         // MODES 2 to 5: increment (see the head of this file)
 };
 
 // The FP32 increment scheme, one value.  Stage 1: g1 = dt R, d1 = B1 g1, s2 = s1 + d1.
@@ -1329,7 +1394,8 @@ __host__ __device__ constexpr size_t surface_smem_bytes(int E) {
 }
 
 // MODE 0: dqdt = R.  MODE 1: FP64 RK stage (g = A g + dt R; q += B g).
-// MODES 2, 3, 4: FP32 increment scheme, stages 1, 2, 3.
+// MODES 2, 3, 4: FP32 increment scheme, stages 1, 2, 3; MODE 5: stage 3 that also writes the
+// next step's s1 (to y: neighbours still read s3 in x).
 // Phase B of block `blk` of one mesh, E elements (the body of k_surface and k_surface_batch).
 // prologue: work that may run before the previous launch has completed.
 template <int P, typename T, bool CUBE>
@@ -1465,8 +1531,8 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
         double q1[4];
         float u[4], v[4], x1[4], g1[4];
         if (MODE == 2 || MODE == 3) row_read(a.x + o + c * 64, x1);
-        if (MODE == 3 || MODE == 4) row_read(a.dlt + o + c * 64, g1);
-        if (MODE == 4) row_read64(a.q + c * C.N + g, wide, q1);
+        if (MODE >= 3) row_read(a.dlt + o + c * 64, g1);
+        if (MODE >= 4) row_read64(a.q + c * C.N + g, wide, q1);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (MODE == 0) q1[i] = double(R[c][i]);
@@ -1486,6 +1552,11 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
 #pragma unroll
             for (int i = 0; i < 4; ++i) out[i] = q1[i];
           }
+          if (MODE == 5) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) u[i] = shifted(q1[i], c, C);
+            row_store(a.y + o + c * 64, u);
+          }
         }
       }
     }
@@ -1504,7 +1575,7 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
 #pragma unroll
       for (int c = 0; c < 5; ++c) x1[c] = a.x[o + c * ns];
     }
-    if (MODE == 3 || MODE == 4) {
+    if (MODE >= 3) {
 #pragma unroll
       for (int c = 0; c < 5; ++c) g1[c] = T(a.dlt[o + c * ns]);
     }
@@ -1512,7 +1583,7 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
 #pragma unroll
       for (int c = 0; c < 5; ++c) g1[c] = rk.A == T(0) ? T(0) : a.g[o + c * ns];
     }
-    if (MODE == 1 || MODE == 4) {
+    if (MODE == 1 || MODE >= 4) {
 #pragma unroll
       for (int c = 0; c < 5; ++c) q1[c] = a.q[c * C.N + g];
     }
@@ -1554,7 +1625,9 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
         a.x[o + c * ns] = s3;
         a.dlt[o + c * ns] = float(w);
       } else {
-        a.q[c * C.N + g] = q1[c] + f2d(float(rk_stage3(rk, R[c], g1[c])));
+        const double qn = q1[c] + f2d(float(rk_stage3(rk, R[c], g1[c])));
+        a.q[c * C.N + g] = qn;
+        if (MODE == 5) a.y[o + c * ns] = shifted(qn, c, C);
       }
     }
   }
@@ -1586,6 +1659,7 @@ struct BatchTable {
   int n;                             // instances in this launch
   int block_start[kMaxBatch + 1];    // first phase-A block of each instance; block_start[n] = grid
   int surf_start[kMaxBatch + 1];     // the same for phase B
+  int state_start[kMaxBatch + 1];    // the same for the state pass (P = 3, FP32)
   T* qs[kMaxBatch];                  // stage state of this stage
   T* rv[kMaxBatch];                  // volume term
   T* vt[kMaxBatch];                  // face-normal viscous fluxes
@@ -1599,6 +1673,14 @@ __device__ __forceinline__ int batch_instance(const int* start, int n, int b) {
   int i = 0;
   while (i + 1 < n && b >= start[i + 1]) ++i;
   return i;
+}
+
+template <typename T>   // float only
+__global__ void __launch_bounds__(256) k_state4_batch(const __grid_constant__ BatchTable<T> tb) {
+  pdl_wait();
+  pdl_release();
+  const int i = batch_instance(tb.state_start, tb.n, blockIdx.x);
+  state4_block(blockIdx.x - tb.state_start[i], tb.a[i].q, tb.qs[i], tb.C[i].nel, tb.C[i]);
 }
 
 template <int P, typename T, int SRC>

@@ -122,10 +122,19 @@ cudaError_t volume_p(const dg_ctx* c, const double* q, cudaStream_t st) {
 
 template <int P, typename T, bool SPLIT>
 cudaError_t volume_src(const dg_ctx* c, const double* q, int src, cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (src != 0) return volume_p<P, T, 1, SPLIT>(c, q, st);
+  if constexpr (use_rows4(P, sizeof(T), SPLIT)) {
+    if (src == 0) {   // the state in a pass of its own (c->cur is then c->qf)
+      const cudaError_t e = launch_pdl(k_state4<T>, dim3((c->nel + kStateElems - 1) / kStateElems), dim3(256), 0, st, q,
+                                       static_cast<T*>(c->qf), c->nel, make_const<T>(c));
+      if (e != cudaSuccess) return e;
+    }
+    return volume_p<P, T, 1, SPLIT>(c, q, st);
+  } else {
+    if constexpr (std::is_same<T, float>::value) {
+      if (src != 0) return volume_p<P, T, 1, SPLIT>(c, q, st);
+    }
+    return volume_p<P, T, 0, SPLIT>(c, q, st);
   }
-  return volume_p<P, T, 0, SPLIT>(c, q, st);
 }
 
 #define DG_FOR_EACH_P(CALL)        \
@@ -199,6 +208,7 @@ cudaError_t surface_mode(const dg_ctx* c, double* q, double* dqdt, const Forcing
       case 2: return surface_p<P, T, 2>(c, q, dqdt, f, rk, st);
       case 3: return surface_p<P, T, 3>(c, q, dqdt, f, rk, st);
       case 4: return surface_p<P, T, 4>(c, q, dqdt, f, rk, st);
+      case 5: return surface_p<P, T, 5>(c, q, dqdt, f, rk, st);
     }
   } else {
     switch (mode) {
@@ -231,13 +241,15 @@ template <typename T>
 void fill_batch(BatchTable<T>* tb, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
                 const RkStage& rk) {
   tb->n = n;
-  int blocks = 0, surf = 0;
+  int blocks = 0, surf = 0, state = 0;
   for (int i = 0; i < n; ++i) {
     const dg_ctx* c = ctx[i];
     tb->block_start[i] = blocks;
     blocks += (owned_elems(c) + c->geom.E - 1) / c->geom.E;
     tb->surf_start[i] = surf;
     surf += (owned_elems(c) + surf_elems(c->P) - 1) / surf_elems(c->P);
+    tb->state_start[i] = state;
+    state += (c->nel + kStateElems - 1) / kStateElems;
     tb->qs[i] = static_cast<T*>(stage_buffer(c, k));
     tb->rv[i] = static_cast<T*>(c->rv);
     tb->vt[i] = static_cast<T*>(c->vt);
@@ -249,6 +261,7 @@ void fill_batch(BatchTable<T>* tb, dg_ctx* const* ctx, double* const* q, const d
   }
   tb->block_start[n] = blocks;
   tb->surf_start[n] = surf;
+  tb->state_start[n] = state;
 }
 
 // Stage k of the RK3 step: the same source and mode sequence as the single-mesh path
@@ -258,13 +271,18 @@ cudaError_t batch_stage_p(const BatchTable<T>& tb, int E, int k, cudaStream_t st
   void (*kg)(const BatchTable<T>);
   void (*kf)(const BatchTable<T>);
   if constexpr (std::is_same<T, float>::value) {
-    kg = k == 0 ? k_volume_batch<P, T, 0> : k_volume_batch<P, T, 1>;
+    if constexpr (use_rows4(P, sizeof(T), false)) kg = k_volume_batch<P, T, 1>;
+    else kg = k == 0 ? k_volume_batch<P, T, 0> : k_volume_batch<P, T, 1>;
     kf = k == 0 ? k_surface_batch<P, T, 2> : k == 1 ? k_surface_batch<P, T, 3> : k_surface_batch<P, T, 4>;
   } else {
     kg = k_volume_batch<P, T, 0>;
     kf = k_surface_batch<P, T, 1>;
   }
   cudaError_t e;
+  if constexpr (use_rows4(P, sizeof(T), false)) {
+    if (k == 0 && (e = launch_pdl(k_state4_batch<T>, dim3(tb.state_start[tb.n]), dim3(256), 0, st, tb)) != cudaSuccess)
+      return e;
+  }
   if ((e = launch_pdl(kg, dim3(tb.block_start[tb.n]), dim3(volume_threads<P, T, false>(E)),
                       volume_smem<P, T, false>(E, false), st, tb)) != cudaSuccess)
     return e;
@@ -276,7 +294,8 @@ cudaError_t batch_stage_p(const BatchTable<T>& tb, int E, int k, cudaStream_t st
 template <int P, typename T>
 cudaError_t batch_prepare_p(int E) {
   const size_t gs = volume_smem<P, T, false>(E, false), fs = surface_smem_bytes<P, T>(surf_elems(P));
-  cudaError_t e = set_smem(k_volume_batch<P, T, 0>, gs);
+  cudaError_t e = cudaSuccess;
+  if constexpr (!use_rows4(P, sizeof(T), false)) e = set_smem(k_volume_batch<P, T, 0>, gs);
   if (e != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
     if ((e = set_smem(k_volume_batch<P, T, 1>, gs)) != cudaSuccess) return e;

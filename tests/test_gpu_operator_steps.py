@@ -1,0 +1,67 @@
+"""Several RK3 steps in one call, and states on addresses that are only 8-byte aligned: the
+branches of the FP32 operator that one step on an aligned state does not reach."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2207_11571_gb300 import inputs  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def dg():
+    from tests.libbuild import ensure_built
+    ensure_built()
+    from paper_2207_11571_gb300 import dg as _dg
+    _dg.lib()
+    return _dg
+
+
+def state(dg, ctx, N):
+    q = torch.empty(5 * N, dtype=torch.float64, device="cuda")
+    dg.dg_init_tgv(ctx, q, torch.from_numpy(inputs.perturbation((5, N), eps=1e-3).ravel()).cuda())
+    return q
+
+
+@pytest.mark.parametrize("K,P,les,split,prec", [(4, 3, 0, 0, 1), (3, 3, 1, 0, 1), (3, 3, 0, 1, 1), (5, 1, 0, 0, 1),
+                                                (3, 2, 1, 0, 1), (3, 4, 0, 0, 1), (2, 5, 1, 0, 1), (3, 6, 0, 0, 1),
+                                                (2, 7, 0, 0, 1), (2, 8, 0, 1, 1), (3, 3, 0, 0, 0)])
+def test_steps_in_one_call_equal_single_steps(dg, K, P, les, split, prec):
+    """Within a call the FP32 operator's last stage also forms the next step's stage state
+    (in the other buffer); the same conversions, so the same bits as a step per call."""
+    N = K ** 3 * (P + 1) ** 3
+    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, les, precision=prec, volume_flux=split)
+    try:
+        q = state(dg, ctx, N)
+        dt = dg.dg_stable_dt(ctx, q, 0.5)
+        one, many = q.clone(), q.clone()
+        for _ in range(5):
+            dg.dg_rk3_step(ctx, one, dt, 1)
+        dg.dg_rk3_step(ctx, many, dt, 3)   # an odd number of steps leaves the buffers exchanged
+        dg.dg_rk3_step(ctx, many, dt, 2)
+        torch.cuda.synchronize()
+        assert torch.isfinite(many).all() and not torch.equal(many, q)
+        assert torch.equal(many, one)
+    finally:
+        dg.dg_destroy(ctx)
+
+
+@pytest.mark.parametrize("K", [3, 4])
+def test_state_on_an_8_byte_boundary_equals_an_aligned_one(dg, K):
+    """At P = 3 the FP64 state moves in 16-byte vectors where its address allows."""
+    P, N = 3, K ** 3 * 64
+    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=1)
+    try:
+        q = state(dg, ctx, N)
+        buf = torch.empty(5 * N + 1, dtype=torch.float64, device="cuda")
+        odd = buf[1:]
+        odd.copy_(q)
+        R, Rbuf = torch.empty_like(q), torch.empty(5 * N + 1, dtype=torch.float64, device="cuda")
+        dg.dg_rhs(ctx, q, R)
+        dg.dg_rhs(ctx, odd, Rbuf[1:])
+        dg.dg_rk3_step(ctx, q, 1e-3, 2)
+        dg.dg_rk3_step(ctx, odd, 1e-3, 2)
+        torch.cuda.synchronize()
+        assert torch.equal(Rbuf[1:], R) and torch.equal(odd, q)
+    finally:
+        dg.dg_destroy(ctx)
