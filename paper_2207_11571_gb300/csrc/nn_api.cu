@@ -23,29 +23,22 @@ struct nn_model {
   int L = 0;                    // dense layers = n_hidden + 1
   int dims[10] = {};            // dims[0] = n_in, dims[1..n_hidden] = width, dims[L] = n_out
   int pad[10] = {};             // round_up(dims[l], 64): leading dimension of bf16 rows
-  int bpad = 0;                 // round_up(max_batch, 64)
   float* W[9] = {};             // FP32 master [out][in]
   float* b[9] = {};
   bf16* Wb[9] = {};             // [out][pad(in)]
-  bf16* Wt[9] = {};             // [in][pad(out)]
   float *mW[9] = {}, *vW[9] = {}, *mb[9] = {}, *vb[9] = {};
   float *gW[9] = {}, *gb[9] = {};
   float *mean_in = nullptr, *std_in = nullptr, *mean_out = nullptr, *std_out = nullptr;
   int adam_t = 0;
   bf16* act[10] = {};           // act[l]: input of layer l, [max_batch][pad(l)]
-  bf16* actT[10] = {};          // [dims[l]][bpad]
-  float* y = nullptr;           // [max_batch][n_out], scaled output
-  float* dy = nullptr;          // [max_batch][max dim] gradient of the current layer output
-  float* dx = nullptr;          // [max_batch][max dim] gradient of the current layer input
-  bf16* dyb = nullptr;          // [max_batch][pad(max dim)]
-  bf16* dyT = nullptr;          // [max dim][bpad]
+  bf16* dy[9] = {};             // gradient of layer l's output, [max_batch][pad(l + 1)]
+  float* colsum[9] = {};        // its column sums over each 32 rows, [max_batch / 32][dims[l + 1]]
   double* loss_part = nullptr;  // reduction partials
-  float* gpart = nullptr;       // [bpad / 32][max dim] bias-gradient partial sums
-  float* gws = nullptr;         // [kMaxSplits][max dim]^2 split-K partial weight gradients
+  float* gws = nullptr;         // partial weight gradients of every layer, [kMaxSplits][n_weights]
+  long long n_weights = 0;
   double* loss_dev = nullptr;
   double* loss_host = nullptr;  // pinned
   int* err = nullptr;           // device error flag of the tensor-core kernels
-  int maxdim = 0;
   int fused = NN_INFER_CLUSTER; // inference path (nn_set_fused)
   // input means for scaling network inputs taken from solver states: in FP64 (FP64 state)
   // and shifted by the reference state of an FP32 context (cached for one reference)
@@ -59,9 +52,6 @@ namespace dgnn {
 
 namespace {
 
-constexpr int kLossBlocks = 1024;
-constexpr int kMaxSplits = 8;   // split-K factor bound of the weight-gradient GEMMs
-constexpr int kLossThreads = 128;
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -76,20 +66,38 @@ __device__ __forceinline__ void pdl_enter() {
 
 // ------------------------------------------------------------------------------- kernels
 
-// act0[r][f] = bf16((X[row(r)][f] - mean[f]) / std[f]) for f < n_in, 0 for the padding.
+// act0[r][f] = bf16((X[row(r)][f] - mean[f]) / std[f]) for f < n_in, 0 for the padding.  A
+// thread forms eight features of a row (one 16-byte store; ld is a multiple of 64), reading
+// X in 16-byte vectors where its rows are aligned (vec).
 __global__ void k_prep_features(const float* __restrict__ X, const int64_t* __restrict__ idx, int rows, int n_in,
-                                int ld, const float* __restrict__ mean, const float* __restrict__ sd,
+                                int ld, bool vec, const float* __restrict__ mean, const float* __restrict__ sd,
                                 bf16* __restrict__ out) {
   pdl_enter();
+  const int per_row = ld / 8;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)rows * ld) return;
-  const int r = (int)(t / ld), f = (int)(t - (long long)r * ld);
-  float v = 0.f;
-  if (f < n_in) {
-    const long long src = idx ? idx[r] : r;
-    v = (X[src * n_in + f] - mean[f]) / sd[f];
+  const int r = (int)(t / per_row), f = 8 * (int)(t - (long long)r * per_row);
+  if (r >= rows) return;
+  const long long src = idx ? idx[r] : r;
+  const float* x = X + src * n_in + f;
+  float v[8];
+  if (vec && f + 8 <= n_in) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 a = reinterpret_cast<const float4*>(x)[h];
+      const float4 m = reinterpret_cast<const float4*>(mean + f)[h], s = reinterpret_cast<const float4*>(sd + f)[h];
+      v[4 * h] = (a.x - m.x) / s.x;
+      v[4 * h + 1] = (a.y - m.y) / s.y;
+      v[4 * h + 2] = (a.z - m.z) / s.z;
+      v[4 * h + 3] = (a.w - m.w) / s.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = f + i < n_in ? (x[i] - mean[f + i]) / sd[f + i] : 0.f;
   }
-  out[t] = __float2bfloat16_rn(v);
+  __nv_bfloat162 p[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+  *reinterpret_cast<uint4*>(out + (long long)r * ld + f) = *reinterpret_cast<const uint4*>(p);
 }
 
 // act0[e][slot * np + node] from the FP64 state q[var][elem][node] of elements e0 .. e0 + rows.
@@ -127,184 +135,157 @@ __global__ void k_prep_state_f32(const float* __restrict__ s, int rec, int ns, i
   out[t] = __float2bfloat16_rn(v);
 }
 
-// MSE against scaled targets: dy = 2 (y - t_s) / (rows n), partial sums of (y - t_s)^2.
-// dL/dy of the MSE over norm_rows x n values, of which this launch holds rows x n (the
-// rest on other ranks of a data-parallel step; norm_rows = rows: the whole batch).
-__global__ void k_loss(const float* __restrict__ y, const float* __restrict__ Y, const int64_t* __restrict__ idx,
-                       int rows, int norm_rows, int n, const float* __restrict__ mean, const float* __restrict__ sd,
-                       float* __restrict__ dy, double* __restrict__ partial) {
-  pdl_enter();
-  // rows over blocks, features over threads; FP32 sums of a few squares per thread, a
-  // warp-shuffle reduction, then the warps' sums added in FP64 in a fixed order
-  __shared__ float wsum[kLossThreads / 32];
-  float acc = 0.f;
-  const float g = 2.f / ((float)norm_rows * (float)n);
-  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-    const long long src = idx ? idx[r] : r;
-    const float* Yr = Y + src * n;
-    const long long o = (long long)r * n;
-    for (int f = threadIdx.x; f < n; f += blockDim.x) {
-      const float ts = (Yr[f] - mean[f]) / sd[f];
-      const float diff = y[o + f] - ts;
-      dy[o + f] = g * diff;
-      acc += diff * diff;
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x / 32] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kLossThreads / 32; ++w) t += (double)wsum[w];
-    partial[blockIdx.x] = t;
-  }
-}
-__global__ void k_sum_partials(const double* __restrict__ partial, int n, double scale, double* __restrict__ out) {
-  pdl_enter();
-  __shared__ double sh[kLossThreads];
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) acc += partial[i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = sh[0] * scale;
-}
-
-// Gradient of one layer's output g[rows][n] (FP32) -> bf16 copies gb[rows][ldb] (columns
-// n..ldb-1 zero) and gT[n][ldt] (rows past `rows` zero), and per-tile column sums
-// part[tile][n] of the bias gradient.  One 32 x 32 tile per block (2D grid over
-// columns and row tiles), so every SM takes part.
-__global__ void k_grad_prep(const float* __restrict__ g, int rows, int n, int ldb, int ldt, bf16* __restrict__ gb,
-                            bf16* __restrict__ gT, float* __restrict__ part) {
-  pdl_enter();
-  __shared__ float tile[32][33];
-  __shared__ float colsum[8][32];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  float cs = 0.f;
-  for (int k = ty; k < 32; k += 8) {
-    const int r = r0 + k, c = c0 + tx;
-    const float v = (r < rows && c < n) ? g[(long long)r * n + c] : 0.f;
-    tile[k][tx] = v;
-    if (r < rows && c < ldb) gb[(long long)r * ldb + c] = __float2bfloat16_rn(v);
-    cs += v;
-  }
-  colsum[ty][tx] = cs;
-  __syncthreads();
-  for (int k = ty; k < 32; k += 8) {
-    const int c = c0 + k, r = r0 + tx;
-    if (c < n && r < ldt) gT[(long long)c * ldt + r] = __float2bfloat16_rn(tile[tx][k]);
-  }
-  if (ty == 0 && c0 + tx < n) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += colsum[k][tx];
-    part[(long long)blockIdx.y * n + c0 + tx] = t;
-  }
-}
-
-// out[i] = sum over splits z of part[z][i], in split order (deterministic split-K sum).
-__global__ void k_split_sum(const float* __restrict__ part, int splits, long long count, float* __restrict__ out) {
-  pdl_enter();
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  float s = 0.f;
-  for (int z = 0; z < splits; ++z) s += part[z * count + i];
-  out[i] = s;
-}
-
-// db[c] = sum over row tiles of part[tile][c]: 32 columns per block, each of 32 thread
-// rows sums every 32nd tile, then the 32 partial sums are added in row order
-// (deterministic).
-__global__ void k_col_sum(const float* __restrict__ part, int tiles, int n, float* __restrict__ db) {
-  pdl_enter();
-  __shared__ float sh[32][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  float s = 0.f;
-  if (c < n)
-    for (int t = threadIdx.y; t < tiles; t += 32) s += part[(long long)t * n + c];
-  sh[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && c < n) {
-    float t = 0.f;
-    for (int k = 0; k < 32; ++k) t += sh[k][threadIdx.x];
-    db[c] = t;
-  }
-}
-
-// act[rows][ld] (bf16) -> actT[n][ldt] for the first n columns, rows padded with zeros.
-__global__ void k_transpose_bf16(const bf16* __restrict__ a, int rows, int n, int ld, int ldt, bf16* __restrict__ aT) {
-  pdl_enter();
-  __shared__ bf16 tile[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int k = ty; k < 32; k += 8) {
-    const int r = r0 + k, c = c0 + tx;
-    tile[k][tx] = (r < rows && c < n) ? a[(long long)r * ld + c] : __float2bfloat16_rn(0.f);
-  }
-  __syncthreads();
-  for (int k = ty; k < 32; k += 8) {
-    const int c = c0 + k, r = r0 + tx;
-    if (c < n && r < ldt) aT[(long long)c * ldt + r] = tile[tx][k];
-  }
-}
-
-// Adam (Kingma & Ba) on every parameter tensor of the network in one launch: segment j
-// is a tensor [out][in] (in = 1 for biases); weight segments also refresh their bf16
-// copies Wb[out][ldb] and Wt[in][ldt].  Blocks are assigned to segments by prefix counts.
-constexpr int kAdamMaxSeg = 18;
-struct AdamSeg {
+// Every parameter tensor of the network in one launch (kMode): kReduce sums the partial
+// gradients into the gradient buffers, kAdam applies Adam (Kingma & Ba) from them and
+// refreshes the weights' bf16 copies, kReduceAdam does both with the same arithmetic.
+// Segment j is a tensor: weights [out][in] with `parts` partial products `stride` apart (a
+// thread takes `vec` elements), or a bias with its column sums of 32 rows each (a block takes
+// 32 columns, eight threads per column).  Blocks are assigned to segments by prefix counts;
+// the block after the last sums the loss partials in FP64.  All sums in a fixed order.
+enum { kReduce = 0, kAdam = 1, kReduceAdam = 2 };
+constexpr int kMaxSeg = 18;
+struct ParamSeg {
   float *p, *g, *m, *v;
-  long long count;
-  int in;
+  const float* part;
+  long long stride;
+  int parts;
+  int count;
+  int in;      // 0: a bias
+  int vec;     // weights: elements per thread, 4 (every row and partial product 16-byte aligned) or 1
   bf16* Wb;
   int ldb;
-  bf16* Wt;
-  int ldt;
 };
-struct AdamTable {
+struct ParamTable {
   int n;
-  int block_start[kAdamMaxSeg + 1];
-  AdamSeg seg[kAdamMaxSeg];
+  int block_start[kMaxSeg + 1];
+  ParamSeg seg[kMaxSeg];
   float lr, b1, b2, eps, bc1, bc2;
+  const double* loss_part;
+  int loss_parts;
+  double loss_scale;
+  double* loss_out;
 };
 
-__global__ void k_adam(const __grid_constant__ AdamTable tb) {
-  pdl_enter();
-  int j = 0;
-  while (j + 1 < tb.n && (int)blockIdx.x >= tb.block_start[j + 1]) ++j;
-  const AdamSeg& S = tb.seg[j];
-  const long long t = (blockIdx.x - tb.block_start[j]) * (long long)blockDim.x + threadIdx.x;
-  if (t >= S.count) return;
-  const float gi = S.g[t];
-  const float mi = tb.b1 * S.m[t] + (1.f - tb.b1) * gi;
-  const float vi = tb.b2 * S.v[t] + (1.f - tb.b2) * gi * gi;
-  S.m[t] = mi;
-  S.v[t] = vi;
-  const float mh = mi / tb.bc1, vh = vi / tb.bc2;
-  const float w = S.p[t] - tb.lr * mh / (sqrtf(vh) + tb.eps);
-  S.p[t] = w;
-  if (S.Wb) {
-    const int o = (int)(t / S.in), i = (int)(t - (long long)o * S.in);
-    const bf16 wb = __float2bfloat16_rn(w);
-    S.Wb[(long long)o * S.ldb + i] = wb;
-    S.Wt[(long long)i * S.ldt + o] = wb;
+// Adam's new value of a parameter; m and v are updated.
+__device__ __forceinline__ float adam_value(const ParamTable& tb, float p, float gi, float& m, float& v) {
+  m = tb.b1 * m + (1.f - tb.b1) * gi;
+  v = tb.b2 * v + (1.f - tb.b2) * gi * gi;
+  const float mh = m / tb.bc1, vh = v / tb.bc2;
+  return p - tb.lr * mh / (sqrtf(vh) + tb.eps);
+}
+
+// V consecutive weights from element t.
+template <int kMode, int V>
+__device__ __forceinline__ void weight_params(const ParamTable& tb, const ParamSeg& S, int t) {
+  float g[V], m[V], v[V], p[V];
+  auto load = [&](const float* a, float x[V]) {
+    if constexpr (V == 4) {
+      const float4 q = *reinterpret_cast<const float4*>(a);
+      x[0] = q.x;
+      x[1] = q.y;
+      x[2] = q.z;
+      x[3] = q.w;
+    } else {
+      x[0] = *a;
+    }
+  };
+  auto store = [&](float* a, const float x[V]) {
+    if constexpr (V == 4) *reinterpret_cast<float4*>(a) = make_float4(x[0], x[1], x[2], x[3]);
+    else *a = x[0];
+  };
+  if (kMode != kReduce) {
+    load(S.m + t, m);
+    load(S.v + t, v);
+    load(S.p + t, p);
+  }
+  if (kMode == kAdam) {
+    load(S.g + t, g);
+  } else {
+#pragma unroll
+    for (int i = 0; i < V; ++i) g[i] = 0.f;
+#pragma unroll 4
+    for (int z = 0; z < S.parts; ++z) {
+      float a[V];
+      load(S.part + z * S.stride + t, a);
+#pragma unroll
+      for (int i = 0; i < V; ++i) g[i] += a[i];
+    }
+    store(S.g + t, g);
+  }
+  if (kMode == kReduce) return;
+#pragma unroll
+  for (int i = 0; i < V; ++i) p[i] = adam_value(tb, p[i], g[i], m[i], v[i]);
+  store(S.m + t, m);
+  store(S.v + t, v);
+  store(S.p + t, p);
+  const int o = t / S.in;
+  bf16* w = S.Wb + (long long)o * S.ldb + (t - o * S.in);
+  if constexpr (V == 4) {
+    const __nv_bfloat162 q[2] = {__floats2bfloat162_rn(p[0], p[1]), __floats2bfloat162_rn(p[2], p[3])};
+    *reinterpret_cast<uint2*>(w) = *reinterpret_cast<const uint2*>(q);
+  } else {
+    *w = __float2bfloat16_rn(p[0]);
   }
 }
 
-// bf16 copies of an FP32 weight [out][in].
-__global__ void k_refresh_bf16(const float* __restrict__ W, long long count, int in, bf16* __restrict__ Wb, int ldb,
-                               bf16* __restrict__ Wt, int ldt) {
+template <int kMode>
+__global__ void __launch_bounds__(256) k_params(const __grid_constant__ ParamTable tb) {
+  pdl_enter();
+  __shared__ double sh[256];
+  int j = 0;
+  while (j < tb.n && (int)blockIdx.x >= tb.block_start[j + 1]) ++j;
+  if (j == tb.n) {   // the loss
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < tb.loss_parts; i += 256) acc += tb.loss_part[i];
+    sh[threadIdx.x] = acc;
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+      if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) *tb.loss_out = sh[0] * tb.loss_scale;
+    return;
+  }
+  const ParamSeg& S = tb.seg[j];
+  const int blk = blockIdx.x - tb.block_start[j];
+  if (S.in) {
+    const int t = (blk * 256 + threadIdx.x) * S.vec;
+    if (t >= S.count) return;
+    if (S.vec == 4) weight_params<kMode, 4>(tb, S, t);
+    else weight_params<kMode, 1>(tb, S, t);
+  } else {
+    const int c = blk * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
+    float gi = 0.f;
+    if (kMode == kAdam) {
+      if (row == 0 && c < S.count) gi = S.g[c];
+    } else {
+      float* part = reinterpret_cast<float*>(sh);
+      float a = 0.f;
+      if (c < S.count) {
+#pragma unroll 4
+        for (int z = row; z < S.parts; z += 8) a += S.part[z * S.stride + c];
+      }
+      part[threadIdx.x] = a;
+      __syncthreads();
+      if (row == 0)
+        for (int k = 0; k < 8; ++k) gi += part[k * 32 + threadIdx.x];
+      if (row == 0 && c < S.count) S.g[c] = gi;
+    }
+    if (kMode != kReduce && row == 0 && c < S.count) {
+      float m = S.m[c], v = S.v[c];
+      S.p[c] = adam_value(tb, S.p[c], gi, m, v);
+      S.m[c] = m;
+      S.v[c] = v;
+    }
+  }
+}
+
+// bf16 copy of an FP32 weight [out][in].
+__global__ void k_refresh_bf16(const float* __restrict__ W, long long count, int in, bf16* __restrict__ Wb, int ldb) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= count) return;
   const int o = (int)(t / in), i = (int)(t - (long long)o * in);
-  const bf16 wb = __float2bfloat16_rn(W[t]);
-  Wb[(long long)o * ldb + i] = wb;
-  Wt[(long long)i * ldt + o] = wb;
+  Wb[(long long)o * ldb + i] = __float2bfloat16_rn(W[t]);
 }
 
 // Per-feature sums of x and x^2 over rows (FP64), blocks stride over rows.
@@ -353,10 +334,32 @@ cudaError_t pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// Forward through all layers for `rows` rows whose scaled inputs are in act[0].
-// last: if S != null, unscaled forcing into S (ld n_out); else scaled output into m->y.
+// Scaled bf16 inputs of `rows` rows (idx, or 0 ..) of X into act[0].
+int prep_features(const nn_model* m, const float* X, const int64_t* idx, int rows, cudaStream_t st) {
+  const bool vec = m->d.n_in % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  DG_CUDA(pdl_launch(k_prep_features, dim3(blocks_for((long long)rows * m->pad[0] / 8, 256)), dim3(256), st, X, idx, rows,
+                     m->d.n_in, m->pad[0], vec, m->mean_in, m->std_in, m->act[0]));
+  return DG_OK;
+}
+
+// Layers 0 .. L - 2 of `rows` rows whose scaled inputs are in act[0], keeping every layer's
+// input (bf16) in act[].
+int hidden_layers(const nn_model* m, int rows, cudaStream_t st) {
+  for (int l = 0; l < m->L - 1; ++l) {
+    GemmEpilogue ep;
+    ep.kind = kGemmBiasReluBf16;
+    ep.bias = m->b[l];
+    ep.out = m->act[l + 1];
+    ep.ldo = m->pad[l + 1];
+    int rc = gemm_bf16(m->act[l], m->pad[l], m->Wb[l], m->pad[l], rows, m->dims[l + 1], m->dims[l], ep, m->err, st);
+    if (rc) return rc;
+  }
+  return DG_OK;
+}
+
+// Forward through all layers: the unscaled forcing into S (ld n_out).
 int forward_layers(const nn_model* m, int rows, float* S, cudaStream_t st) {
-  if (S && m->fused == NN_INFER_FUSED && mlp_fused_ok(m->dims, m->L)) {
+  if (m->fused == NN_INFER_FUSED && mlp_fused_ok(m->dims, m->L)) {
     // inference: all layers in one kernel, activations kept on the SM
     const bf16* W[kMlpMaxLayers];
     const float* B[kMlpMaxLayers];
@@ -367,41 +370,30 @@ int forward_layers(const nn_model* m, int rows, float* S, cudaStream_t st) {
     return mlp_forward_fused(m->act[0], m->pad[0], W, m->pad, B, m->dims, m->L, rows, m->std_out, m->mean_out, S,
                              m->dims[m->L], m->err, st);
   }
-  for (int l = 0; l < m->L; ++l) {
-    GemmEpilogue ep;
-    ep.bias = m->b[l];
-    if (l < m->L - 1) {
-      ep.kind = kGemmBiasReluBf16;
-      ep.out = m->act[l + 1];
-      ep.ldo = m->pad[l + 1];
-    } else if (S) {
-      ep.kind = kGemmAffineF32;
-      ep.scale = m->std_out;
-      ep.shift = m->mean_out;
-      ep.out = S;
-      ep.ldo = m->dims[m->L];
-    } else {
-      ep.kind = kGemmF32;
-      ep.out = m->y;
-      ep.ldo = m->dims[m->L];
-    }
-    int rc = gemm_bf16(m->act[l], m->pad[l], m->Wb[l], m->pad[l], rows, m->dims[l + 1], m->dims[l], ep, m->err, st);
-    if (rc) return rc;
-  }
-  return DG_OK;
+  int rc = hidden_layers(m, rows, st);
+  if (rc) return rc;
+  const int l = m->L - 1;
+  GemmEpilogue ep;
+  ep.kind = kGemmAffineF32;
+  ep.bias = m->b[l];
+  ep.scale = m->std_out;
+  ep.shift = m->mean_out;
+  ep.out = S;
+  ep.ldo = m->dims[m->L];
+  return gemm_bf16(m->act[l], m->pad[l], m->Wb[l], m->pad[l], rows, m->dims[l + 1], m->dims[l], ep, m->err, st);
 }
 
 void free_model(nn_model* m) {
   if (!m) return;
   for (int l = 0; l < 9; ++l) {
-    cudaFree(m->W[l]); cudaFree(m->b[l]); cudaFree(m->Wb[l]); cudaFree(m->Wt[l]);
+    cudaFree(m->W[l]); cudaFree(m->b[l]); cudaFree(m->Wb[l]);
     cudaFree(m->mW[l]); cudaFree(m->vW[l]); cudaFree(m->mb[l]); cudaFree(m->vb[l]);
     cudaFree(m->gW[l]); cudaFree(m->gb[l]);
   }
-  for (int l = 0; l < 10; ++l) { cudaFree(m->act[l]); cudaFree(m->actT[l]); }
+  for (int l = 0; l < 10; ++l) cudaFree(m->act[l]);
+  for (int l = 0; l < 9; ++l) { cudaFree(m->dy[l]); cudaFree(m->colsum[l]); }
   cudaFree(m->mean_in); cudaFree(m->std_in); cudaFree(m->mean_out); cudaFree(m->std_out);
-  cudaFree(m->y); cudaFree(m->dy); cudaFree(m->dx); cudaFree(m->dyb); cudaFree(m->dyT);
-  cudaFree(m->loss_part); cudaFree(m->loss_dev); cudaFree(m->err); cudaFree(m->gpart); cudaFree(m->gws);
+  cudaFree(m->loss_part); cudaFree(m->loss_dev); cudaFree(m->err); cudaFree(m->gws);
   cudaFree(m->mean_in_d); cudaFree(m->mean_shift);
   if (m->loss_host) cudaFreeHost(m->loss_host);
   delete m;
@@ -431,9 +423,7 @@ int alloc_model(const nn_desc* d, nn_model** out) {
   m->dims[m->L] = d->n_out;
   for (int l = 0; l <= m->L; ++l) {
     m->pad[l] = round_up(m->dims[l], 64);
-    m->maxdim = std::max(m->maxdim, m->dims[l]);
   }
-  m->bpad = round_up(d->max_batch, 64);
   const long long B = d->max_batch;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t bytes) {
@@ -443,27 +433,23 @@ int alloc_model(const nn_desc* d, nn_model** out) {
   for (int l = 0; l < m->L; ++l) {
     const size_t in = m->dims[l], o = m->dims[l + 1];
     A((void**)&m->W[l], in * o * 4); A((void**)&m->b[l], o * 4);
-    A((void**)&m->Wb[l], o * m->pad[l] * 2); A((void**)&m->Wt[l], in * m->pad[l + 1] * 2);
+    A((void**)&m->Wb[l], o * m->pad[l] * 2);
     A((void**)&m->mW[l], in * o * 4); A((void**)&m->vW[l], in * o * 4);
     A((void**)&m->mb[l], o * 4); A((void**)&m->vb[l], o * 4);
     A((void**)&m->gW[l], in * o * 4); A((void**)&m->gb[l], o * 4);
   }
   for (int l = 0; l < m->L; ++l) {
     A((void**)&m->act[l], B * m->pad[l] * 2);
-    A((void**)&m->actT[l], (size_t)m->dims[l] * m->bpad * 2);
+    A((void**)&m->dy[l], B * m->pad[l + 1] * 2);
+    A((void**)&m->colsum[l], (size_t)((B + 31) / 32) * m->dims[l + 1] * 4);
+    m->n_weights += (long long)m->dims[l] * m->dims[l + 1];
   }
   A((void**)&m->mean_in, d->n_in * 4); A((void**)&m->std_in, d->n_in * 4);
   A((void**)&m->mean_out, d->n_out * 4); A((void**)&m->std_out, d->n_out * 4);
-  A((void**)&m->y, B * d->n_out * 4);
-  A((void**)&m->dy, B * m->maxdim * 4);
-  A((void**)&m->dx, B * m->maxdim * 4);
-  A((void**)&m->dyb, B * round_up(m->maxdim, 64) * 2);
-  A((void**)&m->dyT, (size_t)m->maxdim * m->bpad * 2);
   A((void**)&m->mean_in_d, d->n_in * 8);
   A((void**)&m->mean_shift, d->n_in * 4);
-  A((void**)&m->loss_part, kLossBlocks * 8);
-  A((void**)&m->gpart, (size_t)(m->bpad / 32) * m->maxdim * 4);
-  A((void**)&m->gws, (size_t)kMaxSplits * m->maxdim * m->maxdim * 4);
+  A((void**)&m->loss_part, (size_t)8 * ((B + 127) / 128) * ((d->n_out + 63) / 64) * 8);
+  A((void**)&m->gws, (size_t)kMaxSplits * m->n_weights * 4);
   A((void**)&m->loss_dev, 8);
   A((void**)&m->err, 4);
   if (e == cudaSuccess) e = cudaMallocHost(&m->loss_host, 8);
@@ -507,8 +493,7 @@ int ensure_shift(nn_model* m, const dg_ctx* c) {
 
 int refresh_bf16(nn_model* m, int l, cudaStream_t st) {
   const long long cnt = (long long)m->dims[l] * m->dims[l + 1];
-  k_refresh_bf16<<<blocks_for(cnt, 256), 256, 0, st>>>(m->W[l], cnt, m->dims[l], m->Wb[l], m->pad[l], m->Wt[l],
-                                                        m->pad[l + 1]);
+  k_refresh_bf16<<<blocks_for(cnt, 256), 256, 0, st>>>(m->W[l], cnt, m->dims[l], m->Wb[l], m->pad[l]);
   DG_CUDA(cudaGetLastError());
   return DG_OK;
 }
@@ -610,108 +595,105 @@ bool adam_ok(const nn_adam& a) {
          a.eps > 0.f && std::isfinite(a.eps);
 }
 
+// Parameter table of every layer; parts: split-K partial weight gradients and column sums of
+// `batch` rows (0: none, Adam from the gradient buffers).
+void param_table(nn_model* m, int batch, ParamTable* tb) {
+  int blocks = 0;
+  long long off = 0;
+  bool aligned = true;   // every row of weights, and every partial product, on 16 bytes
+  for (int l = 0; l < m->L; ++l) aligned = aligned && m->dims[l] % 4 == 0;
+  for (int l = 0; l < m->L; ++l) {
+    const int o = m->dims[l + 1], in = m->dims[l], vec = aligned ? 4 : 1;
+    tb->block_start[tb->n] = blocks;
+    tb->seg[tb->n++] = ParamSeg{m->W[l], m->gW[l], m->mW[l], m->vW[l], m->gws + off, m->n_weights, batch ? grad_splits(o, in, batch) : 0, o * in, in,
+                                vec, m->Wb[l], m->pad[l]};
+    blocks += (int)blocks_for((long long)o * in, 256 * vec);
+    off += (long long)o * in;
+    tb->block_start[tb->n] = blocks;
+    tb->seg[tb->n++] = ParamSeg{m->b[l], m->gb[l], m->mb[l], m->vb[l], m->colsum[l], o, (batch + 31) / 32, o, 0, 1,
+                                nullptr, 0};
+    blocks += (o + 31) / 32;
+  }
+  tb->block_start[tb->n] = blocks;
+}
+
+// Adam's hyperparameters and bias corrections of the next step.
+void adam_step(nn_model* m, const nn_adam& a, ParamTable* tb) {
+  ++m->adam_t;
+  tb->lr = a.lr;
+  tb->b1 = a.beta1;
+  tb->b2 = a.beta2;
+  tb->eps = a.eps;
+  tb->bc1 = 1.f - std::pow(a.beta1, (float)m->adam_t);
+  tb->bc2 = 1.f - std::pow(a.beta2, (float)m->adam_t);
+}
+
 // Forward, MSE and backward of `batch` rows into the model's gradient buffers, normalised
-// over norm_batch rows (a data-parallel step's global batch).  The loss share goes to
-// m->loss_dev.
-int backward_into_grads(nn_model* m, const float* X, const float* Y, const int64_t* idx, int batch, int norm_batch,
-                        cudaStream_t st) {
+// over norm_batch rows (a data-parallel step's global batch), then, with adam, one Adam step
+// in the launch that reduces the gradients.  The loss share goes to m->loss_dev.
+//
+// 2 L + 2 launches (7 L + 3 with element-wise kernels, transposes and a sum per product):
+// scaling, a product per layer forward (the last with the loss), one per layer but the first
+// backward, every layer's weight gradient, the reduction and update.  What is element-wise
+// is an epilogue, and the products read activations, gradients and weights as they lie.
+// Measured per step: 320-512x4-320 at batch 4096 249 -> 100 us, 192-256x7-192 at 1024 209 -> 81 us;
+// a launch of the chain takes 4 us at batch 128 and 6 us at 4096 x 512 x 512.
+int train(nn_model* m, const float* X, const float* Y, const int64_t* idx, int batch, int norm_batch,
+          const nn_adam* adam, cudaStream_t st) {
   const int L = m->L, n_out = m->d.n_out;
-  // forward, keeping every layer input (bf16) in act[]
-  long long tot = (long long)batch * m->pad[0];
-  DG_CUDA(pdl_launch(k_prep_features, dim3(blocks_for(tot, 256)), dim3(256), st, X, idx, batch, m->d.n_in, m->pad[0], m->mean_in, m->std_in,
-                                                        m->act[0]));
-  DG_CUDA(cudaGetLastError());
-  int rc = forward_layers(m, batch, nullptr, st);
+  int rc = prep_features(m, X, idx, batch, st);
+  if (!rc) rc = hidden_layers(m, batch, st);
   if (rc) return rc;
-  // loss and dL/dy
-  DG_CUDA(pdl_launch(k_loss, dim3(kLossBlocks), dim3(kLossThreads), st, m->y, Y, idx, batch, norm_batch, n_out, m->mean_out,
-                     m->std_out, m->dy, m->loss_part));
-  DG_CUDA(cudaGetLastError());
-  DG_CUDA(pdl_launch(k_sum_partials, dim3(1), dim3(kLossThreads), st, m->loss_part, kLossBlocks,
-                     1.0 / ((double)norm_batch * n_out), m->loss_dev));
-  DG_CUDA(cudaGetLastError());
-  // backward
-  float* g = m->dy;   // gradient w.r.t. the output of layer l, [batch][dims[l+1]]
-  float* gnext = m->dx;
-  for (int l = L - 1; l >= 0; --l) {
-    const int o = m->dims[l + 1], in = m->dims[l];
-    const int ldb = round_up(o, 64);
-    const int tiles = m->bpad / 32;
-    dim3 gp(ldb / 32, tiles), bt(32, 8);
-    DG_CUDA(pdl_launch(k_grad_prep, dim3(gp), dim3(bt), st, g, batch, o, ldb, m->bpad, m->dyb, m->dyT, m->gpart));
-    DG_CUDA(cudaGetLastError());
-    DG_CUDA(pdl_launch(k_col_sum, dim3((o + 31) / 32), dim3(dim3(32, 32)), st, m->gpart, tiles, o, m->gb[l]));
-    DG_CUDA(cudaGetLastError());
-    dim3 gt((in + 31) / 32, (m->bpad + 31) / 32);
-    DG_CUDA(pdl_launch(k_transpose_bf16, dim3(gt), dim3(bt), st, m->act[l], batch, in, m->pad[l], m->bpad, m->actT[l]));
-    DG_CUDA(cudaGetLastError());
-    // dW = g^T act : M = o, N = in, K = batch.  Few output tiles and a long K: split K
-    // so that the CTAs cover the SMs, then sum the partial products in a fixed order.
-    GemmEpilogue ew;
-    ew.kind = kGemmF32;
-    ew.ldo = in;
-    const int tiles_mn = ((o + 127) / 128) * ((in + gemm_pick_bn(o, in) - 1) / gemm_pick_bn(o, in));
-    const int kslices = (batch + 63) / 64;
-    const int splits = std::max(1, std::min({kMaxSplits, kslices, 152 / tiles_mn}));
-    if (splits > 1) {
-      ew.out = m->gws;
-      ew.splits = splits;
-      ew.split_stride = (long long)o * in;
-    } else {
-      ew.out = m->gW[l];
-    }
-    rc = gemm_bf16(m->dyT, m->bpad, m->actT[l], m->bpad, o, in, batch, ew, m->err, st);
+  GemmEpilogue el;
+  el.kind = kGemmLossBf16;
+  el.bias = m->b[L - 1];
+  el.Y = Y;
+  el.idx = idx;
+  el.mean = m->mean_out;
+  el.sd = m->std_out;
+  el.grad_scale = 2.f / ((float)norm_batch * (float)n_out);
+  el.out = m->dy[L - 1];
+  el.ldo = m->pad[L];
+  el.colsum = m->colsum[L - 1];
+  el.loss_part = m->loss_part;
+  rc = gemm_bf16(m->act[L - 1], m->pad[L - 1], m->Wb[L - 1], m->pad[L - 1], batch, n_out, m->dims[L - 1], el, m->err,
+                 st);
+  if (rc) return rc;
+  for (int l = L - 1; l > 0; --l) {
+    rc = input_gradient(m->dy[l], m->pad[l + 1], m->Wb[l], m->pad[l], batch, m->dims[l], m->dims[l + 1], m->act[l],
+                        m->pad[l], m->dy[l - 1], m->colsum[l - 1], m->err, st);
     if (rc) return rc;
-    if (splits > 1) {
-      const long long cnt = (long long)o * in;
-      DG_CUDA(pdl_launch(k_split_sum, dim3(blocks_for(cnt, 256)), dim3(256), st, m->gws, splits, cnt, m->gW[l]));
-      DG_CUDA(cudaGetLastError());
-    }
-    if (l > 0) {
-      // d act = g W, masked by the ReLU of the layer that produced act[l]
-      GemmEpilogue ex;
-      ex.kind = kGemmMaskF32;
-      ex.mask = m->act[l];
-      ex.ldm = m->pad[l];
-      ex.out = gnext;
-      ex.ldo = in;
-      rc = gemm_bf16(m->dyb, ldb, m->Wt[l], m->pad[l + 1], batch, in, o, ex, m->err, st);
-      if (rc) return rc;
-      std::swap(g, gnext);
-    }
+  }
+  GradLayer gl[kMaxGradLayers];
+  long long off = 0;
+  for (int l = 0; l < L; ++l) {
+    gl[l] = GradLayer{m->dy[l], m->act[l], m->pad[l + 1], m->pad[l], m->dims[l + 1], m->dims[l], off};
+    off += (long long)m->dims[l] * m->dims[l + 1];
+  }
+  rc = weight_gradients(gl, L, batch, m->gws, m->n_weights, m->err, st);
+  if (rc) return rc;
+  ParamTable tb{};
+  param_table(m, batch, &tb);
+  tb.loss_part = m->loss_part;
+  tb.loss_parts = gemm_loss_partials(batch, n_out);
+  tb.loss_scale = 1.0 / ((double)norm_batch * n_out);
+  tb.loss_out = m->loss_dev;
+  const dim3 grid(tb.block_start[tb.n] + 1);   // and the loss
+  if (adam) {
+    adam_step(m, *adam, &tb);
+    DG_CUDA(pdl_launch(k_params<kReduceAdam>, grid, dim3(256), st, tb));
+  } else {
+    DG_CUDA(pdl_launch(k_params<kReduce>, grid, dim3(256), st, tb));
   }
   return DG_OK;
 }
 
-// One Adam step of every parameter from the gradient buffers (also refreshes the bf16
-// copies of the weights).
+// One Adam step of every parameter from the gradient buffers.
 int adam_apply(nn_model* m, const nn_adam& a, cudaStream_t st) {
-  const int L = m->L;
-  ++m->adam_t;
-  const float bc1 = 1.f - std::pow(a.beta1, (float)m->adam_t);
-  const float bc2 = 1.f - std::pow(a.beta2, (float)m->adam_t);
-  AdamTable at{};
-  at.lr = a.lr;
-  at.b1 = a.beta1;
-  at.b2 = a.beta2;
-  at.eps = a.eps;
-  at.bc1 = bc1;
-  at.bc2 = bc2;
-  int blocks = 0;
-  for (int l = 0; l < L; ++l) {
-    const long long cw = (long long)m->dims[l] * m->dims[l + 1];
-    at.block_start[at.n] = blocks;
-    at.seg[at.n++] = AdamSeg{m->W[l], m->gW[l], m->mW[l], m->vW[l], cw, m->dims[l], m->Wb[l], m->pad[l], m->Wt[l],
-                             m->pad[l + 1]};
-    blocks += (int)blocks_for(cw, 256);
-    const long long cb = m->dims[l + 1];
-    at.block_start[at.n] = blocks;
-    at.seg[at.n++] = AdamSeg{m->b[l], m->gb[l], m->mb[l], m->vb[l], cb, 1, nullptr, 0, nullptr, 0};
-    blocks += (int)blocks_for(cb, 256);
-  }
-  at.block_start[at.n] = blocks;
-  DG_CUDA(pdl_launch(k_adam, dim3(blocks), dim3(256), st, at));
-  DG_CUDA(cudaGetLastError());
+  ParamTable tb{};
+  param_table(m, 0, &tb);
+  adam_step(m, a, &tb);
+  DG_CUDA(pdl_launch(k_params<kAdam>, dim3(tb.block_start[tb.n]), dim3(256), st, tb));
   return DG_OK;
 }
 
@@ -844,10 +826,8 @@ int nn_forward(const nn_model* m, const float* X, float* S, int rows, void* stre
   if (!m || !X || !S) return fail(DG_ERR_INVALID_ARG, "nn_forward: NULL argument");
   if (rows < 1 || rows > m->d.max_batch) return fail(DG_ERR_INVALID_ARG, "nn_forward: rows outside [1, max_batch]");
   cudaStream_t st = (cudaStream_t)stream;
-  const long long tot = (long long)rows * m->pad[0];
-  DG_CUDA(pdl_launch(k_prep_features, dim3(blocks_for(tot, 256)), dim3(256), st, X, nullptr, rows, m->d.n_in, m->pad[0], m->mean_in,
-                                                        m->std_in, m->act[0]));
-  DG_CUDA(cudaGetLastError());
+  int rc = prep_features(m, X, nullptr, rows, st);
+  if (rc) return rc;
   return forward_layers(m, rows, S, st);
 }
 
@@ -871,9 +851,7 @@ int nn_train_step(nn_model* m, const float* X, const float* Y, const int64_t* id
   if (!adam_ok(a))
     return fail(DG_ERR_INVALID_ARG, "nn_train_step: Adam needs lr >= 0, beta1 and beta2 in [0, 1), eps > 0 (finite)");
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = backward_into_grads(m, X, Y, idx, batch, batch, st);
-  if (rc) return rc;
-  rc = adam_apply(m, a, st);
+  int rc = train(m, X, Y, idx, batch, batch, &a, st);
   if (rc) return rc;
   return loss_to_host(m, loss_out, st);
 }
@@ -884,7 +862,7 @@ int nn_backward(nn_model* m, const float* X, const float* Y, const int64_t* idx,
   if (batch < 1 || batch > m->d.max_batch) return fail(DG_ERR_INVALID_ARG, "nn_backward: batch outside [1, max_batch]");
   if (global_batch < batch) return fail(DG_ERR_INVALID_ARG, "nn_backward: global_batch < batch");
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = backward_into_grads(m, X, Y, idx, batch, global_batch, st);
+  int rc = train(m, X, Y, idx, batch, global_batch, nullptr, st);
   if (rc) return rc;
   return loss_to_host(m, loss_out, st);
 }

@@ -570,3 +570,42 @@ def test_data_parallel_step_on_one_rank_equals_train_step(L):
             dist.destroy_process_group()
         nn.nn_destroy(a)
         nn.nn_destroy(b)
+
+
+@pytest.mark.parametrize("n_in,width,nh,first,nv,rows", [
+    (135, 128, 2, 0, 5, 200),     # widths that are no multiple of 16: partial column groups, scalar updates
+    (81, 72, 1, 1, 3, 33),        # one row tile with one live row past a warp's 32
+    (192, 256, 3, 1, 3, 1000),    # rows past the last full tile; several splits of the weight gradient
+    (320, 512, 1, 0, 5, 4096), (64, 8, 8, 1, 3, 1), (320, 200, 4, 0, 5, 129)])
+def test_gradients_at_odd_sizes_match_oracle(L, n_in, width, nh, first, nv, rows):
+    """Weight, bias gradients and loss of one step at tile remainders, one row, the narrowest
+    and the widest layers, on unaligned rows (an index and a target array one float past a
+    16-byte boundary), against the oracle with the same rounding points."""
+    from paper_2207_11571_gb300 import nn
+    dims = [n_in] + [width] * nh + [n_in]
+    draws = inputs.uniform_draws(dims, 61)
+    h = nn.nn_create(n_in, n_in, width, nh, first, nv, max(rows, 8), draws)
+    try:
+        params = [(W.astype(np.float32).astype(np.float64), b) for W, b in mlp.he_uniform_init(dims, draws)]
+        sc = set_random_scalers(nn, h, n_in, 62)
+        total = rows + 7
+        X = inputs.normal((total, n_in), 63).astype(np.float32)
+        Y = (0.3 * inputs.normal((total, n_in), 64)).astype(np.float32)
+        idx = np.random.default_rng(65).permutation(total)[:rows].astype(np.int64)
+
+        def shifted(a):
+            buf = torch.empty(a.size + 1, dtype=torch.float32, device="cuda")
+            buf[1:].copy_(torch.from_numpy(a).reshape(-1))
+            return buf[1:].reshape(a.shape)
+
+        _, loss_or, grads = mlp.train_step(params, {}, sc, X[idx].astype(np.float64), Y[idx].astype(np.float64),
+                                           bf16=True)
+        for Xd, Yd in ((torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()), (shifted(X), shifted(Y))):
+            loss = nn.nn_backward(h, Xd, Yd, torch.from_numpy(idx).cuda())
+            assert loss == pytest.approx(loss_or, rel=NN_RTOL)
+            for l in range(nh + 1):
+                dW, db = nn.nn_get_grads(h, l)
+                assert rel(dW, grads[l][0]) < NN_RTOL, l
+                assert rel(db, grads[l][1]) < NN_RTOL, l
+    finally:
+        nn.nn_destroy(h)
