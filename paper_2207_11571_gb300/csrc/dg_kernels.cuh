@@ -74,6 +74,7 @@ struct OpConst {
   T mu, lam, csd2, lam_t;         // transport
   int les;
   double drho_ref, dE_ref;        // references for shifting the FP64 state
+  int early;                      // phase A lets the next launch in as it starts, not as it ends (make_const)
   FeatureOut feat;                // network features written by phase A (feat.out may be NULL)
   T D[kMaxN1 * kMaxN1];
 };
@@ -958,16 +959,21 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   }
   if (FEAT) {
     // the forcing network's input features, from the stage state: the same arithmetic as the
-    // separate feature kernels of the network
+    // separate feature kernels of the network, four nodes at a time (every array 16-byte
+    // aligned: n^3 = 64 features per variable)
     __nv_bfloat16* fo = static_cast<__nv_bfloat16*>(C.feat.out) + (long long)e * C.feat.ld + 4 * r;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const int slot = v - C.feat.first_var;
       if (slot < 0 || slot >= C.feat.n_vars) continue;
-      const int f = slot * 64 + 4 * r;
+      float sh[4], sd[4], x[4];
+      row_read(C.feat.shift32 + slot * 64 + 4 * r, sh);
+      row_read(C.feat.sd + slot * 64 + 4 * r, sd);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        fo[slot * 64 + i] = __float2bfloat16_rn((s[v][i] - C.feat.shift32[f + i]) / C.feat.sd[f + i]);
+      for (int i = 0; i < 4; ++i) x[i] = (s[v][i] - sh[i]) / sd[i];
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]), hi = __floats2bfloat162_rn(x[2], x[3]);
+      *reinterpret_cast<uint2*>(fo + slot * 64) =
+          make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
     }
   }
   // the other rows of this row's y- and z-line (j ^ m, k ^ m) and their matrix entries
@@ -1198,8 +1204,9 @@ __global__ void __launch_bounds__(volume_max_threads<P, T, SPLIT>(), volume_min_
 k_volume(const double* __restrict__ q, T* __restrict__ qf, T* __restrict__ rv, T* __restrict__ vt,
          const OpConst<T> C) {
   pdl_wait();
-  pdl_release();
+  if (C.early) pdl_release();
   volume_phase<P, T, SRC, CUBE, FEAT, SPLIT>(blockIdx.x, q, qf, rv, vt, C);
+  pdl_release();
 }
 
 // ---------------------------------------------------------------- phase B
@@ -1376,11 +1383,10 @@ __host__ __device__ constexpr int surf_threads(int P) {
   return P == 1 ? 128 : P == 2 ? 224 : P == 3 ? 128 : P == 4 ? 160 : P == 5 ? 224 : P == 6 ? 192 : P == 7 ? 128 : 256;
 }
 __host__ __device__ constexpr int surf_threads_cube(int P) { return P == 1 ? 96 : 192; }
-// Orders whose phase-B blocks are cubes on a whole mesh of even K.  The cube's 36 face
-// evaluations instead of 48 pay where those bound the launch: FP64 (the FP64 pipe; 16^3/P3
-// 910 -> 844, 12^3/P2 248 -> 221 us per RK3 step) and FP32 at P = 3 (8^3 32.8 -> 29.5, 16^3
-// 72.0 -> 57.7, 32^3 327 -> 330 us); in FP32 at P = 2 (16^3 38.2 -> 43.1 us) and P = 1 rows win.
-__host__ __device__ constexpr bool surf_cube(int P, int tsize) { return tsize == 8 ? P <= 3 : P == 3; }
+// Orders whose phase-B blocks may be cubes (on a whole mesh of even K): the cube's 36 face
+// evaluations instead of 48 pay where those bound the launch, on the FP64 pipe; in FP32 rows
+// win (16^3/P3: 48.5 against 52.4 us per RK3 step).
+__host__ __device__ constexpr bool surf_cube(int P, int tsize) { return tsize == 8 && P <= 3; }
 // Blocks per SM the phase-B kernel is compiled for: 64 registers per thread in FP32, 128 in FP64.
 __host__ __device__ constexpr int surf_min_blocks(int threads, int tsize) {
   return tsize == 8 ? 512 / threads : 1024 / threads;
@@ -1634,17 +1640,16 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
   }
 }
 
-template <int P, typename T, int MODE, bool CUBE = false>
-__global__ void __launch_bounds__(CUBE ? surf_threads_cube(P) : surf_threads(P),
-                                  surf_min_blocks(CUBE ? surf_threads_cube(P) : surf_threads(P), sizeof(T)))
+// E elements per block (kCubeElems with CUBE), THREADS threads.
+template <int P, typename T, int MODE, int E, int THREADS, bool CUBE>
+__global__ void __launch_bounds__(THREADS, surf_min_blocks(THREADS, sizeof(T)))
 k_surface(SurfArgs<T> a, Forcing fc, const OpConst<T> C, RkArgs<T> rk) {
-  constexpr int E = CUBE ? kCubeElems : surf_elems(P);
   // last block first: phase A has just written the end of the mesh, which is still in L2
   const int blk = gridDim.x - 1 - blockIdx.x;
   surface_prologue<P, T, CUBE>(blk, E, C);
   pdl_wait();
-  pdl_release();
   surface_block<P, T, MODE, CUBE>(blk, E, a, fc, C, rk);
+  pdl_release();
 }
 
 // ---------------------------------------------------------------------------------------

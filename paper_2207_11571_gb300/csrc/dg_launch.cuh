@@ -36,6 +36,12 @@ OpConst<T> make_const(const dg_ctx* c) {
   k.les = ph.les;
   k.drho_ref = ph.rho_ref;
   k.dE_ref = ph.E_ref;
+  // Where the next launch may start.  Let in early, its blocks fill whichever SMs drain first
+  // instead of spreading over the chip: phase B at 9^3/P3 in FP64 704 -> 250 us per RK3 step
+  // with the release at the end of phase A's blocks, 9^3/P4 44.6 -> 35.6, 16^3/P3 50.2 -> 48.4.
+  // Only the small blocks of a small mesh (512 nodes per SM) leave room for both phases, and
+  // the launch latency saved counts there: 10^3/P3 32.0 -> 29.1, 8^3/P2 23.7 -> 22.3.
+  k.early = std::is_same<T, float>::value && c->P <= 3 && c->N <= 152 * 512;
   k.feat = c->feat_out;
   for (int i = 0; i < kMaxN1 * kMaxN1; ++i) k.D[i] = T(c->geom.D[i]);
   return k;
@@ -173,29 +179,46 @@ SurfArgs<T> surf_args(const dg_ctx* c, double* q, double* dqdt) {
   return a;
 }
 
+template <int P, typename T, int MODE, int E, int THREADS, bool CUBE>
+cudaError_t surface_launch(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, const RkArgs<T>& rk,
+                           cudaStream_t st) {
+  const size_t smem = surface_smem_bytes<P, T>(E);
+  auto kern = k_surface<P, T, MODE, E, THREADS, CUBE>;
+  cudaError_t e = set_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3((owned_elems(c) + E - 1) / E), dim3(THREADS), smem, st, surf_args<T>(c, q, dqdt), f,
+                    make_const<T>(c), rk);
+}
+
 template <int P, typename T, int MODE>
 cudaError_t surface_p(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, const RkArgs<T>& rk,
                       cudaStream_t st) {
-  // cubes wherever they pay and tile the mesh (a slab's layers: rows): the twelve internal
-  // faces' terms are formed once for both sides, to the same bits as per side
-  if constexpr (surf_cube(P, sizeof(T))) {
-    if (!c->part && c->K % 2 == 0) {
-      const size_t smem = surface_smem_bytes<P, T>(kCubeElems);
-      auto kern = k_surface<P, T, MODE, true>;
-      cudaError_t e = set_smem(kern, smem);
-      if (e != cudaSuccess) return e;
-      const int h = c->K / 2;
-      return launch_pdl(kern, dim3(h * h * h), dim3(surf_threads_cube(P)), smem, st, surf_args<T>(c, q, dqdt), f,
-                        make_const<T>(c), rk);
+  const int n = owned_elems(c);
+  // FP64: cubes where they pay (two per SM at least) and tile the mesh (a slab's layers:
+  // rows); the twelve internal faces' terms are formed once for both sides, to the same bits
+  // as per side.  Otherwise few elements per block at P = 2 and 3, so that the FP64 pipes of
+  // all SMs have an equal share.  us per RK3 step, P = 3, cubes / 2 x 96 / 8 x 128 elements x
+  // threads: 8^3 164 / 130 / 196, 11^3 - / 328 / 413, 12^3 365 / 360 / 414, 16^3 770 / 811 / 867.
+  if constexpr (std::is_same<T, double>::value) {
+    if constexpr (surf_cube(P, sizeof(T))) {
+      if (!c->part && c->K % 2 == 0 && n >= 2 * 152 * kCubeElems)
+        return surface_launch<P, T, MODE, kCubeElems, surf_threads_cube(P), true>(c, q, dqdt, f, rk, st);
     }
+    if constexpr (P == 3) return surface_launch<P, T, MODE, 2, 96, false>(c, q, dqdt, f, rk, st);
+    if constexpr (P == 2) return surface_launch<P, T, MODE, 4, 192, false>(c, q, dqdt, f, rk, st);
   }
-  constexpr int E = surf_elems(P);
-  const size_t smem = surface_smem_bytes<P, T>(E);
-  auto kern = k_surface<P, T, MODE>;
-  cudaError_t e = set_smem(kern, smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3((owned_elems(c) + E - 1) / E), dim3(surf_threads(P)), smem, st, surf_args<T>(c, q, dqdt),
-                    f, make_const<T>(c), rk);
+  // P = 3 in FP32: the smallest block whose launch is still one wave (1024 threads per SM at
+  // 64 registers), so that every SM has its share of a small mesh; large meshes want many
+  // elements per block.  us per RK3 step with 2 x 192 / 2 x 96 / 4 x 128 / 8 x 128 elements x
+  // threads: 8^3 28.4 / 29.8 / 29.9 / 31.9, 14^3 44.9 / 41.0 / 42.1 / 42.7, 16^3 53.8 / 49.5 /
+  // 48.5 / 49.3, 32^3 345 / 295 / 294 / 290.
+  if constexpr (P == 3 && std::is_same<T, float>::value) {
+    constexpr int kWave = 152 * 1024;   // threads
+    if (n <= kWave / 192 * 2) return surface_launch<P, T, MODE, 2, 192, false>(c, q, dqdt, f, rk, st);
+    if (n <= kWave / 96 * 2) return surface_launch<P, T, MODE, 2, 96, false>(c, q, dqdt, f, rk, st);
+    if (n <= kWave / 128 * 4) return surface_launch<P, T, MODE, 4, 128, false>(c, q, dqdt, f, rk, st);
+  }
+  return surface_launch<P, T, MODE, surf_elems(P), surf_threads(P), false>(c, q, dqdt, f, rk, st);
 }
 
 // FP64 operator: modes 0 (dq/dt) and 1 (FP64 RK stage).  FP32 operator: modes 0, 2, 3, 4.
