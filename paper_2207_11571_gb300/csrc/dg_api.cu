@@ -58,6 +58,11 @@ cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_
   return f32 ? volume_f32(c, q, src, st) : volume_f64(c, q, src, st);
 }
 
+cudaError_t launch_state(const dg_ctx* c, const double* q, bool* done, cudaStream_t st) {
+  *done = false;
+  return c->opts.precision == DG_PREC_FP32 && !c->geom.split ? state_f32(c, q, done, st) : cudaSuccess;
+}
+
 cudaError_t launch_surface(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,
                            double dt, cudaStream_t st) {
   return c->opts.precision == DG_PREC_FP32 ? surface_f32(c, q, dqdt, f, mode, rk, dt, st)
@@ -82,14 +87,13 @@ static void stage_bytes(const dg_ctx* c, int k, double* grad, double* flux) {
   else *flux += k == 0 ? 10 * T : k == 1 ? 20 * T : 5 * T + 80;
 }
 
-// Evaluates the network forcing on the current state q (all elements) into c->s_buf;
-// features_ready: the phase-A launch before it wrote the network's input features.
-static int forcing_for(dg_ctx* c, const double* q, const nn_model* net, Forcing* f, cudaStream_t st,
-                       bool features_ready = false) {
+// Evaluates the network forcing on the current state q (all elements) into c->s_buf; flags
+// as nn_forcing_on_state.
+static int forcing_for(dg_ctx* c, const double* q, const nn_model* net, Forcing* f, cudaStream_t st, int flags) {
   *f = Forcing{};
   if (!net) return DG_OK;
   int first = 0, nv = 0;
-  int rc = nn_forcing_on_state(net, c, q, c->s_buf, &first, &nv, st, features_ready);
+  int rc = nn_forcing_on_state(net, c, q, c->s_buf, &first, &nv, st, flags);
   if (rc) return rc;
   f->s = c->s_buf;
   f->first_var = first;
@@ -128,23 +132,47 @@ static int exchange_traces(dg_ctx* const* cs, int n, double* const* qs, int what
 static int phase_a_what(const dg_ctx* c, int k) { return (c->opts.precision == DG_PREC_FP32 && k > 0) ? 1 : 0; }
 constexpr int kWhatPhaseB = 2;
 
+// Phase A of n contexts and the forcing network (n == 1; net may be NULL) on one stage state,
+// which is in c->cur (state) or formed from q; written: whoever formed it wrote the network's
+// input features too.  With state and features in hand the network goes first: its few
+// clusters leave most SMs idle, and phase A, which does not need the forcing, runs on those.
+static int phase_a(dg_ctx* const* cs, int n, double* const* qs, const nn_model* net, bool state, bool written, Forcing* f,
+                   cudaStream_t st) {
+  dg_ctx* c = cs[0];
+  FeatureOut features;
+  const bool feats = net && nn_phase_a_features(net, c, &features);
+  if (feats && !state) {
+    c->feat_out = features;
+    const cudaError_t e = launch_state(c, qs[0], &state, st);
+    c->feat_out = FeatureOut{};
+    DG_CUDA(e);
+    written = state;
+  }
+  const bool ahead = feats && written;
+  if (ahead) {
+    const int rc = forcing_for(c, qs[0], net, f, st, kFeaturesReady | kPhaseAFollows);
+    if (rc) return rc;
+    c->beside_forcing = true;
+  } else if (feats && !state) {
+    c->feat_out = features;
+  }
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n && e == cudaSuccess; ++i) e = launch_volume(cs[i], qs[i], state, st);
+  c->feat_out = FeatureOut{};
+  c->beside_forcing = false;
+  DG_CUDA(e);
+  return ahead ? DG_OK : forcing_for(c, qs[0], net, f, st, feats && !state ? kFeaturesReady : 0);
+}
+
 // dq/dt of n contexts: one whole mesh, or the slabs of one mesh exchanging traces.
 static int rhs_into_n(dg_ctx* const* cs, int n, double* const* qs, double* const* outs, const nn_model* net,
                       cudaStream_t st) {
   int rc = exchange_traces(cs, n, qs, phase_a_what(cs[0], 0), st);
   if (rc) return rc;
-  const bool feats = n == 1 && net && nn_phase_a_features(net, cs[0], &cs[0]->feat_out);
-  for (int i = 0; i < n; ++i) {
-    cs[i]->cur = cs[i]->qf;
-    const cudaError_t e = launch_volume(cs[i], qs[i], 0, st);
-    cs[i]->feat_out = FeatureOut{};
-    DG_CUDA(e);
-  }
+  for (int i = 0; i < n; ++i) cs[i]->cur = cs[i]->qf;
   Forcing f;
-  if (n == 1) {
-    rc = forcing_for(cs[0], qs[0], net, &f, st, feats);
-    if (rc) return rc;
-  }
+  rc = phase_a(cs, n, qs, n == 1 ? net : nullptr, false, false, &f, st);
+  if (rc) return rc;
   rc = exchange_traces(cs, n, qs, kWhatPhaseB, st);
   if (rc) return rc;
   for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], outs[i], f, 0, RkStage{}, 0.0, st));
@@ -166,7 +194,8 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
   dg_ctx* c = cs[0];
   const bool post = net && c->forcing_mode == DG_FORCING_POST;
   const bool f32 = c->opts.precision == DG_PREC_FP32;
-  bool ready = false;   // the step's first stage state is in qf
+  bool ready = false;     // the step's first stage state is in qf
+  bool written = false;   // the network's features of the coming stage state are written
   for (int s = 0; s < nsteps; ++s) {
     // slabs rebuild it from the exchanged FP64 state, the post form changes q after the step
     const bool more = s + 1 < nsteps && !c->part && !post;
@@ -175,26 +204,22 @@ static int rk3_steps_n(dg_ctx* const* cs, int n, double* const* qs, double dt, i
       for (int i = 0; i < n; ++i) cs[i]->cur = stage_buffer(cs[i], k);
       int rc = exchange ? exchange_traces(cs, n, qs, phase_a_what(c, k), st) : DG_OK;
       if (rc) return rc;
-      // the forcing's input features come out of the phase-A launch when the network allows
-      const bool want = net && (!post || k == 0);
-      const bool feats = want && n == 1 && nn_phase_a_features(net, c, &c->feat_out);
-      for (int i = 0; i < n; ++i) {
-        const cudaError_t e = launch_volume(cs[i], qs[i], f32 && (k > 0 || ready), st);
-        cs[i]->feat_out = FeatureOut{};
-        DG_CUDA(e);
-      }
       Forcing f;
-      if (want) {
-        rc = forcing_for(c, qs[0], net, &f, st, feats);
-        if (rc) return rc;
-      }
+      rc = phase_a(cs, n, qs, n == 1 && (!post || k == 0) ? net : nullptr, f32 && (k > 0 || ready), written, &f, st);
+      if (rc) return rc;
       if (post) {
         if (k == 0) fpost = f;
         f = Forcing{};
       }
       rc = exchange ? exchange_traces(cs, n, qs, kWhatPhaseB, st) : DG_OK;
       if (rc) return rc;
-      for (int i = 0; i < n; ++i) DG_CUDA(launch_surface(cs[i], qs[i], nullptr, f, stage_mode(c, k, more), rk_stage(k), dt, st));
+      // the FP32 operator's phase B forms the next stage state, and with it the features
+      written = f32 && n == 1 && net && !post && (k < 2 || more) && nn_phase_a_features(net, c, &c->feat_out);
+      cudaError_t e = cudaSuccess;
+      for (int i = 0; i < n && e == cudaSuccess; ++i)
+        e = launch_surface(cs[i], qs[i], nullptr, f, stage_mode(c, k, more), rk_stage(k), dt, st);
+      c->feat_out = FeatureOut{};
+      DG_CUDA(e);
     }
     ready = f32 && more;
     if (ready) std::swap(c->qf, c->qy);   // the next step's s1 is in qy

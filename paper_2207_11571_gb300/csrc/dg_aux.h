@@ -78,6 +78,7 @@ cudaError_t launch_add_forcing(const dg_ctx* c, double* q, const Forcing& f, dou
 // Operator kernels per precision (dg_kernels_*.cu, dg_split.cu, dg_surface_*.cu); src and
 // mode as launch_volume and launch_surface.
 cudaError_t volume_f32(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+cudaError_t state_f32(const dg_ctx* c, const double* q, bool* done, cudaStream_t st);
 cudaError_t volume_f64(const dg_ctx* c, const double* q, int src, cudaStream_t st);
 cudaError_t volume_split_f32(const dg_ctx* c, const double* q, int src, cudaStream_t st);
 cudaError_t volume_split_f64(const dg_ctx* c, const double* q, int src, cudaStream_t st);

@@ -75,9 +75,9 @@ struct Phys {
   double theta_ref;  // p_ref / rho_ref
 };
 
-// Network features that a phase-A launch writes besides its outputs (Sec. 2.2: the
-// element's scaled state): out[e * ld + slot * n^3 + node] = bf16((s_v - mean_f) / sd_f)
-// for v = first_var + slot, from the stage state s the launch forms; mean_f is taken
+// Network features that the launch which forms a stage state s (phase A or its state pass,
+// phase B of the stage before) also writes (Sec. 2.2: the element's scaled state):
+// out[e * ld + slot * n^3 + node] = bf16((s_v - mean_f) / sd_f) for v = first_var + slot; mean_f is taken
 // relative to the operator's reference state (shift32, FP32 operator) or as is (mean64,
 // FP64 operator).  out == nullptr: none.
 struct FeatureOut {
@@ -150,7 +150,10 @@ struct dg_ctx {
   double* host_ring_dev = nullptr;   // the ring's device address (cudaHostGetDevicePointer)
   int forcing_mode = DG_FORCING_STAGE;  // where dg_rk3_step applies a network forcing
   float* s_buf = nullptr;      // forcing buffer [nel][5 n^3]
-  dgnn::FeatureOut feat_out;   // features the next phase-A launch also writes (set per launch)
+  // set per launch: the features that the launch which forms a stage state writes with it,
+  // and whether phase A runs beside the forcing network (launched just before it)
+  dgnn::FeatureOut feat_out;
+  bool beside_forcing = false;
   double* filter_dev[dgnn::kMaxP + 1] = {};  // filter G to each lower order (dg_project)
   double* prolong_dev[dgnn::kMaxP + 1] = {};  // interpolation to each higher order (dg_prolong)
   bool borrowed = false;       // member of a dg_batch: released by dg_batch_destroy only
@@ -173,6 +176,9 @@ inline void* stage_buffer(const dg_ctx* c, int k) {
 // Phase A.  src 0: the stage state is formed from q (FP64) in c->qf; src 1 (FP32 operator,
 // RK stages 2 and 3): it is in c->cur.
 cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_t st);
+// The stage state of phase A's src 0 in a launch of its own, for the orders that have one
+// (*done; phase A then takes src 1).
+cudaError_t launch_state(const dg_ctx* c, const double* q, bool* done, cudaStream_t st);
 // Phase B.  mode 0: dqdt = R (+ s).  mode 1: FP64 RK stage, g = A g + dt R, q += B g.
 // modes 2, 3, 4: FP32 operator RK stages 1, 2, 3 on the FP32 increment; stage 3 adds
 // the increment to the FP64 state.

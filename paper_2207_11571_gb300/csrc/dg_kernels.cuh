@@ -75,7 +75,7 @@ struct OpConst {
   int les;
   double drho_ref, dE_ref;        // references for shifting the FP64 state
   int early;                      // phase A lets the next launch in as it starts, not as it ends (make_const)
-  FeatureOut feat;                // network features written by phase A (feat.out may be NULL)
+  FeatureOut feat;                // network features to write with the stage state (feat.out may be NULL)
   T D[kMaxN1 * kMaxN1];
 };
 
@@ -862,6 +862,29 @@ __device__ __forceinline__ void state_row(const double* __restrict__ q, const fl
 // converts once (32^3 RK3 step 331 -> 306 us, 16^3 58.2 -> 54.1, 8^3 29.7 -> 27.1; a thread per
 // row of four nodes here: 16^3 58.6).  At the other orders, whose kernels hide the
 // conversions, it does not pay (16^3/P8 516 -> 521 us).
+// It also writes the forcing network's input features (C.feat), the same arithmetic as the
+// separate feature kernels of the network.
+__device__ __forceinline__ void feature_store(const FeatureOut& f, int e, int np, int node, int v, float s) {
+  const int slot = v - f.first_var;
+  if (slot < 0 || slot >= f.n_vars) return;
+  const int i = slot * np + node;
+  static_cast<__nv_bfloat16*>(f.out)[(long long)e * f.ld + i] = __float2bfloat16_rn((s - f.shift32[i]) / f.sd[i]);
+}
+// A row of four nodes at P = 3 (every array 16-byte aligned: n^3 = 64 features per variable).
+__device__ __forceinline__ void feature_row(const FeatureOut& f, int e, int node, int v, const float s[4]) {
+  const int slot = v - f.first_var;
+  if (slot < 0 || slot >= f.n_vars) return;
+  const int i = slot * 64 + node;
+  float sh[4], sd[4], x[4];
+  row_read(f.shift32 + i, sh);
+  row_read(f.sd + i, sd);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) x[m] = (s[m] - sh[m]) / sd[m];
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]), hi = __floats2bfloat162_rn(x[2], x[3]);
+  *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(f.out) + (long long)e * f.ld + i) =
+      make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+}
+
 constexpr int kStateElems = 4;   // per block of 256 threads
 __device__ __forceinline__ void state4_block(int blk, const double* __restrict__ q, float* __restrict__ qf, int nel,
                                              const OpConst<float>& C) {
@@ -871,6 +894,10 @@ __device__ __forceinline__ void state4_block(int blk, const double* __restrict__
   state_from_q(q, (long long)e * 64 + node, C, s);
 #pragma unroll
   for (int v = 0; v < 5; ++v) qf[(size_t)e * state_record(4) + v * 64 + node] = s[v];
+  if (C.feat.out != nullptr) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) feature_store(C.feat, e, 64, node, v, s[v]);
+  }
 }
 
 template <typename T>   // float only
@@ -883,7 +910,7 @@ __global__ void __launch_bounds__(256) k_state4(const double* __restrict__ q, T*
 
 constexpr int kRows4Floats = 18 * 64;   // shared floats per element: U, halo rows (4 + 4), y- and z-fluxes (10)
 
-template <int SRC, bool CUBE, bool FEAT>
+template <int SRC, bool CUBE>
 __device__ __forceinline__ void volume4_block(int blk, const double* __restrict__ q, float* qf, float* __restrict__ rv,
                                               float* __restrict__ vt, const OpConst<float>& C) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -956,25 +983,6 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   if (SRC == 0) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) row_store(qf + (size_t)e * state_record(4) + v * 64 + 4 * r, s[v]);
-  }
-  if (FEAT) {
-    // the forcing network's input features, from the stage state: the same arithmetic as the
-    // separate feature kernels of the network, four nodes at a time (every array 16-byte
-    // aligned: n^3 = 64 features per variable)
-    __nv_bfloat16* fo = static_cast<__nv_bfloat16*>(C.feat.out) + (long long)e * C.feat.ld + 4 * r;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      const int slot = v - C.feat.first_var;
-      if (slot < 0 || slot >= C.feat.n_vars) continue;
-      float sh[4], sd[4], x[4];
-      row_read(C.feat.shift32 + slot * 64 + 4 * r, sh);
-      row_read(C.feat.sd + slot * 64 + 4 * r, sd);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] = (s[v][i] - sh[i]) / sd[i];
-      const __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]), hi = __floats2bfloat162_rn(x[2], x[3]);
-      *reinterpret_cast<uint2*>(fo + slot * 64) =
-          make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
-    }
   }
   // the other rows of this row's y- and z-line (j ^ m, k ^ m) and their matrix entries
   f32x2 Dy[4], Dz[4];
@@ -1195,18 +1203,24 @@ __host__ __device__ constexpr int volume_min_blocks() {
 template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
 __device__ __forceinline__ void volume_phase(int blk, const double* __restrict__ q, T* qf, T* __restrict__ rv,
                                              T* __restrict__ vt, const OpConst<T>& C) {
-  if constexpr (use_rows4(P, sizeof(T), SPLIT)) volume4_block<SRC, CUBE, FEAT>(blk, q, qf, rv, vt, C);
+  if constexpr (use_rows4(P, sizeof(T), SPLIT)) volume4_block<SRC, CUBE>(blk, q, qf, rv, vt, C);
   else volume_block<P, T, SRC, CUBE, FEAT, SPLIT>(blk, q, qf, rv, vt, C);
 }
 
-template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
+// BESIDE: launched after the forcing network of the same stage state, to run beside it on the
+// SMs it leaves idle.  That launch released this one after its own wait, so the stage state
+// was complete then; only its lines in this SM's L1 can be old, and the fence drops them.
+// The wait for the network comes last: the next launch waits for this one only.
+template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false, bool BESIDE = false>
 __global__ void __launch_bounds__(volume_max_threads<P, T, SPLIT>(), volume_min_blocks<P, T, SPLIT>())
 k_volume(const double* __restrict__ q, T* __restrict__ qf, T* __restrict__ rv, T* __restrict__ vt,
          const OpConst<T> C) {
-  pdl_wait();
+  if (BESIDE) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  else pdl_wait();
   if (C.early) pdl_release();
   volume_phase<P, T, SRC, CUBE, FEAT, SPLIT>(blockIdx.x, q, qf, rv, vt, C);
   pdl_release();
+  if (BESIDE) pdl_wait();
 }
 
 // ---------------------------------------------------------------- phase B
@@ -1417,7 +1431,7 @@ __device__ __forceinline__ void surface_prologue(int blk, int E, const OpConst<T
   __syncthreads();
 }
 
-template <int P, typename T, int MODE, bool CUBE = false>
+template <int P, typename T, int MODE, bool CUBE = false, bool FEAT = false>
 __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>& a, const Forcing& fc,
                                               const OpConst<T>& C, const RkArgs<T>& rk) {
   constexpr int n = P + 1, n2 = n * n, np = n2 * n, ns = node_stride(n);
@@ -1549,6 +1563,7 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
         if (MODE == 2 || MODE == 3) {
           row_store(a.dlt + o + c * 64, u);
           row_store((MODE == 2 ? a.y : a.x) + o + c * 64, v);
+          if constexpr (FEAT) feature_row(C.feat, e, 4 * r, c, v);
         } else {
           double* out = (MODE == 0 ? a.dqdt : a.q) + c * C.N + g;
           if (wide) {
@@ -1562,6 +1577,7 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
 #pragma unroll
             for (int i = 0; i < 4; ++i) u[i] = shifted(q1[i], c, C);
             row_store(a.y + o + c * 64, u);
+            if constexpr (FEAT) feature_row(C.feat, e, 4 * r, c, u);
           }
         }
       }
@@ -1625,30 +1641,37 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
         rk_stage1(rk, R[c], x1[c], d1, s2);
         a.dlt[o + c * ns] = float(d1);
         a.y[o + c * ns] = s2;
+        if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s2);
       } else if (MODE == 3) {
         T w, s3;
         rk_stage2(rk, R[c], x1[c], g1[c], w, s3);
         a.x[o + c * ns] = s3;
+        if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s3);
         a.dlt[o + c * ns] = float(w);
       } else {
         const double qn = q1[c] + f2d(float(rk_stage3(rk, R[c], g1[c])));
         a.q[c * C.N + g] = qn;
-        if (MODE == 5) a.y[o + c * ns] = shifted(qn, c, C);
+        if (MODE == 5) {
+          const T s1 = shifted(qn, c, C);
+          a.y[o + c * ns] = s1;
+          if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s1);
+        }
       }
     }
   }
   }
 }
 
-// E elements per block (kCubeElems with CUBE), THREADS threads.
-template <int P, typename T, int MODE, int E, int THREADS, bool CUBE>
+// E elements per block (kCubeElems with CUBE), THREADS threads.  FEAT: also writes the network
+// features of the stage state it forms (MODES 2, 3, 5).
+template <int P, typename T, int MODE, int E, int THREADS, bool CUBE, bool FEAT>
 __global__ void __launch_bounds__(THREADS, surf_min_blocks(THREADS, sizeof(T)))
 k_surface(SurfArgs<T> a, Forcing fc, const OpConst<T> C, RkArgs<T> rk) {
   // last block first: phase A has just written the end of the mesh, which is still in L2
   const int blk = gridDim.x - 1 - blockIdx.x;
   surface_prologue<P, T, CUBE>(blk, E, C);
   pdl_wait();
-  surface_block<P, T, MODE, CUBE>(blk, E, a, fc, C, rk);
+  surface_block<P, T, MODE, CUBE, FEAT>(blk, E, a, fc, C, rk);
   pdl_release();
 }
 

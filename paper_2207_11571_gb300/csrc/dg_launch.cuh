@@ -101,11 +101,11 @@ cudaError_t set_smem(K kern, size_t smem) {
 
 // Phase A of one mesh.  src 0: the stage state from q, written to c->qf; else: the stage
 // state in c->cur.
-template <int P, typename T, int SRC, bool CUBE, bool FEAT, bool SPLIT>
+template <int P, typename T, int SRC, bool CUBE, bool FEAT, bool SPLIT, bool BESIDE>
 cudaError_t volume_launch(const dg_ctx* c, const double* q, cudaStream_t st) {
   const int E = CUBE ? kCubeElems : c->geom.E;
   const size_t smem = volume_smem<P, T, SPLIT>(E, CUBE);
-  auto kern = k_volume<P, T, SRC, CUBE, FEAT, SPLIT>;
+  auto kern = k_volume<P, T, SRC, CUBE, FEAT, SPLIT, BESIDE>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int h = c->K / 2;
@@ -114,33 +114,46 @@ cudaError_t volume_launch(const dg_ctx* c, const double* q, cudaStream_t st) {
                     static_cast<T*>(c->rv), static_cast<T*>(c->vt), make_const<T>(c));
 }
 
+// With a forcing network a launch that forms the state writes its features, and one that
+// reads it (the features are then written with it) may run beside the network.
+template <int P, typename T, int SRC, bool CUBE, bool SPLIT>
+cudaError_t volume_shape(const dg_ctx* c, const double* q, cudaStream_t st) {
+  constexpr bool forms = SRC == 0;
+  if (forms ? c->feat_out.out != nullptr : c->beside_forcing)
+    return volume_launch<P, T, SRC, CUBE, forms, SPLIT, !forms>(c, q, st);
+  return volume_launch<P, T, SRC, CUBE, false, SPLIT, false>(c, q, st);
+}
+
 template <int P, typename T, int SRC, bool SPLIT>
 cudaError_t volume_p(const dg_ctx* c, const double* q, cudaStream_t st) {
-  const bool feat = c->feat_out.out != nullptr;
   if constexpr (cube_ok(P) && !SPLIT) {
-    if (c->geom.cube)
-      return feat ? volume_launch<P, T, SRC, true, true, false>(c, q, st)
-                  : volume_launch<P, T, SRC, true, false, false>(c, q, st);
+    if (c->geom.cube) return volume_shape<P, T, SRC, true, false>(c, q, st);
   }
-  return feat ? volume_launch<P, T, SRC, false, true, SPLIT>(c, q, st)
-              : volume_launch<P, T, SRC, false, false, SPLIT>(c, q, st);
+  return volume_shape<P, T, SRC, false, SPLIT>(c, q, st);
+}
+
+// The stage state in a pass of its own (c->cur is then c->qf), where the order has one.
+template <int P, typename T, bool SPLIT>
+cudaError_t state_p(const dg_ctx* c, const double* q, bool* done, cudaStream_t st) {
+  *done = use_rows4(P, sizeof(T), SPLIT);
+  if constexpr (use_rows4(P, sizeof(T), SPLIT))
+    return launch_pdl(k_state4<T>, dim3((c->nel + kStateElems - 1) / kStateElems), dim3(256), 0, st, q,
+                      static_cast<T*>(c->qf), c->nel, make_const<T>(c));
+  return cudaSuccess;
 }
 
 template <int P, typename T, bool SPLIT>
 cudaError_t volume_src(const dg_ctx* c, const double* q, int src, cudaStream_t st) {
-  if constexpr (use_rows4(P, sizeof(T), SPLIT)) {
-    if (src == 0) {   // the state in a pass of its own (c->cur is then c->qf)
-      const cudaError_t e = launch_pdl(k_state4<T>, dim3((c->nel + kStateElems - 1) / kStateElems), dim3(256), 0, st, q,
-                                       static_cast<T*>(c->qf), c->nel, make_const<T>(c));
-      if (e != cudaSuccess) return e;
-    }
-    return volume_p<P, T, 1, SPLIT>(c, q, st);
-  } else {
-    if constexpr (std::is_same<T, float>::value) {
-      if (src != 0) return volume_p<P, T, 1, SPLIT>(c, q, st);
-    }
-    return volume_p<P, T, 0, SPLIT>(c, q, st);
+  bool formed = src != 0;
+  if (!formed) {
+    const cudaError_t e = state_p<P, T, SPLIT>(c, q, &formed, st);
+    if (e != cudaSuccess) return e;
   }
+  if constexpr (std::is_same<T, float>::value) {
+    if (formed) return volume_p<P, T, 1, SPLIT>(c, q, st);
+  }
+  if constexpr (!use_rows4(P, sizeof(T), SPLIT)) return volume_p<P, T, 0, SPLIT>(c, q, st);
+  return cudaErrorInvalidValue;
 }
 
 #define DG_FOR_EACH_P(CALL)        \
@@ -163,6 +176,13 @@ cudaError_t volume_t(const dg_ctx* c, const double* q, int src, cudaStream_t st)
 #undef DG_V
 }
 
+template <typename T>
+cudaError_t state_t(const dg_ctx* c, const double* q, bool* done, cudaStream_t st) {
+#define DG_P(PP) state_p<PP, T, false>(c, q, done, st)
+  DG_FOR_EACH_P(DG_P)
+#undef DG_P
+}
+
 // Operands of phase B of mode `mode` (see k_surface).
 template <typename T>
 SurfArgs<T> surf_args(const dg_ctx* c, double* q, double* dqdt) {
@@ -179,11 +199,14 @@ SurfArgs<T> surf_args(const dg_ctx* c, double* q, double* dqdt) {
   return a;
 }
 
-template <int P, typename T, int MODE, int E, int THREADS, bool CUBE>
+template <int P, typename T, int MODE, int E, int THREADS, bool CUBE, bool FEAT = false>
 cudaError_t surface_launch(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, const RkArgs<T>& rk,
                            cudaStream_t st) {
+  if constexpr (std::is_same<T, float>::value && !FEAT && (MODE == 2 || MODE == 3 || MODE == 5)) {
+    if (c->feat_out.out) return surface_launch<P, T, MODE, E, THREADS, CUBE, true>(c, q, dqdt, f, rk, st);
+  }
   const size_t smem = surface_smem_bytes<P, T>(E);
-  auto kern = k_surface<P, T, MODE, E, THREADS, CUBE>;
+  auto kern = k_surface<P, T, MODE, E, THREADS, CUBE, FEAT>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3((owned_elems(c) + E - 1) / E), dim3(THREADS), smem, st, surf_args<T>(c, q, dqdt), f,

@@ -526,7 +526,7 @@ bool nn_phase_a_features(const nn_model* m, const dg_ctx* c, FeatureOut* out) {
 }
 
 int nn_forcing_on_state(const nn_model* m, const dg_ctx* c, const double* q, float* s, int* first_var, int* n_vars,
-                        cudaStream_t st, bool features_ready) {
+                        cudaStream_t st, int flags) {
   if (!m || !c || !q || !s) return fail(DG_ERR_INVALID_ARG, "forcing: NULL argument");
   const int feat = m->d.n_vars * c->np;
   if (m->d.n_in != feat || m->d.n_out != feat)
@@ -543,8 +543,8 @@ int nn_forcing_on_state(const nn_model* m, const dg_ctx* c, const double* q, flo
   for (int e0 = 0; e0 < c->nel; e0 += m->d.max_batch) {
     const int rows = std::min(m->d.max_batch, c->nel - e0);
     const long long tot = (long long)rows * m->pad[0];
-    if (features_ready && rows == c->nel) {
-      // the phase-A launch before this call wrote the features (nn_phase_a_features)
+    if ((flags & kFeaturesReady) && rows == c->nel) {
+      // the launch that formed the stage state wrote the features (nn_phase_a_features)
     } else if (f32) {
       DG_CUDA(pdl_launch(k_prep_state_f32, dim3(blocks_for(tot, 256)), dim3(256), st, static_cast<const float*>(c->cur), state_record(c->n),
                                                              node_stride(c->n), c->np,
@@ -573,6 +573,7 @@ int nn_forcing_on_state(const nn_model* m, const dg_ctx* c, const double* q, flo
       f.out = s + (long long)e0 * feat;
       f.ldo = feat;
       f.err = m->err;
+      f.release = (flags & kPhaseAFollows) != 0;
       int rc = forcing_fused(f, st);
       if (rc) return rc;
     } else {

@@ -87,6 +87,7 @@ struct ForcingArgs {
   const float* shift;
   float* out;
   int ldo;
+  int release;                    // let the next launch start beside this one
 };
 
 __device__ __forceinline__ int panels_of(int d) { return (d + kPanel - 1) / kPanel; }
@@ -230,6 +231,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
   // programmatic dependent launch: the set-up above overlaps the previous kernel; every
   // global read (stage state, weights: a training step may just have written them) waits
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.release) {
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
 
   if (warp == 0) {
     if (lane == 0) {
@@ -509,6 +514,7 @@ int forcing_fused(const ForcingLaunch& f, cudaStream_t st) {
   a.shift = f.shift;
   a.out = f.out;
   a.ldo = f.ldo;
+  a.release = f.release;
   static bool configured = false;
   if (!configured) {
     DG_CUDA(cudaFuncSetAttribute(k_forcing_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));

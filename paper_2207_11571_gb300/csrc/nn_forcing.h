@@ -22,6 +22,7 @@ struct ForcingLaunch {
   float* out;           // [rows][ldo] FP32, 16-byte aligned rows
   int ldo;
   int* err;             // device error flag (bounded waits)
+  bool release;         // let the next launch start beside this one
 };
 
 // CTAs per cluster (4, 2 or 1) for `rows` elements on `sms` SMs: the largest C whose

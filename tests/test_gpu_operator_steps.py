@@ -87,3 +87,44 @@ def test_phase_b_blocks_of_every_size_give_the_same_bits(dg, K, P, prec):
             assert (alone - qs[0]).abs().max().item() <= 4e-16 * alone.abs().max().item()
     finally:
         dg.dg_batch_destroy(b)
+
+
+@pytest.mark.parametrize("K,P,first,nv", [(6, 3, 0, 5), (5, 3, 1, 3), (6, 2, 0, 5), (4, 5, 1, 3)])
+def test_corrected_steps_in_one_call_equal_single_steps_and_one_rhs(dg, K, P, first, nv):
+    """The network runs ahead of phase A where the stage state and its features exist: within a
+    call phase B writes both, at the start of a call the state pass (P = 3) or phase A does.
+    The same features, so the same bits; and the forced dq/dt of a call on its own agrees
+    with the per-layer path, which forms the features from the state after phase A."""
+    from paper_2207_11571_gb300 import nn
+    N, feat = K ** 3 * (P + 1) ** 3, nv * (P + 1) ** 3
+    dims = [feat, 64, 64, feat]
+    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=1)
+    net = nn.nn_create(feat, feat, 64, 2, first, nv, K ** 3, inputs.uniform_draws(dims, 3))
+    try:
+        # a forcing of order 0.1: larger ones drive the density negative within the steps
+        nn.nn_set_scalers(net, *[v * torch.ones(feat).numpy() for v in (0.0, 1.0, 0.0, 1e-3)])
+        q = state(dg, ctx, N)
+        dt = dg.dg_stable_dt(ctx, q, 0.5)
+        single, many, free = q.clone(), q.clone(), q.clone()
+        for _ in range(3):
+            dg.dg_rk3_step(ctx, single, dt, 1, net)
+        dg.dg_rk3_step(ctx, many, dt, 3, net)
+        dg.dg_rk3_step(ctx, free, dt, 3)
+        torch.cuda.synchronize()
+        assert torch.isfinite(many).all() and not torch.equal(many, free)
+        assert torch.equal(many, single)
+        R, Rl = torch.empty_like(q), torch.empty_like(q)
+        dg.dg_rhs(ctx, q, R, net)
+        nn.nn_set_fused(net, 0)   # a GEMM per layer
+        dg.dg_rhs(ctx, q, Rl, net)
+        plain = torch.empty_like(q)
+        dg.dg_rhs(ctx, q, plain)
+        torch.cuda.synchronize()
+        # both paths sum the same bf16 products in FP32: the forcing itself to 1e-5, on top of
+        # FP32 rounding of dq/dt
+        forcing = (R - plain).abs().max().item()
+        assert forcing > 0
+        assert (R - Rl).abs().max().item() <= 1e-3 * forcing + 1e-6 * plain.abs().max().item()
+    finally:
+        nn.nn_destroy(net)
+        dg.dg_destroy(ctx)
