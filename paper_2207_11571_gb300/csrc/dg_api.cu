@@ -247,17 +247,15 @@ static int diag_enqueue(dg_ctx* c, const double* q, const double* qref, const nn
     if (rc) return rc;
     R = c->rhs_tmp;
   }
-  double* dev_out = c->red + (size_t)c->red_blocks * kDiagLen;
-  DG_CUDA(launch_diagnostics(c, q, R, qref, c->red, c->red_blocks, dev_out, st));
-  // the kernels' error flag rides along in the slot after the diagnostics.  A host-advance
+  DG_CUDA(launch_diagnostics(c, q, R, qref, st));
+  // the kernels' error flag is in the slot after the diagnostics.  A host-advance
   // slot is written by a kernel (its few bytes do not wait behind other streams' state
   // copies on the copy engine); the synchronous paths copy.
   if (slot) {
-    DG_CUDA(launch_store_host(dev_out, kDiagLen, c->err_dev, host, st));
+    DG_CUDA(launch_store_host(c->red, kDiagLen, c->err_dev, host, st));
     return DG_OK;
   }
-  DG_CUDA(cudaMemcpyAsync(host, dev_out, kDiagLen * sizeof(double), cudaMemcpyDeviceToHost, st));
-  DG_CUDA(cudaMemcpyAsync(host + kDiagLen, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+  DG_CUDA(cudaMemcpyAsync(host, c->red, kHostSlot * sizeof(double), cudaMemcpyDeviceToHost, st));
   return DG_OK;
 }
 
@@ -489,10 +487,8 @@ int dg_group_diagnostics(dg_ctx* const* parts, int n, double* const* q, dg_diag*
   std::vector<dg_diag> d(n);
   for (int i = 0; i < n; ++i) {
     dg_ctx* c = parts[i];
-    double* dev_out = c->red + (size_t)c->red_blocks * kDiagLen;
-    DG_CUDA(launch_diagnostics(c, q[i], c->rhs_tmp, nullptr, c->red, c->red_blocks, dev_out, st));
-    DG_CUDA(cudaMemcpyAsync(c->red_host, dev_out, kDiagLen * sizeof(double), cudaMemcpyDeviceToHost, st));
-    DG_CUDA(cudaMemcpyAsync(c->red_host + kDiagLen, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DG_CUDA(launch_diagnostics(c, q[i], c->rhs_tmp, nullptr, st));
+    DG_CUDA(cudaMemcpyAsync(c->red_host, c->red, kHostSlot * sizeof(double), cudaMemcpyDeviceToHost, st));
   }
   for (int i = 0; i < n; ++i) {
     rc = diag_collect(parts[i], true, false, &d[i], st);
@@ -574,7 +570,6 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
     }
   }
   const size_t tsz = f32 ? sizeof(float) : sizeof(double);
-  c->red_blocks = kDiagBlocks;
   cudaError_t e = cudaSuccess;
   const size_t rec = (size_t)c->nel * state_record(c->n), frec = (size_t)c->nel * face_record(c->n);
   if (e == cudaSuccess) e = cudaMalloc(&c->qf, rec * tsz);
@@ -585,7 +580,8 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
   if (f32 && e == cudaSuccess) e = cudaMalloc(&c->dlt, rec * tsz);
   c->cur = c->qf;
   if (e == cudaSuccess) e = cudaMalloc(&c->rhs_tmp, 5 * c->N * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->red, (size_t)(c->red_blocks + 1) * kDiagLen * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&c->red, kDiagBytes);
+  if (e == cudaSuccess) e = cudaMemset(c->red, 0, kDiagOut * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost(&c->red_host, (kDiagLen + 1) * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->err_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(c->err_dev, 0, sizeof(int));

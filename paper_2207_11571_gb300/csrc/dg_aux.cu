@@ -1,6 +1,7 @@
 // Auxiliary kernels: Taylor-Green initial state (Sec. 3.1, Eq. 11), the filter G
 // (Eq. 2, Sec. 2.6), FP64 integral diagnostics (Sec. 2.4, Eq. 9) and the training
 // pairs of Algorithm 1 (Sec. 2.1).
+#include <algorithm>
 #include <cmath>
 
 #include "dg_aux.h"
@@ -103,13 +104,49 @@ cudaError_t launch_prolong(const dg_ctx* lo, const dg_ctx* hi, const double* ql,
 
 // ---------------------------------------------------------------- diagnostics
 
-// Per-node contributions reduced in a fixed order: block tree, then one block over the
-// block partials in index order -> bitwise reproducible for a given launch shape.
-__device__ __forceinline__ void diag_combine(double* a, const double* b) {
+// 1 / x by one Newton-Raphson step of third order, r (1 + e + e^2) with e = 1 - x r, from the
+// FP32 reciprocal (|e| < 2^-22): three FP64 operations, the last rounding the only one that
+// counts.  x outside FP32's range is divided.
+__device__ __forceinline__ double reciprocal64(double x) {
+  const float r32 = 1.f / d2f_rn(x);
+  if (!(fabsf(r32) > 1e-37f && fabsf(r32) < 1e37f)) return 1.0 / x;
+  const double r = f2d(r32), e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+__device__ __forceinline__ bool finite64(double x) {   // on the integer pipe
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) != 0x7FFu;
+}
+
+// max(a, b) of a >= 0 and b >= 0 or NaN (ignored), on the integer pipe.
+__device__ __forceinline__ double max_pos(double a, double b) {
+  const unsigned long long u = __double_as_longlong(a), v = __double_as_longlong(b);
+  return v > u && v <= 0x7FF0000000000000ull ? b : a;
+}
+
+// Warp sums of eight values in a fixed order, the value of lane / 4 in each lane: halves of
+// the values are exchanged at each step, 9 additions per lane instead of 40.
+__device__ __forceinline__ double warp_sum8(const double v[8], int lane) {
+  double a[4], b[2];
 #pragma unroll
-  for (int i = 0; i < kDiagSum; ++i) a[i] += b[i];
+  for (int i = 0; i < 4; ++i) {
+    const bool up = lane & 16;
+    a[i] = (up ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[4 + i], 16);
+  }
 #pragma unroll
-  for (int i = kDiagSum; i < kDiagLen; ++i) a[i] = fmax(a[i], b[i]);
+  for (int i = 0; i < 2; ++i) {
+    const bool up = lane & 8;
+    b[i] = (up ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[2 + i], 8);
+  }
+  const bool up = lane & 4;
+  double s = (up ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  return s + __shfl_xor_sync(0xffffffffu, s, 1);
+}
+__device__ __forceinline__ double warp_max(double x) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x = max_pos(x, __shfl_xor_sync(0xffffffffu, x, off));
+  return x;
 }
 
 // The largest wave speed |v| + c of a node in FP64 (the expression the reference computes).
@@ -122,62 +159,75 @@ __device__ __forceinline__ double wave64(const double qv[5], double gamma) {
 }
 
 // Per-node sums (mass, momenta, energy, kinetic energy, dKE/dt) and maxima (e_inf, wave
-// speed) of the owned nodes.  GB300's FP64 rate is a small fraction of its FP32 rate, so
-// the FP64 work per node is kept to the sums: the quadrature weights come from a table,
-// the kinetic energy is |m|^2 / (2 rho) with one division, and the wave speed is screened
-// in FP32 — the FP64 expression is evaluated only for nodes whose FP32 estimate is within
-// 1e-4 of the thread's running maximum.  Where p/(gamma-1) is at least 1 % of rho e, the
-// FP32 estimate is within 3e-5 of the exact value (rounding of the inputs and of a
-// difference that loses at most two digits); every other node goes to FP64.  The node with
-// the thread's largest exact value is therefore never screened out (its estimate is at
-// least (1 - 6e-5) times every earlier estimate), and the maximum is the FP64 maximum over
-// all nodes, as without the screen.
-__global__ void k_diag_partial(const double* __restrict__ q, const double* __restrict__ R,
-                               const double* __restrict__ qref, NodeGeom ng, double gamma,
-                               double* __restrict__ partial) {
-  __shared__ double sh[kDiagThreads][kDiagLen + 1];
+// speed) of the owned nodes.  GB300's FP64 rate is a small fraction of its FP32 rate and
+// bounds this kernel, so the FP64 work per node is kept to the sums, about 20 operations: the
+// quadrature weights come from a table, one three-operation reciprocal serves the kinetic
+// energy and its derivative, tests and maxima run on the integer pipe, and the wave speed
+// (some 45 operations) is screened in FP32: a thread keeps the node of its largest FP32
+// estimate and evaluates the FP64 expression at the end, if that estimate is within 1e-5 of
+// the block's largest, or at once for a node within 1e-5 of the one it keeps (and of the
+// block's largest so far: on a symmetric flow such nodes are common).  Where
+// p/(gamma-1) is at least a quarter of rho e, the estimate is within 2e-6 of the exact value
+// (rounding of the inputs, and of a difference that multiplies it by four at most); every
+// other node goes to FP64 at once.  The node with the largest exact value is therefore never
+// screened out (its estimate is at least (1 - 4e-6) times every other), and the maximum is
+// the FP64 maximum over all nodes.  Screened against the thread's own running maximum, nearly
+// every warp took the FP64 path at every node.  The last block to finish reduces the block
+// partials (in index order): a launch of one block took 13 us.
+// 16^3/P8 with dq/dt: 352 + 13 -> 208 us (239 MB), 16^3/P3 with a reference 61 + 13 -> 53.
+__global__ void __launch_bounds__(kDiagThreads)
+k_diag_partial(const double* __restrict__ q, const double* __restrict__ R, const double* __restrict__ qref, NodeGeom ng,
+               double gamma, double* partial, const int* __restrict__ flag, unsigned* ticket, double* __restrict__ out) {
+  constexpr int kWarps = kDiagThreads / 32;
+  __shared__ double sh[kWarps][kDiagLen];
+  __shared__ unsigned sm;   // the block's largest estimate so far (bits: estimates are positive)
   __shared__ double sW[kMaxN1 * kMaxN1 * kMaxN1];   // quadrature weight x Jacobian of each node
   double acc[kDiagLen];
   for (int i = 0; i < kDiagLen; ++i) acc[i] = 0.0;
-  const int n = ng.n, np = n * n * n;
+  const int n = ng.n, np = n * n * n, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const double jac = 0.125 * ng.h * ng.h * ng.h;
+  if (threadIdx.x == 0) sm = 0;
   for (int t = threadIdx.x; t < np; t += blockDim.x) {
     const int i = t % n, j = (t / n) % n, k = t / (n * n);
     sW[t] = ng.w[i] * ng.w[j] * ng.w[k] * jac;
   }
   __syncthreads();
   const float gf = (float)gamma;
-  float m32 = 0.f;   // running FP32 estimate of this thread's largest wave speed
+  float m32 = 0.f;             // this thread's largest FP32 estimate of a wave speed
+  long long m_at = -1;         // its node
+  int bad = 0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = ng.t_begin + blockIdx.x * (long long)blockDim.x + threadIdx.x;
   int node = (int)(t0 % np);
   const int dnode = (int)(stride % np);
   for (long long t = t0; t < ng.t_end; t += stride, node = (node + dnode >= np) ? node + dnode - np : node + dnode) {
     const double W = sW[node];
-    double qv[5];
+    double qv[5], rv[4];
+#pragma unroll
     for (int c = 0; c < 5; ++c) qv[c] = q[c * ng.N + t];
+    if (R) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) rv[c] = R[c * ng.N + t];
+    }
     bool finite = true;
-    for (int c = 0; c < 5; ++c) finite = finite && isfinite(qv[c]);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) finite = finite && finite64(qv[c]);
     if (!finite) {
-      acc[kDiagNonfinite] += 1.0;
+      ++bad;
       continue;
     }
-    acc[0] += W * qv[0];
-    acc[1] += W * qv[1];
-    acc[2] += W * qv[2];
-    acc[3] += W * qv[3];
-    acc[4] += W * qv[4];
-    const double ir = 1.0 / qv[0];
-    const double m2 = qv[1] * qv[1] + qv[2] * qv[2] + qv[3] * qv[3];
-    acc[5] += W * 0.5 * (m2 * ir);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) acc[c] += W * qv[c];
+    const double ir = reciprocal64(qv[0]);
+    const double ke2 = (qv[1] * qv[1] + qv[2] * qv[2] + qv[3] * qv[3]) * ir;   // rho v^2
+    acc[5] += W * ke2;   // halved at the end
     if (R) {
-      const double vx = qv[1] * ir, vy = qv[2] * ir, vz = qv[3] * ir;
-      const double v2 = vx * vx + vy * vy + vz * vz;
-      const double dk = vx * R[1 * ng.N + t] + vy * R[2 * ng.N + t] + vz * R[3 * ng.N + t] - 0.5 * v2 * R[t];
+      const double dk = (qv[1] * rv[1] + qv[2] * rv[2] + qv[3] * rv[3]) * ir - 0.5 * (ke2 * ir) * rv[0];
       acc[6] += W * dk;
     }
     if (qref) {
-      for (int c = 0; c < 3; ++c) acc[8 + c] = fmax(acc[8 + c], fabs(qv[1 + c] - qref[(1 + c) * ng.N + t]));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[8 + c] = max_pos(acc[8 + c], fabs(qv[1 + c] - qref[(1 + c) * ng.N + t]));
     }
     // wave speed: FP32 screen, FP64 where it may set the maximum
     const float r = d2f_rn(qv[0]), e = d2f_rn(qv[4]);
@@ -186,43 +236,83 @@ __global__ void k_diag_partial(const double* __restrict__ q, const double* __res
     const float v2f = (mx * mx + my * my + mz * mz) * irf * irf;
     const float pe = e - 0.5f * r * v2f;   // p / (gamma - 1)
     const float wf = sqrtf(v2f) + sqrtf(fmaxf(gf * (gf - 1.f) * pe * irf, 0.f));
-    if (wf >= m32 * (1.f - 1e-4f) || !(pe > 1e-2f * fabsf(e)) || !(r > 0.f)) {
-      acc[11] = fmax(acc[11], wave64(qv, gamma));
-      m32 = fmaxf(m32, wf);
+    const bool sound32 = pe > 0.25f * fabsf(e) && r > 0.f && wf < 1e30f;
+    const bool tie = wf >= m32 * (1.f - 1e-5f) && wf <= m32 * (1.f + 1e-5f);
+    if (sound32) {
+      const unsigned act = __activemask(), top = __reduce_max_sync(act, __float_as_uint(wf));
+      if (lane == __ffs(act) - 1) atomicMax(&sm, top);
+    }
+    if (!sound32 || (tie && wf >= __uint_as_float(*(volatile unsigned*)&sm) * (1.f - 1e-5f))) {
+      acc[11] = max_pos(acc[11], wave64(qv, gamma));
+    } else if (wf > m32 && !tie) {
+      m32 = wf;
+      m_at = t;
     }
   }
-  for (int i = 0; i < kDiagLen; ++i) sh[threadIdx.x][i] = acc[i];
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) diag_combine(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
+  const float bm = __uint_as_float(sm);
+  if (m_at >= 0 && m32 >= bm * (1.f - 1e-5f)) {
+    double qv[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) qv[c] = q[c * ng.N + m_at];
+    acc[11] = max_pos(acc[11], wave64(qv, gamma));
   }
-  if (threadIdx.x == 0)
-    for (int i = 0; i < kDiagLen; ++i) partial[blockIdx.x * kDiagLen + i] = sh[0][i];
+  acc[5] *= 0.5;
+  acc[kDiagNonfinite] = (double)bad;
+  static_assert(kDiagSum == 8, "warp_sum8");
+  const double s8 = warp_sum8(acc, lane);
+  if (lane % 4 == 0) sh[warp][lane / 4] = s8;
+#pragma unroll
+  for (int i = kDiagSum; i < kDiagLen; ++i) {
+    const double x = warp_max(acc[i]);
+    if (lane == 0) sh[warp][i] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < kDiagLen) {
+    double x = sh[0][threadIdx.x];
+    for (int w = 1; w < kWarps; ++w) x = threadIdx.x < kDiagSum ? x + sh[w][threadIdx.x] : max_pos(x, sh[w][threadIdx.x]);
+    partial[threadIdx.x * gridDim.x + blockIdx.x] = x;
+    __threadfence();
+  }
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = warp; i < kDiagLen; i += kWarps) {
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b0 = 0; b0 < (int)gridDim.x; b0 += 128) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int b = b0 + 32 * u + lane;
+        const double y = b < (int)gridDim.x ? __ldcg(partial + (size_t)i * gridDim.x + b) : 0.0;
+        x[u] = i < kDiagSum ? x[u] + y : max_pos(x[u], y);
+      }
+    }
+    double s = x[0];
+#pragma unroll
+    for (int u = 1; u < 4; ++u) s = i < kDiagSum ? s + x[u] : max_pos(s, x[u]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const double y = __shfl_xor_sync(0xffffffffu, s, off);
+      s = i < kDiagSum ? s + y : max_pos(s, y);
+    }
+    if (lane == 0) out[i] = s;
+  }
+  if (threadIdx.x == 0) {   // the error flag in the next slot: one copy carries both
+    *reinterpret_cast<int*>(out + kDiagLen) = *flag;
+    *ticket = 0;
+  }
 }
 
-__global__ void k_diag_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
-  __shared__ double sh[kDiagThreads][kDiagLen + 1];
-  double acc[kDiagLen];
-  for (int i = 0; i < kDiagLen; ++i) acc[i] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) diag_combine(acc, partial + b * kDiagLen);
-  for (int i = 0; i < kDiagLen; ++i) sh[threadIdx.x][i] = acc[i];
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) diag_combine(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int i = 0; i < kDiagLen; ++i) out[i] = sh[0][i];
-}
-
-cudaError_t launch_diagnostics(const dg_ctx* c, const double* q, const double* R, const double* qref,
-                               double* partial, int nblocks, double* out, cudaStream_t st) {
+cudaError_t launch_diagnostics(const dg_ctx* c, const double* q, const double* R, const double* qref, cudaStream_t st) {
   NodeGeom ng = node_geom(c);
-  k_diag_partial<<<nblocks, kDiagThreads, 0, st>>>(q, R, qref, ng, c->opts.gamma, partial);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_diag_final<<<1, kDiagThreads, 0, st>>>(partial, nblocks, out);
+  // two nodes per thread at least: the reduction of a thread's sums costs as much as a node
+  const int nblocks =
+      (int)std::min<long long>(kDiagBlocks, (ng.t_end - ng.t_begin + 2 * kDiagThreads - 1) / (2 * kDiagThreads));
+  k_diag_partial<<<nblocks, kDiagThreads, 0, st>>>(q, R, qref, ng, c->opts.gamma, c->red + kDiagOut, c->err_dev,
+                                                   reinterpret_cast<unsigned*>(c->red + kDiagLen + 1), c->red);
   return cudaGetLastError();
 }
 

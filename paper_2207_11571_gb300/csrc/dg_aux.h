@@ -40,7 +40,10 @@ constexpr int kDiagSum = 8;
 constexpr int kDiagLen = 12;
 constexpr int kDiagNonfinite = 7;
 constexpr int kDiagThreads = 256;
-constexpr int kDiagBlocks = 1024;
+constexpr int kDiagBlocks = 1024;     // at most
+// dg_ctx::red: results, error flag, ticket of the blocks, then the block partials.
+constexpr int kDiagOut = kDiagLen + 2;
+constexpr size_t kDiagBytes = (kDiagOut + (size_t)kDiagBlocks * kDiagLen) * sizeof(double);
 
 cudaError_t launch_init_tgv(const dg_ctx* c, double* q, const double* pert, cudaStream_t st);
 cudaError_t launch_project(const dg_ctx* hi, const dg_ctx* lo, const double* qh, double* ql, const double* Gdev,
@@ -51,8 +54,8 @@ cudaError_t launch_prolong(const dg_ctx* lo, const dg_ctx* hi, const double* ql,
 // host[0..n) = src[0..n), then *flag as an int in the next slot; host is pinned host memory
 // (the SMs write it through the coherent mapping).  n < 1024.
 cudaError_t launch_store_host(const double* src, int n, const int* flag, double* host, cudaStream_t st);
-cudaError_t launch_diagnostics(const dg_ctx* c, const double* q, const double* R, const double* qref,
-                               double* partial, int nblocks, double* out, cudaStream_t st);
+// Into c->red: the diagnostics, then the context's error flag as an int in the next slot.
+cudaError_t launch_diagnostics(const dg_ctx* c, const double* q, const double* R, const double* qref, cudaStream_t st);
 cudaError_t launch_make_pairs(const dg_ctx* lo, const double* qb_n, const double* qnn_np1, const double* qb_np1,
                               double dt, int first_var, int n_vars, float* X, float* Y, cudaStream_t st);
 // Face traces of a slab (element-layer partition).  pack: the owned boundary layers'

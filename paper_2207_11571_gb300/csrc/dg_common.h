@@ -135,7 +135,6 @@ struct dg_ctx {
   float* dlt = nullptr;   // FP32 operator: RK increment, [elem][5][node]
   double* rhs_tmp = nullptr;  // [5][N] FP64 operator value for diagnostics
   double* red = nullptr;  // reduction partials
-  int red_blocks = 0;
   double* red_host = nullptr;  // pinned host copy of the final reduction
   double* q_dev = nullptr;     // device state for dg_advance_host
   int* err_dev = nullptr;      // device error flag: a bounded wait in a kernel expired
