@@ -146,6 +146,18 @@ __device__ __forceinline__ void put16_local(uint8_t* act, int r, int gc, const f
   *reinterpret_cast<uint4*>(pan + panel_offset(r, j + 1)) = hi;
 }
 
+// v = max(v + b, 0), 16 values (b on 16 bytes: slices are multiples of 16 columns).
+__device__ __forceinline__ void bias_relu16(const float* b, float v[16]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 x = reinterpret_cast<const float4*>(b)[i];
+    v[4 * i] = fmaxf(v[4 * i] + x.x, 0.f);
+    v[4 * i + 1] = fmaxf(v[4 * i + 1] + x.y, 0.f);
+    v[4 * i + 2] = fmaxf(v[4 * i + 2] + x.z, 0.f);
+    v[4 * i + 3] = fmaxf(v[4 * i + 3] + x.w, 0.f);
+  }
+}
+
 // Bulk copy (the asynchronous copy engine) of `bytes` of this CTA's shared memory at
 // `src` to the same offset in CTA `cta`, completing its bytes on that CTA's mbarrier `bar`.
 __device__ __forceinline__ void bulk_to_peer(const void* src, uint32_t bytes, uint64_t* bar, uint32_t cta) {
@@ -203,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(copies_landed + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int C = a.csize;
   const int j = (int)cluster_rank();
   const int m0 = (blockIdx.x / C) * kRows;
@@ -237,33 +249,38 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
   }
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // the tile's features, then the weight tiles of this CTA's column slice, layer by
       // layer, chunk by chunk
       const int P0 = panels_of(a.dims[0]);
       mbar_expect_tx(a0_full, P0 * kPanelBytes);
       for (int p = 0; p < P0; ++p) tma_load_2d(act + p * kPanelBytes, &a.act0, a0_full, p * kPanel, m0);
-      int issued = 0;
+      int issued = 0, s = 0;
+      uint32_t ph = 1;
       bool ok = true;
       for (int l = 0; l < a.L && ok; ++l) {
         const int ns = a.dims[l + 1] / C, KP = panels_of(a.dims[l]);
         const int own0 = l == 0 ? 0 : j * (KP / C);   // the K loop's first panel
+        const uint32_t bytes = (uint32_t)(min(kChunk, ns) * kPanel * 2);
+        const CUtensorMap* map = &a.w[l];
+        ok = !*(volatile int*)abort_flag;
         for (int c0 = 0; c0 < ns && ok; c0 += kChunk) {
-          const int nc = min(kChunk, ns - c0);
+          int p = own0;
           for (int i = 0; i < KP; ++i) {
-            const int p = (own0 + i) % KP;
-            const int s = issued % kRing;
-            const uint32_t ph = (issued / kRing) & 1;
-            if (*(volatile int*)abort_flag || !mbar_wait(&empty[s], ph ^ 1)) {
+            if (!mbar_wait(&empty[s], ph)) {
               *(volatile int*)abort_flag = 1;
               atomicExch(err_flag, 21);
               ok = false;
               break;
             }
-            mbar_expect_tx(&full[s], (uint32_t)(min(kChunk, ns) * kPanel * 2));
-            tma_load_2d(ring + s * kTileBytes, &a.w[l], &full[s], p * kPanel, j * ns + c0);
+            mbar_expect_tx(&full[s], bytes);
+            tma_load_2d(ring + s * kTileBytes, map, &full[s], p * kPanel, j * ns + c0);
             ++issued;
-            (void)nc;
+            if (++p == KP) p = 0;
+            if (++s == kRing) {
+              s = 0;
+              ph ^= 1;
+            }
           }
         }
       }
@@ -272,26 +289,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
       if (!mbar_wait(a0_full, 0)) atomicExch(err_flag, 27);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int used = 0;
+    if (elect_one()) {
+      // One thread issues every MMA, and a tile's four MMAs (276 cycles) are accepted no faster
+      // than they run, so whatever else it does per tile adds to them: the panels are taken
+      // source by source with running counters and descriptors (with divisions, a test of the
+      // abort flag and fresh descriptors a tile took 1010 cycles, three times the MMAs).
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
+      const uint64_t act_desc = sw128_desc(smem_u32(act)), ring_desc = sw128_desc(smem_u32(ring));
       for (int l = 0; l < a.L && ok; ++l) {
         const int ns = a.dims[l + 1] / C, KP = panels_of(a.dims[l]);
-        const int pps = l == 0 ? KP : KP / C;   // panels per slice of the input
-        const int own0 = l == 0 ? 0 : j * pps;
-        const uint32_t acc = acc_column(ns, l);
+        const int sources = l == 0 ? 1 : C, pps = KP / sources;   // panels per slice of the input
+        const uint32_t acc = acc_column(ns, l), parity = (uint32_t)(l - 1) & 1u;
         // layer 0: the features by TMA.  Layer l > 0: this CTA's own panels as the epilogue
         // writes them, then each peer's slice when its copies have landed; where this
         // layer's accumulator overlaps the previous one, first the epilogue's last panel
         // (it has read the whole accumulator then).
-        uint32_t have = l == 0 ? 0xFFu : 0u;    // bit p: input panel p is in shared memory
         bool in_ok = true;
         if (l == 0) {
           in_ok = mbar_wait(a0_full, 0);
         } else {
           const int pns = a.dims[l] / C;
           const uint32_t pacc = acc_column(pns, l - 1);
-          if (pacc < acc + ns && acc < pacc + pns) in_ok = mbar_wait(&panel_ready[pps - 1], (l - 1) & 1);
+          if (pacc < acc + ns && acc < pacc + pns) in_ok = mbar_wait(&panel_ready[pps - 1], parity);
         }
         if (*(volatile int*)abort_flag || !in_ok) {
           *(volatile int*)abort_flag = 1;
@@ -301,38 +322,43 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
         fence_async_smem();
         tc_fence_after();
         for (int c0 = 0; c0 < ns && ok; c0 += kChunk) {
-          const uint32_t idesc = idesc_bf16(kRows, min(kChunk, ns - c0));
-          for (int i = 0; i < KP; ++i) {
-            const int p = (own0 + i) % KP;
-            if (!((have >> p) & 1u)) {
-              const int src = p / pps;
-              const bool got = src == j ? mbar_wait(&panel_ready[p - own0], (l - 1) & 1)
-                                        : wait_cluster(&act_from[src], (l - 1) & 1);
-              if (*(volatile int*)abort_flag || !got) {
+          const uint32_t idesc = idesc_bf16(kRows, min(kChunk, ns - c0)), d = tmem + acc + c0;
+          int src = l == 0 ? 0 : j;
+          uint32_t more = 0;   // accumulate
+          for (int n = 0; n < sources && ok; ++n) {
+            uint64_t ad = act_desc + (uint32_t)(src * pps) * (kPanelBytes >> 4);
+            for (int pi = 0; pi < pps; ++pi) {
+              if (l > 0 && c0 == 0 && (n == 0 || pi == 0)) {   // an own panel, a peer's slice
+                if (!(n == 0 ? mbar_wait(&panel_ready[pi], parity) : wait_cluster(&act_from[src], parity))) {
+                  *(volatile int*)abort_flag = 1;
+                  atomicExch(err_flag, 28);
+                  ok = false;
+                  break;
+                }
+                fence_async_smem();
+                tc_fence_after();
+              }
+              if (!mbar_wait(&full[s], ph)) {
                 *(volatile int*)abort_flag = 1;
-                atomicExch(err_flag, 28);
+                atomicExch(err_flag, 24);
                 ok = false;
                 break;
               }
-              fence_async_smem();
               tc_fence_after();
-              have |= src == j ? (1u << p) : (((1u << pps) - 1u) << (src * pps));
-            }
-            const int s = used % kRing;
-            const uint32_t ph = (used / kRing) & 1;
-            if (*(volatile int*)abort_flag || !mbar_wait(&full[s], ph)) {
-              *(volatile int*)abort_flag = 1;
-              atomicExch(err_flag, 24);
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t aa = smem_u32(act + p * kPanelBytes), bb = smem_u32(ring + s * kTileBytes);
+              const uint64_t bd = ring_desc + (uint32_t)s * (kTileBytes >> 4);
 #pragma unroll
-            for (int kk = 0; kk < kPanel / 16; ++kk)
-              umma_bf16(tmem + acc + c0, sw128_desc(aa + kk * 32), sw128_desc(bb + kk * 32), idesc, (i | kk) != 0);
-            umma_commit(&empty[s]);
-            ++used;
+              for (int kk = 0; kk < kPanel / 16; ++kk) {
+                umma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, more);
+                more = 1;
+              }
+              umma_commit(&empty[s]);
+              ad += kPanelBytes >> 4;
+              if (++s == kRing) {
+                s = 0;
+                ph ^= 1;
+              }
+            }
+            if (++src == C) src = 0;
           }
         }
         if (ok) umma_commit(mma_done);
@@ -438,12 +464,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
           const bool two = g + 2 < groups;
           float va[16], vb[16];
           tmem_ld16x2(lane_acc + 16 * g, lane_acc + 16 * (two ? g + 2 : g), va, vb);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) va[i] = fmaxf(va[i] + cb[16 * g + i], 0.f);
+          bias_relu16(cb + 16 * g, va);
           put16_local(act, r, cbase + 16 * g, va);
           if (two) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) vb[i] = fmaxf(vb[i] + cb[16 * (g + 2) + i], 0.f);
+            bias_relu16(cb + 16 * (g + 2), vb);
             put16_local(act, r, cbase + 16 * (g + 2), vb);
           }
           // the panel is read by the copy engine and the tensor core

@@ -255,7 +255,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   if (threadIdx.x == 0) {
     prefetch_map(tmA);
     prefetch_map(tmB);
@@ -303,14 +303,14 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
 
   if (warp == 0) {
     const int early = EARLY ? (KB < STAGES ? KB : STAGES) : 0;
-    if (lane == 0) {
+    if (elect_one()) {
       for (int kb = 0; kb < early; ++kb) {
         mbar_expect_tx(&full[kb], S::kStageBytes);
         load_b(kb);
       }
     }
     enter();
-    if (lane == 0) {
+    if (elect_one()) {
       int issued = 0;
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % STAGES;
@@ -333,7 +333,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
     }
   } else if (warp == 1) {
     enter();
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = idesc_bf16(kBM, BN, A_MN, B_MN);
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % STAGES;

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_fused(const __grid_constant
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       const int P0 = panels_of(a.dims[0]);
       mbar_expect_tx(a0_full, P0 * kPanelBytes);
       for (int p = 0; p < P0; ++p) tma_load_2d(act + p * kPanelBytes, &a.act0, a0_full, p * kPanel, m0);
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_fused(const __grid_constant
       if (!mbar_wait(a0_full, 0)) atomicExch(err_flag, 13);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = mbar_wait(a0_full, 0);
       if (!ok) {
         *(volatile int*)abort_flag = 1;
