@@ -15,18 +15,18 @@
 // Warps: 0 TMA producer (the feature tile, then weight tiles through a 5-stage ring),
 // 1 TMEM allocation and the MMA issuer, 2..9 epilogue: two warps per TMEM lane quarter
 // (one TMEM lane = one element per thread), taking alternate 16-column groups, one 64-column
-// panel of the CTA's slice after the other; 10 the exchange (lane k talks to CTA k): the
-// arrivals at the peers, the slice copies and the receipts, off the epilogue's path.  The layers' biases and the output scaling of
-// this CTA's slices sit in shared memory.  Ordering uses mbarriers only:
+// panel of the CTA's slice after the other; 10 the slice copies and 11 the receipts, one lane
+// per peer, off the epilogue's path and off each other's.  The layers' biases and the output
+// scaling of this CTA's slices sit in shared memory.  Ordering uses mbarriers only:
 //   panel_ready[i] (one arrival per epilogue thread): panel i of this CTA's slice of the
 //       next input is written (a CTA's own panels are free once its own MMAs of the layer
 //       have completed, since only they read them);
 //   act_from[k] (k != own rank): one local arrival carrying the bytes of CTA k's slice,
 //       which CTA k's bulk copies complete;
-//   peers_done (C arrivals): every CTA's MMAs of the current layer have completed, so no
-//       tensor core still reads the panels that the slice copies overwrite, and every
+//   peers_done (C arrivals, each a tensor-core commit multicast to the cluster): every CTA's
+//       MMAs of the current layer have completed, so no tensor core still reads the panels that the slice copies overwrite, and every
 //       earlier slice copy has landed (those MMAs waited for it);
-//   copies_landed (C - 1 arrivals, one from each receiver's exchange warp): this CTA's
+//   copies_landed (C - 1 arrivals, one from each receiver's receipt warp): this CTA's
 //       slice has landed everywhere, so the copy engine no longer reads the panels that
 //       the next slice overwrites.
 // A hidden layer's K loop starts on the CTA's own panels as each is written and then takes
@@ -35,6 +35,11 @@
 // weight tiles stream in the same order.  Where a slice is at most 256 columns, layers
 // alternate between two TMEM accumulators, so the next layer's MMAs may start while the
 // epilogue still reads the last panels of this one.
+// What bounds it: the chain of a layer (MMAs, epilogue, slice copies), not the tensor core,
+// which works a third of the time, nor L2.  4096 elements, 320-512x4-320: about 27 us; the
+// corrected step there 152.5 -> 137.2 us with lighter issue loops, completion announced by the
+// tensor core instead of a thread's remote arrivals, and copies that no longer queue behind
+// the receipts of the layer before.
 // Every wait is bounded (about a second): on expiry a thread sets the error flag and the
 // CTA skips the rest of its work; all threads meet at a final cluster barrier, so that no
 // CTA leaves while a peer may still write into its shared memory.
@@ -64,7 +69,8 @@ constexpr int kRing = 5;
 constexpr int kMaxCluster = 4;
 constexpr int kEpiWarps = 8;                      // two per TMEM lane quarter
 constexpr int kXchgWarp = 2 + kEpiWarps;          // the warp that sends the slices
-constexpr int kThreads = 64 + 32 * kEpiWarps + 32;
+constexpr int kReceiptWarp = kXchgWarp + 1;       // the warp that acknowledges the peers' slices
+constexpr int kThreads = 64 + 32 * kEpiWarps + 64;
 constexpr int kTmemCols = 512;
 constexpr int kActBytes = kMaxPanels * kPanelBytes;
 constexpr int kRingOffset = kActBytes;
@@ -109,6 +115,15 @@ __device__ __forceinline__ uint32_t mapa(uint32_t saddr, uint32_t cta) {
 __device__ __forceinline__ void arrive_remote(uint64_t* bar, uint32_t cta) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(smem_u32(bar), cta))
                : "memory");
+}
+// Arrival, when every MMA issued by this thread has completed, on the mbarrier at the same
+// offset in each CTA of `mask`.
+__device__ __forceinline__ void umma_commit_cluster(uint64_t* bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"(mask)
+      : "memory");
 }
 __device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -362,45 +377,51 @@ __global__ void __launch_bounds__(kThreads, 1) k_forcing_cluster(const __grid_co
           }
         }
         if (ok) umma_commit(mma_done);
+        // every CTA of the cluster hears of it from the tensor core itself
+        if (ok && C > 1 && l + 1 < a.L) umma_commit_cluster(peers_done, (uint16_t)((1u << C) - 1u));
       }
     }
     __syncwarp();
   } else if (warp == kXchgWarp) {
-    if (C > 1) {
-      // per hidden layer: once this CTA's MMAs are done, expect the peers' slices and
-      // announce it to every CTA; once every CTA's are done, copy each panel of this CTA's
-      // slice to every peer as the epilogue finishes it; then tell each peer when its
-      // slice has landed here.  Lane k talks to CTA k (lane i >= 1 copies to CTA j - i),
-      // so the remote operations of one step fly together.
+    // per hidden layer, lane i in [1, C): expect CTA k = j + i's slice; once every CTA's MMAs
+    // are done, copy each panel of this CTA's slice to CTA j - i as the epilogue finishes it
+    // (the first consumer of a slice is the CTA before its owner).  The expected bytes may be
+    // announced after some have arrived: the phase waits for the announcement.
+    if (lane >= 1 && lane < C) {
+      const uint32_t to = (uint32_t)((j - lane + C) % C), from = (uint32_t)((j + lane) % C);
       bool ok = true;
       for (int l = 0; l + 1 < a.L && ok; ++l) {
-        const int ns = a.dims[l + 1] / C, pps = ns / kPanel;
-        const uint32_t slice = (uint32_t)pps * kPanelBytes;
-        ok = mbar_wait(mma_done, l & 1) && !*(volatile int*)abort_flag;
-        if (ok) {
-          if (lane < C && lane != j) mbar_expect_tx(&act_from[lane], slice);
-          __syncwarp();
-          if (lane < C) arrive_remote(peers_done, (uint32_t)lane);
-          ok = wait_cluster(peers_done, l & 1) && !*(volatile int*)abort_flag;
-        }
-        ok = __all_sync(0xffffffffu, ok);
+        const int pps = a.dims[l + 1] / C / kPanel;
+        if (l > 0) ok = wait_cluster(&act_from[from], (l - 1) & 1);   // the phase before has completed
+        if (ok) mbar_expect_tx(&act_from[from], (uint32_t)pps * kPanelBytes);
+        ok = ok && wait_cluster(peers_done, l & 1);
         for (int pi = 0; pi < pps && ok; ++pi) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&panel_ready[pi], l & 1) && !*(volatile int*)abort_flag);
-          if (ok && lane >= 1 && lane < C)
-            bulk_to_peer(act + (j * pps + pi) * kPanelBytes, kPanelBytes, &act_from[j], (uint32_t)((j - lane + C) % C));
+          ok = mbar_wait(&panel_ready[pi], l & 1);
+          if (ok) bulk_to_peer(act + (j * pps + pi) * kPanelBytes, kPanelBytes, &act_from[j], to);
         }
-        if (ok && lane >= 1 && lane < C) {
-          const uint32_t k = (uint32_t)((j + lane) % C);
-          ok = wait_cluster(&act_from[k], l & 1);
-          if (ok) arrive_remote(copies_landed, k);
-        }
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok && lane == 0) {
+        if (!ok || *(volatile int*)abort_flag) {
           *(volatile int*)abort_flag = 1;
           atomicExch(err_flag, 26);
+          ok = false;
         }
       }
     }
+    __syncwarp();
+  } else if (warp == kReceiptWarp) {
+    // lane i in [1, C) tells CTA k = j + i that its slice has landed here
+    if (lane >= 1 && lane < C) {
+      const uint32_t k = (uint32_t)((j + lane) % C);
+      bool ok = true;
+      for (int l = 0; l + 1 < a.L && ok; ++l) {
+        ok = wait_cluster(&act_from[k], l & 1) && !*(volatile int*)abort_flag;
+        if (ok) arrive_remote(copies_landed, k);
+      }
+      if (!ok) {
+        *(volatile int*)abort_flag = 1;
+        atomicExch(err_flag, 30);
+      }
+    }
+    __syncwarp();
   } else {
     // epilogue: warp w owns TMEM lanes (rows) 32 (w % 4) .. +31 and the 16-column groups
     // g of each slice with g % 2 == half
