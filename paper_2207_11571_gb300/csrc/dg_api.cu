@@ -265,7 +265,7 @@ static int diag_parse(dg_ctx* c, const double* r, bool with_rhs, bool with_ref, 
   std::memcpy(&err, r + kDiagLen, sizeof(int));
   if (err) {
     DG_CUDA(cudaMemset(c->err_dev, 0, sizeof(int)));
-    return fail(DG_ERR_TIMEOUT, "a bounded wait in the streamed flux kernel expired (its results are invalid)");
+    return fail(DG_ERR_TIMEOUT, "a bounded wait in an operator kernel expired (its results are invalid)");
   }
   const double vol = 8.0 * M_PI * M_PI * M_PI;
   std::memset(out, 0, sizeof(*out));

@@ -1,24 +1,13 @@
-// TMA bulk copies (cp.async.bulk) and bounded mbarrier waits.
+// A shared-memory mbarrier and bounded waits on it.
 #pragma once
 
 namespace dgnn {
 
-// TMA bulk copies (cp.async.bulk, global -> shared, completion counted in bytes on an
-// mbarrier).  Addresses 16-byte aligned, size a multiple of 16 bytes.
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bulk_bar_init(unsigned long long* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
 }
 __device__ __forceinline__ void bulk_bar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void bulk_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
 // Bounded wait for the phase with the given parity (about a second); false on expiry.
 __device__ __forceinline__ bool bulk_wait(unsigned long long* bar, unsigned parity) {
   const long long t0 = clock64();
@@ -35,6 +24,5 @@ __device__ __forceinline__ bool bulk_wait(unsigned long long* bar, unsigned pari
     if (clock64() - t0 > 2000000000LL) return false;
   }
 }
-
 
 }  // namespace dgnn

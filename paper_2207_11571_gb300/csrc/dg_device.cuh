@@ -131,54 +131,4 @@ __device__ __forceinline__ void viscous_flux(const T vis[9], const T v[3], int d
   f[4] = v[0] * t0 + v[1] * t1 + v[2] * t2 + vis[6 + d];
 }
 
-// Roe dissipation |A~| (qR - qL) in direction +e_d between the left state sL and the
-// right state sR, with Roe-averaged velocity, enthalpy and sound speed; acoustic waves
-// (Vn -/+ c), entropy wave and shear waves (Vn).  The Roe flux is
-// F* = (f(qL) + f(qR))/2 - diss/2.
-template <typename T>
-__device__ __forceinline__ void roe_dissipation(const T sL[5], const Prim<T>& wL, const T sR[5], const Prim<T>& wR,
-                                                int d, T gm1, T Hc, T diss[5]) {
-  const T HL = (sL[4] + wL.pp + Hc) * wL.ir, HR = (sR[4] + wR.pp + Hc) * wR.ir;
-  const T sqL = dsqrt(wL.rho), sqR = dsqrt(wR.rho);
-  const T wden = drcp(sqL + sqR);
-  const T ut[3] = {(sqL * wL.v[0] + sqR * wR.v[0]) * wden, (sqL * wL.v[1] + sqR * wR.v[1]) * wden,
-                   (sqL * wL.v[2] + sqR * wR.v[2]) * wden};
-  const T Ht = (sqL * HL + sqR * HR) * wden;
-  const T ke = T(0.5) * (ut[0] * ut[0] + ut[1] * ut[1] + ut[2] * ut[2]);
-  const T c2 = gm1 * (Ht - ke);
-  const T c = dsqrt(c2);
-  const T rt = sqL * sqR;
-  const T Vn = ut[d];
-  const T dr = sR[0] - sL[0], dp = wR.pp - wL.pp;
-  const T du[3] = {wR.v[0] - wL.v[0], wR.v[1] - wL.v[1], wR.v[2] - wL.v[2]};
-  const T dVn = du[d];
-  const T inv2c2 = T(0.5) * drcp(c2);
-  const T a1 = (dp - rt * c * dVn) * inv2c2;
-  const T a2 = dr - dp * (T(2) * inv2c2);
-  const T a5 = (dp + rt * c * dVn) * inv2c2;
-  const T l1 = fabs(Vn - c) * a1, l2 = fabs(Vn), l5 = fabs(Vn + c) * a5;
-  diss[0] = l1 + l2 * a2 + l5;
-  T shear_dot = T(0);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T sh = (i == d) ? T(0) : rt * du[i];  // shear wave strength (normal part removed)
-    shear_dot += ut[i] * sh;
-    diss[1 + i] = (l1 + l5) * ut[i] + l2 * (a2 * ut[i] + sh);
-  }
-  diss[1 + d] += (l5 - l1) * c;
-  diss[4] = l1 * (Ht - c * Vn) + l2 * (a2 * ke + shear_dot) + l5 * (Ht + c * Vn);
-}
-
-// Roe flux F* = (f(qL) + f(qR))/2 - |A~|(qR - qL)/2 in direction +e_d.
-template <typename T>
-__device__ __forceinline__ void roe_flux(const T sL[5], const Prim<T>& wL, const T sR[5], const Prim<T>& wR, int d,
-                                         T gm1, T Hc, T F[5]) {
-  T fL[5], fR[5], diss[5];
-  euler_flux(sL, wL, Hc, d, fL);
-  euler_flux(sR, wR, Hc, d, fR);
-  roe_dissipation(sL, wL, sR, wR, d, gm1, Hc, diss);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) F[v] = T(0.5) * (fL[v] + fR[v] - diss[v]);
-}
-
 }  // namespace dgnn

@@ -1,6 +1,6 @@
 // The corrective forcing s(q) of an RK stage (Sec. 2.2, Fig. 2; Eq. 4): every layer of
 // the network on the tcgen05 tensor cores in one launch, from the bf16 element features to
-// the unscaled forcing in the layout the flux kernel adds to the operator.
+// the unscaled forcing in the layout phase B adds to the operator.
 //
 // A cluster of C CTAs (C = 1, 2 or 4) carries one tile of 128 elements (MMA M = 128)
 // through the network.  Each CTA loads the tile's features by TMA.  CTA j of the cluster
