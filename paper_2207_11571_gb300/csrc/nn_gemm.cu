@@ -273,24 +273,24 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  auto load_a = [&](int kb) {
-    uint8_t* a = base + (kb % STAGES) * S::kStageBytes;
+  auto load_a = [&](int kb, int s) {
+    uint8_t* a = base + s * S::kStageBytes;
     const int k0 = (kb0 + kb) * kBK;
     if (A_MN) {
 #pragma unroll
-      for (int i = 0; i < kBM / kBK; ++i) tma_load_2d(a + i * kBlk, tmA, &full[kb % STAGES], m0 + i * kBK, k0);
+      for (int i = 0; i < kBM / kBK; ++i) tma_load_2d(a + i * kBlk, tmA, &full[s], m0 + i * kBK, k0);
     } else {
-      tma_load_2d(a, tmA, &full[kb % STAGES], k0, m0);
+      tma_load_2d(a, tmA, &full[s], k0, m0);
     }
   };
-  auto load_b = [&](int kb) {
-    uint8_t* b = base + (kb % STAGES) * S::kStageBytes + S::kABytes;
+  auto load_b = [&](int kb, int s) {
+    uint8_t* b = base + s * S::kStageBytes + S::kABytes;
     const int k0 = (kb0 + kb) * kBK;
     if (B_MN) {
 #pragma unroll
-      for (int i = 0; i < BN / kBK; ++i) tma_load_2d(b + i * kBlk, tmB, &full[kb % STAGES], n0 + i * kBK, k0);
+      for (int i = 0; i < BN / kBK; ++i) tma_load_2d(b + i * kBlk, tmB, &full[s], n0 + i * kBK, k0);
     } else {
-      tma_load_2d(b, tmB, &full[kb % STAGES], k0, n0);
+      tma_load_2d(b, tmB, &full[s], k0, n0);
     }
   };
 
@@ -306,26 +306,29 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
     if (elect_one()) {
       for (int kb = 0; kb < early; ++kb) {
         mbar_expect_tx(&full[kb], S::kStageBytes);
-        load_b(kb);
+        load_b(kb, kb);
       }
     }
     enter();
     if (elect_one()) {
-      int issued = 0;
+      int issued = 0, s = 0;
+      uint32_t ph = 1;
       for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % STAGES;
         if (kb >= early) {
-          const uint32_t ph = (kb / STAGES) & 1;
-          if (*(volatile int*)abort_flag || !mbar_wait(&empty[s], ph ^ 1)) {
+          if (!mbar_wait(&empty[s], ph)) {
             *(volatile int*)abort_flag = 1;
             atomicExch(err_flag, 1);
             break;
           }
           mbar_expect_tx(&full[s], S::kStageBytes);
-          load_b(kb);
+          load_b(kb, s);
         }
-        load_a(kb);
+        load_a(kb, s);
         issued = kb + 1;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1;
+        }
       }
       // drain: every issued copy must land before the CTA exits (bounded)
       for (int kb = (issued > STAGES ? issued - STAGES : 0); kb < issued; ++kb)
@@ -335,23 +338,35 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* tmA, const CUtensor
     enter();
     if (elect_one()) {
       constexpr uint32_t idesc = idesc_bf16(kBM, BN, A_MN, B_MN);
+      // running stage and descriptors: what the issuing thread does besides adds to each slice
+      constexpr uint32_t kStep = 32 >> 4, kStepMn = 2048 >> 4;   // 16 K values: 32 bytes of a row, 16 rows of 128 bytes
+      const uint32_t a0 = smem_u32(base), b0 = a0 + S::kABytes;
+      const uint64_t ad0 = A_MN ? sw128_desc_mn(a0, kBlk) : sw128_desc(a0);
+      const uint64_t bd0 = B_MN ? sw128_desc_mn(b0, kBlk) : sw128_desc(b0);
+      uint64_t ad = ad0, bd = bd0;
+      int s = 0;
+      uint32_t ph = 0, more = 0;
       for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (kb / STAGES) & 1;
-        if (*(volatile int*)abort_flag || !mbar_wait(&full[s], ph)) {
+        if (!mbar_wait(&full[s], ph)) {
           *(volatile int*)abort_flag = 1;
           atomicExch(err_flag, 3);
           break;
         }
         tc_fence_after();
-        const uint32_t a = smem_u32(base + s * S::kStageBytes);
-        const uint32_t b = a + S::kABytes;
-        // 16 K values per instruction: 32 bytes along a K-contiguous row, or 16 rows of 128 bytes
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk)
-          umma_bf16(tmem, A_MN ? sw128_desc_mn(a + kk * 2048, kBlk) : sw128_desc(a + kk * 32),
-                    B_MN ? sw128_desc_mn(b + kk * 2048, kBlk) : sw128_desc(b + kk * 32), idesc, (kb | kk) != 0);
+        for (int kk = 0; kk < kBK / 16; ++kk) {
+          umma_bf16(tmem, ad + kk * (A_MN ? kStepMn : kStep), bd + kk * (B_MN ? kStepMn : kStep), idesc, more);
+          more = 1;
+        }
         umma_commit(&empty[s]);
+        ad += S::kStageBytes >> 4;
+        bd += S::kStageBytes >> 4;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1;
+          ad = ad0;
+          bd = bd0;
+        }
       }
       umma_commit(done);  // fires when every MMA issued above has completed
     }
