@@ -60,7 +60,7 @@ cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_
 
 cudaError_t launch_state(const dg_ctx* c, const double* q, bool* done, cudaStream_t st) {
   *done = false;
-  return c->opts.precision == DG_PREC_FP32 && !c->geom.split ? state_f32(c, q, done, st) : cudaSuccess;
+  return c->opts.precision == DG_PREC_FP32 ? state_f32(c, q, done, st) : cudaSuccess;
 }
 
 cudaError_t launch_surface(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, int mode, const RkStage& rk,

@@ -481,7 +481,7 @@ __host__ __device__ constexpr size_t volume_smem_bytes(int E, int faces, bool sp
 // SRC 0: the stage state is formed from the FP64 state q and written to qf; SRC 1: it is
 // read from qf.  CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the
 // external faces, internal faces take the neighbour's values from the own tile.  FEAT:
-// also write the forcing network's input features (C.feat).  SPLIT: the Euler part of the
+// also write the forcing network's input features (C.feat; FP64, P = 3).  SPLIT: the Euler part of the
 // volume term in the kinetic-energy-preserving split form, 2 sum_m D_im F#(q_i, q_m) along
 // each line with Pirozzoli's two-point flux F# (mass flux {rho}{v_d}; momentum m {v_j} +
 // {p'} delta_jd; energy m {H}), from a tile of primitives; the viscous part keeps the
@@ -570,9 +570,7 @@ __device__ __forceinline__ void volume_block(int blk, const double* __restrict__
         const int slot = v - C.feat.first_var;
         if (slot < 0 || slot >= C.feat.n_vars) continue;
         const int f = slot * np + node;
-        float x;
-        if constexpr (sizeof(T) == 4) x = (float(s[v]) - C.feat.shift32[f]) / C.feat.sd[f];
-        else x = d2f_rn(double(s[v]) - C.feat.mean64[f]) / C.feat.sd[f];
+        const float x = d2f_rn(double(s[v]) - C.feat.mean64[f]) / C.feat.sd[f];
         fo[slot * np] = __float2bfloat16_rn(x);
       }
     }
@@ -1641,21 +1639,15 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
         rk_stage1(rk, R[c], x1[c], d1, s2);
         a.dlt[o + c * ns] = float(d1);
         a.y[o + c * ns] = s2;
-        if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s2);
       } else if (MODE == 3) {
         T w, s3;
         rk_stage2(rk, R[c], x1[c], g1[c], w, s3);
         a.x[o + c * ns] = s3;
-        if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s3);
         a.dlt[o + c * ns] = float(w);
       } else {
         const double qn = q1[c] + f2d(float(rk_stage3(rk, R[c], g1[c])));
         a.q[c * C.N + g] = qn;
-        if (MODE == 5) {
-          const T s1 = shifted(qn, c, C);
-          a.y[o + c * ns] = s1;
-          if constexpr (FEAT) feature_store(C.feat, e, np, node, c, s1);
-        }
+        if (MODE == 5) a.y[o + c * ns] = shifted(qn, c, C);
       }
     }
   }
@@ -1663,7 +1655,7 @@ __device__ __forceinline__ void surface_block(int blk, int E, const SurfArgs<T>&
 }
 
 // E elements per block (kCubeElems with CUBE), THREADS threads.  FEAT: also writes the network
-// features of the stage state it forms (MODES 2, 3, 5).
+// features of the stage state it forms (MODES 2, 3, 5; P = 3).
 template <int P, typename T, int MODE, int E, int THREADS, bool CUBE, bool FEAT>
 __global__ void __launch_bounds__(THREADS, surf_min_blocks(THREADS, sizeof(T)))
 k_surface(SurfArgs<T> a, Forcing fc, const OpConst<T> C, RkArgs<T> rk) {

@@ -114,13 +114,16 @@ cudaError_t volume_launch(const dg_ctx* c, const double* q, cudaStream_t st) {
                     static_cast<T*>(c->rv), static_cast<T*>(c->vt), make_const<T>(c));
 }
 
-// With a forcing network a launch that forms the state writes its features, and one that
-// reads it (the features are then written with it) may run beside the network.
+// With a forcing network (features at P = 3, see nn_phase_a_features) an FP64 launch writes
+// the features of the state it forms; an FP32 launch, whose state was formed with its
+// features before, runs beside the network.
 template <int P, typename T, int SRC, bool CUBE, bool SPLIT>
 cudaError_t volume_shape(const dg_ctx* c, const double* q, cudaStream_t st) {
-  constexpr bool forms = SRC == 0;
-  if (forms ? c->feat_out.out != nullptr : c->beside_forcing)
-    return volume_launch<P, T, SRC, CUBE, forms, SPLIT, !forms>(c, q, st);
+  constexpr bool f64 = std::is_same<T, double>::value;
+  if constexpr (P == 3 && (f64 || SRC == 1)) {
+    if (f64 ? c->feat_out.out != nullptr : c->beside_forcing)
+      return volume_launch<P, T, SRC, CUBE, f64, SPLIT, !f64>(c, q, st);
+  }
   return volume_launch<P, T, SRC, CUBE, false, SPLIT, false>(c, q, st);
 }
 
@@ -202,7 +205,7 @@ SurfArgs<T> surf_args(const dg_ctx* c, double* q, double* dqdt) {
 template <int P, typename T, int MODE, int E, int THREADS, bool CUBE, bool FEAT = false>
 cudaError_t surface_launch(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, const RkArgs<T>& rk,
                            cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value && !FEAT && (MODE == 2 || MODE == 3 || MODE == 5)) {
+  if constexpr (P == 3 && std::is_same<T, float>::value && !FEAT && (MODE == 2 || MODE == 3 || MODE == 5)) {
     if (c->feat_out.out) return surface_launch<P, T, MODE, E, THREADS, CUBE, true>(c, q, dqdt, f, rk, st);
   }
   const size_t smem = surface_smem_bytes<P, T>(E);

@@ -512,7 +512,9 @@ static int sm_count() {
 
 bool nn_phase_a_features(const nn_model* m, const dg_ctx* c, FeatureOut* out) {
   const int feat = m->d.n_vars * c->np;
-  if (m->fused != NN_INFER_CLUSTER || c->nel > m->d.max_batch || m->d.n_in != feat || feat != m->pad[0]) return false;
+  // whole 64-column panels of at most 512 features: P = 3 (192 or 320) alone has them
+  if (c->P != 3 || m->fused != NN_INFER_CLUSTER || c->nel > m->d.max_batch || m->d.n_in != feat || feat != m->pad[0])
+    return false;
   if (forcing_cluster_size(m->dims, m->L, c->nel, sm_count()) <= 0) return false;
   if (c->opts.precision == DG_PREC_FP32 && ensure_shift(const_cast<nn_model*>(m), c) != DG_OK) return false;
   out->out = m->act[0];

@@ -89,8 +89,9 @@ def test_phase_b_blocks_of_every_size_give_the_same_bits(dg, K, P, prec):
         dg.dg_batch_destroy(b)
 
 
-@pytest.mark.parametrize("K,P,first,nv", [(6, 3, 0, 5), (5, 3, 1, 3), (6, 2, 0, 5), (4, 5, 1, 3)])
-def test_corrected_steps_in_one_call_equal_single_steps_and_one_rhs(dg, K, P, first, nv):
+@pytest.mark.parametrize("K,P,first,nv,split", [(6, 3, 0, 5, 0), (5, 3, 1, 3, 0), (5, 3, 0, 5, 1), (6, 2, 0, 5, 0),
+                                                (4, 5, 1, 3, 0)])
+def test_corrected_steps_in_one_call_equal_single_steps_and_one_rhs(dg, K, P, first, nv, split):
     """The network runs ahead of phase A where the stage state and its features exist: within a
     call phase B writes both, at the start of a call the state pass (P = 3) or phase A does.
     The same features, so the same bits; and the forced dq/dt of a call on its own agrees
@@ -98,7 +99,7 @@ def test_corrected_steps_in_one_call_equal_single_steps_and_one_rhs(dg, K, P, fi
     from paper_2207_11571_gb300 import nn
     N, feat = K ** 3 * (P + 1) ** 3, nv * (P + 1) ** 3
     dims = [feat, 64, 64, feat]
-    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=1)
+    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=1, volume_flux=split)
     net = nn.nn_create(feat, feat, 64, 2, first, nv, K ** 3, inputs.uniform_draws(dims, 3))
     try:
         # a forcing of order 0.1: larger ones drive the density negative within the steps
