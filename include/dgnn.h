@@ -196,9 +196,9 @@ int dg_batch_member(dg_batch* batch, int i, dg_ctx** out);
  * pointers, dt values or elements-per-block change) and replayed nsteps times on stream;
  * the call must then not be made while that stream is being captured.  With
  * DG_BATCH_PERSISTENT each RK stage of every member, of every order, is one cooperative
- * launch whose blocks walk the gradient phase of all members, meet at a grid barrier
+ * launch whose blocks walk phase A of all members, meet at a grid barrier
  * (a bounded wait: on expiry the first member's error flag is set, reported by its
- * dg_diagnostics as DG_ERR_TIMEOUT) and walk the flux phase; the per-element arithmetic
+ * dg_diagnostics as DG_ERR_TIMEOUT) and walk phase B; the per-element arithmetic
  * is that of dg_rk3_step. */
 int dg_batch_rk3_step(dg_batch* batch, double* const* q, const double* dt, int nsteps, int flags,
                       void* stream);

@@ -29,10 +29,10 @@
 // Every component of a node or face node is then at a compile-time offset from one address.
 //
 // Phase A: a block owns E consecutive elements (or, at P <= 3 on even K, a 2 x 2 x 2 cube
-// of elements whose twelve internal faces need no halo), one thread per node.  Phase B: a
-// block owns surf_elems(P) elements; its interface terms are dense work items, one per
-// (element, face, face node), so that every lane does useful Roe work, and its nodes add
-// the lifted results in a fixed order.  All constants arrive in the operator precision
+// of elements whose twelve internal faces need no halo), one thread per node (P = 3 in FP32:
+// per row of four).  Phase B: a block owns a few elements, the more the larger the mesh; its
+// interface terms are dense work items, one per (element, face, face node), so that every
+// lane does useful Roe work, and its nodes add the lifted results in a fixed order.  All constants arrive in the operator precision
 // (OpConst): no FP64 arithmetic or conversion runs per node except where the FP64 state
 // is read or written.
 #pragma once
@@ -46,9 +46,9 @@
 namespace dgnn {
 
 // Programmatic dependent launch between the operator's launches: a kernel waits until its
-// predecessor in the stream has completed and its writes are visible, then lets its
-// successor be launched (which happens once every block of this grid has got here, i.e.
-// in its last wave), so the next launch overlaps this one's tail.  Kernels launched
+// predecessor in the stream has completed and its writes are visible, and lets its
+// successor be launched (which happens once every block of this grid has said so: where
+// along a block that pays is in make_const), so the next launch's start overlaps its tail.  Kernels launched
 // without the attribute pass the wait at once.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
