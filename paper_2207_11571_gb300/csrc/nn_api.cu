@@ -259,16 +259,20 @@ __global__ void __launch_bounds__(256) k_params(const __grid_constant__ ParamTab
     if (kMode == kAdam) {
       if (row == 0 && c < S.count) gi = S.g[c];
     } else {
-      float* part = reinterpret_cast<float*>(sh);
-      float a = 0.f;
-      if (c < S.count) {
+      // partial sums z, z + 32, .. for each z < 32, then z = 0 .. 31: a fixed order
+      __shared__ float part[32][32];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float a = 0.f;
+        if (c < S.count) {
 #pragma unroll 4
-        for (int z = row; z < S.parts; z += 8) a += S.part[z * S.stride + c];
+          for (int z = row + 8 * u; z < S.parts; z += 32) a += S.part[z * S.stride + c];
+        }
+        part[row + 8 * u][threadIdx.x & 31] = a;
       }
-      part[threadIdx.x] = a;
       __syncthreads();
       if (row == 0)
-        for (int k = 0; k < 8; ++k) gi += part[k * 32 + threadIdx.x];
+        for (int k = 0; k < 32; ++k) gi += part[k][threadIdx.x];
       if (row == 0 && c < S.count) S.g[c] = gi;
     }
     if (kMode != kReduce && row == 0 && c < S.count) {

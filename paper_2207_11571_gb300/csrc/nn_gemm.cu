@@ -69,32 +69,55 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
 }
 
 // Sum over the warp's 32 lanes (rows) of each of 16 columns: lanes 2 c and 2 c + 1 return
-// column c.  Halves of the columns are exchanged at each step, 16 shuffles in all; the order
-// of the additions is fixed.
+// column c.  Halves of the columns are exchanged at each step (24 shuffles).  The order of
+// the additions is fixed: rows r, r + 8, r + 16, r + 24, then r = 0 .. 7.
 __device__ __forceinline__ float warp_column_sums(const float v[16], int lane) {
-  float a[8], b[4], c[2];
+  float a[2][8], s[4], b[2][2], c[4], d[8];   // a: rows r, r + 16 (r < 16)
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const bool up = lane & 16;
-    const float keep = up ? v[8 + i] : v[i], give = up ? v[i] : v[8 + i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    const float keep = up ? v[8 + i] : v[i], got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[8 + i], 16);
+    a[0][i] = up ? got : keep;
+    a[1][i] = up ? keep : got;
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const bool up = lane & 8;
-    const float keep = up ? a[4 + i] : a[i], give = up ? a[i] : a[4 + i];
-    b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    float lo[2], hi[2];   // rows r (+ 16), r + 8 (+ 16), r < 8
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float keep = up ? a[k][4 + i] : a[k][i];
+      const float got = __shfl_xor_sync(0xffffffffu, up ? a[k][i] : a[k][4 + i], 8);
+      lo[k] = up ? got : keep;
+      hi[k] = up ? keep : got;
+    }
+    s[i] = ((lo[0] + hi[0]) + lo[1]) + hi[1];
   }
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < 2; ++i) {   // b[k]: r % 4 + 4 k
     const bool up = lane & 4;
-    const float keep = up ? b[2 + i] : b[i], give = up ? b[i] : b[2 + i];
-    c[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    const float keep = up ? s[2 + i] : s[i], got = __shfl_xor_sync(0xffffffffu, up ? s[i] : s[2 + i], 4);
+    b[0][i] = up ? got : keep;
+    b[1][i] = up ? keep : got;
   }
-  const bool up = lane & 2;
-  const float keep = up ? c[1] : c[0], give = up ? c[0] : c[1];
-  const float s = keep + __shfl_xor_sync(0xffffffffu, give, 2);
-  return s + __shfl_xor_sync(0xffffffffu, s, 1);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {   // c[2 k + h]: r % 2 + 2 h + 4 k
+    const bool up = lane & 2;
+    const float keep = up ? b[k][1] : b[k][0], got = __shfl_xor_sync(0xffffffffu, up ? b[k][0] : b[k][1], 2);
+    c[2 * k] = up ? got : keep;
+    c[2 * k + 1] = up ? keep : got;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool up = lane & 1;
+    const float got = __shfl_xor_sync(0xffffffffu, c[k], 1);
+    d[2 * k] = up ? got : c[k];
+    d[2 * k + 1] = up ? c[k] : got;
+  }
+  float t = d[0];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) t += d[k];
+  return t;
 }
 
 // 16 consecutive floats, as vectors where the address allows (vec); 0 past `left` of them.
