@@ -807,16 +807,15 @@ __device__ __forceinline__ void row_read(const float* p, float v[4]) {
   v[2] = a.z;
   v[3] = a.w;
 }
-// d[0] own + sum_{m = 1..3} d[m] row(at[m - 1]) of the rows at base + at[...]: the thread's own
-// row of a line and the three others.
-__device__ __forceinline__ void rows_contract(const float own[4], const float* base, const int at[3],
-                                              const f32x2 d[4], float out[4]) {
+// sum_m d[m] row_m over a line of four rows: row 0 the thread's own, the others at base + at[...]
+// (m: the exclusive-or of their positions along the line).  Farthest row first, own row last:
+// of the orders that an exclusive-or gives, the one no less accurate than along the line.
+__device__ __forceinline__ void rows_contract(const Row& own, const float* base, const int at[3], const f32x2 d[4],
+                                              float out[4]) {
   Row acc{0ull, 0ull};
-  fma2(acc.lo, d[0], pack2(own[0], own[1]));
-  fma2(acc.hi, d[0], pack2(own[2], own[3]));
 #pragma unroll
-  for (int m = 1; m < 4; ++m) {
-    const Row r = row_load(base + at[m - 1]);
+  for (int m = 3; m >= 0; --m) {
+    const Row r = m ? row_load(base + at[m - 1]) : own;
     fma2(acc.lo, d[m], r.lo);
     fma2(acc.hi, d[m], r.hi);
   }
@@ -1011,8 +1010,9 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
     }
     G[0][a][0] = fma_(-lift, UL[a] - U[a][0], G[0][a][0]);
     G[0][a][3] = fma_(lift, UR[a] - U[a][3], G[0][a][3]);
-    rows_contract(U[a], sU + a * 64, yat, Dy, G[1][a]);
-    rows_contract(U[a], sU + a * 64, zat, Dz, G[2][a]);
+    const Row own{pack2(U[a][0], U[a][1]), pack2(U[a][2], U[a][3])};
+    rows_contract(own, sU + a * 64, yat, Dy, G[1][a]);
+    rows_contract(own, sU + a * 64, zat, Dz, G[2][a]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       G[1][a][i] = mul_(C.s2h, G[1][a][i]);
@@ -1139,40 +1139,42 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
         }
       } else {
         row_store(sF + (5 * (d - 1) + c) * 64 + 4 * r, F[c]);
-        if (c < 4) {   // the own row's share now, the others' after the exchange
-          float own, other;
-          unpack2(d == 1 ? Dy[0] : Dz[0], own, other);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h * own, F[c][i], R[c][i]);
-        }
       }
     }
   }
   __syncwarp(half);
+  // Each line is summed before it is scaled and added: D's large entries make every partial
+  // sum several times the derivative, and R must not be rounded at that size.  The energy
+  // flux goes relative to the own row, as along x.
   float* re = rv + (size_t)e * state_record(4) + 4 * r;
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    Row acc{0ull, 0ull}, y0, z0;
-    if (c == 4) {   // the energy flux relative to the own row, as above
-      y0 = row_load(sF + c * 64 + 4 * r);
-      z0 = row_load(sF + (5 + c) * 64 + 4 * r);
-    }
+    const float* fy = sF + c * 64;
+    const float* fz = fy + 5 * 64;
+    const Row y0 = row_load(fy + 4 * r), z0 = row_load(fz + 4 * r);
+    if (c == 4) {
+      Row acc{0ull, 0ull};
 #pragma unroll
-    for (int m = 1; m < 4; ++m) {
-      Row y = row_load(sF + c * 64 + yat[m - 1]), z = row_load(sF + (5 + c) * 64 + zat[m - 1]);
-      if (c == 4) {
-        y = Row{line_sub(y.lo, y0.lo), line_sub(y.hi, y0.hi)};
-        z = Row{line_sub(z.lo, z0.lo), line_sub(z.hi, z0.hi)};
+      for (int m = 1; m < 4; ++m) {
+        const Row y = row_load(fy + yat[m - 1]), z = row_load(fz + zat[m - 1]);
+        fma2(acc.lo, Dy[m], line_sub(y.lo, y0.lo));
+        fma2(acc.hi, Dy[m], line_sub(y.hi, y0.hi));
+        fma2(acc.lo, Dz[m], line_sub(z.lo, z0.lo));
+        fma2(acc.hi, Dz[m], line_sub(z.hi, z0.hi));
       }
-      fma2(acc.lo, Dy[m], y.lo);
-      fma2(acc.hi, Dy[m], y.hi);
-      fma2(acc.lo, Dz[m], z.lo);
-      fma2(acc.hi, Dz[m], z.hi);
-    }
-    float g[4];
-    row_unpack(acc, g);
+      float g[4];
+      row_unpack(acc, g);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
+      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
+    } else {
+      float g[4];
+      rows_contract(y0, fy, yat, Dy, g);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
+      rows_contract(z0, fz, zat, Dz, g);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
+    }
     row_store(re + c * 64, R[c]);
   }
 }
