@@ -309,82 +309,73 @@ __host__ __device__ constexpr bool use_lines(int P) {
 __host__ __device__ constexpr int line_row(int n) { return n | 1; }
 __host__ __device__ constexpr int line_nodes(int n) { return line_row(n) * n * n; }
 
-// The derivative matrix changes sign when rows and columns are reversed, D[P-i][P-m] =
-// -D[i][m], so a line's derivative splits into the sums and differences of its mirrored
-// values: with e_m = f_m + f_{P-m}, o_m = f_m - f_{P-m},
-//   E_i = sum_m (D[i][m] + D[i][P-m])/2 e_m (+ D[i][c] f_c),  O_i = sum_m (D[i][m] - D[i][P-m])/2 o_m,
-//   out_i = O_i + E_i,  out_{P-i} = O_i - E_i,  m < n/2, c the middle node of an odd n.
-// That is about half the multiply-adds and half the matrix entries.  The energy flux has a
-// large common part at low Mach numbers, whose rounding the sums e_m would double; D
-// annihilates constants, so its lines (REF) are taken relative to a node r of the line,
-// e_m = (f_m - f_r) + (f_{P-m} - f_r), with r = c for an odd n and n/2 - 1 for an even one
-// (16^3/P8 RK3 step against 64 bits: 4.6e-10 as a plain sum, 5.7e-10 without r, 4.3e-10 with).
-// c_D32 holds the entries of every order as duplicated FP32 pairs, in constant memory (one
-// copy per translation unit, filled by upload_const_D on the host before the first launch):
-// row i (i <= n/2): the E entries (n+1)/2, then the O entries n/2.  Read with compile-time
-// indices.
+// c_D32 holds the derivative matrices of every order as duplicated FP32 pairs, row-major, in
+// constant memory (one copy per translation unit, filled by upload_const_D on the host before
+// the first launch), read with compile-time indices.
 __constant__ float2 c_D32[kMaxP + 1][kMaxN1 * kMaxN1];
 
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 line_add(f32x2 a, f32x2 b) { return add2(a, b); }
 __device__ __forceinline__ f32x2 line_sub(f32x2 a, f32x2 b) {   // a - b in one instruction: -1 x b + a
   fma2(a, 0xBF800000BF800000ull, b);
   return a;
 }
-__device__ __forceinline__ float line_add(float a, float b) { return a + b; }
 __device__ __forceinline__ float line_sub(float a, float b) { return a - b; }
+__device__ __forceinline__ float line_neg(float a) { return -a; }
+__device__ __forceinline__ f32x2 line_neg(f32x2 a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ void line_fma(f32x2& acc, float2 d, f32x2 v) { fma2(acc, pack2(d.x, d.y), v); }
 __device__ __forceinline__ void line_fma(float& acc, float2 d, float v) { acc = fmaf(d.x, v, acc); }
 
 // out[node(i)] = sum_m D[i][m] f[node(m)], i = 0..P, for the line of nodes along direction
 // D with tangential index ab; f and out may be the same array (the line's values are all
-// read before any is written, and no other task touches the line).
-template <int P, int D, bool REF, typename V>
+// read before any is written, and no other task touches the line).  D[P-i][P-m] = -D[i][m]:
+// an entry, once read, serves the two mirrored rows.
+//
+// The sums run over the plain values.  The sums and differences f_m +- f_{P-m} would halve
+// the multiply-adds, but they are rounded before D weighs them: the error of dq/dt in density
+// and momenta grew up to 1.6 times (16^3/P8 RK3 step 504 us with them, 518 without).
+//
+// REL: D annihilates constants, so a line may be taken relative to one of its nodes.  The
+// energy flux has a large common part at low Mach numbers, whose rounding the plain sum
+// carries into the result; it goes relative to node 1 in the lower half and P - 1 in the
+// upper, which on a coarse mesh are near enough to every row's own node (one middle node
+// doubled the error of the energy on 2^3 elements at P = 8).
+template <int P, int D, bool REL, typename V>
 __device__ __forceinline__ void line_derivative(const V* f, V* out, int ab) {
-  constexpr int n = P + 1, rs = line_row(n), h = n / 2, he = (n + 1) / 2;
-  constexpr int ne = REF ? h : he;   // the reference is the middle node of an odd n: its entry drops out
+  constexpr int n = P + 1, rs = line_row(n);
   const int a = ab % n, b = ab / n;
   const int base = D == 0 ? rs * (a + n * b) : D == 1 ? a + rs * n * b : a + rs * b;
   constexpr int st = D == 0 ? 1 : D == 1 ? rs : rs * n;
-  V e[ne], o[h];
-  V r = V(0);
-  if (REF) r = f[base + (n & 1 ? h : h - 1) * st];
+  V v[n], u[n];   // the line and its mirror image
 #pragma unroll
-  for (int m = 0; m < h; ++m) {
-    const V x = f[base + m * st], y = f[base + (P - m) * st];
-    if (!REF) e[m] = line_add(x, y);
-    else if (!(n & 1) && m == h - 1) e[m] = line_sub(y, r);   // f_m is the reference itself
-    else e[m] = line_add(line_sub(x, r), line_sub(y, r));
-    o[m] = line_sub(x, y);
+  for (int m = 0; m < n; ++m) v[m] = f[base + m * st];
+#pragma unroll
+  for (int m = 0; m < n; ++m) u[m] = v[P - m];
+  if (REL) {
+    const V r = v[1], s = u[1];
+#pragma unroll
+    for (int m = 0; m < n; ++m) {
+      v[m] = line_sub(v[m], r);
+      u[m] = line_sub(u[m], s);
+    }
   }
-  if (!REF && (n & 1)) e[ne - 1] = f[base + h * st];
 #pragma unroll
-  for (int i = 0; i < h; ++i) {
-    V E = V(0), O = V(0);
+  for (int i = 0; i < (n + 1) / 2; ++i) {
+    V lo = V(0), hi = V(0);
 #pragma unroll
-    for (int m = 0; m < ne; ++m) line_fma(E, c_D32[P][i * n + m], e[m]);
-#pragma unroll
-    for (int m = 0; m < h; ++m) line_fma(O, c_D32[P][i * n + he + m], o[m]);
-    out[base + i * st] = line_add(O, E);
-    out[base + (P - i) * st] = line_sub(O, E);
-  }
-  if (n & 1) {   // the middle row: D[c][P-m] = -D[c][m]
-    V O = V(0);
-#pragma unroll
-    for (int m = 0; m < h; ++m) line_fma(O, c_D32[P][h * n + he + m], o[m]);
-    out[base + h * st] = O;
+    for (int m = 0; m < n; ++m) {
+      if ((m == i && i > 0) || (REL && m == 1)) continue;   // D[i][i] = 0 inside; v[1] = u[1] = 0
+      line_fma(lo, c_D32[P][i * n + m], v[m]);
+      if (2 * i < P) line_fma(hi, c_D32[P][i * n + m], u[m]);
+    }
+    out[base + i * st] = lo;
+    if (2 * i < P) out[base + (P - i) * st] = line_neg(hi);
   }
 }
 
-template <int P, bool REF, typename V>
+template <int P, bool REL, typename V>
 __device__ __forceinline__ void line_derivative_dir(int d, const V* f, V* out, int ab) {
-  if (d == 0) line_derivative<P, 0, REF>(f, out, ab);
-  else if (d == 1) line_derivative<P, 1, REF>(f, out, ab);
-  else line_derivative<P, 2, REF>(f, out, ab);
+  if (d == 0) line_derivative<P, 0, REL>(f, out, ab);
+  else if (d == 1) line_derivative<P, 1, REL>(f, out, ab);
+  else line_derivative<P, 2, REL>(f, out, ab);
 }
 
 template <typename T>

@@ -60,16 +60,7 @@ static cudaError_t upload_const_D() {
   for (int P = 1; P <= kMaxP; ++P) {
     Basis1D b;
     if (build_basis(P, &b) != 0) return cudaErrorInvalidValue;
-    const int n = P + 1, he = (n + 1) / 2;
-    for (int i = 0; i <= P / 2; ++i) {
-      const double* D = b.D + i * n;
-      for (int m = 0; m < n / 2; ++m) {
-        const float s = (float)(0.5 * (D[m] + D[P - m])), d = (float)(0.5 * (D[m] - D[P - m]));
-        h[P][i * n + m] = make_float2(s, s);
-        h[P][i * n + he + m] = make_float2(d, d);
-      }
-      if (n & 1) h[P][i * n + n / 2] = make_float2((float)D[n / 2], (float)D[n / 2]);
-    }
+    for (int i = 0; i < (P + 1) * (P + 1); ++i) h[P][i] = make_float2((float)b.D[i], (float)b.D[i]);
   }
   e = cudaMemcpyToSymbol(c_D32, h, sizeof(h));
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;

@@ -20,6 +20,13 @@ PLAIN_LINES = {
     (16, 3, 1600.0): (2.883e-07, 2.951e-06, 2.952e-06, 1.936e-07, 1.609e-04),
     (8, 3, 30.0): (1.489e-07, 1.560e-06, 1.572e-06, 1.056e-07, 8.185e-05),
     (7, 3, 200.0): (1.290e-07, 1.282e-06, 1.287e-06, 8.647e-08, 7.047e-05),
+    (8, 5, 1600.0): (3.445e-07, 2.960e-06, 3.044e-06, 2.038e-07, 1.745e-04),
+    (8, 5, 30.0): (3.445e-07, 3.320e-06, 3.407e-06, 2.752e-07, 1.749e-04),
+    (8, 6, 30.0): (5.536e-07, 4.604e-06, 4.563e-06, 4.178e-07, 2.404e-04),
+    (6, 7, 30.0): (5.508e-07, 4.284e-06, 4.244e-06, 3.795e-07, 2.283e-04),
+    (6, 8, 1600.0): (5.201e-07, 4.356e-06, 4.326e-06, 3.070e-07, 2.568e-04),
+    (6, 8, 30.0): (5.201e-07, 5.282e-06, 5.247e-06, 4.987e-07, 2.574e-04),
+    (3, 8, 1600.0): (2.670e-07, 2.260e-06, 2.063e-06, 1.536e-07, 1.291e-04),
 }
 
 
