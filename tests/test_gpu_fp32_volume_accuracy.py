@@ -17,6 +17,9 @@ from paper_2207_11571_gb300 import inputs  # noqa: E402
 
 # (K, P, Re) -> RMS error of dq/dt per variable (density, momenta, energy)
 PLAIN_LINES = {
+    (16, 1, 1600.0): (4.687e-08, 6.910e-07, 6.956e-07, 3.659e-08, 2.912e-05),
+    (16, 2, 1600.0): (1.610e-07, 1.683e-06, 1.704e-06, 1.067e-07, 8.823e-05),
+    (12, 4, 1600.0): (3.546e-07, 3.242e-06, 3.223e-06, 2.224e-07, 1.830e-04),
     (16, 3, 1600.0): (2.883e-07, 2.951e-06, 2.952e-06, 1.936e-07, 1.609e-04),
     (8, 3, 30.0): (1.489e-07, 1.560e-06, 1.572e-06, 1.056e-07, 8.185e-05),
     (7, 3, 200.0): (1.290e-07, 1.282e-06, 1.287e-06, 8.647e-08, 7.047e-05),
@@ -39,6 +42,18 @@ def dg():
     return _dg
 
 
+@pytest.fixture(scope="module")
+def measured(dg):
+    """RMS errors of a case, measured once."""
+    seen = {}
+
+    def get(*case):
+        if case not in seen:
+            seen[case] = rms_errors(dg, *case)
+        return seen[case]
+    return get
+
+
 def rms_errors(dg, K, P, Re, eps=1e-3):
     flow, mesh = physics.Flow(Re=Re), dgsem.Mesh(K, P)
     q = dgsem.tgv_state(mesh, flow, inputs.perturbation((5, K ** 3 * (P + 1) ** 3), eps=eps))
@@ -54,6 +69,16 @@ def rms_errors(dg, K, P, Re, eps=1e-3):
 
 
 @pytest.mark.parametrize("K,P,Re", sorted(PLAIN_LINES))
-def test_no_variable_loses_more_than_the_plain_lines(dg, K, P, Re):
-    e = rms_errors(dg, K, P, Re)
+def test_no_variable_loses_more_than_the_plain_lines(measured, K, P, Re):
+    e = measured(K, P, Re)
     assert (e <= 1.05 * np.array(PLAIN_LINES[K, P, Re])).all(), (e, e / PLAIN_LINES[K, P, Re])
+
+
+@pytest.mark.parametrize("K,P,Re", sorted(PLAIN_LINES))
+def test_energy_flux_is_rounded_alike_in_the_volume_and_at_the_faces(measured, K, P, Re):
+    """At Mach 0.1 the energy flux is 250 times its divergence.  Its rounding at a face node
+    enters the volume term and the lifted interface term with opposite signs, as one number;
+    rounded a second way, the error of the energy is 2 to 4 % larger at low order.  1 %: the
+    share of another order of the volume's sums."""
+    e = measured(K, P, Re)[4]
+    assert e <= 1.01 * PLAIN_LINES[K, P, Re][4], (e, e / PLAIN_LINES[K, P, Re][4])
