@@ -1292,13 +1292,15 @@ __device__ __forceinline__ void face_state(FaceState<T>& f, const OpConst<T>& C)
 // Densities of both sides of a face, their reciprocals, rt = sqrt(rho_o rho_b) and
 // wd = 1 / (sqrt rho_o + sqrt rho_b)^2 = 1 / (rho_o + rho_b + 2 rt).  FP64: one division
 // serves all three reciprocals (the FP64 pipe bounds that operator).
+// Negative densities on both sides have a positive product: the root is then taken of one of
+// them, so that a flow that has left the physical states gives NaN and not plausible fluxes.
 __device__ __forceinline__ void face_densities(FaceState<float>& o, FaceState<float>& b, float rho_ref, float& rt,
                                                float& wd) {
   o.rho = add_(o.s[0], rho_ref);
   b.rho = add_(b.s[0], rho_ref);
   o.ir = drcp(o.rho);
   b.ir = drcp(b.rho);
-  rt = dsqrt(mul_(o.rho, b.rho));
+  rt = dsqrt(o.rho < 0.f ? o.rho : mul_(o.rho, b.rho));
   wd = drcp(fma_(2.f, rt, add_(o.rho, b.rho)));
 }
 __device__ __forceinline__ void face_densities(FaceState<double>& o, FaceState<double>& b, double rho_ref, double& rt,
@@ -1306,7 +1308,7 @@ __device__ __forceinline__ void face_densities(FaceState<double>& o, FaceState<d
   o.rho = add_(o.s[0], rho_ref);
   b.rho = add_(b.s[0], rho_ref);
   const double pr = mul_(o.rho, b.rho);
-  rt = sqrt(pr);
+  rt = sqrt(o.rho < 0.0 ? o.rho : pr);
   const double den = fma_(2.0, rt, add_(o.rho, b.rho));
   const double inv = 1.0 / mul_(pr, den), ipr = mul_(inv, den);
   wd = mul_(inv, pr);

@@ -129,3 +129,26 @@ def test_corrected_steps_in_one_call_equal_single_steps_and_one_rhs(dg, K, P, fi
     finally:
         nn.nn_destroy(net)
         dg.dg_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("sides", ["both", "one"])
+def test_negative_density_gives_nan(dg, prec, sides):
+    """A flow that has left the physical states is told by NaN, also where the densities (and
+    pressures) on both sides of a face are negative and their product is not."""
+    K, P = 3, 3
+    N = K ** 3 * (P + 1) ** 3
+    ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=prec)
+    try:
+        q = state(dg, ctx, N)
+        if sides == "both":
+            q.neg_()
+        else:
+            q.view(5, K ** 3, -1)[:, 13].neg_()
+        R = torch.empty_like(q)
+        dg.dg_rhs(ctx, q, R)
+        faces = R.view(5, K ** 3, 4, 4, 4)[:, 13, 0]
+        torch.cuda.synchronize()
+        assert torch.isnan(faces).all()
+    finally:
+        dg.dg_destroy(ctx)
