@@ -101,10 +101,10 @@ cudaError_t prepare_batch_persist_constants();
 // (dg_batch_f32.cu / dg_batch_f64.cu): q[i] is instance i's FP64 state, dt[i] its step.
 cudaError_t batch_stage_f32(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
                             const RkStage& rk, cudaStream_t st);
-// Sets the kernels' shared-memory attributes for order P at E elements per block; call
-// before batch_stage_* (never inside a stream capture).
-cudaError_t batch_prepare_f32(int P, int E);
-cudaError_t batch_prepare_f64(int P, int E);
+// Sets the kernels' shared-memory attributes for `elems` elements of order P in all, E per
+// phase-A block; call before batch_stage_* (never inside a stream capture).
+cudaError_t batch_prepare_f32(int P, int elems, int E);
+cudaError_t batch_prepare_f64(int P, int elems, int E);
 cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
                             const RkStage& rk, cudaStream_t st);
 

@@ -68,7 +68,9 @@ cudaError_t stage_group(const dg_batch* b, const Group& g, double* const* q, con
 cudaError_t prepare_groups(const dg_batch* b) {
   for (const Group& g : b->groups) {
     const int E = b->inst[g.members[0]]->geom.E;
-    cudaError_t e = b->precision == DG_PREC_FP32 ? batch_prepare_f32(g.P, E) : batch_prepare_f64(g.P, E);
+    int elems = 0;
+    for (int m : g.members) elems += b->inst[m]->nel;
+    cudaError_t e = b->precision == DG_PREC_FP32 ? batch_prepare_f32(g.P, elems, E) : batch_prepare_f64(g.P, elems, E);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -8,5 +8,5 @@ cudaError_t batch_stage_f64(int P, dg_ctx* const* ctx, double* const* q, const d
                            const RkStage& rk, cudaStream_t st) {
   return batch_stage_t<double>(P, ctx, q, dt, n, k, rk, st);
 }
-cudaError_t batch_prepare_f64(int P, int E) { return batch_prepare_t<double>(P, E); }
+cudaError_t batch_prepare_f64(int P, int elems, int E) { return batch_prepare_t<double>(P, elems, E); }
 }  // namespace dgnn

@@ -74,7 +74,7 @@ struct OpConst {
   T mu, lam, csd2, lam_t;         // transport
   int les;
   double drho_ref, dE_ref;        // references for shifting the FP64 state
-  int early;                      // phase A lets the next launch in as it starts, not as it ends (make_const)
+  int early;                      // phase A lets the next launch in as it starts, not as it ends (release_early)
   FeatureOut feat;                // network features to write with the stage state (feat.out may be NULL)
   T D[kMaxN1 * kMaxN1];
 };
@@ -1675,6 +1675,7 @@ constexpr int kMaxBatch = 16;
 template <typename T>
 struct BatchTable {
   int n;                             // instances in this launch
+  int early;                         // phase A lets the next launch in as it starts, not as it ends
   int block_start[kMaxBatch + 1];    // first phase-A block of each instance; block_start[n] = grid
   int surf_start[kMaxBatch + 1];     // the same for phase B
   int state_start[kMaxBatch + 1];    // the same for the state pass (P = 3, FP32)
@@ -1705,21 +1706,22 @@ template <int P, typename T, int SRC>
 __global__ void __launch_bounds__(volume_max_threads<P, T, false>(), volume_min_blocks<P, T, false>())
 k_volume_batch(const __grid_constant__ BatchTable<T> tb) {
   pdl_wait();
-  pdl_release();
+  if (tb.early) pdl_release();
   const int i = batch_instance(tb.block_start, tb.n, blockIdx.x);
   volume_phase<P, T, SRC>(blockIdx.x - tb.block_start[i], tb.a[i].q, tb.qs[i], tb.rv[i], tb.vt[i], tb.C[i]);
+  pdl_release();
 }
 
-template <int P, typename T, int MODE>
-__global__ void __launch_bounds__(surf_threads(P), surf_min_blocks(surf_threads(P), sizeof(T)))
+template <int P, typename T, int MODE, int E, int THREADS>
+__global__ void __launch_bounds__(THREADS, surf_min_blocks(THREADS, sizeof(T)))
 k_surface_batch(const __grid_constant__ BatchTable<T> tb) {
   const int b = gridDim.x - 1 - blockIdx.x;
   const int i = batch_instance(tb.surf_start, tb.n, b);
   const int blk = b - tb.surf_start[i];
-  surface_prologue<P, T, false>(blk, surf_elems(P), tb.C[i]);
+  surface_prologue<P, T, false>(blk, E, tb.C[i]);
   pdl_wait();
+  surface_block<P, T, MODE>(blk, E, tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);
   pdl_release();
-  surface_block<P, T, MODE>(blk, surf_elems(P), tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);
 }
 
 }  // namespace dgnn

@@ -13,6 +13,16 @@ namespace dgnn {
 // Elements a launch processes: the whole mesh, or a slab's own layers.
 inline int owned_elems(const dg_ctx* c) { return c->e_end - c->e_begin; }
 
+// Where phase A of a launch of `nodes` nodes lets the next launch in.  Let in early, its blocks
+// fill whichever SMs drain first instead of spreading over the chip: phase B at 9^3/P3 in FP64
+// 704 -> 250 us per RK3 step with the release at the end of phase A's blocks, 9^3/P4 44.6 -> 35.6,
+// 16^3/P3 50.2 -> 48.4.  Only the small blocks of a small mesh (512 nodes per SM) leave room for
+// both phases, and the launch latency saved counts there: 10^3/P3 32.0 -> 29.1, 8^3/P2 23.7 -> 22.3.
+template <typename T>
+bool release_early(int P, long long nodes) {
+  return std::is_same<T, float>::value && P <= 3 && nodes <= 152 * 512;
+}
+
 template <typename T>
 OpConst<T> make_const(const dg_ctx* c) {
   OpConst<T> k;
@@ -36,12 +46,7 @@ OpConst<T> make_const(const dg_ctx* c) {
   k.les = ph.les;
   k.drho_ref = ph.rho_ref;
   k.dE_ref = ph.E_ref;
-  // Where the next launch may start.  Let in early, its blocks fill whichever SMs drain first
-  // instead of spreading over the chip: phase B at 9^3/P3 in FP64 704 -> 250 us per RK3 step
-  // with the release at the end of phase A's blocks, 9^3/P4 44.6 -> 35.6, 16^3/P3 50.2 -> 48.4.
-  // Only the small blocks of a small mesh (512 nodes per SM) leave room for both phases, and
-  // the launch latency saved counts there: 10^3/P3 32.0 -> 29.1, 8^3/P2 23.7 -> 22.3.
-  k.early = std::is_same<T, float>::value && c->P <= 3 && c->N <= 152 * 512;
+  k.early = release_early<T>(c->P, c->N);
   k.feat = c->feat_out;
   for (int i = 0; i < kMaxN1 * kMaxN1; ++i) k.D[i] = T(c->geom.D[i]);
   return k;
@@ -207,35 +212,48 @@ cudaError_t surface_launch(const dg_ctx* c, double* q, double* dqdt, const Forci
                     make_const<T>(c), rk);
 }
 
+// Elements and threads of phase B's blocks for n elements in a launch: f(E, THREADS) as
+// integral constants.
+// FP64: few elements per block at P = 2 and 3, so that the FP64 pipes of all SMs have an equal
+// share.  us per RK3 step, P = 3, 2 x 96 / 8 x 128 elements x threads: 8^3 130 / 196, 11^3
+// 328 / 413, 12^3 360 / 414, 16^3 811 / 867; a batch of 8^3, 6^3 and 4^3 222 / 683.
+// P = 3 in FP32: the smallest block whose launch is still one wave (1024 threads per SM at
+// 64 registers), so that every SM has its share of a small mesh; large meshes want many
+// elements per block.  us per RK3 step with 2 x 192 / 2 x 96 / 4 x 128 / 8 x 128 elements x
+// threads: 8^3 28.4 / 29.8 / 29.9 / 31.9, 14^3 44.9 / 41.0 / 42.1 / 42.7, 16^3 53.8 / 49.5 /
+// 48.5 / 49.3, 32^3 345 / 295 / 294 / 290.
+template <int N>
+using Int = std::integral_constant<int, N>;
+template <int P, typename T, typename F>
+auto with_surf_block(int n, F f) {
+  if constexpr (std::is_same<T, double>::value) {
+    if constexpr (P == 3) return f(Int<2>{}, Int<96>{});
+    if constexpr (P == 2) return f(Int<4>{}, Int<192>{});
+  }
+  if constexpr (P == 3 && std::is_same<T, float>::value) {
+    constexpr int kWave = 152 * 1024;   // threads
+    if (n <= kWave / 192 * 2) return f(Int<2>{}, Int<192>{});
+    if (n <= kWave / 96 * 2) return f(Int<2>{}, Int<96>{});
+    if (n <= kWave / 128 * 4) return f(Int<4>{}, Int<128>{});
+  }
+  return f(Int<surf_elems(P)>{}, Int<surf_threads(P)>{});
+}
+
 template <int P, typename T, int MODE>
 cudaError_t surface_p(const dg_ctx* c, double* q, double* dqdt, const Forcing& f, const RkArgs<T>& rk,
                       cudaStream_t st) {
   const int n = owned_elems(c);
   // FP64: cubes where they pay (two per SM at least) and tile the mesh (a slab's layers:
   // rows); the twelve internal faces' terms are formed once for both sides, to the same bits
-  // as per side.  Otherwise few elements per block at P = 2 and 3, so that the FP64 pipes of
-  // all SMs have an equal share.  us per RK3 step, P = 3, cubes / 2 x 96 / 8 x 128 elements x
-  // threads: 8^3 164 / 130 / 196, 11^3 - / 328 / 413, 12^3 365 / 360 / 414, 16^3 770 / 811 / 867.
-  if constexpr (std::is_same<T, double>::value) {
-    if constexpr (surf_cube(P, sizeof(T))) {
-      if (!c->part && c->K % 2 == 0 && n >= 2 * 152 * kCubeElems)
-        return surface_launch<P, T, MODE, kCubeElems, surf_threads_cube(P), true>(c, q, dqdt, f, rk, st);
-    }
-    if constexpr (P == 3) return surface_launch<P, T, MODE, 2, 96, false>(c, q, dqdt, f, rk, st);
-    if constexpr (P == 2) return surface_launch<P, T, MODE, 4, 192, false>(c, q, dqdt, f, rk, st);
+  // as per side.  us per RK3 step, P = 3, cubes / rows: 8^3 164 / 130, 12^3 365 / 360, 16^3
+  // 770 / 811.
+  if constexpr (surf_cube(P, sizeof(T))) {
+    if (!c->part && c->K % 2 == 0 && n >= 2 * 152 * kCubeElems)
+      return surface_launch<P, T, MODE, kCubeElems, surf_threads_cube(P), true>(c, q, dqdt, f, rk, st);
   }
-  // P = 3 in FP32: the smallest block whose launch is still one wave (1024 threads per SM at
-  // 64 registers), so that every SM has its share of a small mesh; large meshes want many
-  // elements per block.  us per RK3 step with 2 x 192 / 2 x 96 / 4 x 128 / 8 x 128 elements x
-  // threads: 8^3 28.4 / 29.8 / 29.9 / 31.9, 14^3 44.9 / 41.0 / 42.1 / 42.7, 16^3 53.8 / 49.5 /
-  // 48.5 / 49.3, 32^3 345 / 295 / 294 / 290.
-  if constexpr (P == 3 && std::is_same<T, float>::value) {
-    constexpr int kWave = 152 * 1024;   // threads
-    if (n <= kWave / 192 * 2) return surface_launch<P, T, MODE, 2, 192, false>(c, q, dqdt, f, rk, st);
-    if (n <= kWave / 96 * 2) return surface_launch<P, T, MODE, 2, 96, false>(c, q, dqdt, f, rk, st);
-    if (n <= kWave / 128 * 4) return surface_launch<P, T, MODE, 4, 128, false>(c, q, dqdt, f, rk, st);
-  }
-  return surface_launch<P, T, MODE, surf_elems(P), surf_threads(P), false>(c, q, dqdt, f, rk, st);
+  return with_surf_block<P, T>(n, [&](auto E, auto threads) {
+    return surface_launch<P, T, MODE, E.value, threads.value, false>(c, q, dqdt, f, rk, st);
+  });
 }
 
 // FP64 operator: modes 0 (dq/dt) and 1 (FP64 RK stage).  FP32 operator: modes 0, 2, 3, 4.
@@ -277,17 +295,40 @@ cudaError_t surface_t(const dg_ctx* c, double* q, double* dqdt, const Forcing& f
 // Batched RK stage: one phase-A and one phase-B launch for all instances of order P.
 // Instances must share the operator precision T and the elements-per-block E.
 
+// Elements per phase-B block of a launch of n elements of order P in all.
+template <typename T>
+int surf_block_elems(int P, int n) {
+  const auto elems = [](auto E, auto) { return (int)E.value; };
+  switch (P) {
+    case 1: return with_surf_block<1, T>(n, elems);
+    case 2: return with_surf_block<2, T>(n, elems);
+    case 3: return with_surf_block<3, T>(n, elems);
+    case 4: return with_surf_block<4, T>(n, elems);
+    case 5: return with_surf_block<5, T>(n, elems);
+    case 6: return with_surf_block<6, T>(n, elems);
+    case 7: return with_surf_block<7, T>(n, elems);
+  }
+  return with_surf_block<8, T>(n, elems);
+}
+
 template <typename T>
 void fill_batch(BatchTable<T>* tb, dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
                 const RkStage& rk) {
   tb->n = n;
-  int blocks = 0, surf = 0, state = 0;
+  int blocks = 0, surf = 0, state = 0, elems = 0;
+  long long nodes = 0;
+  for (int i = 0; i < n; ++i) {
+    elems += owned_elems(ctx[i]);
+    nodes += ctx[i]->N;
+  }
+  tb->early = release_early<T>(ctx[0]->P, nodes);
+  const int E = surf_block_elems<T>(ctx[0]->P, elems);
   for (int i = 0; i < n; ++i) {
     const dg_ctx* c = ctx[i];
     tb->block_start[i] = blocks;
     blocks += (owned_elems(c) + c->geom.E - 1) / c->geom.E;
     tb->surf_start[i] = surf;
-    surf += (owned_elems(c) + surf_elems(c->P) - 1) / surf_elems(c->P);
+    surf += (owned_elems(c) + E - 1) / E;
     tb->state_start[i] = state;
     state += (c->nel + kStateElems - 1) / kStateElems;
     tb->qs[i] = static_cast<T*>(stage_buffer(c, k));
@@ -304,19 +345,26 @@ void fill_batch(BatchTable<T>* tb, dg_ctx* const* ctx, double* const* q, const d
   tb->state_start[n] = state;
 }
 
+// The phase-B kernel of stage k.
+template <int P, typename T, int E, int THREADS>
+auto batch_surface(int k) {
+  if constexpr (std::is_same<T, float>::value)
+    return k == 0 ? k_surface_batch<P, T, 2, E, THREADS>
+                  : k == 1 ? k_surface_batch<P, T, 3, E, THREADS> : k_surface_batch<P, T, 4, E, THREADS>;
+  else return k_surface_batch<P, T, 1, E, THREADS>;
+}
+
 // Stage k of the RK3 step: the same source and mode sequence as the single-mesh path
-// (FP32 operator: sources 0, 1, 1 and modes 2, 3, 4; FP64 operator: source 0, mode 1).
+// (FP32 operator: sources 0, 1, 1 and modes 2, 3, 4; FP64 operator: source 0, mode 1), and
+// its rules for phase B's blocks and for the release, over all members.
 template <int P, typename T>
-cudaError_t batch_stage_p(const BatchTable<T>& tb, int E, int k, cudaStream_t st) {
+cudaError_t batch_stage_p(const BatchTable<T>& tb, int elems, int E, int k, cudaStream_t st) {
   void (*kg)(const BatchTable<T>);
-  void (*kf)(const BatchTable<T>);
   if constexpr (std::is_same<T, float>::value) {
     if constexpr (use_rows4(P, sizeof(T), false)) kg = k_volume_batch<P, T, 1>;
     else kg = k == 0 ? k_volume_batch<P, T, 0> : k_volume_batch<P, T, 1>;
-    kf = k == 0 ? k_surface_batch<P, T, 2> : k == 1 ? k_surface_batch<P, T, 3> : k_surface_batch<P, T, 4>;
   } else {
     kg = k_volume_batch<P, T, 0>;
-    kf = k_surface_batch<P, T, 1>;
   }
   cudaError_t e;
   if constexpr (use_rows4(P, sizeof(T), false)) {
@@ -326,38 +374,40 @@ cudaError_t batch_stage_p(const BatchTable<T>& tb, int E, int k, cudaStream_t st
   if ((e = launch_pdl(kg, dim3(tb.block_start[tb.n]), dim3(volume_threads<P, T, false>(E)),
                       volume_smem<P, T, false>(E, false), st, tb)) != cudaSuccess)
     return e;
-  return launch_pdl(kf, dim3(tb.surf_start[tb.n]), dim3(surf_threads(P)), surface_smem_bytes<P, T>(surf_elems(P)), st, tb);
+  return with_surf_block<P, T>(elems, [&](auto SE, auto threads) {
+    return launch_pdl(batch_surface<P, T, SE.value, threads.value>(k), dim3(tb.surf_start[tb.n]), dim3(threads.value),
+                      surface_smem_bytes<P, T>(SE.value), st, tb);
+  });
 }
 
 // Dynamic shared-memory attributes of the batched kernels of order P at E elements per
-// block; set before any launch (and outside stream capture).
+// block of phase A; set before any launch (and outside stream capture).
 template <int P, typename T>
-cudaError_t batch_prepare_p(int E) {
-  const size_t gs = volume_smem<P, T, false>(E, false), fs = surface_smem_bytes<P, T>(surf_elems(P));
+cudaError_t batch_prepare_p(int elems, int E) {
+  const size_t gs = volume_smem<P, T, false>(E, false);
   cudaError_t e = cudaSuccess;
   if constexpr (!use_rows4(P, sizeof(T), false)) e = set_smem(k_volume_batch<P, T, 0>, gs);
-  if (e != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
-    if ((e = set_smem(k_volume_batch<P, T, 1>, gs)) != cudaSuccess) return e;
-    if ((e = set_smem(k_surface_batch<P, T, 2>, fs)) != cudaSuccess) return e;
-    if ((e = set_smem(k_surface_batch<P, T, 3>, fs)) != cudaSuccess) return e;
-    return set_smem(k_surface_batch<P, T, 4>, fs);
-  } else {
-    return set_smem(k_surface_batch<P, T, 1>, fs);
+    if (e == cudaSuccess) e = set_smem(k_volume_batch<P, T, 1>, gs);
   }
+  return with_surf_block<P, T>(elems, [&](auto SE, auto threads) {
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k)
+      e = set_smem(batch_surface<P, T, SE.value, threads.value>(k), surface_smem_bytes<P, T>(SE.value));
+    return e;
+  });
 }
 
 template <typename T>
-cudaError_t batch_prepare_t(int P, int E) {
+cudaError_t batch_prepare_t(int P, int elems, int E) {
   switch (P) {
-    case 1: return batch_prepare_p<1, T>(E);
-    case 2: return batch_prepare_p<2, T>(E);
-    case 3: return batch_prepare_p<3, T>(E);
-    case 4: return batch_prepare_p<4, T>(E);
-    case 5: return batch_prepare_p<5, T>(E);
-    case 6: return batch_prepare_p<6, T>(E);
-    case 7: return batch_prepare_p<7, T>(E);
-    case 8: return batch_prepare_p<8, T>(E);
+    case 1: return batch_prepare_p<1, T>(elems, E);
+    case 2: return batch_prepare_p<2, T>(elems, E);
+    case 3: return batch_prepare_p<3, T>(elems, E);
+    case 4: return batch_prepare_p<4, T>(elems, E);
+    case 5: return batch_prepare_p<5, T>(elems, E);
+    case 6: return batch_prepare_p<6, T>(elems, E);
+    case 7: return batch_prepare_p<7, T>(elems, E);
+    case 8: return batch_prepare_p<8, T>(elems, E);
   }
   return cudaErrorInvalidValue;
 }
@@ -369,15 +419,17 @@ cudaError_t batch_stage_t(int P, dg_ctx* const* ctx, double* const* q, const dou
   BatchTable<T> tb;
   fill_batch<T>(&tb, ctx, q, dt, n, k, rk);
   const int E = ctx[0]->geom.E;
+  int elems = 0;
+  for (int i = 0; i < n; ++i) elems += owned_elems(ctx[i]);
   switch (P) {
-    case 1: return batch_stage_p<1, T>(tb, E, k, st);
-    case 2: return batch_stage_p<2, T>(tb, E, k, st);
-    case 3: return batch_stage_p<3, T>(tb, E, k, st);
-    case 4: return batch_stage_p<4, T>(tb, E, k, st);
-    case 5: return batch_stage_p<5, T>(tb, E, k, st);
-    case 6: return batch_stage_p<6, T>(tb, E, k, st);
-    case 7: return batch_stage_p<7, T>(tb, E, k, st);
-    case 8: return batch_stage_p<8, T>(tb, E, k, st);
+    case 1: return batch_stage_p<1, T>(tb, elems, E, k, st);
+    case 2: return batch_stage_p<2, T>(tb, elems, E, k, st);
+    case 3: return batch_stage_p<3, T>(tb, elems, E, k, st);
+    case 4: return batch_stage_p<4, T>(tb, elems, E, k, st);
+    case 5: return batch_stage_p<5, T>(tb, elems, E, k, st);
+    case 6: return batch_stage_p<6, T>(tb, elems, E, k, st);
+    case 7: return batch_stage_p<7, T>(tb, elems, E, k, st);
+    case 8: return batch_stage_p<8, T>(tb, elems, E, k, st);
   }
   return cudaErrorInvalidValue;
 }
