@@ -157,8 +157,12 @@ def ptr(t):
 
 
 def stream_ptr(stream=None):
+    """Handle of ``stream``, or of the current stream.  Every call asks for it: through a
+    torch.cuda.Stream object it took 3.9 us of a call's 15, more than two kernel launches."""
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         if not torch.cuda.is_available():
             return None
         stream = torch.cuda.current_stream()

@@ -152,3 +152,26 @@ def test_negative_density_gives_nan(dg, prec, sides):
         assert torch.isnan(faces).all()
     finally:
         dg.dg_destroy(ctx)
+
+
+def test_current_stream_handle_follows_torch_and_costs_little(dg):
+    """At 8^3/P3 and below a call is bound by the host: the state pass added a launch to it, and
+    looking the current stream up as an object costs more than that launch."""
+    import time
+    st = torch.cuda.Stream()
+    assert not dg.stream_ptr().value == st.cuda_stream
+    with torch.cuda.stream(st):
+        assert dg.stream_ptr().value == st.cuda_stream == torch.cuda.current_stream().cuda_stream
+        assert dg.stream_ptr(torch.cuda.default_stream()).value in (None, 0)
+    assert dg.stream_ptr().value in (None, 0)
+
+    def us(f, n=2000):
+        best = float("inf")
+        for _ in range(5):
+            t = time.perf_counter()
+            for _ in range(n):
+                f()
+            best = min(best, time.perf_counter() - t)
+        return best / n * 1e6
+
+    assert us(dg.stream_ptr) < 0.8 * us(torch.cuda.current_stream)
