@@ -12,6 +12,7 @@ namespace dgnn {
 
 constexpr int kMaxP = 8;
 constexpr int kMaxN1 = kMaxP + 1;
+constexpr int kSMs = 152;   // of a GB300
 
 // Element-major workspace records (dg_kernels.cuh), n = P + 1: node stride of a component,
 // and sizes of the state and face records in values.

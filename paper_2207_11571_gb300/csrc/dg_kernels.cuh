@@ -1399,7 +1399,8 @@ __host__ __device__ constexpr int surf_threads_cube(int P) { return P == 1 ? 96 
 __host__ __device__ constexpr bool surf_cube(int P, int tsize) { return tsize == 8 && P <= 3; }
 // Blocks per SM the phase-B kernel is compiled for: 64 registers per thread in FP32, 128 in FP64.
 __host__ __device__ constexpr int surf_min_blocks(int threads, int tsize) {
-  return tsize == 8 ? 512 / threads : 1024 / threads;
+  const int blocks = (tsize == 8 ? 512 : 1024) / threads;
+  return blocks > 0 ? blocks : 1;
 }
 
 // Shared memory of a phase-B block: neighbour elements [6 E] (int), lifted interface terms

@@ -222,6 +222,10 @@ cudaError_t surface_launch(const dg_ctx* c, double* q, double* dqdt, const Forci
 // elements per block.  us per RK3 step with 2 x 192 / 2 x 96 / 4 x 128 / 8 x 128 elements x
 // threads: 8^3 28.4 / 29.8 / 29.9 / 31.9, 14^3 44.9 / 41.0 / 42.1 / 42.7, 16^3 53.8 / 49.5 /
 // 48.5 / 49.3, 32^3 345 / 295 / 294 / 290.
+// P >= 6: a block per element.  Where every element has an SM to itself, a thread per node, as
+// nothing else hides the block's latency (us per RK3 step against the general threads: FP32 3^3/P7
+// 30.4 -> 23.1, 4^3/P6 22.7 -> 21.4, 5^3/P8 40.7 -> 29.6; FP64 5^3/P8 400 -> 316, 5^3/P6 207 -> 154);
+// with two elements per SM the general threads overlap better (7^3/P8 61.0 against 69.6).
 template <int N>
 using Int = std::integral_constant<int, N>;
 template <int P, typename T, typename F>
@@ -235,6 +239,9 @@ auto with_surf_block(int n, F f) {
     if (n <= kWave / 192 * 2) return f(Int<2>{}, Int<192>{});
     if (n <= kWave / 96 * 2) return f(Int<2>{}, Int<96>{});
     if (n <= kWave / 128 * 4) return f(Int<4>{}, Int<128>{});
+  }
+  if constexpr (P >= 6) {
+    if (n <= kSMs) return f(Int<1>{}, Int<max_threads_for(P)>{});
   }
   return f(Int<surf_elems(P)>{}, Int<surf_threads(P)>{});
 }

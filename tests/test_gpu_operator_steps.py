@@ -175,3 +175,52 @@ def test_current_stream_handle_follows_torch_and_costs_little(dg):
         return best / n * 1e6
 
     assert us(dg.stream_ptr) < 0.8 * us(torch.cuda.current_stream)
+
+
+@pytest.mark.parametrize("K,P,prec", [(3, 3, 1), (12, 3, 1), (15, 3, 1), (2, 6, 1), (5, 6, 1), (3, 7, 1), (5, 7, 1), (1, 8, 1),
+                                      (5, 8, 1), (5, 6, 0), (3, 7, 0), (5, 8, 0)])
+def test_phase_b_blocks_of_a_mesh_and_of_a_large_batch_give_the_same_bits(dg, K, P, prec):
+    """A batch takes its blocks by the elements of all members: beside a large one the widest
+    (P = 3) or those of many elements per SM (P >= 6), where the mesh alone takes small blocks or
+    a thread per node.  Each face term is the same arithmetic."""
+    other = 20 if P == 3 else 6
+    b = dg.dg_create_batch([(K, P, 400.0, 0.1, 0.71, 0), (other, P, 200.0, 0.1, 0.71, 0)], precision=prec)
+    try:
+        qs = [state(dg, dg.dg_batch_member(b, i), k ** 3 * (P + 1) ** 3) for i, k in enumerate((K, other))]
+        alone = qs[0].clone()
+        dg.dg_batch_rk3_step(b, qs, [1e-3, 1e-3], 2)
+        dg.dg_rk3_step(dg.dg_batch_member(b, 0), alone, 1e-3, 2)
+        torch.cuda.synchronize()
+        assert torch.isfinite(alone).all()
+        if prec == 1:
+            assert torch.equal(alone, qs[0])
+        else:   # separate compilations may contract a multiply-add differently: a rounding of the state
+            assert (alone - qs[0]).abs().max().item() <= 4e-16 * alone.abs().max().item()
+    finally:
+        dg.dg_batch_destroy(b)
+
+
+@pytest.mark.parametrize("P,prec", [(8, 0), (8, 1), (6, 0), (7, 0)])
+def test_meshes_of_one_element_per_sm_take_the_same_time(dg, P, prec):
+    """4^3 and 5^3 elements at P >= 6 are one block per SM in both phases, so they take the same
+    time.  Interface blocks of a few warps took 1.2 to 1.3 times as long on 5^3; 1.12 leaves room
+    for the larger launch."""
+    def us(K):
+        N = K ** 3 * (P + 1) ** 3
+        ctx = dg.dg_create(K, P, 400.0, 0.1, 0.71, 0, precision=prec)
+        try:
+            q = state(dg, ctx, N)
+            best = float("inf")
+            for _ in range(6):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                for _ in range(30):
+                    dg.dg_rk3_step(ctx, q, 1e-6)
+                b.record()
+                b.synchronize()
+                best = min(best, a.elapsed_time(b) / 30 * 1e3)
+            return best
+        finally:
+            dg.dg_destroy(ctx)
+    small, large = us(4), us(5)
+    assert large <= 1.12 * small, (small, large)
