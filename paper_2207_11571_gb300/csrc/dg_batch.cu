@@ -90,16 +90,16 @@ cudaError_t step_direct(const dg_batch* b, double* const* q, const double* dt, c
 
 // One RK3 step of every member as three persistent launches (one per stage, every order
 // together), after a reset of the grid barrier's counters.
-cudaError_t step_persistent(const dg_batch* b, double* const* q, const double* dt, size_t smem, int grid,
+cudaError_t step_persistent(const dg_batch* b, double* const* q, const double* dt, int grid,
                             cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), st);
   const int n = (int)b->inst.size();
   for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-    e = batch_persistent_stage(b->inst.data(), q, dt, n, k, rk_stage(k), b->bar, smem, grid, st);
+    e = batch_persistent_stage(b->inst.data(), q, dt, n, k, rk_stage(k), b->bar, grid, st);
   return e;
 }
 
-int prepare_persistent(const dg_batch* b, size_t* smem, int* grid) {
+int prepare_persistent(const dg_batch* b, int* grid) {
   if (b->precision != DG_PREC_FP32)
     return fail(DG_ERR_UNSUPPORTED, "dg_batch_rk3_step: the persistent stage kernel runs the FP32 operator");
   std::vector<int> orders;
@@ -108,17 +108,16 @@ int prepare_persistent(const dg_batch* b, size_t* smem, int* grid) {
       return fail(DG_ERR_UNSUPPORTED, "dg_batch_rk3_step: the persistent stage kernel takes orders 1 to 6");
     orders.push_back(c->P);
   }
-  DG_CUDA(batch_persistent_prepare(orders.data(), (int)orders.size(), smem, grid));
+  DG_CUDA(batch_persistent_prepare(orders.data(), (int)orders.size(), grid));
   return DG_OK;
 }
 
 // Records one step with the groups as parallel branches: fork from cap[0], each group on
 // its own stream, join back into cap[0].  persistent: three cooperative launches on cap[0].
 int record_step(dg_batch* b, double* const* q, const double* dt, bool persistent) {
-  size_t psmem = 0;
   int pgrid = 0;
   if (persistent) {
-    int rc = prepare_persistent(b, &psmem, &pgrid);
+    int rc = prepare_persistent(b, &pgrid);
     if (rc) return rc;
   }
   // kernel attributes (dynamic shared memory) are set outside the recording
@@ -131,7 +130,7 @@ int record_step(dg_batch* b, double* const* q, const double* dt, bool persistent
   cudaStream_t s0 = b->cap[0];
   DG_CUDA(cudaStreamBeginCapture(s0, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaEventRecord(b->fork, s0);
-  if (persistent && e == cudaSuccess) e = step_persistent(b, q, dt, psmem, pgrid, s0);
+  if (persistent && e == cudaSuccess) e = step_persistent(b, q, dt, pgrid, s0);
   for (size_t gi = 0; gi < b->groups.size() && e == cudaSuccess && !persistent; ++gi) {
     cudaStream_t s = b->cap[gi];
     if (gi > 0) e = cudaStreamWaitEvent(s, b->fork, 0);
@@ -269,11 +268,10 @@ int dg_batch_rk3_step(dg_batch* b, double* const* q, const double* dt, int nstep
   cudaStream_t st = (cudaStream_t)stream;
   if (flags & DG_BATCH_NO_GRAPH) {
     if (persistent) {
-      size_t smem = 0;
       int grid = 0;
-      int rc = prepare_persistent(b, &smem, &grid);
+      int rc = prepare_persistent(b, &grid);
       if (rc) return rc;
-      for (int s = 0; s < nsteps; ++s) DG_CUDA(step_persistent(b, q, dt, smem, grid, st));
+      for (int s = 0; s < nsteps; ++s) DG_CUDA(step_persistent(b, q, dt, grid, st));
       return DG_OK;
     }
     for (int s = 0; s < nsteps; ++s) DG_CUDA(step_direct(b, q, dt, st));

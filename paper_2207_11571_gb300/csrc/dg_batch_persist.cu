@@ -16,6 +16,7 @@
 namespace dgnn {
 
 constexpr int kPersistThreads = 384;
+// Elements per work item of order P, at most (P = 3, 16 threads per element: see persist_elems_of).
 __host__ __device__ constexpr int persist_elems(int P) {
   return kPersistThreads / (use_rows4(P, sizeof(float), false) ? 16 : (P + 1) * (P + 1) * (P + 1));
 }
@@ -82,8 +83,8 @@ __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const _
     switch (pt.P[i]) {
 #define DG_PB(PP)                                                                                   \
   case PP:                                                                                          \
-    surface_prologue<PP, float, false>(blk, persist_elems(PP), tb.C[i]);                            \
-    surface_block<PP, float, MODE>(blk, persist_elems(PP), tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);  \
+    surface_prologue<PP, float, false>(blk, tb.C[i].E, tb.C[i]);                                    \
+    surface_block<PP, float, MODE>(blk, tb.C[i].E, tb.a[i], Forcing{}, tb.C[i], tb.rk[i]);          \
     break;
       DG_PB(1) DG_PB(2) DG_PB(3) DG_PB(4) DG_PB(5) DG_PB(6)
 #undef DG_PB
@@ -94,17 +95,25 @@ __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const _
 
 namespace {
 
-// Shared memory of one work item of order P in the persistent kernel (the larger phase).
-size_t persist_smem_p(int P) {
+// Shared memory of a work item of E elements of order P (the larger phase).
+size_t persist_smem_p(int P, int E) {
   switch (P) {
-#define DG_SM(PP)                                                                                                     \
-  case PP:                                                                                                            \
-    return std::max(volume_smem<PP, float, false>(persist_elems(PP), false),                                          \
-                    surface_smem_bytes<PP, float>(persist_elems(PP)));
+#define DG_SM(PP) \
+  case PP: return std::max(volume_smem<PP, float, false>(E, false), surface_smem_bytes<PP, float>(E));
     DG_SM(1) DG_SM(2) DG_SM(3) DG_SM(4) DG_SM(5) DG_SM(6)
 #undef DG_SM
   }
   return 0;
+}
+
+// Elements per work item of order P, `elems` of them in the launch.  P = 3: a full block of rows
+// (24 elements) leaves most of the chip idle on small meshes, so as many as give every block
+// of the grid an item, and at least a node per thread of phase B.  us per RK3 step with 24 /
+// 6 / one item per block: 8^3 83 / 49 / 54, twelve 5^3 88 / 63 / 70, 16^3 + 12^3 128 / 174 / 112.
+int persist_elems_of(int P, int elems, int grid) {
+  if (!use_rows4(P, sizeof(float), false)) return persist_elems(P);
+  const int nodes = kPersistThreads / ((P + 1) * (P + 1) * (P + 1));
+  return std::max(nodes, std::min(persist_elems(P), (elems + grid - 1) / grid));
 }
 
 using PersistKernel = void (*)(const PersistTable);
@@ -120,9 +129,9 @@ cudaError_t prepare_batch_persist_constants() { return upload_const_D(); }
 
 bool batch_persistent_ok(int P) { return P >= 1 && P <= 6; }
 
-cudaError_t batch_persistent_prepare(const int* orders, int n, size_t* smem_out, int* grid_out) {
+cudaError_t batch_persistent_prepare(const int* orders, int n, int* grid_out) {
   size_t smem = 0;
-  for (int i = 0; i < n; ++i) smem = std::max(smem, persist_smem_p(orders[i]));
+  for (int i = 0; i < n; ++i) smem = std::max(smem, persist_smem_p(orders[i], persist_elems(orders[i])));
   int grid = 0;
   for (int k = 0; k < 3; ++k) {
     PersistKernel kern = persist_kernel(k);
@@ -138,25 +147,29 @@ cudaError_t batch_persistent_prepare(const int* orders, int n, size_t* smem_out,
     grid = (k == 0) ? g : std::min(grid, g);
   }
   if (grid < 1) return cudaErrorInvalidConfiguration;
-  *smem_out = smem;
   *grid_out = grid;
   return cudaSuccess;
 }
 
 cudaError_t batch_persistent_stage(dg_ctx* const* ctx, double* const* q, const double* dt, int n, int k,
-                                   const RkStage& rk, unsigned* bar, size_t smem, int grid, cudaStream_t st) {
+                                   const RkStage& rk, unsigned* bar, int grid, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
   PersistTable pt;
   fill_batch<float>(&pt.tb, ctx, q, dt, n, k, rk);
   // work items of E_P elements per member, whatever blocking the member uses alone
-  int items = 0;
+  int items = 0, elems[kMaxP + 1] = {};
+  size_t smem = 0;
   for (int i = 0; i < n; ++i) {
-    const int P = ctx[i]->P;
-    if (!batch_persistent_ok(P)) return cudaErrorInvalidValue;
+    if (!batch_persistent_ok(ctx[i]->P)) return cudaErrorInvalidValue;
+    elems[ctx[i]->P] += owned_elems(ctx[i]);
+  }
+  for (int i = 0; i < n; ++i) {
+    const int P = ctx[i]->P, E = persist_elems_of(P, elems[P], grid);
+    smem = std::max(smem, persist_smem_p(P, E));   // no more than it needs: the rest is L1
     pt.P[i] = P;
-    pt.tb.C[i].E = persist_elems(P);
+    pt.tb.C[i].E = E;
     pt.tb.block_start[i] = items;
-    items += (owned_elems(ctx[i]) + persist_elems(P) - 1) / persist_elems(P);
+    items += (owned_elems(ctx[i]) + E - 1) / E;
   }
   pt.tb.block_start[n] = items;
   pt.bar = bar;

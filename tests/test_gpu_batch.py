@@ -225,3 +225,36 @@ def test_a_small_mesh_in_a_batch_takes_no_longer_than_alone(dg, K, prec):
         assert batch <= 1.4 * alone, (batch, alone)
     finally:
         dg.dg_batch_destroy(b)
+
+
+@pytest.mark.parametrize("members", [[(8, 3)], [(5, 3)] * 12, [(4, 3), (4, 3)], [(16, 3), (7, 3)]])
+def test_persistent_work_items_of_every_size_give_the_same_bits(dg, members):
+    """At P = 3 a work item takes 6 to 24 elements by the size of the batch (16^3 + 7^3: 15, with
+    ragged last items).  Its kernel is the single mesh's, so the members keep their bits."""
+    members = [(K, P, 200.0, 0.1, 0.71, 0) for K, P in members]
+    b = dg.dg_create_batch(members, precision=1)
+    try:
+        qs = init_states(dg, b, members)
+        dts = [1e-3] * len(members)
+        ref = alone(dg, b, qs, dts, 2)
+        dg.dg_batch_rk3_step(b, qs, dts, 2, flags=dg.DG_BATCH_PERSISTENT)
+        torch.cuda.synchronize()
+        for q, r in zip(qs, ref):
+            assert torch.isfinite(q).all()
+            assert torch.equal(q, r)
+    finally:
+        dg.dg_batch_destroy(b)
+
+
+def test_a_small_persistent_batch_uses_the_chip(dg):
+    """One 8^3 mesh at P = 3 takes no longer than one 8^3 mesh at P = 4, which has twice its nodes:
+    with work items of 24 elements 22 blocks did all the work (83 against 59 us)."""
+    def us(P):
+        members = [(8, P, 200.0, 0.1, 0.71, 0)]
+        b = dg.dg_create_batch(members, precision=1)
+        try:
+            qs = init_states(dg, b, members)
+            return _us(lambda: dg.dg_batch_rk3_step(b, qs, [1e-6], flags=dg.DG_BATCH_PERSISTENT))
+        finally:
+            dg.dg_batch_destroy(b)
+    assert us(3) <= 1.05 * us(4)
