@@ -205,6 +205,30 @@ __device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a,
 __device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// A value (four consecutive ones) that another launch may have written after this SM last
+// cached its line: read at the L2, the point of coherence, in program order.
+__device__ __forceinline__ float ld_l2(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_l2(const double* p) {
+  double v;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void ld4_l2(const float* p, float v[4]) {
+  asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "l"(p)
+               : "memory");
+}
+// A value of the stage state, by phase A's source (see k_volume).
+template <int SRC, typename T>
+__device__ __forceinline__ T state_value(const T* p) {
+  return SRC == 2 ? ld_l2(p) : *p;
+}
+
 // ---------------------------------------------------------------- shared-memory tiles
 
 // Four values of a node in shared memory, read and written as vectors: FP32 one plane of
@@ -470,7 +494,7 @@ __host__ __device__ constexpr size_t volume_smem_bytes(int E, int faces, bool sp
 
 // Phase A of block `blk` of one mesh (the body of k_volume and k_volume_batch).
 // SRC 0: the stage state is formed from the FP64 state q and written to qf; SRC 1: it is
-// read from qf.  CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the
+// read from qf; SRC 2: the same, at the L2 (BESIDE, see k_volume).  CUBE: the block is a 2 x 2 x 2 cube of elements; the halo holds only the
 // external faces, internal faces take the neighbour's values from the own tile.  FEAT:
 // also write the forcing network's input features (C.feat; FP64, P = 3).  SPLIT: the Euler part of the
 // volume term in the kinetic-energy-preserving split form, 2 sum_m D_im F#(q_i, q_m) along
@@ -478,7 +502,7 @@ __host__ __device__ constexpr size_t volume_smem_bytes(int E, int faces, bool sp
 // {p'} delta_jd; energy m {H}), from a tile of primitives; the viscous part keeps the
 // standard form.
 template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false>
-__device__ __forceinline__ void volume_block(int blk, const double* __restrict__ q, T* __restrict__ qf,
+__device__ __forceinline__ void volume_block(int blk, const double* __restrict__ q, T* qf,
                                              T* __restrict__ rv, T* __restrict__ vt, const OpConst<T>& C) {
   constexpr int n = P + 1, n2 = n * n, np = n2 * n, ns = node_stride(n);
   constexpr bool kLines = use_lines<T>(P);
@@ -510,7 +534,7 @@ __device__ __forceinline__ void volume_block(int blk, const double* __restrict__
       for (int v = 0; v < 5; ++v) qe[v * ns] = s[v];
     } else {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) s[v] = qe[v * ns];
+      for (int v = 0; v < 5; ++v) s[v] = state_value<SRC>(qe + v * ns);
     }
   }
   // set-up that the own loads' latency covers
@@ -534,7 +558,7 @@ __device__ __forceinline__ void volume_block(int blk, const double* __restrict__
     } else {
       const T* qn = qf + (size_t)enb * state_record(n) + fn;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sn[v] = qn[v * ns];
+      for (int v = 0; v < 5; ++v) sn[v] = state_value<SRC>(qn + v * ns);
     }
     const Prim<T> wn = prim_c(sn, C);
     gradient_vars(sn, wn, C.theta_ref, Un);
@@ -838,6 +862,8 @@ __device__ __forceinline__ void state_row(const double* __restrict__ q, const fl
       row_read64(q + v * C.N + (long long)e * 64 + node, wide, d);
 #pragma unroll
       for (int i = 0; i < 4; ++i) s[v][i] = shifted(d[i], v, C);
+    } else if (SRC == 2) {
+      ld4_l2(qf + (size_t)e * state_record(4) + v * 64 + node, s[v]);
     } else {
       row_read(qf + (size_t)e * state_record(4) + v * 64 + node, s[v]);
     }
@@ -936,9 +962,9 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
       state_from_q(q, (long long)exr * 64 + 4 * r, C, xr);
     } else {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) xl[v] = qf[(size_t)exl * state_record(4) + v * 64 + 4 * r + 3];
+      for (int v = 0; v < 5; ++v) xl[v] = state_value<SRC>(qf + (size_t)exl * state_record(4) + v * 64 + 4 * r + 3);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) xr[v] = qf[(size_t)exr * state_record(4) + v * 64 + 4 * r];
+      for (int v = 0; v < 5; ++v) xr[v] = state_value<SRC>(qf + (size_t)exr * state_record(4) + v * 64 + 4 * r);
     }
     float hU[4][4];
 #pragma unroll
@@ -1199,17 +1225,21 @@ __device__ __forceinline__ void volume_phase(int blk, const double* __restrict__
 }
 
 // BESIDE: launched after the forcing network of the same stage state, to run beside it on the
-// SMs it leaves idle.  That launch released this one after its own wait, so the stage state
-// was complete then; only its lines in this SM's L1 can be old, and the fence drops them.
-// The wait for the network comes last: the next launch waits for this one only.
+// SMs it leaves idle.  The network releases this launch after its own wait, so the stage state
+// was complete, and at the L2, before any block here starts.  This launch has waited for
+// nothing itself, and this SM's L1 may hold lines of the former contents: the fence pairs with the
+// network's ahead of its release, and the state is read past the L1, by loads the compiler can
+// neither move above the fence nor take for read-only.  Everything else read here is a kernel
+// parameter.  The wait for the network comes last: the next launch, which waits for this one
+// only, must be one that waits before it touches memory (phase B).
 template <int P, typename T, int SRC, bool CUBE = false, bool FEAT = false, bool SPLIT = false, bool BESIDE = false>
 __global__ void __launch_bounds__(volume_max_threads<P, T, SPLIT>(), volume_min_blocks<P, T, SPLIT>())
-k_volume(const double* __restrict__ q, T* __restrict__ qf, T* __restrict__ rv, T* __restrict__ vt,
-         const OpConst<T> C) {
+k_volume(const double* __restrict__ q, T* qf, T* __restrict__ rv, T* __restrict__ vt, const OpConst<T> C) {
+  static_assert(!BESIDE || SRC == 1, "beside the network the stage state exists");
   if (BESIDE) asm volatile("fence.acq_rel.gpu;" ::: "memory");
   else pdl_wait();
   if (C.early) pdl_release();
-  volume_phase<P, T, SRC, CUBE, FEAT, SPLIT>(blockIdx.x, q, qf, rv, vt, C);
+  volume_phase<P, T, BESIDE ? 2 : SRC, CUBE, FEAT, SPLIT>(blockIdx.x, q, qf, rv, vt, C);
   pdl_release();
   if (BESIDE) pdl_wait();
 }

@@ -224,3 +224,34 @@ def test_meshes_of_one_element_per_sm_take_the_same_time(dg, P, prec):
             dg.dg_destroy(ctx)
     small, large = us(4), us(5)
     assert large <= 1.12 * small, (small, large)
+
+
+@pytest.mark.parametrize("K,split,width,hidden", [(16, 0, 512, 4), (13, 0, 256, 3), (10, 1, 256, 4), (6, 0, 128, 2)])
+def test_phase_a_beside_the_network_equals_phase_a_before_it(dg, K, split, width, hidden):
+    """Phase A reads the stage state while the network runs.  A network whose max_batch takes the
+    elements in two parts goes after phase A, which then waits as usual; its clusters are the
+    same, so every bit must be.  Many steps on changing states: a stale line is a wrong state."""
+    from paper_2207_11571_gb300 import nn
+    N, feat = K ** 3 * 64, 320
+    dims = [feat] + [width] * hidden + [feat]
+    ctx = dg.dg_create(K, 3, 400.0, 0.1, 0.71, 1, precision=1, volume_flux=split)
+    draws = inputs.uniform_draws(dims, 5)
+    nets = [nn.nn_create(feat, feat, width, hidden, 0, 5, rows, draws) for rows in (K ** 3, (K ** 3 + 1) // 2)]
+    try:
+        for net in nets:
+            nn.nn_set_scalers(net, *[v * torch.ones(feat).numpy() for v in (0.0, 1.0, 0.0, 1e-4)])
+        q = state(dg, ctx, N)
+        dt = dg.dg_stable_dt(ctx, q, 0.4)
+        beside, before, R, Rb = q.clone(), q.clone(), torch.empty_like(q), torch.empty_like(q)
+        for steps in (1, 4, 2, 3, 1, 1, 5):
+            dg.dg_rk3_step(ctx, beside, dt, steps, nets[0])
+            dg.dg_rhs(ctx, beside, R, nets[0])
+            dg.dg_rk3_step(ctx, before, dt, steps, nets[1])
+            dg.dg_rhs(ctx, before, Rb, nets[1])
+            torch.cuda.synchronize()
+            assert torch.isfinite(before).all()
+            assert torch.equal(beside, before) and torch.equal(R, Rb)
+    finally:
+        for net in nets:
+            nn.nn_destroy(net)
+        dg.dg_destroy(ctx)
