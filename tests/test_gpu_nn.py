@@ -609,3 +609,35 @@ def test_gradients_at_odd_sizes_match_oracle(L, n_in, width, nh, first, nv, rows
                 assert rel(db, grads[l][1]) < NN_RTOL, l
     finally:
         nn.nn_destroy(h)
+
+
+@pytest.mark.parametrize("n_in,width,nh,rows", [(320, 512, 4, 1024), (192, 256, 7, 300), (320, 64, 2, 33)])
+def test_training_steps_in_a_row_equal_steps_apart(L, n_in, width, nh, rows):
+    """The launches of a step and of the next overlap: a launch starts before the ones ahead of it
+    have ended.  Many steps in a row give the bits of the same steps with the GPU idle between
+    them, so nothing is read before its writer is done."""
+    from paper_2207_11571_gb300 import nn
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    X = torch.randn((rows, n_in), generator=g, device="cuda")
+    Y = torch.randn((rows, n_in), generator=g, device="cuda")
+    first, nv = (0, 5) if n_in == 320 else (1, 3)
+    nets = [make_net(nn, n_in, width, nh, 3, max_batch=rows, first_var=first, n_vars=nv)[0] for _ in range(2)]
+    try:
+        for _ in range(3):
+            for _ in range(12):
+                nn.nn_train_step(nets[0], X, Y, lr=1e-3, want_loss=False)
+            for _ in range(12):
+                nn.nn_train_step(nets[1], X, Y, lr=1e-3, want_loss=False)
+                torch.cuda.synchronize()
+            S = [torch.empty_like(Y) for _ in nets]
+            for net, s in zip(nets, S):
+                nn.nn_forward(net, X, s)
+            torch.cuda.synchronize()
+            assert torch.isfinite(S[0]).all() and torch.equal(S[0], S[1])
+            for layer in range(nh + 1):
+                for a, b in zip(nn.nn_get_params(nets[0], layer), nn.nn_get_params(nets[1], layer)):
+                    assert np.array_equal(a, b)
+    finally:
+        for net in nets:
+            nn.nn_destroy(net)
