@@ -192,7 +192,7 @@ k_diag_partial(const double* __restrict__ q, const double* __restrict__ R, const
     sW[t] = ng.w[i] * ng.w[j] * ng.w[k] * jac;
   }
   __syncthreads();
-  const float gf = (float)gamma;
+  const float gg = (float)(gamma * (gamma - 1.0));   // rounded once: gamma may be near 1
   float m32 = 0.f;             // this thread's largest FP32 estimate of a wave speed
   long long m_at = -1;         // its node
   int bad = 0;
@@ -233,10 +233,11 @@ k_diag_partial(const double* __restrict__ q, const double* __restrict__ R, const
     const float r = d2f_rn(qv[0]), e = d2f_rn(qv[4]);
     const float mx = d2f_rn(qv[1]), my = d2f_rn(qv[2]), mz = d2f_rn(qv[3]);
     const float irf = 1.f / r;
-    const float v2f = (mx * mx + my * my + mz * mz) * irf * irf;
-    const float pe = e - 0.5f * r * v2f;   // p / (gamma - 1)
-    const float wf = sqrtf(v2f) + sqrtf(fmaxf(gf * (gf - 1.f) * pe * irf, 0.f));
-    const bool sound32 = pe > 0.25f * fabsf(e) && r > 0.f && wf < 1e30f;
+    const float vx = mx * irf, vy = my * irf, vz = mz * irf;
+    const float pe = e - 0.5f * (mx * vx + my * vy + mz * vz);   // p / (gamma - 1)
+    const float wf = sqrtf(vx * vx + vy * vy + vz * vz) + sqrtf(fmaxf(gg * pe * irf, 0.f));
+    // the bounds on r and wf: what FP32 flushes to zero is below 1e-6 of the estimate
+    const bool sound32 = pe > 0.25f * fabsf(e) && r > 1e-20f && wf > 1e-3f && wf < 1e18f;
     const bool tie = wf >= m32 * (1.f - 1e-5f) && wf <= m32 * (1.f + 1e-5f);
     if (sound32) {
       const unsigned act = __activemask(), top = __reduce_max_sync(act, __float_as_uint(wf));

@@ -342,6 +342,30 @@ def test_max_wave_screen_keeps_the_fp64_maximum(dg, case):
     assert d["max_wave"] == pytest.approx(ref, rel=1e-15, abs=0), (d["max_wave"], ref)
 
 
+@pytest.mark.parametrize("gamma,scale", [(1.0005, 1.0), (1.002, 1.0), (1.4, 1.0), (1.0005, 1e-18), (1.4, 1e-21)])
+def test_max_wave_screen_near_gamma_one_and_at_small_scales(dg, gamma, scale):
+    """One node whose wave speed is all sound exceeds one (of the same thread block) that is nearly
+    all velocity by 1e-6.  An
+    FP32 estimate with gamma rounded before 1 is subtracted is off by 6e-5 in the sound alone at
+    gamma 1.0005, and one that squares momenta loses them where density and momentum are
+    small: either ranks the nodes wrongly."""
+    import numpy as np
+    gammas = gamma + np.arange(0, 2000) * 1e-9   # one that FP32 rounds down
+    gamma = float(gammas[np.argmin((np.float32(gammas).astype(float) - 1.0) / (gammas - 1.0))])
+    c = Ctx(dg, 6, 3, gamma=gamma)
+    N = c.N
+    q = torch.zeros(5, N, dtype=torch.float64, device="cuda")
+    q[0], q[4] = 1.0, 1e-3 / (gamma * (gamma - 1.0))          # at rest, c about 0.03
+    v, pe = 1.0, 0.5 / 0.7 * 0.3                              # 30 % of rho e is internal
+    w = v + (gamma * (gamma - 1.0) * pe) ** 0.5
+    q[1, 7], q[4, 7] = v, 0.5 * v * v + pe
+    q[4, 70] = (w * (1.0 + 1e-6)) ** 2 / (gamma * (gamma - 1.0))
+    q *= scale
+    d = dg.dg_diagnostics(c.h, q.view(-1))
+    ref = _max_wave_brute(q.view(-1), N, gamma)
+    assert d["max_wave"] == pytest.approx(ref, rel=1e-15, abs=0), (d["max_wave"] / ref - 1.0, gamma)
+
+
 def test_diagnostics_flag_nonfinite_state(dg):
     c = Ctx(dg, 2, 3)
     q, _ = c.tgv()
