@@ -586,6 +586,9 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
   if (e == cudaSuccess) e = cudaMalloc(&c->err_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(c->err_dev, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->s_buf, 5 * c->N * sizeof(float));
+  // the memsets and table copies above run on the legacy stream, which the caller's
+  // (non-blocking) streams do not wait for: the diagnostics' ticket must be zero before the first call
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     dg_destroy(c);
     return cuda_fail(e, "dg_create: workspace allocation");
