@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "dg_aux.h"
-#include "dg_bulk.cuh"
+#include "dg_barrier.cuh"
 #include "dg_kernels.cuh"
 #include "nn_bridge.h"
 #include "tc_common.cuh"
@@ -911,34 +911,40 @@ extern "C" int dg_set_forcing_mode(dg_ctx* c, int mode) {
 }
 
 namespace dgnn {
-// Two bounded waits on mbarriers that never complete (no arrivals): out[0] from the
-// bulk-copy wait, out[1] from the tensor-core wait; 1 = reported completion.
-__global__ void k_wait_selfcheck(int* out) {
-  __shared__ unsigned long long bars[2];
-  if (threadIdx.x == 0) {
-    bulk_bar_init(&bars[0]);
-    bulk_bar_init(&bars[1]);
-    bulk_bar_fence_init();
+// Two bounded waits that nothing completes: block 0 in the persistent kernel's grid barrier,
+// which expects one block more than arrives, block 1 in the tensor-core kernels' mbarrier wait.
+// out[block]: 1 = reported completion.
+__global__ void k_wait_selfcheck(unsigned* bar, int* out) {
+  __shared__ uint64_t mbar;
+  bool done;
+  if (blockIdx.x == 0) {
+    done = grid_barrier_bounded(bar, 2);
+  } else {
+    if (threadIdx.x == 0) {
+      tc::mbar_init(&mbar, 1);
+      tc::mbar_fence_init();
+    }
+    __syncthreads();
+    done = tc::mbar_wait(&mbar, 0);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) out[0] = bulk_wait(&bars[0], 0u) ? 1 : 0;
-  if (threadIdx.x == 32) out[1] = tc::mbar_wait(reinterpret_cast<uint64_t*>(&bars[1]), 0u) ? 1 : 0;
+  if (threadIdx.x == 0) out[blockIdx.x] = done ? 1 : 0;
 }
 }  // namespace dgnn
 
 extern "C" int dg_check_bounded_waits(double* seconds, void* stream) {
   using namespace dgnn;
   cudaStream_t st = (cudaStream_t)stream;
-  int* d = nullptr;
-  DG_CUDA(cudaMalloc(&d, 2 * sizeof(int)));
+  int* d = nullptr;   // the two results, then the barrier's counters
+  DG_CUDA(cudaMalloc(&d, 4 * sizeof(int)));
   int h[2] = {-1, -1};
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e == cudaSuccess) e = cudaMemsetAsync(d, 0xFF, 2 * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d + 2, 0, 2 * sizeof(int), st);
   if (e == cudaSuccess) e = cudaEventRecord(a, st);
   if (e == cudaSuccess) {
-    k_wait_selfcheck<<<1, 64, 0, st>>>(d);
+    k_wait_selfcheck<<<2, 64, 0, st>>>(reinterpret_cast<unsigned*>(d + 2), d);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaEventRecord(b, st);

@@ -11,6 +11,7 @@
 // flag and returns.  The launches of a step form one CUDA graph, after a reset of the
 // barrier's counter.
 #include "dg_aux.h"
+#include "dg_barrier.cuh"
 #include "dg_launch.cuh"
 
 namespace dgnn {
@@ -26,35 +27,6 @@ struct PersistTable {
   int P[kMaxBatch];
   unsigned* bar;          // [0] arrivals at the barrier, [1] its generation
 };
-
-// Bounded grid barrier: every block's thread 0 counts its arrival; the last to arrive
-// resets the count and advances the generation, the others wait for the new generation.
-// Writes before the barrier are visible after it (fences around the count).  Returns
-// false in every thread of a block whose wait expired.
-__device__ __forceinline__ bool grid_barrier_bounded(unsigned* bar) {
-  __syncthreads();
-  int expired = 0;
-  if (threadIdx.x == 0) {
-    volatile unsigned* gen = bar + 1;
-    const unsigned g = *gen;
-    __threadfence();
-    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*gen == g) {
-        if (clock64() - t0 > 2000000000LL) {
-          expired = 1;
-          break;
-        }
-      }
-    }
-    __threadfence();
-  }
-  return __syncthreads_or(expired) == 0;
-}
 
 template <int SRC, int MODE>
 __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const __grid_constant__ PersistTable pt) {
@@ -73,7 +45,7 @@ __global__ void __launch_bounds__(kPersistThreads, 2) k_batch_persistent(const _
     }
     __syncthreads();   // the next item reuses the shared memory
   }
-  if (!grid_barrier_bounded(pt.bar)) {
+  if (!grid_barrier_bounded(pt.bar, gridDim.x)) {
     if (threadIdx.x == 0 && tb.err[0]) atomicExch(tb.err[0], 1);
     return;
   }

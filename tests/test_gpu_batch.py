@@ -258,3 +258,22 @@ def test_a_small_persistent_batch_uses_the_chip(dg):
         finally:
             dg.dg_batch_destroy(b)
     assert us(3) <= 1.05 * us(4)
+
+
+def test_the_persistent_barrier_gives_up_and_batches_run_on(dg):
+    """The self-check holds a block in the persistent kernel's grid barrier for one that never
+    arrives: it gives up within its limit, and a persistent batch runs afterwards."""
+    secs = dg.dg_check_bounded_waits()
+    assert 0.2 < secs < 3.0, secs   # the two waits side by side, each about a second
+    members = [(3, 3, 200.0, 0.1, 0.71, 0), (2, 5, 200.0, 0.1, 0.71, 0)]
+    b = dg.dg_create_batch(members, precision=1)
+    try:
+        qs = init_states(dg, b, members)
+        ref = alone(dg, b, qs, [1e-3, 1e-3], 2)
+        dg.dg_batch_rk3_step(b, qs, [1e-3, 1e-3], 2, flags=dg.DG_BATCH_PERSISTENT)
+        torch.cuda.synchronize()
+        for i, (q, r) in enumerate(zip(qs, ref)):
+            assert (q - r).abs().max().item() <= 1e-12 * r.abs().max().item()
+            dg.dg_diagnostics(dg.dg_batch_member(b, i), q)   # the error flag is clear
+    finally:
+        dg.dg_batch_destroy(b)
