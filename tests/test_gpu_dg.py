@@ -342,6 +342,23 @@ def test_max_wave_screen_keeps_the_fp64_maximum(dg, case):
     assert d["max_wave"] == pytest.approx(ref, rel=1e-15, abs=0), (d["max_wave"], ref)
 
 
+def test_kinetic_energy_keeps_its_digits_at_every_density(dg):
+    """The diagnostics divide by the density through an FP32 reciprocal and one third-order step,
+    and by a division where the density is outside FP32's range.  Uniform states of unit
+    momentum: ke = 1 / (2 rho), within the rounding of the weighted sum (8 nodes)."""
+    c = Ctx(dg, 1, 1)
+    q = torch.zeros(5, c.N, dtype=torch.float64, device="cuda")
+    q[1] = 1.0
+    rng = np.random.default_rng(7)
+    rho = np.concatenate([10.0 ** rng.uniform(-3, 3, 60), 10.0 ** rng.uniform(-60, 60, 60), 2.0 ** np.arange(-150, 151, 25.0),
+                          [1e-37, 1.1754943508222875e-38, 1.17e-38, 3.4028234663852886e38, 3.5e38, 1e37, 1e-300, 1e300, -2.0]])
+    for r in rho:
+        q[0] = r
+        q[4] = 2.0 / abs(r) + 1.0
+        d = dg.dg_diagnostics(c.h, q.view(-1))
+        assert d["ke"] == pytest.approx(0.5 / r, rel=2e-15, abs=0), (r, d["ke"] * 2 * r - 1)
+
+
 @pytest.mark.parametrize("gamma,scale", [(1.0005, 1.0), (1.002, 1.0), (1.4, 1.0), (1.0005, 1e-18), (1.4, 1e-21)])
 def test_max_wave_screen_near_gamma_one_and_at_small_scales(dg, gamma, scale):
     """One node whose wave speed is all sound exceeds one (of the same thread block) that is nearly
