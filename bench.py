@@ -33,6 +33,7 @@ WORKLOAD_NAME = "tgv-re1600-m0.1: 32^3/P3 + 16^3/P6 + 16^3/P8, FP32 operator, FP
 RE, MACH, PR, CFL = 1600.0, 0.1, 0.71, 0.7
 METRIC = "DOF-stage updates/s (TGV 32^3/P3, 16^3/P6, 16^3/P8 per RK3 step)"
 UNIT = "DOF-stage updates/s"
+PROFILE_STEPS = 3   # of dg_profile_rk3 per mesh
 # Algorithmic floor of one DOF-stage update: read the FP64 state (5 x 8 B), read and write
 # the FP64 RK register (2 x 5 x 8 B), write the state (5 x 8 B)
 FLOOR_BYTES = 160.0
@@ -601,7 +602,7 @@ def run_ours(args, rank, ws):
     # per-kernel device times (CUDA events around each launch, on the launching stream)
     prof = []
     for (K, P), c, q, dt in zip(WORKLOAD, ctxs, states, dts):
-        p = dg.dg_profile_rk3(c, q, dt, 3, stream)
+        p = dg.dg_profile_rk3(c, q, dt, PROFILE_STEPS, stream)
         p["workload"] = f"{K}^3/P{P}"
         prof.append(p)
     total_ms = sum(p["ms_gradient"] + p["ms_flux"] for p in prof)
@@ -629,11 +630,12 @@ def run_ours(args, rank, ws):
                 "traffic": sum(traffics) if all(t is not None for t in traffics) else None,
                 "per_mesh": {m: round(v["frac"], 4) for m, v in per_mesh.items()},
                 "note": "algorithmic floor 160 B per DOF-stage (q read, RK register read + write, q write, "
-                        "FP64); traffic = ncu DRAM bytes of the six launches of one stage, null unless taken "
-                        "on the current kernel sources"}
+                        "FP64); traffic = ncu DRAM bytes of k_volume and k_surface of the three meshes, null "
+                        "unless taken on the current kernel sources"}
     # the implementation's own bytes (stage states, volume terms, face fluxes, FP32 increments: each
     # value read or written once) over the whole timed step and for the dominant kernel
-    step_bytes = sum(3 * (p["flux_bytes_per_launch"] + p["gradient_bytes_per_launch"]) for p in prof)
+    step_bytes = sum(p["flux_bytes_per_launch"] * p["launches_flux"] + p["gradient_bytes_per_launch"] * p["launches_gradient"]
+                     for p in prof) / PROFILE_STEPS
     step_gbs = step_bytes / (ms / args.steps / 1e3) / 1e9
     roofline["implementation"] = {
         "bytes_per_dof_stage": step_bytes / updates_per_step, "achieved": step_gbs, "frac": step_gbs / peak,
@@ -734,17 +736,24 @@ def run_ours(args, rank, ws):
                 "batched": batched,
                 "algorithm1": alg1,
                 "cpu_baseline": cpu, "e2e": e2e,
-                "gpu_launches": 6 * len(WORKLOAD) * args.steps, "clocks": clk}
+                "gpu_launches": sum(step_launches(P) for _, P in WORKLOAD) * args.steps, "clocks": clk}
         print(json.dumps(line), flush=True)
     return 0
 
 
 # ----------------------------------------------------------------------------- batched instances
 
+def step_launches(P):
+    """Launches of one RK3 step of the FP32 operator: two per stage, and at P = 3 the pass that
+    forms the first stage state."""
+    return 7 if P == 3 else 6
+
+
 def step_bytes_per_node(P):
-    """FP32-operator algorithmic bytes per node of one RK3 step (both launches of all
-    stages): 500 of node values and 96 / (P + 1) of face fluxes six times."""
-    return 500.0 + 576.0 / (P + 1)
+    """FP32-operator algorithmic bytes per node of one RK3 step (all launches of all
+    stages): 500 of node values, 20 more where phase A reads the first stage state back
+    (P = 3), and 96 / (P + 1) of face fluxes six times."""
+    return 500.0 + (20.0 if P == 3 else 0.0) + 576.0 / (P + 1)
 
 
 BATCH_NAME = ("12 independent TGV instances, (K, P, Re) drawn with seed 12 from {8,12,16} x {3,6} x "
@@ -837,7 +846,7 @@ def batched_measure(args, rank, ws, steps, with_clocks=False):
     floor = FLOOR_BYTES * value / ws / 1e9
     step_bytes = sum(step_bytes_per_node(P) * n for (_, P, _), n in zip(members, nodes))
     impl = step_bytes * steps / (ms / 1e3) / 1e9
-    groups = len({P for _, P, _ in members})
+    launches = sum(step_launches(P) for P in {P for _, P, _ in members})
     dg.dg_batch_destroy(b)
     return {"value": value, "unit": UNIT, "ms_per_step": ms / steps, "steps": steps, "clocks": clk,
             "members": [f"{K}^3/P{P}/Re{int(Re)}" for K, P, Re in members], "nodes": sum(nodes),
@@ -848,7 +857,7 @@ def batched_measure(args, rank, ws, steps, with_clocks=False):
                          "kernel": "whole batched step (all launches)", "traffic": None,
                          "implementation": {"bytes_per_dof_stage": step_bytes / (3 * sum(nodes)), "achieved": impl,
                                             "frac": impl / peak}},
-            "e2e": e2e, "gpu_launches": 6 * groups * steps}
+            "e2e": e2e, "gpu_launches": launches * steps}
 
 
 def run_batched(args, rank, ws):

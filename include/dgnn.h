@@ -268,12 +268,12 @@ int dg_make_pairs(const dg_ctx* lo, const double* q_bar_n, const double* q_nn_np
                   float* X, float* Y, void* stream);
 
 /* Measurement: advances q like dg_rk3_step (nsteps RK3 steps, no forcing) while
- * recording CUDA events on `stream` around every kernel launch.  Returns the summed
- * device time in milliseconds of the phase-A (BR1 gradient) and phase-B (flux, lift,
- * RK update) kernels, the number of launches of each, and the algorithmic bytes one
- * launch of each phase moves, averaged over the three RK stages (state, stage state,
- * stresses and RK increment: each value read or written once; neighbour reads not
- * counted).  All outputs are HOST pointers; any may be NULL.  Synchronises. */
+ * recording CUDA events on `stream` around every phase.  Returns the summed
+ * device time in milliseconds of the phase-A (gradient and volume term; at P = 3 in FP32
+ * with the pass that forms the first stage state) and phase-B (interface, RK update)
+ * kernels, the number of launches of each, and the algorithmic bytes one launch of each
+ * phase moves on average (state, stage state, volume term, face fluxes and RK increment:
+ * each value read or written once; neighbour reads not counted).  All outputs are HOST pointers; any may be NULL.  Synchronises. */
 int dg_profile_rk3(dg_ctx* ctx, double* q, double dt, int nsteps, double* ms_gradient,
                    double* ms_flux, int* launches_gradient, int* launches_flux,
                    double* flux_bytes_per_launch, double* gradient_bytes_per_launch,

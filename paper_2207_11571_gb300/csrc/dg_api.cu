@@ -76,12 +76,19 @@ static int stage_mode(const dg_ctx* c, int k, bool more) {
   return k == 2 && more ? 5 : 2 + k;
 }
 
-// Algorithmic bytes per node of the phase-A and phase-B launches of stage k: every value
-// the kernel must read or write once (neighbour interface reads are L2 hits, not counted).
+// Whether phase A of stage 1 is two launches: the stage state in a pass of its own first.
+static bool state_pass(const dg_ctx* c) {
+  return use_rows4(c->P, c->opts.precision == DG_PREC_FP32 ? 4 : 8, c->geom.split != 0);
+}
+
+// Algorithmic bytes per node of the phase-A (the state pass with it) and phase-B launches of
+// stage k of a step on its own: every value a kernel must read or write once (neighbour
+// interface reads are L2 hits, not counted).
 static void stage_bytes(const dg_ctx* c, int k, double* grad, double* flux) {
   const bool f32 = c->opts.precision == DG_PREC_FP32;
   const double T = f32 ? 4 : 8, face = 24.0 * T / c->n;   // four viscous values on six faces
   *grad = (f32 && k > 0 ? 5 * T : 40 + 5 * T) + 5 * T + face;
+  if (k == 0 && state_pass(c)) *grad += 5 * T;   // read back by phase A
   *flux = 10 * T + face;
   if (!f32) *flux += 40 + (k ? 40 : 0) + 80;
   else *flux += k == 0 ? 10 * T : k == 1 ? 20 * T : 5 * T + 80;
@@ -833,10 +840,11 @@ int dg_profile_rk3(dg_ctx* c, double* q, double dt, int nsteps, double* ms_gradi
   if (e != cudaSuccess) return cuda_fail(e, "dg_profile_rk3");
   if (ms_gradient) *ms_gradient = tg;
   if (ms_flux) *ms_flux = tf;
-  if (launches_gradient) *launches_gradient = nl;
+  const int ng = nl + (state_pass(c) ? nsteps : 0);
+  if (launches_gradient) *launches_gradient = ng;
   if (launches_flux) *launches_flux = nl;
   if (flux_bytes) *flux_bytes = bf / nl * (double)c->N;
-  if (grad_bytes) *grad_bytes = bg / nl * (double)c->N;
+  if (grad_bytes) *grad_bytes = bg / ng * (double)c->N;
   return DG_OK;
 }
 

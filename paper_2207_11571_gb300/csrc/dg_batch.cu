@@ -3,8 +3,8 @@
 // Each member is an ordinary context (its own mesh, flow, closure and workspace).  A
 // batched RK3 step groups the members by order P: every group runs one phase-A and one
 // phase-B launch per stage covering all of its members' element blocks (k_volume_batch,
-// k_surface_batch), so twelve small meshes cost six launches per step per order instead of
-// six per mesh.  Groups of different orders do not depend on each other and run as
+// k_surface_batch), so twelve small meshes cost six launches per step per order (seven at P = 3
+// in FP32, whose first stage state has a pass of its own) instead of as many per mesh.  Groups of different orders do not depend on each other and run as
 // parallel branches.  The whole step is recorded once into a CUDA graph on private
 // streams and replayed on the caller's stream; it is recorded again when the member
 // states, step sizes or elements-per-block change.

@@ -342,6 +342,21 @@ def test_max_wave_screen_keeps_the_fp64_maximum(dg, case):
     assert d["max_wave"] == pytest.approx(ref, rel=1e-15, abs=0), (d["max_wave"], ref)
 
 
+@pytest.mark.parametrize("K,P,split,prec", [(4, 3, 0, 1), (4, 3, 1, 1), (4, 3, 0, 0), (3, 2, 0, 1), (2, 6, 0, 1)])
+def test_profile_counts_every_launch_and_its_bytes(dg, K, P, split, prec):
+    """Two launches per stage; at P = 3 in FP32 the first stage state has a pass of its own, which
+    writes 20 bytes per node that phase A reads back."""
+    c = Ctx(dg, K, P, precision=prec, volume_flux=split)
+    q, _ = c.tgv()
+    p = dg.dg_profile_rk3(c.h, q, 1e-4, 2)
+    own_pass = P == 3 and prec == 1 and split == 0
+    assert (p["launches_gradient"], p["launches_flux"]) == (8 if own_pass else 6, 6)
+    if prec == 1:
+        per_node = (p["gradient_bytes_per_launch"] * p["launches_gradient"]
+                    + p["flux_bytes_per_launch"] * p["launches_flux"]) / (2 * c.N)
+        assert per_node == pytest.approx(500 + (20 if own_pass else 0) + 576 / (P + 1), rel=1e-12)
+
+
 def test_kinetic_energy_keeps_its_digits_at_every_density(dg):
     """The diagnostics divide by the density through an FP32 reciprocal and one third-order step,
     and by a division where the density is outside FP32's range.  Uniform states of unit
