@@ -12,7 +12,9 @@ namespace dgnn {
 
 constexpr int kMaxP = 8;
 constexpr int kMaxN1 = kMaxP + 1;
-constexpr int kSMs = 152;   // of a GB300
+// SMs of a GB300: the size rules of the launches go by it (the order of some sums does too, so it
+// is not asked of the device)
+constexpr int kSMs = 152;
 
 // Element-major workspace records (dg_kernels.cuh), n = P + 1: node stride of a component,
 // and sizes of the state and face records in values.

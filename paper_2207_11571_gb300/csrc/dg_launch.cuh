@@ -20,7 +20,7 @@ inline int owned_elems(const dg_ctx* c) { return c->e_end - c->e_begin; }
 // both phases, and the launch latency saved counts there: 10^3/P3 32.0 -> 29.1, 8^3/P2 23.7 -> 22.3.
 template <typename T>
 bool release_early(int P, long long nodes) {
-  return std::is_same<T, float>::value && P <= 3 && nodes <= 152 * 512;
+  return std::is_same<T, float>::value && P <= 3 && nodes <= kSMs * 512;
 }
 
 template <typename T>
@@ -235,7 +235,7 @@ auto with_surf_block(int n, F f) {
     if constexpr (P == 2) return f(Int<4>{}, Int<192>{});
   }
   if constexpr (P == 3 && std::is_same<T, float>::value) {
-    constexpr int kWave = 152 * 1024;   // threads
+    constexpr int kWave = kSMs * 1024;   // threads
     if (n <= kWave / 192 * 2) return f(Int<2>{}, Int<192>{});
     if (n <= kWave / 96 * 2) return f(Int<2>{}, Int<96>{});
     if (n <= kWave / 128 * 4) return f(Int<4>{}, Int<128>{});
@@ -255,7 +255,7 @@ cudaError_t surface_p(const dg_ctx* c, double* q, double* dqdt, const Forcing& f
   // as per side.  us per RK3 step, P = 3, cubes / rows: 8^3 164 / 130, 12^3 365 / 360, 16^3
   // 770 / 811.
   if constexpr (surf_cube(P, sizeof(T))) {
-    if (!c->part && c->K % 2 == 0 && n >= 2 * 152 * kCubeElems)
+    if (!c->part && c->K % 2 == 0 && n >= 2 * kSMs * kCubeElems)
       return surface_launch<P, T, MODE, kCubeElems, surf_threads_cube(P), true>(c, q, dqdt, f, rk, st);
   }
   return with_surf_block<P, T>(n, [&](auto E, auto threads) {

@@ -587,11 +587,11 @@ int launch_gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb
   return DG_OK;
 }
 
-// Tile width: enough CTAs to cover the 152 SMs when possible, wider tiles otherwise.
+// Tile width: enough CTAs to cover the SMs when possible, wider tiles otherwise.
 int pick_bn(int M, int N) {
   const int mt = (M + kBM - 1) / kBM;
-  if (N > 128 && mt * ((N + 255) / 256) >= 152) return 256;
-  if (N > 64 && mt * ((N + 127) / 128) >= 152) return 128;
+  if (N > 128 && mt * ((N + 255) / 256) >= kSMs) return 256;
+  if (N > 64 && mt * ((N + 127) / 128) >= kSMs) return 128;
   return 64;
 }
 
@@ -664,7 +664,7 @@ int input_gradient(const __nv_bfloat16* dy, int ldy, const __nv_bfloat16* W, int
 // other way moves the next step's gradients by up to half a percent.)
 int grad_splits(int M, int N, int rows) {
   const int bn = pick_bn(M, N), tiles = ((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
-  return std::max(1, std::min({kMaxSplits, (rows + kBK - 1) / kBK, 152 / tiles}));
+  return std::max(1, std::min({kMaxSplits, (rows + kBK - 1) / kBK, kSMs / tiles}));
 }
 
 int weight_gradients(const GradLayer* layers, int L, int rows, float* out, long long split_stride, int* err_flag,
