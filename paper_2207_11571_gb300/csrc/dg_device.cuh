@@ -1,6 +1,6 @@
-// Device-side physics of the compressible Navier-Stokes operator (Appendix A) and
-// the interface fluxes of Sec. 3.1 (Roe advective, BR1 viscous), templated on the
-// arithmetic type T (float: FP32 operator, double: FP64 parity operator).
+// Device-side physics of the compressible Navier-Stokes operator (Appendix A), templated
+// on the arithmetic type T (float: FP32 operator, double: FP64 parity operator).  The
+// interface fluxes of Sec. 3.1 are face_terms in dg_kernels.cuh.
 //
 // States are reference-shifted: s = (r, m1, m2, m3, e) with r = rho - rho_ref and
 // e = rho e - E_ref (Phys); with zero references these are the conserved variables.

@@ -32,9 +32,9 @@
 // of elements whose twelve internal faces need no halo), one thread per node (P = 3 in FP32:
 // per row of four).  Phase B: a block owns a few elements, the more the larger the mesh; its
 // interface terms are dense work items, one per (element, face, face node), so that every
-// lane does useful Roe work, and its nodes add the lifted results in a fixed order.  All constants arrive in the operator precision
-// (OpConst): no FP64 arithmetic or conversion runs per node except where the FP64 state
-// is read or written.
+// lane does useful Roe work, and its nodes add the lifted results in a fixed order.  All
+// constants arrive in the operator precision (OpConst): in the FP32 operator no FP64
+// arithmetic or conversion runs per node except where the FP64 state is read or written.
 #pragma once
 
 #include <cuda_bf16.h>

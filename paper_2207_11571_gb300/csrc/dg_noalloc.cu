@@ -4,13 +4,14 @@
 // allowed or not wanted -- an in-situ analysis hook inside another solver's time loop
 // whose device memory was budgeted and locked at start-up, or a host thread that must
 // not take the allocator's locks or synchronise the device (cudaMalloc and cudaFree may
-// do both).  dg_create allocates its workspace (stage state, volume term and face fluxes); this entry point instead uses one fixed scratch array that
-// lives in the library's own device image.
+// do both).  dg_create allocates its workspace (stage state, volume term and face fluxes);
+// this entry point instead uses one fixed scratch array that lives in the library's own
+// device image.
 //
 // The scratch array holds the three intermediate fields of one operator evaluation: the
 // stage state and the volume term (5 values per node each) and the viscous fluxes normal to
-// the faces (4 values per face node), at most kNoallocMaxNodes nodes.  Every GPU that loads the library keeps it
-// (5.8 MB) until the process exits.  All calls on a device share it and it keeps the
+// the faces (4 values per face node), at most kNoallocMaxNodes nodes.  Every GPU that loads
+// the library keeps it (5.8 MB) until the process exits.  All calls on a device share it and it keeps the
 // last call's contents; nothing in it needs to start at zero, because the first kernel
 // of every call writes every entry it later reads.  Calls whose work overlaps on the GPU
 // (different streams, or different host threads) race on the array: serialise them.

@@ -644,7 +644,7 @@ void adam_step(nn_model* m, const nn_adam& a, ParamTable* tb) {
 // scaling, a product per layer forward (the last with the loss), one per layer but the first
 // backward, every layer's weight gradient, the reduction and update.  What is element-wise
 // is an epilogue, and the products read activations, gradients and weights as they lie.
-// Measured per step: 320-512x4-320 at batch 4096 250 -> 96 us, 192-256x7-192 at 1024 210 -> 75 us;
+// Measured per step: 320-512x4-320 at batch 4096 251 -> 98 us, 192-256x7-192 at 1024 211 -> 78 us;
 // a launch of the chain takes 4 us at batch 128 and 6 us at 4096 x 512 x 512.
 int train(nn_model* m, const float* X, const float* Y, const int64_t* idx, int batch, int norm_batch,
           const nn_adam* adam, cudaStream_t st) {

@@ -70,9 +70,9 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
-// One lane of a converged warp.  tcgen05 and TMA instructions take their operands from
-// uniform registers; behind an elected lane the compiler knows that one thread runs them,
-// behind a test of the lane number it wraps each in a loop over the warp's values.
+// One lane of a converged warp, for the threads that issue tcgen05 and TMA instructions.
+// Against a test of the lane number: corrected 16^3/P3 step 147 -> 141.8 us, training step of
+// 320-512x4-320 at batch 4096 100.5 -> 95.2.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
