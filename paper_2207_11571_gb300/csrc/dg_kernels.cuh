@@ -1144,14 +1144,11 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       if (d == 0) {
-        // the energy flux relative to the row's first node: D annihilates constants, and the
-        // large common part at low Mach numbers stays out of the rounding
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float g = 0.f;
 #pragma unroll
-          for (int m = c == 4 ? 1 : 0; m < 4; ++m)
-            g = fma_(C.D[4 * i + m], c == 4 ? add_(F[4][m], -F[4][0]) : F[c][m], g);
+          for (int m = 0; m < 4; ++m) g = fma_(C.D[4 * i + m], F[c][m], g);
           R[c][i] = mul_(-C.s2h, g);
         }
       } else {
@@ -1161,37 +1158,19 @@ __device__ __forceinline__ void volume4_block(int blk, const double* __restrict_
   }
   __syncwarp(half);
   // Each line is summed before it is scaled and added: D's large entries make every partial
-  // sum several times the derivative, and R must not be rounded at that size.  The energy
-  // flux goes relative to the own row, as along x.
+  // sum several times the derivative, and R must not be rounded at that size.
   float* re = rv + (size_t)e * state_record(4) + 4 * r;
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     const float* fy = sF + c * 64;
     const float* fz = fy + 5 * 64;
-    const Row y0 = row_load(fy + 4 * r), z0 = row_load(fz + 4 * r);
-    if (c == 4) {
-      Row acc{0ull, 0ull};
+    float g[4];
+    rows_contract(row_load(fy + 4 * r), fy, yat, Dy, g);
 #pragma unroll
-      for (int m = 1; m < 4; ++m) {
-        const Row y = row_load(fy + yat[m - 1]), z = row_load(fz + zat[m - 1]);
-        fma2(acc.lo, Dy[m], line_sub(y.lo, y0.lo));
-        fma2(acc.hi, Dy[m], line_sub(y.hi, y0.hi));
-        fma2(acc.lo, Dz[m], line_sub(z.lo, z0.lo));
-        fma2(acc.hi, Dz[m], line_sub(z.hi, z0.hi));
-      }
-      float g[4];
-      row_unpack(acc, g);
+    for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
+    rows_contract(row_load(fz + 4 * r), fz, zat, Dz, g);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
-    } else {
-      float g[4];
-      rows_contract(y0, fy, yat, Dy, g);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
-      rows_contract(z0, fz, zat, Dz, g);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
-    }
+    for (int i = 0; i < 4; ++i) R[c][i] = fma_(-C.s2h, g[i], R[c][i]);
     row_store(re + c * 64, R[c]);
   }
 }

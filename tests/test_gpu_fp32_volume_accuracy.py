@@ -20,6 +20,8 @@ PLAIN_LINES = {
     (16, 1, 1600.0): (4.687e-08, 6.910e-07, 6.956e-07, 3.659e-08, 2.912e-05),
     (16, 2, 1600.0): (1.610e-07, 1.683e-06, 1.704e-06, 1.067e-07, 8.823e-05),
     (12, 4, 1600.0): (3.546e-07, 3.242e-06, 3.223e-06, 2.224e-07, 1.830e-04),
+    (3, 3, 1600.0): (5.832e-08, 5.190e-07, 5.714e-07, 3.706e-08, 3.059e-05),
+    (3, 3, 30.0): (5.832e-08, 5.304e-07, 5.791e-07, 3.723e-08, 3.044e-05),
     (16, 3, 1600.0): (2.883e-07, 2.951e-06, 2.952e-06, 1.936e-07, 1.609e-04),
     (8, 3, 30.0): (1.489e-07, 1.560e-06, 1.572e-06, 1.056e-07, 8.185e-05),
     (7, 3, 200.0): (1.290e-07, 1.282e-06, 1.287e-06, 8.647e-08, 7.047e-05),
