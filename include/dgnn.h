@@ -65,7 +65,8 @@ typedef struct {
   double Cs;          /* Smagorinsky constant, default 0.1 */
   double Prt;         /* turbulent Prandtl number, default 0.9 */
   double les_delta;   /* LES filter width; <= 0 selects h/(P+1) (default) */
-  int elems_per_block;/* elements per CUDA block; <= 0 selects the tuned default for P */
+  int elems_per_block;/* elements per block of the gradient and volume phase; <= 0 selects the
+                         tuned default for P */
   int block_shape;    /* blocks of the gradient and volume phase: 0: elems_per_block
                          consecutive elements (default); 1: 2 x 2 x 2 cubes of elements
                          (P <= 3 and even K only, else DG_ERR_INVALID_ARG), whose twelve
