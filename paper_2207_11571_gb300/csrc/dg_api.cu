@@ -50,6 +50,15 @@ int cuda_fail(cudaError_t err, const char* what) {
   return fail(DG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
 }
 
+cudaError_t zero_device(void* p, size_t bytes) {
+  cudaStream_t s = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, bytes, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (s) cudaStreamDestroy(s);
+  return e;
+}
+
 RkStage rk_stage(int k) { return RkStage{kRkA[k], kRkB[k], 1.0 / kRkB[0], kRkB[2] * kRkA[2]}; }
 
 cudaError_t launch_volume(const dg_ctx* c, const double* q, int src, cudaStream_t st) {
@@ -588,14 +597,11 @@ int dg_create_local(int K, int P, double Re, double Mach, double Pr, int closure
   c->cur = c->qf;
   if (e == cudaSuccess) e = cudaMalloc(&c->rhs_tmp, 5 * c->N * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->red, kDiagBytes);
-  if (e == cudaSuccess) e = cudaMemset(c->red, 0, kDiagOut * sizeof(double));
+  if (e == cudaSuccess) e = zero_device(c->red, kDiagOut * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost(&c->red_host, (kDiagLen + 1) * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->err_dev, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(c->err_dev, 0, sizeof(int));
+  if (e == cudaSuccess) e = zero_device(c->err_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->s_buf, 5 * c->N * sizeof(float));
-  // the memsets and table copies above run on the legacy stream, which the caller's
-  // (non-blocking) streams do not wait for: the diagnostics' ticket must be zero before the first call
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     dg_destroy(c);
     return cuda_fail(e, "dg_create: workspace allocation");

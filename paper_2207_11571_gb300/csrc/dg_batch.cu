@@ -231,8 +231,7 @@ int dg_create_batch(const dg_instance_desc* desc, int n, const dg_opts* opts, dg
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[gi], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->bar, 2 * sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(b->bar, 0, 2 * sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // done before any stream uses it
+  if (e == cudaSuccess) e = zero_device(b->bar, 2 * sizeof(unsigned));
   if (e != cudaSuccess) {
     dg_batch_destroy(b);
     return cuda_fail(e, "dg_create_batch: streams, events and barrier");
